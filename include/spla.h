@@ -207,8 +207,9 @@ int spla_decode_selected(spla_cache_t *cache, const void *q, const float *rms_we
  *   sel_idx:      DEVICE int32 [batch][T][H_kv][top_k] or NULL: the blocks each position selected.
  *   workspace:    DEVICE scratch, 256-byte aligned, of at least the `min_bytes` that spla_query_prefill_workspace
  *                 reports for this T; with more (up to `good_bytes`) more positions are processed per kernel launch.
- * Built on the general kernels (any group size up to 16, fp32 or bf16, d 64 or 128); strided selection windows are not
- * supported (SPLA_ERR_UNSUPPORTED).  Returns SPLA_ERR_CAPACITY, with nothing enqueued, if the chunk does not fit.
+ * bf16 caches and queries with at most 16384 blocks per sequence run on the tensor cores (all positions of a chunk as
+ * contractions); fp32, longer sequences and SPLA_GENERAL_KERNELS take the general kernels, one virtual unit per
+ * position.  Strided selection windows are not supported (SPLA_ERR_UNSUPPORTED).  Returns SPLA_ERR_CAPACITY, with nothing enqueued, if the chunk does not fit.
  */
 int spla_prefill(spla_cache_t *cache, const void *k_new, const void *v_new, const void *q, int32_t T,
                  const float *rms_weight, float *out, int32_t *sel_idx, void *workspace, size_t workspace_bytes,

@@ -1,4 +1,5 @@
-// Prefill- / training-shaped forward: the output of every query position of a chunk of T new tokens.
+// Prefill- / training-shaped forward on the general kernels: the output of every query position of a chunk of T new
+// tokens, for what the tensor-core path (prefill_attend.cu) does not serve: fp32, very long sequences.
 //
 // The paper develops the method on the decode step and says that it carries over to training and prefilling
 // (Section 2, opening; Section 3.3 "Kernel Design": the kernels serve both).  The reading taken: the query at

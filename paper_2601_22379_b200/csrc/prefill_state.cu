@@ -1,0 +1,246 @@
+// Per-position pieces of the tensor-core prefill path that precede the scoring: the log mass of every position's own,
+// growing block, and the recurrent state at the start of every range of SB tokens.
+//
+// Section 3.1 (Eq. taylor-2nd) and Section 3.2 (Eq. rla-impl-1) of the paper, for every prefix that ends inside the
+// chunk.  Nothing here touches more than the chunk's own tokens (and the open block before it).
+#include "prefill_chunk.h"
+#include "umma.cuh"
+
+namespace spla {
+
+namespace {
+
+constexpr int kOwnThreads = 256;
+constexpr int kOwnGroup = 32;              // positions whose prefix statistics are in shared memory together
+
+// One CTA per (block the chunk touches, unit).  D threads walk the block's tokens, one channel each: running sum and
+// running sum of squared deviations (each token's deviation from the mean before and after it: Welford's update, no
+// cancellation), so that the statistics of ALL prefixes of the block cost one pass instead of one pass per prefix.
+// After every 32 tokens the eight warps form the dots of those prefixes with their positions' queries.
+// Bound by that serial chain (16 cycles per token).  64-token blocks, d = 128: 50 us -> 6 us for 144 CTAs against two
+// passes per prefix.
+template <int D>
+__global__ void __launch_bounds__(kOwnThreads) prefill_own_kernel(const Params p, const PrefillChunk pc,
+                                                                  const __nv_bfloat16* __restrict__ q, float* __restrict__ out,
+                                                                  int* __restrict__ sel_user) {
+  constexpr int VEC = D / 32;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* mean_s = reinterpret_cast<float*>(smem_raw);          // [kOwnGroup][D]
+  float* var_s = mean_s + kOwnGroup * D;                       // [kOwnGroup][D]
+  __shared__ float inv_s[128];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const PrefillUnit r = prefill_unit_of(p, pc, blockIdx.y);
+  const int G = p.G;
+  if (r.first < 0 && blockIdx.x == 0) {                        // positions of a refused append: empty prefix, zero output
+    for (int t = 0; t < min(pc.T, -r.first); ++t) {
+      for (int x = tid; x < G * D; x += kOwnThreads) out[(((size_t)r.b * pc.T + t) * p.Hq + (size_t)r.h * G) * D + x] = 0.f;
+      for (int x = tid; x < p.top_k; x += kOwnThreads) {
+        pc.sel[((size_t)r.u * pc.T + t) * p.top_k + x] = -1;
+        if (sel_user) sel_user[(((size_t)r.b * pc.T + t) * p.Hkv + r.h) * p.top_k + x] = -1;
+      }
+    }
+  }
+  const int blk = r.L0 / p.B + blockIdx.x;
+  const int t0 = blk * p.B;
+  if (t0 >= r.L_end) return;                                   // CTA-uniform
+  if ((p.flags & kDebugBounds) && blk >= p.max_blocks) {       // checked build
+    if (tid == 0) atomicExch(p.status, kStatusBounds);
+    return;
+  }
+  const int cnt = min(p.B, r.L_end - t0);
+  if (tid < 128) inv_s[tid] = 1.f / (float)(tid + 1);
+  const __nv_bfloat16* kc = reinterpret_cast<const __nv_bfloat16*>(p.k_cache) + ((size_t)r.u * p.max_blocks * p.B + t0) * D;
+  const bool round16 = (p.flags & kStatsBf16) != 0;
+  float sum = 0.f, m2 = 0.f, mean = 0.f;
+  __syncthreads();
+  for (int g0 = 0; g0 < cnt; g0 += kOwnGroup) {
+    const int ng = min(kOwnGroup, cnt - g0);
+    if (tid < D) {
+      __nv_bfloat16 x[kOwnGroup];
+#pragma unroll
+      for (int j = 0; j < kOwnGroup; ++j) x[j] = j < ng ? kc[(size_t)(g0 + j) * D + tid] : __nv_bfloat16();
+#pragma unroll
+      for (int j = 0; j < kOwnGroup; ++j) {
+        const float v = __bfloat162float(x[j]), inv = inv_s[min(g0 + j, 127)];
+        const float before = v - mean;
+        sum += v;
+        mean = sum * inv;
+        m2 = g0 + j == 0 ? 0.f : fmaf(before, v - mean, m2);
+        float mm = mean, vv = m2 * inv;
+        if (round16) { mm = __bfloat162float(__float2bfloat16_rn(mm)); vv = __bfloat162float(__float2bfloat16_rn(vv)); }
+        mean_s[j * D + tid] = mm;
+        var_s[j * D + tid] = vv;
+      }
+    }
+    __syncthreads();
+    for (int j = warp; j < ng; j += kOwnThreads / 32) {
+      const int pos = t0 + g0 + j;
+      if (pos < r.L0) continue;                                // a token from before the chunk
+      const int t = pos - r.first;
+      float mv[VEC], vv[VEC];
+      load_vec<VEC>(mean_s + j * D + lane * VEC, mv);
+      load_vec<VEC>(var_s + j * D + lane * VEC, vv);
+      const __nv_bfloat16* qp = q + (((size_t)r.b * pc.T + t) * p.Hq + (size_t)r.h * G) * D + lane * VEC;
+      for (int g = 0; g < G; ++g) {
+        float x[VEC], d2[2] = {0.f, 0.f};
+        load_vec<VEC>(qp + (size_t)g * D, x);
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) {
+          const float qh = x[v] * p.sm_scale;
+          d2[0] = fmaf(qh, mv[v], d2[0]);
+          d2[1] = fmaf(0.5f * qh * qh, vv[v], d2[1]);
+        }
+        warp_reduce_multi<2>(d2, lane);                        // lanes 0..15: the mean dot, 16..31: the variance dot
+        const float dv = (p.flags & 2u) ? 0.f : __shfl_sync(0xffffffffu, d2[0], 16);
+        if (lane == 0) pc.ell_own[((size_t)r.u * pc.T + t) * G + g] = logf((float)(g0 + j + 1)) + d2[0] + __logf(1.f + dv);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// What the chunk's tokens of one SB range add to the recurrent state: phi(K)^T V, [d][d] per CTA, warp-level tensor-core
+// products.  phi enters as three bf16 parts (24 significant bits), V exactly; the sums are fp32 over at most 128 tokens.
+// Warp w takes the rows (features) 16 (w % (D / 16)) .. + 15 and its share of the columns.
+template <int D>
+__global__ void __launch_bounds__(256) prefill_local_state_kernel(const Params p, const PrefillChunk pc) {
+  constexpr int PAD = 8;                                       // 16-byte row offset: ldmatrix without bank conflicts
+  constexpr int LD = D + PAD;
+  constexpr int MT = D / 16;                                   // row tiles
+  constexpr int WPM = 8 / MT;                                  // warps per row tile
+  constexpr int NT = D / 8 / WPM;                              // column tiles of a warp
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __nv_bfloat16* phi = reinterpret_cast<__nv_bfloat16*>(smem_raw);    // [3][64][LD]
+  __nv_bfloat16* vs = phi + 3 * 64 * LD;                              // [64][LD]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const PrefillUnit r = prefill_unit_of(p, pc, blockIdx.y);
+  const int start = prefill_range_start(pc, r, blockIdx.x);
+  const int lo = max(start, r.L0), hi = min(start + pc.SB, r.L_end);  // tokens of this range
+  const size_t tok0 = (size_t)r.u * p.max_blocks * p.B;
+  const uint4* kc = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.k_cache) + tok0 * D);
+  const uint4* vc = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.v_cache) + tok0 * D);
+  const float a2 = p.phi_scale * kLog2e;
+  const int mt = warp % MT, wn = warp / MT;
+  const int g = lane >> 2, t = lane & 3, mi = lane >> 3, r8 = lane & 7;
+  float acc[NT][4];
+#pragma unroll
+  for (int n = 0; n < NT; ++n) { acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f; }
+  constexpr int CH = D / 8;                                    // 16-byte chunks per token
+  for (int s0 = start; s0 < hi; s0 += 64) {
+    if (s0 > start) __syncthreads();
+    for (int idx = tid; idx < 64 * CH; idx += 256) {
+      const int row = idx / CH, ch = idx % CH, pos = s0 + row;
+      uint4 kk = make_uint4(0u, 0u, 0u, 0u), vv = kk;
+      float nl2 = -INFINITY;
+      if (pos >= lo && pos < hi) {
+        kk = kc[(size_t)pos * CH + ch];
+        vv = vc[(size_t)pos * CH + ch];
+        nl2 = -p.tok_lse[tok0 + pos] * kLog2e;
+      }
+      const uint32_t w[4] = {kk.x, kk.y, kk.z, kk.w};
+      uint32_t h[4], m[4], l[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float f0 = ex2(fmaf(bf16_lo(w[e]), a2, nl2)), f1 = ex2(fmaf(bf16_hi(w[e]), a2, nl2));
+        h[e] = pack_bf16(f0, f1);
+        const float r0 = f0 - bf16_lo(h[e]), r1 = f1 - bf16_hi(h[e]);
+        m[e] = pack_bf16(r0, r1);
+        l[e] = pack_bf16(r0 - bf16_lo(m[e]), r1 - bf16_hi(m[e]));
+      }
+      *reinterpret_cast<uint4*>(phi + (size_t)row * LD + ch * 8) = make_uint4(h[0], h[1], h[2], h[3]);
+      *reinterpret_cast<uint4*>(phi + (size_t)(64 + row) * LD + ch * 8) = make_uint4(m[0], m[1], m[2], m[3]);
+      *reinterpret_cast<uint4*>(phi + (size_t)(128 + row) * LD + ch * 8) = make_uint4(l[0], l[1], l[2], l[3]);
+      *reinterpret_cast<uint4*>(vs + (size_t)row * LD + ch * 8) = vv;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {                           // 16 tokens per step
+      uint32_t a[3][4];
+#pragma unroll
+      for (int part = 0; part < 3; ++part) {
+        // A[m][k] = phi[token k][feature m]: four transposed 8x8 matrices (m 0-7, k 0-7), (m 8-15, k 0-7), (m 0-7, k 8-15), ...
+        const uint32_t addr = smem_u32(phi + (size_t)(part * 64 + ks * 16 + (mi >> 1) * 8 + r8) * LD + mt * 16 + (mi & 1) * 8);
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(a[part][0]), "=r"(a[part][1]), "=r"(a[part][2]), "=r"(a[part][3]) : "r"(addr));
+      }
+#pragma unroll
+      for (int np = 0; np < NT / 2; ++np) {
+        uint32_t b[4];
+        const uint32_t addr = smem_u32(vs + (size_t)(ks * 16 + (mi & 1) * 8 + r8) * LD + (wn * NT + np * 2 + (mi >> 1)) * 8);
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]) : "r"(addr));
+#pragma unroll
+        for (int part = 0; part < 3; ++part) {
+          mma_bf16(acc[2 * np], a[part][0], a[part][1], a[part][2], a[part][3], b[0], b[1]);
+          mma_bf16(acc[2 * np + 1], a[part][0], a[part][1], a[part][2], a[part][3], b[2], b[3]);
+        }
+      }
+    }
+  }
+  float* dst = pc.snap + ((size_t)r.u * pc.n_sb + blockIdx.x) * D * D;
+#pragma unroll
+  for (int n = 0; n < NT; ++n) {
+    const int col = (wn * NT + n) * 8 + 2 * t;
+    *reinterpret_cast<float2*>(dst + (size_t)(mt * 16 + g) * D + col) = make_float2(acc[n][0], acc[n][1]);
+    *reinterpret_cast<float2*>(dst + (size_t)(mt * 16 + g + 8) * D + col) = make_float2(acc[n][2], acc[n][3]);
+  }
+}
+
+// The ranges' contributions become, in place, the state before each range; the cache's state is advanced over the chunk.
+// One thread per four entries; bound by the memory traffic (64 KB read and written per range and unit at d = 128).
+template <int D>
+__global__ void __launch_bounds__(128) prefill_scan_state_kernel(const Params p, const PrefillChunk pc) {
+  constexpr int N4 = D * D / 4, AHEAD = 8;
+  const int idx = blockIdx.x * 128 + threadIdx.x;
+  const int u = blockIdx.y;
+  float4* st = reinterpret_cast<float4*>(p.state + (size_t)u * D * D) + idx;
+  float4* x = reinterpret_cast<float4*>(pc.snap + (size_t)u * pc.n_sb * D * D) + idx;
+  float4 s = *st;
+  for (int i0 = 0; i0 < pc.n_sb; i0 += AHEAD) {
+    float4 a[AHEAD];
+#pragma unroll
+    for (int j = 0; j < AHEAD; ++j)
+      if (i0 + j < pc.n_sb) a[j] = x[(size_t)(i0 + j) * N4];
+#pragma unroll
+    for (int j = 0; j < AHEAD; ++j) {
+      if (i0 + j < pc.n_sb) {
+        x[(size_t)(i0 + j) * N4] = s;
+        s.x += a[j].x; s.y += a[j].y; s.z += a[j].z; s.w += a[j].w;
+      }
+    }
+  }
+  *st = s;
+}
+
+template <int D>
+cudaError_t own_d(const Params& p, const PrefillChunk& c, const void* q, float* out, int* sel_user, cudaStream_t s) {
+  const size_t smem = (size_t)2 * kOwnGroup * D * 4;
+  prefill_own_kernel<D><<<dim3((c.T + p.B - 2) / p.B + 1, p.batch * p.Hkv), kOwnThreads, smem, s>>>(
+      p, c, reinterpret_cast<const __nv_bfloat16*>(q), out, sel_user);
+  ++g_launch_count;
+  return cudaGetLastError();
+}
+
+template <int D>
+cudaError_t state_d(const Params& p, const PrefillChunk& c, cudaStream_t s) {
+  const size_t smem = (size_t)4 * 64 * (D + 8) * 2;
+  auto kern = prefill_local_state_kernel<D>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<dim3(c.n_sb, p.batch * p.Hkv), 256, smem, s>>>(p, c);
+  ++g_launch_count;
+  prefill_scan_state_kernel<D><<<dim3(D * D / 4 / 128, p.batch * p.Hkv), 128, 0, s>>>(p, c);
+  ++g_launch_count;
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_prefill_own(const Params& p, const PrefillChunk& c, const void* q, float* out, int* sel_user, cudaStream_t s) {
+  return p.d == 128 ? own_d<128>(p, c, q, out, sel_user, s) : own_d<64>(p, c, q, out, sel_user, s);
+}
+cudaError_t launch_prefill_state(const Params& p, const PrefillChunk& c, cudaStream_t s) {
+  return p.d == 128 ? state_d<128>(p, c, s) : state_d<64>(p, c, s);
+}
+
+}  // namespace spla

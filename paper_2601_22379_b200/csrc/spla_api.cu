@@ -8,6 +8,7 @@
 #include <cuda.h>
 
 #include "../../include/spla.h"
+#include "prefill_chunk.h"
 #include "spla_internal.h"
 
 using namespace spla;
@@ -23,6 +24,7 @@ struct spla_cache {
   int sm_count;
   AttendMaps maps;
   AttendMaps state_maps;   // the same caches in boxes of 64 tokens, for the tensor-core state kernel
+  AttendMaps prefill_maps; // ... of one block, at most 64 tokens, for the tensor-core prefill path
 };
 
 static thread_local char g_cuda_err[256] = "";
@@ -118,6 +120,14 @@ static int validate_config(const spla_config_t* c) {
   if (c->window_size > c->block_size) return SPLA_ERR_INVALID_ARG;
   if (windows_per_block(c) > kMaxWindows) return SPLA_ERR_UNSUPPORTED;
   return SPLA_OK;
+}
+
+// The tensor-core prefill path serves bf16 caches and queries with whole-block statistics (see prefill_attend.cu).
+static bool prefill_on_tensor_cores(const spla_config_t* c) {
+  const int64_t max_blocks = ((int64_t)c->max_context + c->block_size - 1) / c->block_size;
+  const int64_t rows = (int64_t)c->batch * c->n_kv_heads * max_blocks * c->block_size;
+  return c->kv_dtype == SPLA_BF16 && c->q_dtype == SPLA_BF16 && c->window_size == 0 && !(c->flags & SPLA_GENERAL_KERNELS) &&
+         max_blocks <= kPfMaxBlocks && rows < (1ll << 31);
 }
 
 struct WorkspaceLayout {
@@ -223,6 +233,7 @@ extern "C" int spla_init_cache(const spla_config_t* config, const spla_buffers_t
 
   c->maps.valid = false;
   c->state_maps.valid = false;
+  c->prefill_maps.valid = false;
   if (p.kv_bf16) {
     const unsigned long long rows = (unsigned long long)p.batch * p.Hkv * p.max_blocks * p.B;
     c->maps.valid = make_kv_tile_map(c->maps.k, b->k_cache, p.d, p.tile_rows, rows) &&
@@ -230,6 +241,9 @@ extern "C" int spla_init_cache(const spla_config_t* config, const spla_buffers_t
     c->state_maps.valid = p.d == 128 && rows >= 64 && rows < (1ull << 31) && !(config->flags & SPLA_GENERAL_KERNELS) &&
                           make_kv_map(c->state_maps.k, b->k_cache, p.d, 64, rows) &&
                           make_kv_map(c->state_maps.v, b->v_cache, p.d, 64, rows);
+    const int box = p.B < 64 ? p.B : 64;
+    c->prefill_maps.valid = prefill_on_tensor_cores(config) && rows < (1ull << 31) && make_kv_map(c->prefill_maps.k, b->k_cache, p.d, box, rows) &&
+                            make_kv_map(c->prefill_maps.v, b->v_cache, p.d, box, rows);
   }
 
   cudaStream_t s = (cudaStream_t)stream;
@@ -477,23 +491,81 @@ static int prefill_batch_cap(const spla_config_t* c) {   // virtual units are th
   return (int)(65535 / U);
 }
 
+// Workspace of the tensor-core path: tables for the whole chunk, then the log masses of `ns` ranges of SB positions.
+struct PrefillChunkLayout {
+  size_t ell_own, snap, sel, ell, total;
+};
+
+static PrefillChunkLayout prefill_chunk_layout(const spla_config_t* c, int T, int ns) {
+  PrefillChunkLayout w;
+  const size_t U = (size_t)c->batch * c->n_kv_heads, G = c->n_q_heads / c->n_kv_heads, d = c->head_dim;
+  const size_t max_blocks = ((size_t)c->max_context + c->block_size - 1) / c->block_size;
+  int SB, P, nt;
+  prefill_tiling((int)G, c->block_size, &SB, &P, &nt);
+  size_t off = 0;
+  auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
+  w.ell_own = take(U * T * G * 4);
+  w.snap = take((c->flags & SPLA_NO_RLA) ? 0 : U * prefill_ranges(T, SB) * d * d * 4);
+  w.sel = take(U * T * c->top_k * 4);
+  w.ell = take(U * ns * SB * G * align_up(max_blocks, 32) * 4);
+  w.total = off;
+  return w;
+}
+
 extern "C" int spla_query_prefill_workspace(const spla_config_t* config, int32_t T, size_t* min_bytes, size_t* good_bytes) {
   int rc = validate_config(config);
   if (rc) return rc;
   if (T < 1 || (!min_bytes && !good_bytes)) return SPLA_ERR_INVALID_ARG;
   if (prefill_batch_cap(config) < 1) return SPLA_ERR_UNSUPPORTED;
-  const size_t one = prefill_layout(config, T, 1).total;
+  const bool fast = prefill_on_tensor_cores(config);
+  int SB, P, nt;
+  prefill_tiling(config->n_q_heads / config->n_kv_heads, config->block_size, &SB, &P, &nt);
+  auto total = [&](int units) { return fast ? prefill_chunk_layout(config, T, units).total : prefill_layout(config, T, units).total; };
+  const long long most = fast ? prefill_ranges(T, SB) : (T < prefill_batch_cap(config) ? T : prefill_batch_cap(config));
+  const size_t one = total(1);
   if (min_bytes) *min_bytes = one;
   if (good_bytes) {
     // about 256 MB of per-batch scratch, at most the whole chunk at once
-    const size_t per_pos = prefill_layout(config, T, 2).total - one;
-    long long tb = (long long)((256ull << 20) / (per_pos ? per_pos : 1));
-    if (tb < 1) tb = 1;
-    if (tb > T) tb = T;
-    if (tb > prefill_batch_cap(config)) tb = prefill_batch_cap(config);
-    *good_bytes = prefill_layout(config, T, (int)tb).total;
+    const size_t per = total(2) - one;
+    long long n = (long long)((256ull << 20) / (per ? per : 1));
+    if (n < 1) n = 1;
+    if (n > most) n = most;
+    *good_bytes = total((int)n);
   }
   return SPLA_OK;
+}
+
+// The chunk on the tensor cores.  The chunk's tokens are in the cache and the lengths advanced; the state is not.
+static int prefill_chunked(spla_cache* c, const void* q, int T, const float* rms_weight, float* out, int32_t* sel_idx, char* ws,
+                           size_t workspace_bytes, cudaStream_t s) {
+  PrefillChunk pc;
+  memset(&pc, 0, sizeof(pc));
+  pc.T = T;
+  prefill_tiling(c->p.G, c->p.B, &pc.SB, &pc.P, &pc.nt);
+  pc.n_sb = prefill_ranges(T, pc.SB);
+  const PrefillChunkLayout w = prefill_chunk_layout(&c->cfg, T, 1);
+  const int blocks = (int)((c->len_bound + c->p.B - 1) / c->p.B);
+  pc.stride = (int)align_up(blocks, 32);
+  // SB ranges per launch: as many as the workspace holds at this sequence length
+  const size_t per = (size_t)c->p.batch * c->p.Hkv * pc.SB * c->p.G * pc.stride * 4;
+  long long ns = (long long)((workspace_bytes - w.ell) / per);
+  if (ns > pc.n_sb) ns = pc.n_sb;
+  if (ns > 65535 / pc.nt) ns = 65535 / pc.nt;             // (a grid dimension)
+  if (ns < 1) ns = 1;                                     // (the minimum workspace holds one range at the largest length)
+  pc.ell_own = (float*)(ws + w.ell_own);
+  pc.snap = (float*)(ws + w.snap);
+  pc.sel = (int*)(ws + w.sel);
+  pc.ell = (float*)(ws + w.ell);
+  cudaError_t e = launch_prefill_own(c->p, pc, q, out, sel_idx, s);
+  if (e == cudaSuccess && !(c->cfg.flags & SPLA_NO_RLA)) e = launch_prefill_state(c->p, pc, s);
+  for (int s0 = 0; s0 < pc.n_sb && e == cudaSuccess; s0 += (int)ns) {
+    pc.s0 = s0;
+    pc.ns = (int)(ns < pc.n_sb - s0 ? ns : pc.n_sb - s0);
+    e = launch_prefill_score(c->p, pc, q, blocks, c->sm_count, s);
+    if (e == cudaSuccess) e = launch_prefill_select(c->p, pc, blocks, sel_idx, s);
+    if (e == cudaSuccess) e = launch_prefill_attend(c->p, pc, c->prefill_maps, q, rms_weight, out, s);
+  }
+  return e == cudaSuccess ? SPLA_OK : cuda_fail(e, "spla_prefill");
 }
 
 extern "C" int spla_prefill(spla_cache_t* c, const void* k_new, const void* v_new, const void* q, int32_t T,
@@ -505,17 +577,12 @@ extern "C" int spla_prefill(spla_cache_t* c, const void* k_new, const void* v_ne
     return SPLA_ERR_INVALID_ARG;
   if (c->p.NW != 1) return SPLA_ERR_UNSUPPORTED;                 // whole-block statistics only
   if (c->len_bound + T > c->cfg.max_context) return SPLA_ERR_CAPACITY;
-  // positions per launch: as many as the workspace holds
   const int cap = prefill_batch_cap(&c->cfg);
   if (cap < 1) return SPLA_ERR_UNSUPPORTED;
-  const size_t one = prefill_layout(&c->cfg, T, 1).total;
+  const bool fast = prefill_on_tensor_cores(&c->cfg);
+  if (fast && !c->prefill_maps.valid) return SPLA_ERR_UNSUPPORTED;   // (the driver refused the tensor maps)
+  const size_t one = fast ? prefill_chunk_layout(&c->cfg, T, 1).total : prefill_layout(&c->cfg, T, 1).total;
   if (workspace_bytes < one) return SPLA_ERR_INVALID_ARG;
-  const size_t per_pos = prefill_layout(&c->cfg, T, 2).total - one;
-  long long tb = 1 + (long long)((workspace_bytes - one) / (per_pos ? per_pos : 1));
-  if (tb > T) tb = T;
-  if (tb > cap) tb = cap;
-  while (tb > 1 && prefill_layout(&c->cfg, T, (int)tb).total > workspace_bytes) --tb;   // (alignment padding)
-  const PrefillLayout w = prefill_layout(&c->cfg, T, (int)tb);
   char* ws = reinterpret_cast<char*>(workspace);
   cudaStream_t s = (cudaStream_t)stream;
   const int qb = c->cfg.q_dtype == SPLA_BF16;
@@ -529,6 +596,15 @@ extern "C" int spla_prefill(spla_cache_t* c, const void* k_new, const void* v_ne
     if (e != cudaSuccess) return cuda_fail(e, "spla_prefill/append");
     c->len_bound += T;
   }
+  if (fast) return prefill_chunked(c, q, T, rms_weight, out, sel_idx, ws, workspace_bytes, s);
+
+  // positions per launch: as many as the workspace holds
+  const size_t per_pos = prefill_layout(&c->cfg, T, 2).total - one;
+  long long tb = 1 + (long long)((workspace_bytes - one) / (per_pos ? per_pos : 1));
+  if (tb > T) tb = T;
+  if (tb > cap) tb = cap;
+  while (tb > 1 && prefill_layout(&c->cfg, T, (int)tb).total > workspace_bytes) --tb;   // (alignment padding)
+  const PrefillLayout w = prefill_layout(&c->cfg, T, (int)tb);
   // 2. per-position statistics of the growing block, o_bar of every position, S_bar advanced over the chunk
   float* vstats = reinterpret_cast<float*>(ws + w.vstats);
   float* vobar = reinterpret_cast<float*>(ws + w.vobar);

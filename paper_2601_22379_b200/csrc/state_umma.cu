@@ -29,9 +29,8 @@
 //
 // Every wait is an mbarrier poll with an iteration limit; on expiry the CTA raises its abort flag, all roles
 // leave their loops, tensor memory is released and the time-out status is latched.  No multicast anywhere.
-#include <cuda.h>
-
 #include "spla_internal.h"
+#include "umma.cuh"
 
 namespace spla {
 
@@ -49,59 +48,9 @@ constexpr int kSuSmemBytes = kSuStages * kSuStageBytes;      // 192 KB
 constexpr int kSuGroup = 2;                                  // tiles accumulated in tensor memory before a flush
 constexpr int kSuTmemCols = 256;                             // two 128-column accumulators, used in turn
 
-// tcgen05 instruction descriptor, kind::f16: fp32 accumulator (bit 4), A and B bf16 (bits 7, 10), A and B
-// MN-major (bits 15, 16), N / 8 at bit 17, M / 16 at bit 24.
-constexpr uint32_t kSuIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((kSuD / 8) << 17) | ((kSuD / 16) << 24);
-
-// Shared-memory matrix descriptor of an MN-major bf16 operand in the 128-byte swizzle: start address / 16,
-// leading byte offset / 16 at bit 16 (distance between the two 64-channel halves), stride byte offset / 16 at
-// bit 32 (distance between groups of 8 tokens), descriptor version 1 at bit 46, layout type 2 at bit 61.
-__device__ __forceinline__ uint64_t umma_desc(uint32_t smem_addr) {
-  const uint64_t lo = (uint64_t)((smem_addr >> 4) & 0x3fffu) | ((uint64_t)(kSuHalfBytes >> 4) << 16);
-  const uint64_t hi = (uint64_t)(1024 >> 4) | (1ull << 14) | (2ull << 29);
-  return lo | (hi << 32);
-}
-
-__device__ __forceinline__ void tma_load_box(uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
-  asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-               "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar))
-               : "memory");
-}
-__device__ __forceinline__ void mbar_arrive1(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}"
-      ::"r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(kSuIdesc), "r"(accumulate), "r"(0u)
-      : "memory");
-}
-// Arrives on the barrier once every tcgen05.mma issued so far by this thread has completed.
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// 32 consecutive accumulator columns of this thread's tensor-memory lane.
-__device__ __forceinline__ void tmem_ld32(uint32_t addr, float (&v)[32]) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(addr)
-      : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
+// A and B MN-major bf16, 128 x 128
+constexpr uint32_t kSuIdesc = umma_idesc(true, true, true, kSuD, kSuD);
+__device__ __forceinline__ uint64_t su_desc(uint32_t smem_addr) { return umma_desc_sw128(smem_addr, kSuHalfBytes); }
 
 }  // namespace
 
@@ -140,8 +89,7 @@ __global__ void __launch_bounds__(kSuThreads, 1)
     abort_s = 0;
   }
   if (warp == 1) {                                       // tensor memory for the 128 x 128 fp32 accumulator
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(kSuTmemCols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    tmem_alloc(&tmem_base_s, kSuTmemCols);
   }
   tc_fence_before();
   __syncthreads();
@@ -185,8 +133,8 @@ __global__ void __launch_bounds__(kSuThreads, 1)
           for (int part = 0; part < 2; ++part)           // head of phi, then its remainder
 #pragma unroll
             for (int kk = 0; kk < kSuTile / 16; ++kk)    // 16 tokens (two swizzle atoms of 8 rows) per instruction
-              umma_bf16(tmem + ab * kSuD, umma_desc(base + part * kSuTileBytes + kk * 2048),
-                        umma_desc(base + 2 * kSuTileBytes + kk * 2048), (!first || part > 0 || kk > 0) ? 1u : 0u);
+              umma_ss(tmem + ab * kSuD, su_desc(base + part * kSuTileBytes + kk * 2048),
+                      su_desc(base + 2 * kSuTileBytes + kk * 2048), kSuIdesc, (!first || part > 0 || kk > 0) ? 1u : 0u);
           umma_commit(&empty[s]);                        // the stage may be refilled once these have read it
           if (last) umma_commit(&acc_full[ab]);          // and the group's sum may be drained
         }
@@ -273,7 +221,7 @@ __global__ void __launch_bounds__(kSuThreads, 1)
           *kp = hi4;
           *lp = lo4;
         }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the tensor core's reads
+        proxy_fence();                                   // generic writes -> visible to the tensor core's reads
         __syncwarp();
         if (lane == 0) mbar_arrive1(&ready[s]);
         // one accumulator group behind the issuer: by now those instructions have long completed
@@ -302,7 +250,7 @@ __global__ void __launch_bounds__(kSuThreads, 1)
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kSuTmemCols) : "memory");
+    tmem_free(tmem, kSuTmemCols);
   }
   if (tid == 0 && abort_s) atomicExch(p.status, kStatusTimeout);
   if (S == 1) return;

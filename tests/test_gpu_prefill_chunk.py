@@ -1,0 +1,110 @@
+"""The tensor-core prefill path against the general kernels (fp32 products, one virtual unit per position) on the same
+inputs: every group size, block size and head dim class it has code for, at the edges of its tiles and ranges.
+
+Tolerance: probabilities and linear coefficients enter their products as two bf16 parts (2^-17 relative per term), phi as
+22 bits, everything else in fp32, so single outputs agree to a few 1e-5; the residual's error is that of its operands,
+2^-17 |o_bar|, times the RMSNorm's amplification 1 / |o_rla|, which the sizes below keep under about 10 (near-complete
+selection, where it is larger, is the last case, with its own bound)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2601_22379_b200 import binding, runner, synth
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+RTOL, ATOL = 3e-4, 3e-5
+
+CASES = [
+    # batch, hkv, G, d, B, top_k, n_sink, n_local, L0, T, flags
+    (1, 2, 4, 128, 64, 8, 1, 2, 0, 64, 0),             # exactly one range
+    (2, 2, 4, 128, 64, 6, 1, 2, 63, 130, 0),           # a chunk that starts on a block's last token
+    (1, 1, 4, 128, 64, 16, 1, 4, 64 * 40, 1, 0),       # a single position
+    (1, 2, 4, 128, 128, 6, 1, 2, 1000, 200, 0),        # two tiles of tokens per block
+    (1, 2, 4, 128, 32, 8, 1, 4, 700, 97, 0),           # two blocks per tile
+    (1, 2, 4, 128, 16, 8, 0, 0, 333, 75, 0),           # four blocks per tile; own block not always selected
+    (1, 1, 1, 128, 64, 5, 1, 1, 900, 140, 0),          # groups of 1, 2, 3, 5, 8, 16
+    (1, 1, 2, 64, 32, 5, 1, 1, 500, 70, 0),
+    (1, 1, 3, 128, 64, 6, 1, 2, 700, 66, 0),
+    (2, 2, 5, 128, 64, 8, 1, 4, 1500, 131, 0),
+    (1, 2, 8, 64, 64, 8, 1, 2, 801, 65, 0),
+    (1, 1, 16, 128, 64, 8, 1, 4, 64 * 21 + 1, 90, 0),
+    (1, 2, 4, 64, 64, 8, 1, 2, 64 * 30 + 5, 300, binding.SPLA_STATS_BF16),
+    (1, 2, 4, 128, 64, 64, 1, 4, 64 * 90, 100, 0),     # longest selection
+    (1, 1, 4, 128, 64, 8, 1, 2, 700, 90, binding.SPLA_FIRST_ORDER),
+    (1, 1, 4, 128, 64, 8, 0, 0, 700, 90, binding.SPLA_NO_RLA),
+    (1, 1, 4, 128, 16, 8, 1, 4, 16 * 600, 40, 0),      # more than 512 blocks: a CTA selects
+    (1, 1, 4, 64, 16, 8, 1, 4, 16 * 1100, 33, binding.SPLA_DEBUG_BOUNDS),
+]
+
+
+def _inputs(case, seed=11):
+    batch, hkv, G, d, B, top_k, ns, nl, L0, T, flags = case
+    w = synth.Workload("case", seed, batch=batch, n_q_heads=hkv * G, n_kv_heads=hkv, head_dim=d, block_size=B, top_k=top_k,
+                       context=max(L0, 1), n_sink=ns, n_local=nl, n_outlier_channels=4, outlier_scale=3.0, n_steps=T)
+    g = torch.Generator(device=DEV).manual_seed(seed)
+    K0, V0, _ = runner.generate_prefill(w, DEV)
+    k = torch.randn(batch, hkv, T, d, generator=g, device=DEV)
+    k[..., :3] *= 3.0
+    v = torch.randn(batch, hkv, T, d, generator=g, device=DEV)
+    q0 = synth.query_directions(w).to(DEV).repeat_interleave(G, dim=1)[:, None]
+    q = (q0 + torch.randn(batch, T, hkv * G, d, generator=g, device=DEV)) / 1.4
+    return w, K0[:, :, :L0].contiguous(), V0[:, :, :L0].contiguous(), *(x.to(torch.bfloat16).contiguous() for x in (k, v, q))
+
+
+def _run(w, K0, V0, k, v, q, flags, **kw):
+    cache = binding.SplaCache(runner.config_for(w, flags=flags), DEV)
+    for t in (cache.bufs.k_cache, cache.bufs.v_cache):
+        t.fill_(float("nan"))                           # nothing past a sequence's end may reach a result
+    if K0.shape[2]:
+        cache.append_tokens(K0, V0)
+    T = k.shape[2]
+    sel = torch.full((w.batch, T, w.n_kv_heads, w.top_k), -7, dtype=torch.int32, device=DEV)
+    out = cache.prefill(k, v, q, synth.gamma(w).to(DEV), sel_idx=sel, **kw)
+    torch.cuda.synchronize()
+    assert cache.sync_status() == 0
+    return out, sel, cache
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: "-".join(map(str, c)))
+def test_tensor_core_prefill_equals_the_general_kernels(case):
+    w, K0, V0, k, v, q = _inputs(case)
+    flags = case[-1]
+    n0 = binding.launch_count()
+    a, sel_a, ca = _run(w, K0, V0, k, v, q, flags)
+    n1 = binding.launch_count()
+    b, sel_b, cb = _run(w, K0, V0, k, v, q, flags | binding.SPLA_GENERAL_KERNELS)
+    assert n1 > n0 and torch.isfinite(a).all()
+    same = (sel_a == sel_b).all(dim=-1)                 # [batch, T, hkv]; near-ties may fall the other way
+    assert same.float().mean().item() >= (0.97 if flags & binding.SPLA_STATS_BF16 else 0.99)
+    rows = same.repeat_interleave(w.group, dim=2)
+    np.testing.assert_allclose(a[rows].cpu().numpy(), b[rows].cpu().numpy(), rtol=RTOL, atol=ATOL)
+    if not flags & binding.SPLA_NO_RLA:
+        rel = (ca.bufs.rla_state - cb.bufs.rla_state).norm() / cb.bufs.rla_state.norm()
+        assert rel.item() < parity.STATE_TOL_TENSOR + parity.STATE_TOL_FMA   # (the history went in on either kernel)
+    least, _, _ = _run(w, K0, V0, k, v, q, flags, workspace_bytes=1)
+    assert torch.equal(least, a)                        # positions per launch change nothing
+
+
+def test_tensor_core_prefill_under_near_complete_selection():
+    """All blocks but one or two selected: |o_bar| is 20 to 40 times |o_rla| here, and with it the tolerance."""
+    case = (1, 2, 4, 128, 64, 30, 1, 4, 64 * 30 + 9, 60, 0)
+    w, K0, V0, k, v, q = _inputs(case)
+    a, sel_a, _ = _run(w, K0, V0, k, v, q, 0)
+    b, sel_b, _ = _run(w, K0, V0, k, v, q, binding.SPLA_GENERAL_KERNELS)
+    rows = (sel_a == sel_b).all(dim=-1).repeat_interleave(w.group, dim=2)
+    np.testing.assert_allclose(a[rows].cpu().numpy(), b[rows].cpu().numpy(), rtol=40 * RTOL, atol=40 * ATOL)
+
+
+def test_a_wait_that_runs_out_is_reported_and_leaves_the_device_usable():
+    case = CASES[1]
+    w, K0, V0, k, v, q = _inputs(case)
+    cache = binding.SplaCache(runner.config_for(w), DEV)
+    cache.append_tokens(K0, V0)
+    cache.debug_wait_hook(2000, 16)
+    cache.prefill(k, v, q, synth.gamma(w).to(DEV))
+    torch.cuda.synchronize()
+    assert cache.sync_status() == binding.SPLA_ERR_TIMEOUT
+    a, _, _ = _run(w, K0, V0, k, v, q, 0)
+    assert torch.isfinite(a).all()
