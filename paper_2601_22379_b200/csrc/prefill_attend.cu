@@ -26,9 +26,13 @@
 // coefficients, drain and epilogue (4 warps); phi(K) (4 warps).  Two-deep rings everywhere, released as early as each
 // operand allows.  setmaxnreg moves registers to the linear warps, whose row of R takes 128.
 //
-// Bound by the tensor pipe (about 2560 cycles per tile: 10 products of 128 x 64 x 128, the four whose left operand comes
-// from shared memory at 3/4 of the rate).  A prompt of 8192 tokens (8 KV heads, G = 4, d = 128, 32 of up to 128 blocks of
-// 64): 2.46 ms of the call's 2.87 ms, which took 60.6 ms as one virtual unit per position on the general kernels.
+// The tensor pipe needs about 2560 cycles per tile (8 products of 128 x 64 x 128; the four whose left operand comes from
+// shared memory run at 3/4 of the rate).  What bounds the kernel above that is issuing: four roles with different code share
+// each scheduler, so code size counts (with every loop unrolled 43 % of all stalls were instruction fetches, 9000 cycles per
+// tile; with 16-token loop bodies 3600), and the MMA warp runs converged with one elected lane (a one-lane branch cost 75 to
+// 110 cycles per MMA instead of 50 to 65).  A prompt of 8192 tokens (8 KV heads, G = 4, d = 128, 32 of up to 128 blocks of
+// 64): 60.6 ms as one virtual unit per position on the general kernels, 2.87 ms with this kernel unrolled, 1.72 ms now, of
+// which it takes 1.3 ms.
 //
 // Every wait is an mbarrier poll with an iteration limit; on expiry the CTA raises its abort flag, all roles leave their
 // loops, tensor memory is released and the time-out status is latched.  No multicast anywhere.
@@ -62,7 +66,7 @@ struct PaSmem {
   static constexpr int kBitmap = kPhi + 4 * kTileBytes;          // [512] words: the union of the selected blocks
   static constexpr int kLse = kBitmap + kPfMaxBlocks / 8;        // float [2][64]
   static constexpr int kBars = kLse + 2 * kPaTile * 4;
-  static constexpr int kMisc = kBars + 18 * 8;                   // tensor-memory base, abort flag, tile count
+  static constexpr int kMisc = kBars + 22 * 8;                   // tensor-memory base, abort flag, tile count
   static constexpr int kBytes = kMisc + 32;
   static_assert(kBytes <= 227 * 1024, "shared memory of the attend kernel");
   static_assert(2 * H * D * 128 <= 4 * kTileBytes, "S_base fits the phi(K) ring");
@@ -89,6 +93,13 @@ struct TileWalk {
   uint32_t word;
   int blk[4], off;
   __device__ __forceinline__ void start(const uint32_t* bitmap, int B_) { bm = bitmap; w = 0; B = B_; word = bm[0]; off = B_; blk[0] = -1; }
+  // Block number s of a tile of small blocks (of a short last tile: the first again).  A select, so that blk[] stays in registers.
+  __device__ __forceinline__ int sub_block(int s) const {
+    int r = blk[0];
+#pragma unroll
+    for (int x = 1; x < 4; ++x) r = s == x ? blk[x] : r;
+    return r < 0 ? blk[0] : r;
+  }
   __device__ __forceinline__ int next_bit() {
     while (word == 0u) {
       if (++w >= kPfMaxBlocks / 32) { w = kPfMaxBlocks / 32; return -1; }
@@ -110,27 +121,42 @@ struct TileWalk {
   }
 };
 
-// A position's ascending selection list, followed along the walk.
+// A position's ascending selection list, followed along the walk; the entry after the current one is already loaded.
 struct SelCursor {
   const int* list;
-  int j, k, cur;
-  __device__ __forceinline__ void start(const int* l, int top_k) { list = l; j = 0; k = top_k; cur = (l && k > 0) ? l[0] : -1; }
+  int left, cur, nxt;
+  __device__ __forceinline__ void start(const int* l, int top_k) {
+    list = l;
+    left = l ? top_k : 0;
+    cur = left > 0 ? l[0] : -1;
+    nxt = left > 1 ? l[1] : -1;
+  }
   __device__ __forceinline__ bool at(int blk) const { return cur == blk; }
-  __device__ __forceinline__ void pass() { ++j; cur = j < k ? list[j] : -1; }
+  __device__ __forceinline__ void pass() {
+    cur = nxt;
+    --left;
+    ++list;
+    nxt = left > 1 ? list[1] : -1;
+  }
 };
 
 // The tokens of the current tile that row `pos` attends to (bit j: token j of the tile), and those after `base` it leaves
 // out (the two halves of the linear branch).  Moves the cursor.
 __device__ __forceinline__ void tile_masks(const TileWalk& tw, SelCursor& sc, int pos, int base, uint64_t& sel, uint64_t& neg, uint64_t& posv) {
   sel = neg = posv = 0ull;
-  if (pos < 0) return;
   if (tw.B >= kPaTile) {
     const int tok0 = tw.blk[0] * tw.B + tw.off;
-    const bool s = sc.at(tw.blk[0]);
+    const bool s = sc.at(tw.blk[0]);                             // (never for a row without a position: its list is empty)
     if (s && tw.off + kPaTile >= tw.B) sc.pass();
+    if (tok0 + kPaTile <= base) {                                // (uniform: wholly before the tile's positions)
+      sel = neg = s ? ~0ull : 0ull;
+      return;
+    }
+    if (pos < 0) return;
     const uint64_t seen = low_bits(pos + 1 - tok0), old = low_bits(base - tok0);
     if (s) { sel = seen; neg = seen & old; } else { posv = seen & ~old; }
   } else {
+    if (pos < 0) return;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       if (q * tw.B >= kPaTile || tw.blk[q] < 0) continue;
@@ -143,6 +169,16 @@ __device__ __forceinline__ void tile_masks(const TileWalk& tw, SelCursor& sc, in
   }
 }
 
+// Whether the tile holds rows past the sequence's end (the open block; of a short last tile the repeated first block).
+__device__ __forceinline__ bool tile_past(const TileWalk& tw, int L_end) {
+  if (tw.B >= kPaTile) return tw.blk[0] * tw.B + tw.off + kPaTile > L_end;
+  bool past = false;
+#pragma unroll
+  for (int s = 0; s < 4; ++s)
+    if (s * tw.B < kPaTile) past |= ((tw.blk[s] < 0 ? tw.blk[0] : tw.blk[s]) + 1) * tw.B > L_end;
+  return past;
+}
+
 template <int D, bool RLA>
 __global__ void __launch_bounds__(kPaThreads, 1)
     prefill_attend_kernel(const Params p, const PrefillChunk pc, const __grid_constant__ CUtensorMap map_k,
@@ -153,7 +189,7 @@ __global__ void __launch_bounds__(kPaThreads, 1)
   extern __shared__ __align__(1024) unsigned char smem[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SM::kBars);
   uint64_t *k_full = bars, *k_empty = bars + 2, *v_full = bars + 4, *v_empty = bars + 6, *phi_ready = bars + 8, *phi_empty = bars + 10,
-           *sa_full = bars + 12, *pa_ready = bars + 14, *r_full = bars + 16, *r_empty = bars + 17;
+           *s_full = bars + 12, *a_full = bars + 14, *p_ready = bars + 16, *c_ready = bars + 18, *r_full = bars + 20, *r_empty = bars + 21;
   uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(smem + SM::kMisc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + SM::kMisc + 4);
   int* n_set_s = reinterpret_cast<int*>(smem + SM::kMisc + 8);
@@ -179,7 +215,8 @@ __global__ void __launch_bounds__(kPaThreads, 1)
       mbar_init(&k_full[s], 1);  mbar_init(&k_empty[s], 5);   // four transform warps and the MMA
       mbar_init(&v_full[s], 1);  mbar_init(&v_empty[s], 1);
       mbar_init(&phi_ready[s], 4);  mbar_init(&phi_empty[s], 1);
-      mbar_init(&sa_full[s], 1);  mbar_init(&pa_ready[s], RLA ? 8 : 4);
+      mbar_init(&s_full[s], 1);  mbar_init(&a_full[s], 1);
+      mbar_init(&p_ready[s], 4);  mbar_init(&c_ready[s], 4);
     }
     mbar_init(r_full, 1);
     mbar_init(r_empty, 4);
@@ -329,76 +366,77 @@ __global__ void __launch_bounds__(kPaThreads, 1)
       }
       if (*abort_flag)                                            // let the copies in flight land before the CTA leaves
         for (int j = max(0, issued - 2); j < issued; ++j) mbar_wait(&full[j & 1], (j >> 1) & 1, lim);
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
       // ------------------------------------------------------------ MMA issuer -------------------------------------
       constexpr uint32_t id_s = umma_idesc(true, false, false, kPfRows, kPaTile);
       constexpr uint32_t id_a = umma_idesc(false, false, false, kPfRows, kPaTile);
       constexpr uint32_t id_o = umma_idesc(true, false, true, kPfRows, D);
       constexpr uint32_t id_r0 = umma_idesc(false, false, true, kPfRows, D);
+      const uint32_t one = elect_one();                           // (the whole warp runs this loop: see umma_ss_one)
       bool ok = true;
-      // (operand offset of k-step kk: 32 bytes inside the 128-byte rows, then the next array of rows)
-      auto qoff = [](int kk) { return (uint32_t)((kk >> 2) * (kPfRows * 128) + (kk & 3) * 32); };
-      auto koff = [](int kk) { return (uint32_t)((kk >> 2) * SM::kHalf + (kk & 3) * 32); };
+      // The loops are rolled as far as they can be (four products per trip): the roles of a CTA run on the same schedulers
+      // and their code competes for the instruction cache.
+      const uint32_t q0 = umma_desc_lo(sbase + SM::kQ, 16), fh0 = umma_desc_lo(sbase + SM::kFh, 16), fl0 = umma_desc_lo(sbase + SM::kFl, 16);
+      constexpr uint32_t kQStep = kPfRows * 128 / 16, kKStep = SM::kHalf / 16;   // to the next 64 channels of q, of a K tile
+      // D (+)= X Y^T over all channels: both K-major, 16 channels = 32 bytes per step, 64 per array of rows
+      auto xyT = [&](uint32_t d, uint32_t x, uint32_t y, uint32_t idesc, uint32_t acc) {
+#pragma unroll
+        for (int hh = 0; hh < H; ++hh) umma_ss4_one<2, 2>(one, d, x + hh * kQStep, y + hh * kKStep, idesc, hh > 0 ? 1u : acc);
+      };
+      // D (+)= C V for the two parts of C, 16 tokens per step
+      auto cv = [&](uint32_t d, uint32_t c, uint32_t v, uint32_t acc) {
+#pragma unroll
+        for (int part = 0; part < 2; ++part) umma_ts4_one<16, 2048 / 16>(one, d, c + part * 8, v, id_o, part > 0 ? 1u : acc);
+      };
       auto first_products = [&](int i) {                          // S and A of tile i
         const int b = i & 1, par = (i >> 1) & 1;
         const uint32_t d = tSA + b * 128;
-        const uint32_t kt = sbase + SM::kK + b * SM::kTileBytes;
-        if (!mbar_wait(&k_full[b], par, lim)) { ok = false; return; }
+        if (!warp_waits(&k_full[b], par, lim)) { ok = false; return; }
         tc_fence_after();
-#pragma unroll
-        for (int kk = 0; kk < KS; ++kk)
-          umma_ss(d, umma_desc_sw128(sbase + SM::kQ + qoff(kk), 16), umma_desc_sw128(kt + koff(kk), 16), id_s, kk > 0);
-        umma_commit(&k_empty[b]);
-        if (!mbar_wait(&phi_ready[b], par, lim)) { ok = false; return; }
+        xyT(d, q0, umma_desc_lo(sbase + SM::kK + b * SM::kTileBytes, 16), id_s, 0u);
+        umma_commit_one(one, &k_empty[b]);
+        umma_commit_one(one, &s_full[b]);
+        if (!warp_waits(&phi_ready[b], par, lim)) { ok = false; return; }
         if constexpr (RLA) {
           tc_fence_after();
-          const uint32_t ph = sbase + SM::kPhi + b * 2 * SM::kTileBytes, pl = ph + SM::kTileBytes;
-#pragma unroll
+          const uint32_t ph = umma_desc_lo(sbase + SM::kPhi + b * 2 * SM::kTileBytes, 16);
+#pragma unroll 1
           for (int part = 0; part < 3; ++part)                    // head x head, remainder x head, head x remainder
-#pragma unroll
-            for (int kk = 0; kk < KS; ++kk)
-              umma_ss(d + 64, umma_desc_sw128(sbase + (part == 1 ? SM::kFl : SM::kFh) + qoff(kk), 16),
-                      umma_desc_sw128((part == 2 ? pl : ph) + koff(kk), 16), id_a, part > 0 || kk > 0);
-          umma_commit(&phi_empty[b]);
+            xyT(d + 64, part == 1 ? fl0 : fh0, part == 2 ? ph + SM::kTileBytes / 16 : ph, id_a, part > 0);
+          umma_commit_one(one, &phi_empty[b]);
+          umma_commit_one(one, &a_full[b]);
         }
-        umma_commit(&sa_full[b]);
       };
       if constexpr (RLA) {                                        // R = phi(q) S_base
-        const uint32_t sh = sbase + SM::kPhi, sl = sh + H * D * 128;
-#pragma unroll
-        for (int part = 0; part < 3; ++part)
-#pragma unroll
+#pragma unroll 1
+        for (int part = 0; part < 3; ++part) {
+          const uint32_t x = part == 1 ? fl0 : fh0, y = umma_desc_lo(sbase + SM::kPhi + (part == 2 ? H * D * 128 : 0), D * 128);
+#pragma unroll 1
           for (int kk = 0; kk < KS; ++kk)
-            umma_ss(tR, umma_desc_sw128(sbase + (part == 1 ? SM::kFl : SM::kFh) + qoff(kk), 16),
-                    umma_desc_sw128((part == 2 ? sl : sh) + kk * 2048, D * 128), id_r0, part > 0 || kk > 0);
-        umma_commit(&phi_empty[0]);
-        umma_commit(&phi_empty[1]);
+            umma_ss_one(one, tR, umma_desc_of(x + (kk >> 2) * kQStep + (kk & 3) * 2), umma_desc_of(y + kk * (2048 / 16)), id_r0, part > 0 || kk > 0);
+        }
+        umma_commit_one(one, &phi_empty[0]);
+        umma_commit_one(one, &phi_empty[1]);
       }
-      first_products(0);
-      for (int i = 0; i < n_tiles && ok && !*abort_flag; ++i) {
+#pragma unroll 1
+      for (int i = -1; i < n_tiles && ok && !warp_aborted(abort_flag); ++i) {
         if (i + 1 < n_tiles) first_products(i + 1);
         if (!ok) break;
+        if (i < 0) continue;
         const int b = i & 1, par = (i >> 1) & 1;
-        if (!mbar_wait(&pa_ready[b], par, lim) || !mbar_wait(&v_full[b], par, lim)) { ok = false; break; }
+        if (!warp_waits(&p_ready[b], par, lim) || !warp_waits(&v_full[b], par, lim)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t a = tSA + b * 128, vt = sbase + SM::kV + b * SM::kTileBytes;
-#pragma unroll
-        for (int part = 0; part < 2; ++part)
-#pragma unroll
-          for (int ks = 0; ks < kPaTile / 16; ++ks)
-            umma_ts(tO, a + part * 32 + ks * 8, umma_desc_sw128(vt + ks * 2048, SM::kHalf), id_o, i > 0 || part > 0 || ks > 0);
+        const uint32_t a = tSA + b * 128, v = umma_desc_lo(sbase + SM::kV + b * SM::kTileBytes, SM::kHalf);
+        cv(tO, a, v, i > 0);
         if constexpr (RLA) {
           const bool fresh = i > 0 && i % kFlush == 0;            // R was drained: the sum starts over
-          if (fresh && !mbar_wait(r_empty, (i / kFlush - 1) & 1, lim)) { ok = false; break; }
+          if (fresh && !warp_waits(r_empty, (i / kFlush - 1) & 1, lim)) { ok = false; break; }
+          if (!warp_waits(&c_ready[b], par, lim)) { ok = false; break; }
           tc_fence_after();
-#pragma unroll
-          for (int part = 0; part < 2; ++part)
-#pragma unroll
-            for (int ks = 0; ks < kPaTile / 16; ++ks)
-              umma_ts(tR, a + 64 + part * 32 + ks * 8, umma_desc_sw128(vt + ks * 2048, SM::kHalf), id_o, !fresh || part > 0 || ks > 0);
+          cv(tR, a + 64, v, !fresh);
         }
-        umma_commit(&v_empty[b]);
-        if (i % kFlush == kFlush - 1 || i == n_tiles - 1) umma_commit(r_full);
+        umma_commit_one(one, &v_empty[b]);
+        if (i % kFlush == kFlush - 1 || i == n_tiles - 1) umma_commit_one(one, r_full);
       }
       if (!ok) *abort_flag = 1;
     }
@@ -418,28 +456,40 @@ __global__ void __launch_bounds__(kPaThreads, 1)
     for (int i = 0; i < n_tiles && !warp_aborted(abort_flag); ++i) {
       tw.next();
       uint64_t sel, neg, posv;
-      tile_masks(tw, cur, pos, 0, sel, neg, posv);
+      tile_masks(tw, cur, pos, base, sel, neg, posv);
       const int b = i & 1;
       const uint32_t src = tSA + b * 128 + lane_off;
-      if (!warp_waits(&sa_full[b], (i >> 1) & 1, lim)) { ok = false; break; }
+      if (!warp_waits(&s_full[b], (i >> 1) & 1, lim)) { ok = false; break; }
       tc_fence_after();
-      uint32_t s0[32], s1[32];
-      tmem_ld32_async(src, s0);
-      tmem_ld32_async(src + 32, s1);
-      tmem_ld_wait32(s0);
-      tmem_ld_wait32(s1);
-      const uint32_t m0 = (uint32_t)sel, m1 = (uint32_t)(sel >> 32);
-      if (!__all_sync(0xffffffffu, sel == ~0ull)) {
+      // Rows that attend to all of the tile or to none of it need no mask per token (a row that attends to none gets its
+      // zeros from an infinite offset); tiles that reach past the sequence's end always take the masked form: what lies
+      // there may be anything.
+      const bool plain = __all_sync(0xffffffffu, sel == ~0ull || sel == 0ull) && !tile_past(tw, r.L_end);
+      float mt = -INFINITY;
+      {
+        uint32_t s0[32], s1[32];
+        tmem_ld32_async(src, s0);
+        tmem_ld32_async(src + 32, s1);
+        tmem_ld_wait32(s0);
+        tmem_ld_wait32(s1);
+        if (plain) {
+          float mx0 = -INFINITY, mx1 = -INFINITY;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          if (!(m0 & (1u << j))) s0[j] = 0xff800000u;
-          if (!(m1 & (1u << j))) s1[j] = 0xff800000u;
+          for (int j = 0; j < 32; j += 2) {
+            mx0 = fmaxf(mx0, fmaxf(__uint_as_float(s0[j]), __uint_as_float(s0[j + 1])));
+            mx1 = fmaxf(mx1, fmaxf(__uint_as_float(s1[j]), __uint_as_float(s1[j + 1])));
+          }
+          if (sel) mt = fmaxf(mx0, mx1) * sc2;                    // (sc2 > 0)
+        } else {
+          const uint32_t m0 = (uint32_t)sel, m1 = (uint32_t)(sel >> 32);
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            if (m0 & (1u << j)) mt = fmaxf(mt, __uint_as_float(s0[j]));
+            if (m1 & (1u << j)) mt = fmaxf(mt, __uint_as_float(s1[j]));
+          }
+          mt *= sc2;
         }
       }
-      float mx0 = -INFINITY, mx1 = -INFINITY;
-#pragma unroll
-      for (int j = 0; j < 32; ++j) { mx0 = fmaxf(mx0, __uint_as_float(s0[j])); mx1 = fmaxf(mx1, __uint_as_float(s1[j])); }
-      const float mt = fmaxf(mx0, mx1) * sc2;                     // (sc2 > 0; -inf where nothing is selected)
       // The first selected tile of a row sets its maximum (its row of O is zero so far); later ones only move it when it
       // would let a probability exceed 2^8.
       const bool grow = mt > m + 8.f && m > -INFINITY;
@@ -452,45 +502,49 @@ __global__ void __launch_bounds__(kPaThreads, 1)
         const float f = m > -INFINITY ? ex2(m - m_new) : 1.f;
         m = m_new;
         l *= f;
-#pragma unroll
+#pragma unroll 1
         for (int c = 0; c < D; c += 16) {
           uint32_t o[16];
-          asm volatile(
-              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
-              "tcgen05.wait::ld.sync.aligned;"
-              : "=r"(o[0]), "=r"(o[1]), "=r"(o[2]), "=r"(o[3]), "=r"(o[4]), "=r"(o[5]), "=r"(o[6]), "=r"(o[7]), "=r"(o[8]),
-                "=r"(o[9]), "=r"(o[10]), "=r"(o[11]), "=r"(o[12]), "=r"(o[13]), "=r"(o[14]), "=r"(o[15])
-              : "r"(tO + lane_off + c)
-              : "memory");
+          tmem_ld16_async(tO + lane_off + c, o);
+          tmem_ld_wait16(o);
 #pragma unroll
           for (int x = 0; x < 16; ++x) o[x] = __float_as_uint(__uint_as_float(o[x]) * f);
           tmem_st16(tO + lane_off + c, o);
         }
       }
-      const float mm = m > -INFINITY ? m : 0.f;
-      float sum0 = 0.f, sum1 = 0.f;
-      uint32_t lo[32];
+      const float nm = sel ? -m : -INFINITY;                      // (m is finite for a row that has selected anything)
+      float2 sum = make_float2(0.f, 0.f);
+      auto probs = [&](uint32_t (&s)[16], int c) {                // 16 tokens: scores -> head and remainder, in place
+        if (!plain) {
+          const uint32_t bits = (uint32_t)(sel >> (16 * c));
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const float p0 = ex2(fmaf(__uint_as_float(s0[2 * j]), sc2, -mm)), p1 = ex2(fmaf(__uint_as_float(s0[2 * j + 1]), sc2, -mm));
-        sum0 += p0; sum1 += p1;
-        s0[j] = pack_bf16(p0, p1);
-        lo[j] = pack_bf16(p0 - bf16_lo(s0[j]), p1 - bf16_hi(s0[j]));
-      }
+          for (int j = 0; j < 16; ++j)
+            if (!(bits & (1u << j))) s[j] = 0xff800000u;
+        }
+        uint32_t pk[16];
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const float p0 = ex2(fmaf(__uint_as_float(s1[2 * j]), sc2, -mm)), p1 = ex2(fmaf(__uint_as_float(s1[2 * j + 1]), sc2, -mm));
-        sum0 += p0; sum1 += p1;
-        s0[16 + j] = pack_bf16(p0, p1);
-        lo[16 + j] = pack_bf16(p0 - bf16_lo(s0[16 + j]), p1 - bf16_hi(s0[16 + j]));
+        for (int j = 0; j < 8; ++j) {
+          const float2 x = __ffma2_rn(make_float2(__uint_as_float(s[2 * j]), __uint_as_float(s[2 * j + 1])), make_float2(sc2, sc2), make_float2(nm, nm));
+          const float2 pr = make_float2(ex2(x.x), ex2(x.y));
+          sum = __fadd2_rn(sum, pr);
+          pk[j] = pack_bf16(pr.x, pr.y);
+          const float2 lo = __fadd2_rn(pr, make_float2(-bf16_lo(pk[j]), -bf16_hi(pk[j])));
+          pk[8 + j] = pack_bf16(lo.x, lo.y);
+        }
+        tmem_st16(src + 16 * c, pk);
+      };
+#pragma unroll 1
+      for (int c = 0; c < 4; ++c) {                               // (rolled, like the other roles' loops: see the top)
+        uint32_t cur16[16];
+        tmem_ld16_async(src + 16 * c, cur16);
+        tmem_ld_wait16(cur16);
+        probs(cur16, c);
       }
-      l += sum0 + sum1;
-      tmem_st32(src, s0);
-      tmem_st32(src + 32, lo);
+      l += sum.x + sum.y;
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive1(&pa_ready[b]);
+      if (lane == 0) mbar_arrive1(&p_ready[b]);
     }
     if (!ok) *abort_flag = 1;
     l_s[row] = l;                                                 // (every S product has completed, or the CTA gives up)
@@ -510,74 +564,72 @@ __global__ void __launch_bounds__(kPaThreads, 1)
       const float cs = exp2f((float)(s_exp - kPhiExp));           // A carries 2^28, R shall carry 2^(14 + s_exp)
 #pragma unroll
       for (int x = 0; x < D; ++x) acc[x] = 0.f;
-      auto drain = [&](int grp) {
-        if (!warp_waits(r_full, grp & 1, lim)) { ok = false; return; }
-        tc_fence_after();
+#pragma unroll 1
+      for (int i = 0; i <= n_tiles && !warp_aborted(abort_flag); ++i) {
+        if (i == n_tiles || (i > 0 && i % kFlush == 0)) {         // a finished group of tiles, hidden behind the next one's first products
+          if (!warp_waits(r_full, ((i - 1) / kFlush) & 1, lim)) { ok = false; break; }
+          tc_fence_after();
 #pragma unroll
-        for (int c = 0; c < D; c += 32) {
-          float v[32];
-          tmem_ld32(tR + lane_off + c, v);
+          for (int c = 0; c < D; c += 32) {
+            float v[32];
+            tmem_ld32(tR + lane_off + c, v);
 #pragma unroll
-          for (int x = 0; x < 32; ++x) acc[c + x] += v[x];
+            for (int x = 0; x < 32; ++x) acc[c + x] += v[x];
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive1(r_empty);
+          if (i == n_tiles) break;
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive1(r_empty);
-      };
-      for (int i = 0; i < n_tiles && !warp_aborted(abort_flag); ++i) {
         tw.next();
         uint64_t sel, neg, posv;
         tile_masks(tw, cur, pos, base, sel, neg, posv);
         const int b = i & 1;
         const uint32_t src = tSA + b * 128 + 64 + lane_off;
-        if (!warp_waits(&sa_full[b], (i >> 1) & 1, lim)) { ok = false; break; }
+        if (!warp_waits(&a_full[b], (i >> 1) & 1, lim)) { ok = false; break; }
         tc_fence_after();
-        uint32_t a0[32], a1[32];
-        tmem_ld32_async(src, a0);
-        tmem_ld32_async(src + 32, a1);
-        tmem_ld_wait32(a0);
-        tmem_ld_wait32(a1);
         // signed coefficients: -A for selected tokens before the base, +A for unselected ones from it on, else 0 (never
         // 0 x A: a column past the sequence's end may hold anything)
-        const bool plain = posv == 0ull && (neg == 0ull || neg == ~0ull);
-        if (__all_sync(0xffffffffu, plain)) {
-          const bool on = neg != 0ull;
+        const bool plain = __all_sync(0xffffffffu, posv == 0ull && (neg == 0ull || neg == ~0ull)) && !tile_past(tw, r.L_end);
+        const float mul = neg ? -cs : 0.f;
+        auto coefs = [&](uint32_t (&x)[16], int c) {              // 16 tokens: A -> head and remainder, in place
+          if (plain) {
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            a0[j] = on ? __float_as_uint(__uint_as_float(a0[j]) * -cs) : 0u;
-            a1[j] = on ? __float_as_uint(__uint_as_float(a1[j]) * -cs) : 0u;
+            for (int j = 0; j < 16; j += 2) {
+              const float2 y = __fmul2_rn(make_float2(__uint_as_float(x[j]), __uint_as_float(x[j + 1])), make_float2(mul, mul));
+              x[j] = __float_as_uint(y.x);
+              x[j + 1] = __float_as_uint(y.y);
+            }
+          } else {
+            const uint32_t nb = (uint32_t)(neg >> (16 * c)), pb = (uint32_t)(posv >> (16 * c));
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              const float y = __uint_as_float(x[j]) * cs;
+              x[j] = (nb & (1u << j)) ? __float_as_uint(-y) : (pb & (1u << j)) ? __float_as_uint(y) : 0u;
+            }
           }
-        } else {
-          const uint32_t n0 = (uint32_t)neg, n1 = (uint32_t)(neg >> 32), q0 = (uint32_t)posv, q1 = (uint32_t)(posv >> 32);
+          uint32_t pk[16];
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const float x0 = __uint_as_float(a0[j]) * cs, x1 = __uint_as_float(a1[j]) * cs;
-            a0[j] = (n0 & (1u << j)) ? __float_as_uint(-x0) : (q0 & (1u << j)) ? __float_as_uint(x0) : 0u;
-            a1[j] = (n1 & (1u << j)) ? __float_as_uint(-x1) : (q1 & (1u << j)) ? __float_as_uint(x1) : 0u;
+          for (int j = 0; j < 8; ++j) {
+            const float2 c = make_float2(__uint_as_float(x[2 * j]), __uint_as_float(x[2 * j + 1]));
+            pk[j] = pack_bf16(c.x, c.y);
+            const float2 lo = __fadd2_rn(c, make_float2(-bf16_lo(pk[j]), -bf16_hi(pk[j])));
+            pk[8 + j] = pack_bf16(lo.x, lo.y);
           }
-        }
-        uint32_t hi[32];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const float c0 = __uint_as_float(a0[2 * j]), c1 = __uint_as_float(a0[2 * j + 1]);
-          hi[j] = pack_bf16(c0, c1);
-          a0[j] = pack_bf16(c0 - bf16_lo(hi[j]), c1 - bf16_hi(hi[j]));
-        }
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const float c0 = __uint_as_float(a1[2 * j]), c1 = __uint_as_float(a1[2 * j + 1]);
-          hi[16 + j] = pack_bf16(c0, c1);
-          a0[16 + j] = pack_bf16(c0 - bf16_lo(hi[16 + j]), c1 - bf16_hi(hi[16 + j]));
-        }
-        tmem_st32(src, hi);
-        tmem_st32(src + 32, a0);
+          tmem_st16(src + 16 * c, pk);
+        };
+#pragma unroll 1
+      for (int c = 0; c < 4; ++c) {                               // (rolled, like the other roles' loops: see the top)
+        uint32_t cur16[16];
+        tmem_ld16_async(src + 16 * c, cur16);
+        tmem_ld_wait16(cur16);
+        coefs(cur16, c);
+      }
         tmem_st_wait();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive1(&pa_ready[b]);
-        if (i > 0 && i % kFlush == 0) { drain(i / kFlush - 1); if (!ok) break; }
+        if (lane == 0) mbar_arrive1(&c_ready[b]);
       }
-      if (ok && !warp_aborted(abort_flag)) drain((n_tiles - 1) / kFlush);
     } else {
       if (!warp_waits(r_full, ((n_tiles - 1) / kFlush) & 1, lim)) ok = false;
     }
@@ -636,7 +688,7 @@ __global__ void __launch_bounds__(kPaThreads, 1)
         // only inside their row, and phi is elementwise given the token's log-sum-exp
         const unsigned char* kt = smem + SM::kK + b * SM::kTileBytes + tg * 16;
         unsigned char* ph = smem + SM::kPhi + b * 2 * SM::kTileBytes + tg * 16;
-#pragma unroll
+#pragma unroll 2
         for (int j = 0; j < SM::kTileBytes / 2048; ++j) {
           const float nl2 = fmaf(-lse_s[b * kPaTile + (tg >> 3) + 16 * (j & 3)], kLog2e, (float)kPhiExp);
           const uint4 raw = *reinterpret_cast<const uint4*>(kt + j * 2048);
@@ -644,27 +696,22 @@ __global__ void __launch_bounds__(kPaThreads, 1)
           uint32_t h[4], lo[4];
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            const float f0 = ex2(fmaf(bf16_lo(w[e]), a2, nl2)), f1 = ex2(fmaf(bf16_hi(w[e]), a2, nl2));
-            h[e] = pack_h2(f0, f1);
-            lo[e] = pack_h2(f0 - h2_lo(h[e]), f1 - h2_hi(h[e]));
+            const float2 x = __ffma2_rn(make_float2(bf16_lo(w[e]), bf16_hi(w[e])), make_float2(a2, a2), make_float2(nl2, nl2));
+            const float2 f = make_float2(ex2(x.x), ex2(x.y));
+            h[e] = pack_h2(f.x, f.y);
+            const float2 d = __fadd2_rn(f, make_float2(-h2_lo(h[e]), -h2_hi(h[e])));
+            lo[e] = pack_h2(d.x, d.y);
           }
           *reinterpret_cast<uint4*>(ph + j * 2048) = make_uint4(h[0], h[1], h[2], h[3]);
           *reinterpret_cast<uint4*>(ph + SM::kTileBytes + j * 2048) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
         }
       }
       // rows past the sequence's end hold whatever the cache memory holds; 0 x V must be 0
-      bool tail = false;
-      const int rows = B < kPaTile ? B : kPaTile;
-#pragma unroll
-      for (int s = 0; s < 4; ++s)
-        if (s * rows < kPaTile && tw.blk[s] >= 0 && tw.blk[s] * B + tw.off + rows > r.L_end) tail = true;
-      if (B < kPaTile && tw.blk[kPaTile / B - 1] < 0 && tw.blk[0] * B + rows > r.L_end) tail = true;
-      if (tail) {                                                 // uniform over the four warps
+      if (tile_past(tw, r.L_end)) {                               // uniform over the four warps
         if (!warp_waits(&v_full[b], par, lim)) { ok = false; break; }
         for (int x = tg; x < kPaTile * (D / 8); x += 128) {
           const int rw = x / (D / 8), ch = x % (D / 8);
-          int blk = B < kPaTile ? tw.blk[rw / B] : tw.blk[0];
-          if (blk < 0) blk = tw.blk[0];
+          const int blk = B < kPaTile ? tw.sub_block(rw / B) : tw.blk[0];
           const int tok = blk * B + tw.off + (B < kPaTile ? rw % B : rw);
           if (tok >= r.L_end)
             *reinterpret_cast<uint4*>(smem + SM::kV + b * SM::kTileBytes + (ch >> 3) * SM::kHalf + rw * 128 + (((ch & 7) ^ (rw & 7)) << 4)) =

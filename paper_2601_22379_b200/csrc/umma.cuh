@@ -29,6 +29,12 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t smem_addr, uint32_t
   return lo | (hi << 32);
 }
 
+// The same descriptor in two words, for loops that step through an operand: the low word grows by bytes / 16 (shared memory
+// ends below the 18 bits that the address field covers, so it never carries), the high word is the same for all.
+constexpr uint32_t kUmmaDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t umma_desc_lo(uint32_t smem_addr, uint32_t lead_bytes) { return (smem_addr >> 4) | ((lead_bytes >> 4) << 16); }
+__device__ __forceinline__ uint64_t umma_desc_of(uint32_t lo) { return ((uint64_t)kUmmaDescHi << 32) | lo; }
+
 // D (tensor memory) (+)= A B, A and B in shared memory.
 __device__ __forceinline__ void umma_ss(uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
@@ -38,14 +44,67 @@ __device__ __forceinline__ void umma_ss(uint32_t tmem_d, uint64_t desc_a, uint64
       ::"r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate), "r"(0u)
       : "memory");
 }
-// The same with A in tensor memory (row m in lane m, two 16-bit k per 32-bit column).
-__device__ __forceinline__ void umma_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate) {
+// The same for a whole warp whose lanes all hold the operands, `one` non-zero in the lane that issues.  Operands that are
+// the same in every lane of a converged warp can stay in uniform registers; issued from a branch that only one lane takes,
+// an MMA cost 75 to 110 cycles in a loop beside busy warps, this way 50 to 65.
+__device__ __forceinline__ void umma_ss_one(uint32_t one, uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p, q;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {%5, %5, %5, %5}, p;\n\t}"
-      ::"r"(tmem_d), "r"(tmem_a), "l"(desc_b), "r"(idesc), "r"(accumulate), "r"(0u)
+      "setp.ne.b32 q, %6, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}"
+      ::"r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate), "r"(0u), "r"(one)
       : "memory");
+}
+// Four k-steps in one go (the predicates are formed once): D (+)= A B + three more that always accumulate.  DA, DB: what the
+// low descriptor words grow by per step.
+template <uint32_t DA, uint32_t DB>
+__device__ __forceinline__ void umma_ss4_one(uint32_t one, uint32_t tmem_d, uint32_t lo_a, uint32_t lo_b, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %10, 0;\n\t"
+      "setp.ne.b32 q, %12, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %5, %9, {%11, %11, %11, %11}, p;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %2, %6, %9, {%11, %11, %11, %11}, 1;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %3, %7, %9, {%11, %11, %11, %11}, 1;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %4, %8, %9, {%11, %11, %11, %11}, 1;\n\t}"
+      ::"r"(tmem_d), "l"(umma_desc_of(lo_a)), "l"(umma_desc_of(lo_a + DA)), "l"(umma_desc_of(lo_a + 2 * DA)), "l"(umma_desc_of(lo_a + 3 * DA)),
+        "l"(umma_desc_of(lo_b)), "l"(umma_desc_of(lo_b + DB)), "l"(umma_desc_of(lo_b + 2 * DB)), "l"(umma_desc_of(lo_b + 3 * DB)),
+        "r"(idesc), "r"(accumulate), "r"(0u), "r"(one)
+      : "memory");
+}
+// ... with A in tensor memory (row m in lane m, two 16-bit k per 32-bit column), DA columns further per step.
+template <uint32_t DA, uint32_t DB>
+__device__ __forceinline__ void umma_ts4_one(uint32_t one, uint32_t tmem_d, uint32_t tmem_a, uint32_t lo_b, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %10, 0;\n\t"
+      "setp.ne.b32 q, %12, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %5, %9, {%11, %11, %11, %11}, p;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%2], %6, %9, {%11, %11, %11, %11}, 1;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%3], %7, %9, {%11, %11, %11, %11}, 1;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%4], %8, %9, {%11, %11, %11, %11}, 1;\n\t}"
+      ::"r"(tmem_d), "r"(tmem_a), "r"(tmem_a + DA), "r"(tmem_a + 2 * DA), "r"(tmem_a + 3 * DA),
+        "l"(umma_desc_of(lo_b)), "l"(umma_desc_of(lo_b + DB)), "l"(umma_desc_of(lo_b + 2 * DB)), "l"(umma_desc_of(lo_b + 3 * DB)),
+        "r"(idesc), "r"(accumulate), "r"(0u), "r"(one)
+      : "memory");
+}
+__device__ __forceinline__ void umma_commit_one(uint32_t one, uint64_t* bar) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar)), "r"(one)
+      : "memory");
+}
+// One lane of a converged warp.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b32 d;\n\t"
+      "elect.sync d|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r));
+  return r;
 }
 // Arrives on the barrier once every tcgen05.mma issued so far by this thread has completed.
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
@@ -85,6 +144,20 @@ __device__ __forceinline__ void tmem_ld_wait32(uint32_t (&r)[32]) {
                  "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
                :: "memory");
 }
+__device__ __forceinline__ void tmem_ld16_async(uint32_t addr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                 "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(addr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait16(uint32_t (&r)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :: "memory");
+}
 __device__ __forceinline__ void tmem_ld32(uint32_t addr, float (&v)[32]) {
   uint32_t r[32];
   tmem_ld32_async(addr, r);
@@ -92,22 +165,12 @@ __device__ __forceinline__ void tmem_ld32(uint32_t addr, float (&v)[32]) {
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
-// 16 / 32 consecutive columns of this thread's lane written; tmem_st_wait() before anybody is told.
+// 16 consecutive columns of this thread's lane written; tmem_st_wait() before anybody is told.
 __device__ __forceinline__ void tmem_st16(uint32_t addr, const uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
       ::"r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
         "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-      : "memory");
-}
-__device__ __forceinline__ void tmem_st32(uint32_t addr, const uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
-      ::"r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]),
-        "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]),
-        "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
       : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
