@@ -89,10 +89,18 @@ __device__ __forceinline__ uint64_t low_bits(int n) { return n >= 64 ? ~0ull : (
 // `off` inside it; smaller ones: 64 / B consecutive set bits together (blk[s] < 0: none left).
 struct TileWalk {
   const uint32_t* bm;
-  int w, B;
+  int w, w_end, B;
   uint32_t word;
   int blk[4], off;
-  __device__ __forceinline__ void start(const uint32_t* bitmap, int B_) { bm = bitmap; w = 0; B = B_; word = bm[0]; off = B_; blk[0] = -1; }
+  __device__ __forceinline__ void start(const uint32_t* bitmap, int B_, int last_blk) {
+    bm = bitmap;
+    w = 0;
+    w_end = (last_blk >> 5) + 1;
+    B = B_;
+    word = bm[0];
+    off = B_;
+    blk[0] = -1;
+  }
   // Block number s of a tile of small blocks (of a short last tile: the first again).  A select, so that blk[] stays in registers.
   __device__ __forceinline__ int sub_block(int s) const {
     int r = blk[0];
@@ -102,7 +110,7 @@ struct TileWalk {
   }
   __device__ __forceinline__ int next_bit() {
     while (word == 0u) {
-      if (++w >= kPfMaxBlocks / 32) { w = kPfMaxBlocks / 32; return -1; }
+      if (++w >= w_end) { w = w_end; return -1; }                 // (a tile of small blocks may run past the last one)
       word = bm[w];
     }
     const int i = w * 32 + __ffs(word) - 1;
@@ -344,7 +352,7 @@ __global__ void __launch_bounds__(kPaThreads, 1)
       uint64_t *full = is_k ? k_full : v_full, *empty = is_k ? k_empty : v_empty;
       const CUtensorMap* map = is_k ? &map_k : &map_v;
       TileWalk tw;
-      tw.start(bitmap, B);
+      tw.start(bitmap, B, own_hi);
       int issued = 0;
       for (int i = 0; i < n_tiles && !*abort_flag; ++i) {
         tw.next();
@@ -448,7 +456,7 @@ __global__ void __launch_bounds__(kPaThreads, 1)
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
     const float sc2 = p.sm_scale * kLog2e;
     TileWalk tw;
-    tw.start(bitmap, B);
+    tw.start(bitmap, B, own_hi);
     SelCursor cur;
     cur.start(pos >= 0 ? pc.sel + ((size_t)r.u * pc.T + (pos - r.first)) * p.top_k : nullptr, p.top_k);
     float m = -INFINITY, l = 0.f;
@@ -558,7 +566,7 @@ __global__ void __launch_bounds__(kPaThreads, 1)
     float acc[RLA ? D : 1];
     if constexpr (RLA) {
       TileWalk tw;
-      tw.start(bitmap, B);
+      tw.start(bitmap, B, own_hi);
       SelCursor cur;
       cur.start(pos >= 0 ? pc.sel + ((size_t)r.u * pc.T + (pos - r.first)) * p.top_k : nullptr, p.top_k);
       const float cs = exp2f((float)(s_exp - kPhiExp));           // A carries 2^28, R shall carry 2^(14 + s_exp)
@@ -676,7 +684,7 @@ __global__ void __launch_bounds__(kPaThreads, 1)
     const int tg = tid - 384;
     const float a2 = p.phi_scale * kLog2e;
     TileWalk tw;
-    tw.start(bitmap, B);
+    tw.start(bitmap, B, own_hi);
     bool ok = true;
     for (int i = 0; i < n_tiles && !warp_aborted(abort_flag); ++i) {
       tw.next();
