@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kPsThreads, 2) prefill_score_kernel(const Para
 // (counting the keys at or above a candidate, with a stop as soon as exactly k are), which needs no scratch and no sort;
 // the list then comes out in ascending order by ballots.
 template <int W, int NK>
-__global__ void __launch_bounds__(256) prefill_select_kernel(const Params p, const PrefillChunk pc, int* __restrict__ sel_user) {
+__global__ void __launch_bounds__(256, 2) prefill_select_kernel(const Params p, const PrefillChunk pc, int* __restrict__ sel_user) {
   __shared__ float red_s[8][2];
   __shared__ int cnt_s[2][8];
   constexpr int L = W * 32;                                    // lanes of a position
@@ -336,13 +336,14 @@ cudaError_t launch_prefill_score(const Params& p, const PrefillChunk& c, const v
   return p.d == 128 ? score_d<128, false>(p, c, q, max_blocks_seen, sm_count, s) : score_d<64, false>(p, c, q, max_blocks_seen, sm_count, s);
 }
 
-// Selection for the same positions.  Up to 512 blocks a warp holds a position's keys; above, a CTA does.
+// Selection for the same positions.  Up to 1024 blocks a warp holds a position's keys; above, a CTA does (513 blocks, 512 positions x 16
+// units: 121 us by CTAs, whose barriers cost more than the wider registers of one warp, 55 us by warps).
 cudaError_t launch_prefill_select(const Params& p, const PrefillChunk& c, int max_blocks_seen, int* sel_user, cudaStream_t s) {
   if (max_blocks_seen <= 32 * 2) return select_w<1, 2>(p, c, sel_user, s);
   if (max_blocks_seen <= 32 * 4) return select_w<1, 4>(p, c, sel_user, s);
   if (max_blocks_seen <= 32 * 8) return select_w<1, 8>(p, c, sel_user, s);
   if (max_blocks_seen <= 32 * 16) return select_w<1, 16>(p, c, sel_user, s);
-  if (max_blocks_seen <= 256 * 4) return select_w<8, 4>(p, c, sel_user, s);
+  if (max_blocks_seen <= 32 * 32) return select_w<1, 32>(p, c, sel_user, s);
   if (max_blocks_seen <= 256 * 16) return select_w<8, 16>(p, c, sel_user, s);
   return select_w<8, 64>(p, c, sel_user, s);
 }

@@ -12,13 +12,15 @@ namespace {
 
 constexpr int kOwnThreads = 256;
 constexpr int kOwnGroup = 32;              // positions whose prefix statistics are in shared memory together
+constexpr int kOwnRows = 4;                // (position, head) rows a warp works on side by side
+template <int VEC> struct QueryVec { using type = uint2; };      // a lane's VEC query elements
+template <> struct QueryVec<2> { using type = uint32_t; };
 
 // One CTA per (block the chunk touches, unit).  D threads walk the block's tokens, one channel each: running sum and
 // running sum of squared deviations (each token's deviation from the mean before and after it: Welford's update, no
 // cancellation), so that the statistics of ALL prefixes of the block cost one pass instead of one pass per prefix.
 // After every 32 tokens the eight warps form the dots of those prefixes with their positions' queries.
-// Bound by that serial chain (16 cycles per token).  64-token blocks, d = 128: 50 us -> 6 us for 144 CTAs against two
-// passes per prefix.
+// Bound by that serial chain and the load latencies around it.
 template <int D>
 __global__ void __launch_bounds__(kOwnThreads) prefill_own_kernel(const Params p, const PrefillChunk pc,
                                                                   const __nv_bfloat16* __restrict__ q, float* __restrict__ out,
@@ -52,6 +54,20 @@ __global__ void __launch_bounds__(kOwnThreads) prefill_own_kernel(const Params p
   const __nv_bfloat16* kc = reinterpret_cast<const __nv_bfloat16*>(p.k_cache) + ((size_t)r.u * p.max_blocks * p.B + t0) * D;
   const bool round16 = (p.flags & kStatsBf16) != 0;
   float sum = 0.f, m2 = 0.f, mean = 0.f;
+  // Queries of kOwnRows (position, head) rows of the group that starts at token g0, requested before they are needed:
+  // fetched one row at a time where they are used, their latency was half of this kernel's time (33 -> 15 us for 144 CTAs).
+  using QV = typename QueryVec<VEC>::type;
+  QV qn[kOwnRows];
+  auto fetch = [&](int g0, int row0, int ng) {
+#pragma unroll
+    for (int i = 0; i < kOwnRows; ++i) {
+      const int row = row0 + i, pos = t0 + g0 + row / G;
+      const bool ok = row < ng * G && pos >= r.L0;
+      const size_t off = (((size_t)r.b * pc.T + (ok ? pos - r.first : 0)) * p.Hq + (size_t)r.h * G + row % G) * D + lane * VEC;
+      qn[i] = ok ? __ldg(reinterpret_cast<const QV*>(q + off)) : QV();
+    }
+  };
+  fetch(0, warp * kOwnRows, min(kOwnGroup, cnt));
   __syncthreads();
   for (int g0 = 0; g0 < cnt; g0 += kOwnGroup) {
     const int ng = min(kOwnGroup, cnt - g0);
@@ -73,28 +89,33 @@ __global__ void __launch_bounds__(kOwnThreads) prefill_own_kernel(const Params p
       }
     }
     __syncthreads();
-    for (int j = warp; j < ng; j += kOwnThreads / 32) {
-      const int pos = t0 + g0 + j;
-      if (pos < r.L0) continue;                                // a token from before the chunk
-      const int t = pos - r.first;
-      float mv[VEC], vv[VEC];
-      load_vec<VEC>(mean_s + j * D + lane * VEC, mv);
-      load_vec<VEC>(var_s + j * D + lane * VEC, vv);
-      const __nv_bfloat16* qp = q + (((size_t)r.b * pc.T + t) * p.Hq + (size_t)r.h * G) * D + lane * VEC;
-      for (int g = 0; g < G; ++g) {
-        float x[VEC], d2[2] = {0.f, 0.f};
-        load_vec<VEC>(qp + (size_t)g * D, x);
+    for (int row0 = warp * kOwnRows; row0 < ng * G; row0 += kOwnRows * (kOwnThreads / 32)) {
+      float vals[2 * kOwnRows];
+#pragma unroll
+      for (int i = 0; i < kOwnRows; ++i) {
+        const int j = min((row0 + i) / G, ng - 1);
+        float x[VEC], mv[VEC], vv[VEC], dm = 0.f, dv = 0.f;
+        load_vec<VEC>(reinterpret_cast<const __nv_bfloat16*>(&qn[i]), x);
+        load_vec<VEC>(mean_s + j * D + lane * VEC, mv);
+        load_vec<VEC>(var_s + j * D + lane * VEC, vv);
 #pragma unroll
         for (int v = 0; v < VEC; ++v) {
           const float qh = x[v] * p.sm_scale;
-          d2[0] = fmaf(qh, mv[v], d2[0]);
-          d2[1] = fmaf(0.5f * qh * qh, vv[v], d2[1]);
+          dm = fmaf(qh, mv[v], dm);
+          dv = fmaf(0.5f * qh * qh, vv[v], dv);
         }
-        warp_reduce_multi<2>(d2, lane);                        // lanes 0..15: the mean dot, 16..31: the variance dot
-        const float dv = (p.flags & 2u) ? 0.f : __shfl_sync(0xffffffffu, d2[0], 16);
-        if (lane == 0) pc.ell_own[((size_t)r.u * pc.T + t) * G + g] = logf((float)(g0 + j + 1)) + d2[0] + __logf(1.f + dv);
+        vals[i] = dm;
+        vals[kOwnRows + i] = dv;
       }
+      fetch(g0, row0 + kOwnRows * (kOwnThreads / 32), ng);       // the next rows of this group ...
+      warp_reduce_multi<2 * kOwnRows>(vals, lane);               // value lane / 4: the mean dots, then the variance dots
+      float dv = __shfl_xor_sync(0xffffffffu, vals[0], 16);
+      if (p.flags & 2u) dv = 0.f;
+      const int row = row0 + (lane >> 2), j = row / G, pos = t0 + g0 + j;
+      if (lane < 16 && (lane & 3) == 0 && row < ng * G && pos >= r.L0)
+        pc.ell_own[((size_t)r.u * pc.T + (pos - r.first)) * G + row % G] = logf((float)(g0 + j + 1)) + vals[0] + __logf(1.f + dv);
     }
+    if (g0 + kOwnGroup < cnt) fetch(g0 + kOwnGroup, warp * kOwnRows, min(kOwnGroup, cnt - g0 - kOwnGroup));   // ... or the first of the next
     __syncthreads();
   }
 }
@@ -187,25 +208,34 @@ __global__ void __launch_bounds__(256) prefill_local_state_kernel(const Params p
 }
 
 // The ranges' contributions become, in place, the state before each range; the cache's state is advanced over the chunk.
-// One thread per four entries; bound by the memory traffic (64 KB read and written per range and unit at d = 128).
+// One thread per two entries, the next eight ranges requested before this eight are written.  Bound by the memory traffic
+// (64 KB read and written per range and unit at d = 128): 129 ranges x 8 units (135 MB) 19 us = 7 TB/s, partly from L2;
+// with four entries a thread and nothing ahead 74 us.
 template <int D>
 __global__ void __launch_bounds__(128) prefill_scan_state_kernel(const Params p, const PrefillChunk pc) {
-  constexpr int N4 = D * D / 4, AHEAD = 8;
+  constexpr int N2 = D * D / 2, AHEAD = 8;
   const int idx = blockIdx.x * 128 + threadIdx.x;
   const int u = blockIdx.y;
-  float4* st = reinterpret_cast<float4*>(p.state + (size_t)u * D * D) + idx;
-  float4* x = reinterpret_cast<float4*>(pc.snap + (size_t)u * pc.n_sb * D * D) + idx;
-  float4 s = *st;
-  for (int i0 = 0; i0 < pc.n_sb; i0 += AHEAD) {
-    float4 a[AHEAD];
+  float2* st = reinterpret_cast<float2*>(p.state + (size_t)u * D * D) + idx;
+  float2* x = reinterpret_cast<float2*>(pc.snap + (size_t)u * pc.n_sb * D * D) + idx;
+  float2 s = *st;
+  float2 nx[AHEAD];
+  auto fetch = [&](int i0) {
 #pragma unroll
     for (int j = 0; j < AHEAD; ++j)
-      if (i0 + j < pc.n_sb) a[j] = x[(size_t)(i0 + j) * N4];
+      if (i0 + j < pc.n_sb) nx[j] = x[(size_t)(i0 + j) * N2];
+  };
+  fetch(0);
+  for (int i0 = 0; i0 < pc.n_sb; i0 += AHEAD) {
+    float2 a[AHEAD];
+#pragma unroll
+    for (int j = 0; j < AHEAD; ++j) a[j] = nx[j];
+    fetch(i0 + AHEAD);
 #pragma unroll
     for (int j = 0; j < AHEAD; ++j) {
       if (i0 + j < pc.n_sb) {
-        x[(size_t)(i0 + j) * N4] = s;
-        s.x += a[j].x; s.y += a[j].y; s.z += a[j].z; s.w += a[j].w;
+        x[(size_t)(i0 + j) * N2] = s;
+        s.x += a[j].x; s.y += a[j].y;
       }
     }
   }
@@ -229,7 +259,7 @@ cudaError_t state_d(const Params& p, const PrefillChunk& c, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   kern<<<dim3(c.n_sb, p.batch * p.Hkv), 256, smem, s>>>(p, c);
   ++g_launch_count;
-  prefill_scan_state_kernel<D><<<dim3(D * D / 4 / 128, p.batch * p.Hkv), 128, 0, s>>>(p, c);
+  prefill_scan_state_kernel<D><<<dim3(D * D / 2 / 128, p.batch * p.Hkv), 128, 0, s>>>(p, c);
   ++g_launch_count;
   return cudaGetLastError();
 }
