@@ -3,13 +3,13 @@
 // state S_bar += phi(k_t)^T v_t in fp32 (Section 3.2, Eq. rla-impl-1, "Numerical Stability").
 //
 // Appends of up to 32 tokens per sequence (the decode loop) run as ONE fused kernel, see append_fused_kernel.
-// Bulk appends (prefill) run as three kernels in stream order, all reading the OLD sequence lengths until the
-// last one bumps them:
+// Longer appends of a bf16 cache with d = 128 run as one pass on the tensor cores (append_bulk.cu); all others as three
+// kernels in stream order, all reading the OLD sequence lengths until the last one bumps them:
 //   block  : one CTA per touched block: its keys (cached ones below the old length, new ones above) are staged in
 //            shared memory once; from there the new tokens go to the cache (k_new, v_new -> cache), their
 //            logsumexp of phi_scale * k to tok_lse, and the block's mean / variance records are recomputed (two
 //            exact passes, so the result does not depend on how the tokens were split across append calls)
-//   state  : rank-n update of S_bar (tensor cores for long bf16 appends, else rows tiled over CTAs on the FMA pipe)
+//   state  : rank-n update of S_bar (rows tiled over CTAs on the FMA pipe)
 //   lengths: seq_lens += n_new
 #include "spla_internal.h"
 
@@ -17,7 +17,6 @@ namespace spla {
 
 constexpr int kStateRows = 16;     // rows of S_bar per CTA
 constexpr int kStateTokens = 32;   // tokens staged per inner step
-constexpr int kStateUmmaMinTokens = 256;   // appends at least this long take the tensor-core state kernel
 
 __device__ __forceinline__ int tokens_to_add(const Params& p, const int* n_new, int max_new, int b, int L) {
   int n = n_new ? n_new[b] : max_new;
@@ -173,15 +172,8 @@ __global__ void __launch_bounds__(kStatThreads) append_block_kernel(const Params
   for (int t = t_new + warp; t < cnt; t += kStatThreads / 32) {
     float k[VEC];
     load_vec<VEC>(tile + (size_t)t * D + lane * VEC, k);
-    float mx = -INFINITY;
-#pragma unroll
-    for (int v = 0; v < VEC; ++v) { k[v] *= p.phi_scale; mx = fmaxf(mx, k[v]); }
-    mx = warp_max(mx);
-    float s = 0.f;
-#pragma unroll
-    for (int v = 0; v < VEC; ++v) s += expf(k[v] - mx);
-    s = warp_sum(s);
-    if (lane == 0) p.tok_lse[blk_tok0 + t] = mx + logf(s);
+    const float lse = token_lse<VEC>(k, p.phi_scale);
+    if (lane == 0) p.tok_lse[blk_tok0 + t] = lse;
   }
 
   const int c = tid % D;
@@ -246,7 +238,7 @@ __global__ void append_lengths_kernel(const Params p, const int* __restrict__ n_
 // log-sum-exp is recomputed from the new keys).  Every CTA reads the old lengths; the last CTA to have read them
 // (atomic ticket at the start, nobody waits) advances them.
 constexpr int kFusedThreads = 256;
-constexpr int kFusedMaxNew = 32;
+constexpr int kFusedMaxNew = kAppendStepMax;
 
 template <typename T, int D, bool WIN>
 __global__ void __launch_bounds__(kFusedThreads, 4) append_fused_kernel(const Params p, const T* __restrict__ k_new,
@@ -307,15 +299,8 @@ __global__ void __launch_bounds__(kFusedThreads, 4) append_fused_kernel(const Pa
       load_vec<VEC>(kn + (size_t)i * D + lane * VEC, k);
       copy_bytes<VEC * sizeof(T)>(reinterpret_cast<T*>(p.k_cache) + pos * D + lane * VEC, kn + (size_t)i * D + lane * VEC);
       copy_bytes<VEC * sizeof(T)>(reinterpret_cast<T*>(p.v_cache) + pos * D + lane * VEC, vn + (size_t)i * D + lane * VEC);
-      float mx = -INFINITY;
-#pragma unroll
-      for (int v = 0; v < VEC; ++v) { k[v] *= p.phi_scale; mx = fmaxf(mx, k[v]); }
-      mx = warp_max(mx);
-      float sm = 0.f;
-#pragma unroll
-      for (int v = 0; v < VEC; ++v) sm += expf(k[v] - mx);
-      sm = warp_sum(sm);
-      if (lane == 0) p.tok_lse[pos] = mx + logf(sm);
+      const float lse = token_lse<VEC>(k, p.phi_scale);
+      if (lane == 0) p.tok_lse[pos] = lse;
     }
   } else if ((role -= n_copy) < n_stats) {
     // ---- statistics role: one touched block; cached keys below the old length, new keys above it -----------
@@ -391,7 +376,7 @@ __global__ void __launch_bounds__(kFusedThreads, 4) append_fused_kernel(const Pa
 
 template <typename T, int D>
 static cudaError_t launch_typed(const Params& p, const void* k_new, const void* v_new, const int* n_new, int max_new,
-                                const AttendMaps* state_maps, cudaStream_t stream) {
+                                const AttendMaps* maps, const AttendMaps* fresh_maps, cudaStream_t stream) {
   const int U = p.batch * p.Hkv;
   const T* kn = reinterpret_cast<const T*>(k_new);
   const T* vn = reinterpret_cast<const T*>(v_new);
@@ -405,6 +390,9 @@ static cudaError_t launch_typed(const Params& p, const void* k_new, const void* 
     return launch_ex(kern, dim3(n_copy + n_stats + n_state, U), dim3(kFusedThreads), 0, stream, 0, true,
                      p, kn, vn, n_new, max_new, n_copy, n_stats);
   }
+  // bf16 with d = 128: everything in one pass, the state on the tensor cores; the rest in three kernels
+  if (sizeof(T) == 2 && D == 128 && maps && maps->valid && fresh_maps && fresh_maps->valid)
+    return launch_append_bulk(p, *maps, *fresh_maps, n_new, max_new, stream);
   {
     const size_t tile_bytes = (size_t)p.B * D * sizeof(T);
     auto kern = append_block_kernel<T, D>;
@@ -413,15 +401,8 @@ static cudaError_t launch_typed(const Params& p, const void* k_new, const void* 
     ++g_launch_count;
   }
   if (!(p.flags & 4u)) {
-    // long appends of a bf16 cache with d = 128: the rank-n update is a dense contraction, done on the tensor cores
-    // from the tokens the copy kernel has just stored; everything else on the FMA pipe
-    if (sizeof(T) == 2 && D == 128 && state_maps && state_maps->valid && max_new >= kStateUmmaMinTokens) {
-      const cudaError_t e = launch_state_umma(p, state_maps, n_new, max_new, stream);
-      if (e != cudaSuccess) return e;
-    } else {
-      append_state_kernel<T, D><<<dim3(D / kStateRows, U), D, 0, stream>>>(p, kn, vn, n_new, max_new);
-      ++g_launch_count;
-    }
+    append_state_kernel<T, D><<<dim3(D / kStateRows, U), D, 0, stream>>>(p, kn, vn, n_new, max_new);
+    ++g_launch_count;
   }
   append_lengths_kernel<<<(p.batch + 127) / 128, 128, 0, stream>>>(p, n_new, max_new);
   ++g_launch_count;
@@ -429,12 +410,12 @@ static cudaError_t launch_typed(const Params& p, const void* k_new, const void* 
 }
 
 cudaError_t launch_append(const Params& p, const void* k_new, const void* v_new, const int* n_new, int max_new,
-                          const AttendMaps* state_maps, cudaStream_t stream) {
+                          const AttendMaps* maps, const AttendMaps* fresh_maps, cudaStream_t stream) {
   if (p.kv_bf16)
-    return p.d == 128 ? launch_typed<__nv_bfloat16, 128>(p, k_new, v_new, n_new, max_new, state_maps, stream)
-                      : launch_typed<__nv_bfloat16, 64>(p, k_new, v_new, n_new, max_new, state_maps, stream);
-  return p.d == 128 ? launch_typed<float, 128>(p, k_new, v_new, n_new, max_new, state_maps, stream)
-                    : launch_typed<float, 64>(p, k_new, v_new, n_new, max_new, state_maps, stream);
+    return p.d == 128 ? launch_typed<__nv_bfloat16, 128>(p, k_new, v_new, n_new, max_new, maps, fresh_maps, stream)
+                      : launch_typed<__nv_bfloat16, 64>(p, k_new, v_new, n_new, max_new, maps, fresh_maps, stream);
+  return p.d == 128 ? launch_typed<float, 128>(p, k_new, v_new, n_new, max_new, maps, fresh_maps, stream)
+                    : launch_typed<float, 64>(p, k_new, v_new, n_new, max_new, maps, fresh_maps, stream);
 }
 
 }  // namespace spla

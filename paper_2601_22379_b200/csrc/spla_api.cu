@@ -23,7 +23,7 @@ struct spla_cache {
   int attend_occ[5] = {-2, -2, -2, -2, -2};   // by log2 of the cluster size
   int sm_count;
   AttendMaps maps;
-  AttendMaps state_maps;   // the same caches in boxes of 64 tokens, for the tensor-core state kernel
+  AttendMaps state_maps;   // the same caches in boxes of 64 tokens, for the one-pass bulk append
   AttendMaps prefill_maps; // ... of one block, at most 64 tokens, for the tensor-core prefill path
 };
 
@@ -131,7 +131,7 @@ static bool prefill_on_tensor_cores(const spla_config_t* c) {
 }
 
 struct WorkspaceLayout {
-  size_t ell, chunk_part, scores, obar_part, sel, n_sel, att_acc, att_ml, score_ticket, attend_ticket, append_ticket, state_part, state_ticket, status, total;
+  size_t ell, chunk_part, scores, obar_part, sel, n_sel, att_acc, att_ml, score_ticket, attend_ticket, append_ticket, state_part, status, total;
   int max_chunks;
 };
 
@@ -154,8 +154,7 @@ static WorkspaceLayout workspace_layout(const spla_config_t* c) {
   w.score_ticket = take(U * 4);
   w.attend_ticket = take(U * 4);
   w.append_ticket = take(256);
-  w.state_part = take(state_umma_part_bytes((int)U, (int)d));
-  w.state_ticket = take(U * 4);
+  w.state_part = take(append_bulk_part_bytes((int)U, (int)d));
   w.status = take(256);
   w.total = off;
   return w;
@@ -225,7 +224,7 @@ extern "C" int spla_init_cache(const spla_config_t* config, const spla_buffers_t
   p.att_acc = (float*)(ws + w.att_acc); p.att_ml = (float*)(ws + w.att_ml);
   p.score_ticket = (int*)(ws + w.score_ticket); p.attend_ticket = (int*)(ws + w.attend_ticket);
   p.append_ticket = (int*)(ws + w.append_ticket);
-  p.state_part = (float*)(ws + w.state_part); p.state_ticket = (int*)(ws + w.state_ticket);
+  p.state_part = (float*)(ws + w.state_part);
   p.status = (int*)(ws + w.status);
   p.max_chunks = w.max_chunks;
   p.tile_rows = (p.B * p.d * 2 > 16384 && p.B % 32 == 0) ? p.B / 2 : p.B;
@@ -271,12 +270,23 @@ extern "C" int spla_set_length_bound(spla_cache_t* c, int32_t max_seq_len) {
   return SPLA_OK;
 }
 
+// The append with tensor maps over the caller's new tokens where the one-pass kernel wants them.
+static cudaError_t append_launch(const spla_cache* c, const Params& p, const void* k_new, const void* v_new, const int32_t* n_new,
+                                 int32_t max_new, cudaStream_t s) {
+  AttendMaps fresh;
+  fresh.valid = false;
+  const unsigned long long rows = (unsigned long long)p.batch * p.Hkv * max_new;
+  if (c->state_maps.valid && max_new > kAppendStepMax && rows >= 64 && rows < (1ull << 31))
+    fresh.valid = make_kv_map(fresh.k, const_cast<void*>(k_new), p.d, 64, rows) && make_kv_map(fresh.v, const_cast<void*>(v_new), p.d, 64, rows);
+  return launch_append(p, k_new, v_new, n_new, max_new, &c->state_maps, &fresh, s);
+}
+
 extern "C" int spla_append_tokens(spla_cache_t* c, const void* k_new, const void* v_new, const int32_t* n_new,
                                   int32_t max_new, void* stream) {
   if (!c || !k_new || !v_new || max_new < 1) return SPLA_ERR_INVALID_ARG;
   if (!aligned(k_new, 16) || !aligned(v_new, 16)) return SPLA_ERR_INVALID_ARG;
   if (c->len_bound + max_new > c->cfg.max_context) return SPLA_ERR_CAPACITY;
-  cudaError_t e = launch_append(c->p, k_new, v_new, n_new, max_new, &c->state_maps, (cudaStream_t)stream);
+  cudaError_t e = append_launch(c, c->p, k_new, v_new, n_new, max_new, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "spla_append_tokens");
   c->len_bound += max_new;
   return SPLA_OK;
@@ -592,7 +602,7 @@ extern "C" int spla_prefill(spla_cache_t* c, const void* k_new, const void* v_ne
   {
     Params pa = c->p;
     pa.flags |= SPLA_NO_RLA;
-    cudaError_t e = launch_append(pa, k_new, v_new, nullptr, T, nullptr, s);
+    cudaError_t e = append_launch(c, pa, k_new, v_new, nullptr, T, s);
     if (e != cudaSuccess) return cuda_fail(e, "spla_prefill/append");
     c->len_bound += T;
   }

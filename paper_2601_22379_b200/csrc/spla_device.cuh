@@ -58,8 +58,7 @@ struct Params {
   int* score_ticket;   // [U]
   int* attend_ticket;  // [U]
   int* append_ticket;  // [1]
-  float* state_part;   // [U][splits][d][d]  partial S_bar updates of the tensor-core state kernel
-  int* state_ticket;   // [U]
+  float* state_part;   // [U][splits][d][d]  partial S_bar updates of the one-pass bulk append
   int* status;         // [1]
   int max_chunks;
   // Prefill-shaped forward (general kernels only): the grid's second dimension then counts *virtual* units, one per
@@ -109,6 +108,11 @@ __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 
+// Log-sum-exp of phi_scale * k from its base-2 pieces: mx2 = max(k) * (phi_scale log2 e), sum = sum_c 2^(k_c phi_scale log2 e
+// - mx2).  Every append path forms mx2 by one rounded product and sums the terms in the same order (four consecutive
+// channels, then halves of the token: + 64, + 32, ... channels), so that tok_lse has the same bits whichever wrote it.
+__device__ __forceinline__ float lse_from_base2(float mx2, float sum) { return __fmul_rn(__fadd_rn(mx2, log2f(sum)), kLn2); }
+
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -118,6 +122,20 @@ __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+
+// The log-sum-exp of one token by one warp, VEC = d / 32 channels per lane.
+template <int VEC>
+__device__ __forceinline__ float token_lse(const float (&k)[VEC], float phi_scale) {
+  const float a2 = phi_scale * kLog2e;
+  float mx = -INFINITY;
+#pragma unroll
+  for (int v = 0; v < VEC; ++v) mx = fmaxf(mx, k[v]);
+  const float mx2 = __fmul_rn(warp_max(mx), a2);
+  float s = ex2(fmaf(k[0], a2, -mx2));
+#pragma unroll
+  for (int v = 1; v < VEC; ++v) s += ex2(fmaf(k[v], a2, -mx2));
+  return lse_from_base2(mx2, warp_sum(s));
 }
 
 // Sums N (a power of two, <= 32) per-lane values across the warp with N - 1 + log2(32 / N) shuffles instead

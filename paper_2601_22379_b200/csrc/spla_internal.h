@@ -87,10 +87,10 @@ struct AttendMaps {                      // TMA tensor maps (CUtensorMap) of the
   alignas(64) unsigned char v[128];
   bool valid;
 };
-// state_umma.cu (bulk S_bar update on tcgen05 tensor cores: bf16 cache, d = 128; maps with boxes of 64 tokens)
-int state_umma_splits(int units);
-size_t state_umma_part_bytes(int units, int d);
-cudaError_t launch_state_umma(const Params& p, const AttendMaps* maps, const int* n_new, int max_new, cudaStream_t stream);
+// append_bulk.cu (one-pass bulk append with S_bar on the tensor cores: bf16 cache, d = 128; maps with boxes of 64 tokens)
+size_t append_bulk_part_bytes(int units, int d);
+cudaError_t launch_append_bulk(const Params& p, const AttendMaps& cache, const AttendMaps& fresh, const int* n_new, int max_new,
+                               cudaStream_t stream);
 // attend_merge.cu
 cudaError_t launch_attend_merge(const Params& p, const AttendMaps* maps, const void* q, int q_is_bf16,
                                 const float* rms_weight, const int* sel_in, float* out, float* dbg_o_sparse,
@@ -109,9 +109,10 @@ cudaError_t launch_decode_fused(const Params& p, const AttendMaps& maps, const v
                                 float* dbg_o_sparse, float* dbg_o_rla, int* sel_user, int pending_new, cudaStream_t stream);
 int decode_fused_max_clusters(const Params& p);   // clusters of p.cs CTAs resident at once; -1 if unknown
 // append.cu
-// `state_maps` (may be null): tensor maps with boxes of 64 tokens; when given, bulk appends of a bf16 cache with
-// d = 128 update S_bar on the tensor cores instead of the FMA kernel.
+// `maps`, `fresh_maps` (may be null): tensor maps with boxes of 64 tokens over the cache and over k_new / v_new; with both,
+// appends of more than 32 tokens per sequence to a bf16 cache with d = 128 take the one-pass kernel.
 cudaError_t launch_append(const Params& p, const void* k_new, const void* v_new, const int* n_new, int max_new,
-                          const AttendMaps* state_maps, cudaStream_t stream);
+                          const AttendMaps* maps, const AttendMaps* fresh_maps, cudaStream_t stream);
+constexpr int kAppendStepMax = 32;      // up to so many new tokens per sequence the decode-step kernel serves an append
 
 }  // namespace spla

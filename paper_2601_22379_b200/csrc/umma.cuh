@@ -23,30 +23,15 @@ __host__ __device__ constexpr uint32_t umma_idesc(bool bf16, bool a_mn, bool b_m
 //                    bytes further inside the row, the next 64 in the next array of rows;
 //   MN-major operand (a row holds 64 consecutive m / n of one k):  the leading offset is the distance between the arrays
 //                    of rows that hold neighbouring groups of 64 m / n; the next 16 k are 16 rows = 2048 bytes further.
-__device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t smem_addr, uint32_t lead_bytes) {
-  const uint64_t lo = (uint64_t)((smem_addr >> 4) & 0x3fffu) | ((uint64_t)(lead_bytes >> 4) << 16);
-  const uint64_t hi = (uint64_t)(1024 >> 4) | (1ull << 14) | (2ull << 29);
-  return lo | (hi << 32);
-}
-
-// The same descriptor in two words, for loops that step through an operand: the low word grows by bytes / 16 (shared memory
-// ends below the 18 bits that the address field covers, so it never carries), the high word is the same for all.
+// In two words, for loops that step through an operand: the low word grows by bytes / 16 (shared memory ends below the 18
+// bits that the address field covers, so it never carries), the high word is the same for all.
 constexpr uint32_t kUmmaDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
 __device__ __forceinline__ uint32_t umma_desc_lo(uint32_t smem_addr, uint32_t lead_bytes) { return (smem_addr >> 4) | ((lead_bytes >> 4) << 16); }
 __device__ __forceinline__ uint64_t umma_desc_of(uint32_t lo) { return ((uint64_t)kUmmaDescHi << 32) | lo; }
 
-// D (tensor memory) (+)= A B, A and B in shared memory.
-__device__ __forceinline__ void umma_ss(uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}"
-      ::"r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate), "r"(0u)
-      : "memory");
-}
-// The same for a whole warp whose lanes all hold the operands, `one` non-zero in the lane that issues.  Operands that are
-// the same in every lane of a converged warp can stay in uniform registers; issued from a branch that only one lane takes,
-// an MMA cost 75 to 110 cycles in a loop beside busy warps, this way 50 to 65.
+// D (tensor memory) (+)= A B, A and B in shared memory; for a whole warp whose lanes all hold the operands, `one` non-zero
+// in the lane that issues.  Operands that are the same in every lane of a converged warp can stay in uniform registers;
+// issued from a branch that only one lane takes, an MMA cost 75 to 110 cycles in a loop beside busy warps, this way 50 to 65.
 __device__ __forceinline__ void umma_ss_one(uint32_t one, uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p, q;\n\t"
@@ -89,6 +74,7 @@ __device__ __forceinline__ void umma_ts4_one(uint32_t one, uint32_t tmem_d, uint
         "r"(idesc), "r"(accumulate), "r"(0u), "r"(one)
       : "memory");
 }
+// Arrives on the barrier once every tcgen05.mma issued so far by this thread has completed.
 __device__ __forceinline__ void umma_commit_one(uint32_t one, uint64_t* bar) {
   asm volatile(
       "{\n\t.reg .pred q;\n\t"
@@ -105,10 +91,6 @@ __device__ __forceinline__ uint32_t elect_one() {
       "selp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(r));
   return r;
-}
-// Arrives on the barrier once every tcgen05.mma issued so far by this thread has completed.
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }

@@ -1,0 +1,83 @@
+"""The one-pass bulk append (bf16, d = 128, more than 32 tokens) against the three-kernel one (SPLA_GENERAL_KERNELS), at the
+edges of its 64-token tiles, of blocks and of its shares: K/V, statistics and log-sum-exps bit for bit, nothing written past
+the end.  S_bar: phi enters as 16 bits from 256 tokens on (2^-18 relative per term, undiminished in sums of signed terms: the
+tensor-core tolerance), as 24 below, where what is left is the tensor core's accumulation (cut after two tiles) and fp32."""
+import pytest
+import torch
+
+from paper_2601_22379_b200 import binding, runner, synth
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+CASES = [
+    # batch, hkv, B, window, [tokens per append, longest sequence], ragged, flags
+    (2, 2, 64, None, [64], False, 0),                        # one whole tile
+    (2, 2, 64, None, [33, 40, 100], False, 0),               # shorter than a tile; across a boundary
+    (1, 2, 64, None, [63, 65, 64], False, 0),                # ends on, starts before a boundary
+    (1, 1, 64, None, [64 * 37 + 1], False, 0),               # 16 shares of one unit
+    (3, 8, 64, None, [700, 333], True, 0),
+    (20, 8, 64, None, [150, 64], True, 0),                   # 160 units: more CTAs than SMs, one share each
+    (2, 2, 128, None, [70, 190, 1000], False, 0),            # blocks of two tiles; a block opened in its second half
+    (2, 3, 128, None, [300, 65], True, 0),
+    (2, 2, 32, None, [47, 200], False, 0),
+    (2, 2, 16, None, [50, 131], True, 0),
+    (2, 2, 64, (32, 16), [77, 240], False, 0),               # strided windows
+    (1, 2, 128, (32, 16), [150, 500], True, 0),
+    (2, 2, 64, None, [130, 77], False, binding.SPLA_STATS_BF16),
+    (2, 2, 64, None, [130, 77], False, binding.SPLA_NO_RLA),
+    (1, 2, 64, None, [500, 301], True, binding.SPLA_DEBUG_BOUNDS),
+]
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: "-".join(map(str, c)))
+def test_one_pass_append_equals_the_three_kernel_append(case):
+    batch, hkv, B, window, sizes, ragged, flags = case
+    w = synth.Workload("case", 5, batch=batch, n_q_heads=hkv, n_kv_heads=hkv, head_dim=128, block_size=B, top_k=8,
+                       context=sum(sizes), n_outlier_channels=4, outlier_scale=3.0)
+    caches = [binding.SplaCache(runner.config_for(w, flags=f, window=window, extra_context=B), DEV)
+              for f in (flags, flags | binding.SPLA_GENERAL_KERNELS)]
+    for c in caches:
+        c.bufs.k_cache.fill_(float("nan"))
+        c.bufs.v_cache.fill_(float("nan"))
+    g = torch.Generator(device=DEV).manual_seed(3)
+    state = torch.zeros(batch, hkv, 128, 128, dtype=torch.float64, device=DEV)
+    for n in sizes:
+        k, v = (torch.randn(batch, hkv, n, 128, generator=g, device=DEV).to(torch.bfloat16) for _ in range(2))
+        n_new = torch.randint(0, n + 1, (batch,), generator=torch.Generator().manual_seed(n), dtype=torch.int32).to(DEV) if ragged else None
+        before = binding.launch_count()
+        caches[0].append_tokens(k, v, n_new)
+        assert binding.launch_count() - before <= 2
+        caches[1].append_tokens(k, v, n_new)
+        phi = torch.softmax(k.double(), dim=-1)
+        if ragged:
+            phi = phi * (torch.arange(n, device=DEV)[None, :] < n_new[:, None])[:, None, :, None]
+        state += phi.transpose(-1, -2) @ v.double()
+    torch.cuda.synchronize()
+    a, b = caches
+    assert a.sync_status() == 0 and b.sync_status() == 0
+    assert torch.equal(a.bufs.seq_lens, b.bufs.seq_lens)
+    for name in ("k_cache", "v_cache"):
+        assert torch.equal(getattr(a.bufs, name).view(torch.int16), getattr(b.bufs, name).view(torch.int16)), name
+    for name in ("stats", "tok_lse"):
+        assert torch.equal(getattr(a.bufs, name), getattr(b.bufs, name)), name
+    if flags & binding.SPLA_NO_RLA:
+        assert not a.bufs.rla_state.any()
+    else:
+        err = (a.bufs.rla_state.double() - state).flatten(2).norm(dim=-1) / state.flatten(2).norm(dim=-1).clamp_min(1e-30)
+        assert err.max().item() < (parity.STATE_TOL_TENSOR if max(sizes) >= 256 else parity.STATE_TOL_FMA)
+
+
+def test_one_pass_append_skips_and_reports_a_sequence_that_would_overflow():
+    w = synth.Workload("case", 6, batch=2, n_q_heads=2, n_kv_heads=2, head_dim=128, block_size=64, top_k=8, context=300)
+    cache = binding.SplaCache(runner.config_for(w), DEV)
+    k = torch.randn(2, 2, 200, 128, device=DEV).to(torch.bfloat16)
+    cache.append_tokens(k, k, torch.tensor([200, 100], dtype=torch.int32, device=DEV))
+    before = cache.bufs.rla_state.clone()
+    cache.set_length_bound(0)                                # the host is told too little: the device has to notice
+    cache.append_tokens(k, k)
+    torch.cuda.synchronize()
+    assert cache.sync_status() == binding.SPLA_ERR_CAPACITY
+    assert cache.bufs.seq_lens.cpu().tolist() == [200, 300]
+    assert torch.equal(cache.bufs.rla_state[0], before[0]) and not torch.equal(cache.bufs.rla_state[1], before[1])
