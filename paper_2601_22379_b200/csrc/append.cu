@@ -240,7 +240,10 @@ __global__ void append_lengths_kernel(const Params p, const int* __restrict__ n_
 constexpr int kFusedThreads = 256;
 constexpr int kFusedMaxNew = kAppendStepMax;
 
-template <typename T, int D, bool WIN>
+// ROWS: rows of S_bar per CTA of the state role.  Few rows spread a unit over many SMs where there are few units; with many
+// units the launch is bound by the number of its CTAs, and each takes more (512 units: 28 -> 20 us with
+// 32 rows and one statistics CTA per block that one token can touch; 64 and 128 rows 20 and 24 us).
+template <typename T, int D, bool WIN, int ROWS>
 __global__ void __launch_bounds__(kFusedThreads, 4) append_fused_kernel(const Params p, const T* __restrict__ k_new,
                                                                      const T* __restrict__ v_new,
                                                                      const int* __restrict__ n_new, int max_new, int n_copy,
@@ -249,7 +252,7 @@ __global__ void __launch_bounds__(kFusedThreads, 4) append_fused_kernel(const Pa
   constexpr int TG = kFusedThreads / D;            // thread groups of D threads
   __shared__ float red_s[TG][D];
   __shared__ float mean_s[D];
-  __shared__ float phi_s[kFusedMaxNew][kStateRows];
+  __shared__ float phi_s[kFusedMaxNew][ROWS];
   __shared__ float lse_s[kFusedMaxNew];
   __shared__ int last_s;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -307,14 +310,14 @@ __global__ void __launch_bounds__(kFusedThreads, 4) append_fused_kernel(const Pa
     const int blk = L / p.B + (WIN ? role / p.NW : role);
     block_stats_role<T, D, WIN>(p, u, blk, WIN ? role % p.NW : 0, L, L + max(n, 0), kn, n > 0 && blk * p.B < L + n, red_s, mean_s);
   } else if (!(p.flags & 4u)) {
-    // ---- state role: S_bar[row0 .. row0 + 15][:] += sum_t phi(k_t)[row] v_t ------------------------------------
+    // ---- state role: S_bar[row0 .. row0 + ROWS - 1][:] += sum_t phi(k_t)[row] v_t ------------------------------------
     role -= n_stats;
-    const int row0 = role * kStateRows;
+    const int row0 = role * ROWS;
     const int nn = max(n, 0);
     const float a2 = p.phi_scale * kLog2e;
     // The rows of S_bar this thread will update are requested first: the load comes from DRAM and would
     // otherwise sit at the end of the role's dependency chain.
-    constexpr int RPT = kStateRows / TG;                         // rows per thread
+    constexpr int RPT = ROWS / TG;                         // rows per thread
     const int tg = tid / D, j = tid % D;
     float* S = p.state + (size_t)u * D * D + (size_t)(row0 + tg * RPT) * D + j;
     float s_old[RPT];
@@ -353,9 +356,9 @@ __global__ void __launch_bounds__(kFusedThreads, 4) append_fused_kernel(const Pa
       if (t < nn && part == 0) lse_s[t] = mx + log2f(sm);        // base-2 domain
     }
     __syncthreads();
-    for (int idx = tid; idx < kFusedMaxNew * kStateRows; idx += kFusedThreads) {
-      const int t = idx / kStateRows, r = idx % kStateRows;
-      phi_s[t][r] = t < nn ? exp2f(to_float(kn[(size_t)t * D + row0 + r]) * a2 - lse_s[t]) : 0.f;
+    for (int idx = tid; idx < nn * ROWS; idx += kFusedThreads) {
+      const int t = idx / ROWS, r = idx % ROWS;
+      phi_s[t][r] = exp2f(to_float(kn[(size_t)t * D + row0 + r]) * a2 - lse_s[t]);
     }
     __syncthreads();
     float acc[RPT];
@@ -382,10 +385,13 @@ static cudaError_t launch_typed(const Params& p, const void* k_new, const void* 
   const T* vn = reinterpret_cast<const T*>(v_new);
   if (max_new <= kFusedMaxNew) {
     const int n_copy = (max_new + kFusedThreads / 32 - 1) / (kFusedThreads / 32);
-    const int n_stats = ((max_new + p.B - 1) / p.B + 1) * p.NW;   // one CTA per window of every block that can be touched
-    const int n_state = (p.flags & 4u) ? 0 : D / kStateRows;
+    const int n_stats = ((max_new + p.B - 2) / p.B + 1) * p.NW;   // one CTA per window of every block that can be touched
+    const bool wide = (long long)U * (D / kStateRows) > 4LL * 148;   // more small state CTAs than run at once
+    constexpr int kWideRows = 32;
+    const int n_state = (p.flags & 4u) ? 0 : D / (wide ? kWideRows : kStateRows);
     // Same shared-memory carve-out as the decode kernels around it: a change of carve-out drains the SMs.
-    auto kern = p.NW > 1 ? append_fused_kernel<T, D, true> : append_fused_kernel<T, D, false>;
+    auto kern = p.NW > 1 ? (wide ? append_fused_kernel<T, D, true, kWideRows> : append_fused_kernel<T, D, true, kStateRows>)
+                         : (wide ? append_fused_kernel<T, D, false, kWideRows> : append_fused_kernel<T, D, false, kStateRows>);
     cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     return launch_ex(kern, dim3(n_copy + n_stats + n_state, U), dim3(kFusedThreads), 0, stream, 0, true,
                      p, kn, vn, n_new, max_new, n_copy, n_stats);

@@ -195,10 +195,8 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
   float* ell_s = reinterpret_cast<float*>(smem_raw + SM::kEll);          // [G][chunk] log mass per block
   __shared__ int err_s;
 
-  const int chunk = p.chunk;                      // blocks per CTA
+  const int chunk = p.chunk;                      // blocks per CTA, at most (and the stride of its table of log masses)
   const int NW = WIN ? p.NW : 1;                  // selection windows per block; a "record" is one window
-  const int cta_blk0 = rank * chunk;              // first block of this CTA's share
-  const int rec_begin = cta_blk0 * NW;            // (a CTA that has records starts at its share's first block)
   const ST* stats_u = reinterpret_cast<const ST*>(p.stats) + (size_t)u * p.max_blocks * NW * 2 * D;
   if (tid == 0) {                               // nothing here depends on the preceding kernel
     if constexpr (SM::kMma) { for (int s = 0; s < SM::kSlots; ++s) mbar_init(&full[s], 1); }
@@ -312,10 +310,17 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
   }
   int L = L0;
   int nblk = (L + p.B - 1) / p.B;
+  // This CTA's share of the unit's blocks.  The launch is sized for the longest sequence; a shorter one is dealt out evenly
+  // over the cluster, so that its CTAs finish together (64 sequences of 4K to 64K tokens on clusters of two: with fixed
+  // shares the first CTA had up to 512 blocks and the second what was left; score launch 97 -> 80 us).  EARLY: the CTAs may have
+  // read different lengths, the shares are the fixed ones.
+  const int share = EARLY ? chunk : min(chunk, ((nblk + CS - 1) / CS + 7) / 8 * 8);
+  const int cta_blk0 = rank * share;              // first block of the share
+  const int rec_begin = cta_blk0 * NW;            // (a CTA that has records starts at its share's first block)
   const int nblk_stream = EARLY ? max(0, L0 - pending_new) / p.B : nblk;    // blocks whose records the ring may fetch
-  const int n_stream = max(0, min(cta_blk0 + chunk, nblk_stream) - cta_blk0) * NW;
+  const int n_stream = max(0, min(cta_blk0 + share, nblk_stream) - cta_blk0) * NW;
   int blk_begin = min(nblk, cta_blk0);
-  int nb_my = min(nblk, blk_begin + chunk) - blk_begin;   // blocks of this CTA (EARLY: refreshed after the wait)
+  int nb_my = min(nblk, blk_begin + share) - blk_begin;   // blocks of this CTA (EARLY: refreshed after the wait)
   int n_my = nb_my * NW;                          // records of this CTA
   const int n_rounds = (n_stream + kStageRec - 1) / kStageRec;
 
@@ -566,7 +571,7 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
       L = cover_len(p, checked_len(p, b), (long long)CS * chunk * p.B);
       nblk = (L + p.B - 1) / p.B;
       blk_begin = min(nblk, cta_blk0);
-      nb_my = min(nblk, blk_begin + chunk) - blk_begin;
+      nb_my = min(nblk, blk_begin + share) - blk_begin;
       n_my = nb_my * NW;
       nblk_fin = nblk;
       n_last = L - (nblk - 1) * p.B;
@@ -690,12 +695,12 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
         st_async_v2(map_to_rank(mine, (uint32_t)r), __float_as_uint(m), __float_as_uint(s), map_to_rank(bar, (uint32_t)r));
     }
   }
-  const int nblk_pad = min(nblk, CS * chunk);
+  const int nblk_pad = min(nblk, CS * share);
   if (tid == 32) {
     mbar_expect_tx(pbar, (uint32_t)(CS * G * 8));
     if (key_dest) {                               // the keys arrive two at a time: every CTA sends ceil(its blocks / 2) pairs
       uint32_t bytes = 0;
-      for (int r = 0; r < CS; ++r) bytes += (uint32_t)((max(0, min(nblk_pad, (r + 1) * chunk) - min(nblk_pad, r * chunk)) + 1) / 2) * 8u;
+      for (int r = 0; r < CS; ++r) bytes += (uint32_t)((max(0, min(nblk_pad, (r + 1) * share) - min(nblk_pad, r * share)) + 1) / 2) * 8u;
       mbar_expect_tx(kbar, bytes);
     }
   }

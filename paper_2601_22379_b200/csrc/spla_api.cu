@@ -405,6 +405,7 @@ static int launch_decode(spla_cache* c, const void* q, const float* rms_weight, 
   }
   plan_score_grid(c, &p, false);
   plan_attend(c, &p);
+  if ((long long)p.batch * p.Hkv * p.cs > 2LL * c->sm_count) pending = 0;   // several waves: most clusters start after the append anyway, and deal out their blocks evenly once the length is known
   e = launch_score(p, q, qb, sel_idx, s, pending);
   if (e == cudaSuccess) e = launch_attend_merge(p, &c->maps, q, qb, rms_weight, nullptr, out, dbg_o_sparse, dbg_o_rla, s);
   return e == cudaSuccess ? SPLA_OK : cuda_fail(e, where);

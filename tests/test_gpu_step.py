@@ -158,3 +158,26 @@ def test_many_one_call_steps_on_one_cache_in_one_graph():
     assert torch.equal(sel_a, sel_b)
     assert torch.equal(outs_a, outs_b)
     _same_cache(a, b)
+
+
+@pytest.mark.parametrize("batch,lo,hi", [(40, 130, 9000), (64, 64, 700), (37, 63, 64 * 33 + 1)])
+def test_many_ragged_units_deal_their_blocks_out_evenly(batch, lo, hi):
+    """More clusters than run at once: shares follow each sequence's own length (down to one block for several CTAs), state
+    CTAs take more rows.  Against the general kernels: same selections (ties aside) and outputs to bf16 accuracy."""
+    w = synth.BY_NAME["ragged_serving"].scaled(batch=batch, context=hi, context_min=lo, n_steps=4)
+    a, K, V, lens = runner.build_cache(w, DEV)
+    b, _, _, _ = runner.build_cache(w, DEV, prefill=(K, V, lens), flags=binding.SPLA_GENERAL_KERNELS)
+    gamma = synth.gamma(w).to(DEV)
+    for i in range(2):
+        k1, v1 = synth.step_kv(w, i, DEV)
+        q = synth.step_queries(w, i, DEV)
+        sa, sb = a.new_sel_buffer(), b.new_sel_buffer()
+        oa, ob = a.append_decode(k1, v1, q, gamma, sel_idx=sa), b.append_decode(k1, v1, q, gamma, sel_idx=sb)
+        torch.cuda.synchronize()
+        assert a.sync_status() == 0 and b.sync_status() == 0
+        same = (sa == sb).all(dim=-1)
+        assert same.float().mean().item() > 0.99
+        rows = same.repeat_interleave(w.group, dim=1)
+        assert parity.rel_l2(oa[rows].cpu().numpy(), ob[rows].cpu().numpy()) < 5e-3
+        assert torch.equal(a.bufs.stats, b.bufs.stats)
+        assert parity.rel_l2(a.bufs.rla_state.cpu().numpy(), b.bufs.rla_state.cpu().numpy()) < 2 * parity.STATE_TOL_TENSOR   # (the contexts went in on different kernels)
