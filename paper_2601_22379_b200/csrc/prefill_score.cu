@@ -1,39 +1,66 @@
 // Block scores and selection of every position of a prefill chunk (Section 3.1, Eq. taylor-2nd; Section 2.2, grouped
 // BlockScore; Section 2.1, Select), as a contraction instead of one pass over the statistics per position.
 //
-// For the complete blocks the Taylor log masses of 128 query rows (P positions x G heads) and 32 records are two
-// matrix products, q . mean and (q^2) . var, on the warp-level tensor cores.  Precision is that of fp32 products: q is
-// bf16 already and its square has 16 significant bits, exactly two bf16 parts; an fp32 record element enters as three
-// bf16 parts (24 bits), a 16-bit one as itself; scale factors are applied to the fp32 sums.  Eight products per record
-// and row with fp32 records, three with 16-bit ones.
+// For the complete blocks the Taylor log masses of 128 query rows (P positions x G heads) and 64 records are two matrix
+// products, q . mean and (q^2) . var, on the 5th-generation tensor cores.  Precision is that of fp32 products: q is bf16
+// already and its square has 16 significant bits, exactly two bf16 parts; an fp32 record element enters as three bf16 parts
+// (24 bits), a 16-bit one as itself; scale factors are applied to the fp32 sums.  Eight products per record and row with
+// fp32 records, three with 16-bit ones.
 #include "prefill_chunk.h"
+#include "umma.cuh"
 
 namespace spla {
 
 namespace {
 
-constexpr int kPsThreads = 256;
-constexpr int kPsRec = 32;                 // records staged together
+constexpr int kPsThreads = 416;            // 4 warps: rows in, log masses out; 8: records; 1: products
+constexpr int kPsLoaders = 256;
+constexpr int kPsRec = 64;                 // records of a tile: the N of the products
+constexpr uint32_t kPsTmemCols = 512;
 
-__device__ __forceinline__ void ldm_x4(uint32_t (&r)[4], uint32_t addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+template <int D, bool R16>
+struct PsSmem {
+  static constexpr int H = D / 64;                             // arrays of 128-byte rows per part
+  static constexpr int NP = R16 ? 1 : 3;                       // parts of a record element
+  static constexpr int kHalf = kPsRec * 128;
+  static constexpr int kPart = H * kHalf;
+  static constexpr int kStage = 2 * NP * kPart;                // means, variances: 96 KB (d = 128, fp32)
+  static constexpr int kBars = 2 * kStage;
+  static constexpr int kMisc = kBars + 10 * 8;                 // tensor-memory base, abort flag
+  static constexpr int kBytes = kMisc + 16;
+};
+
+__device__ __forceinline__ bool warp_waits(uint64_t* bar, uint32_t parity, int limit) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit));
+}
+__device__ __forceinline__ bool warp_aborted(volatile int* flag) { return __any_sync(0xffffffffu, *flag != 0); }
+__device__ __forceinline__ void store8(float* dst, const float (&v)[8]) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
+               "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
 }
 
-// One CTA: one tile of query rows, `rec_per_cta` consecutive records.  Warp w holds rows 16 w .. 16 w + 15 as the left
-// operand in registers; the records' parts are staged in shared memory once per 32 records, the next 32 already on their
-// way into registers.
+// One CTA: one tile of query rows, `rec_per_cta` consecutive records, 64 at a time.  The rows (q and the two parts of q^2)
+// stay in tensor memory as the left operand; eight warps cut the records into their parts, two tiles in shared memory and a
+// third on its way in registers; one warp issues the products into two pairs of accumulators; four warps turn finished sums
+// into log masses, one row per thread, in whole 32-byte sectors.
+//
+// Bound by the tensor pipe: 64 products of 128 x 64 x 16 per tile, 45 cycles each (2900 per
+// tile), and by a CTA's start where it has few tiles.  512 tokens on 32768 x 2 (16 units, 513 blocks, fp32): 132 us on the
+// warp-level tensor cores (the same products, operands through ldmatrix), 52 us now; the 8192-token prompt: 145 us, 115 us.
+//
+// Every wait has an iteration limit; on expiry all roles leave, tensor memory is released and the time-out is latched.
 template <int D, bool R16>
-__global__ void __launch_bounds__(kPsThreads, 2) prefill_score_kernel(const Params p, const PrefillChunk pc,
+__global__ void __launch_bounds__(kPsThreads, 1) prefill_score_kernel(const Params p, const PrefillChunk pc,
                                                                       const __nv_bfloat16* __restrict__ q, int rec_per_cta) {
-  constexpr int LD = D + 8;                                    // padded row: ldmatrix without bank conflicts
-  constexpr int NP = R16 ? 1 : 3;                              // parts of a record element
-  constexpr int KS = D / 16;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __nv_bfloat16* ms = reinterpret_cast<__nv_bfloat16*>(smem_raw);   // [NP][kPsRec][LD]
-  __nv_bfloat16* vs = ms + NP * kPsRec * LD;                        // [NP][kPsRec][LD]
+  using SM = PsSmem<D, R16>;
+  constexpr int H = SM::H, NP = SM::NP;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SM::kBars);
+  uint64_t *r_full = bars, *r_empty = bars + 2, *c_full = bars + 4, *c_empty = bars + 6, *q_ready = bars + 8, *done = bars + 9;
+  uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(smem + SM::kMisc);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + SM::kMisc + 4);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int g8 = lane >> 2, t4 = lane & 3;
   const PrefillUnit r = prefill_unit_of(p, pc, blockIdx.z);
   const int G = p.G;
   const int sb = pc.s0 + blockIdx.y / pc.nt, tile = blockIdx.y % pc.nt;
@@ -48,112 +75,174 @@ __global__ void __launch_bounds__(kPsThreads, 2) prefill_score_kernel(const Para
     if (tid == 0) atomicExch(p.status, kStatusBounds);
     return;
   }
-
-  // the rows this thread holds: warp * 16 + g8 and + 8
-  int pos_r[2];
-  bool ok_r[2];
-  uint32_t qa[KS][4];
-#pragma unroll
-  for (int hf = 0; hf < 2; ++hf) {
-    const int row = warp * 16 + g8 + 8 * hf;
-    pos_r[hf] = pos0 + row / G;
-    ok_r[hf] = row < pc.P * G && pos_r[hf] >= r.L0 && pos_r[hf] < pos_hi;
-    const size_t off = (((size_t)r.b * pc.T + (ok_r[hf] ? pos_r[hf] - r.first : 0)) * p.Hq + (size_t)r.h * G + row % G) * D;
-    const uint32_t* qr = reinterpret_cast<const uint32_t*>(q + off);
-#pragma unroll
-    for (int kk = 0; kk < KS; ++kk) {
-      qa[kk][hf] = ok_r[hf] ? __ldg(qr + 8 * kk + t4) : 0u;
-      qa[kk][2 + hf] = ok_r[hf] ? __ldg(qr + 8 * kk + 4 + t4) : 0u;
+  const int n_tiles = (rec1 - rec0 + kPsRec - 1) / kPsRec;
+  const int lim = p.wait_limit;
+  if (tid == 0) {
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&r_full[s], kPsLoaders / 32);  mbar_init(&r_empty[s], 1);
+      mbar_init(&c_full[s], 1);  mbar_init(&c_empty[s], 4);
     }
+    mbar_init(q_ready, 4);
+    mbar_init(done, 1);
+    mbar_init_done();
+    *abort_flag = 0;
   }
+  if (warp == 12) tmem_alloc(tmem_base_s, kPsTmemCols);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_base_s;
+  const uint32_t tQ = tmem + 256;                              // q, then q^2 head and remainder, D / 2 columns each
+  bool ok = true;
 
-  // staging: thread t takes 16-byte pieces t, t + 256, ... of the 32 records
-  constexpr int kPieces = kPsRec * 2 * D * (R16 ? 2 : 4) / 16 / kPsThreads;    // per thread: 8 (d = 128, fp32) .. 2
-  constexpr int kPerRec = 2 * D * (R16 ? 2 : 4) / 16;                           // pieces of a record
-  const uint4* recs = reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned char*>(p.stats) +
-                                                     (size_t)r.u * p.max_blocks * 2 * D * (R16 ? 2 : 4));
-  uint4 st[kPieces];
-  auto fetch = [&](int base) {
+  if (warp < 4) {
+    // ---------------------------------------------------------------- rows in, log masses out: one row per thread ----
+    const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
+    const int row = tid, pos = pos0 + row / G;
+    const bool live = row < pc.P * G && pos >= r.L0 && pos < pos_hi;
+    {
+      const uint4* qr = reinterpret_cast<const uint4*>(
+          q + (((size_t)r.b * pc.T + (live ? pos - r.first : 0)) * p.Hq + (size_t)r.h * G + row % G) * D);
+      uint4 raw[D / 8];
 #pragma unroll
-    for (int j = 0; j < kPieces; ++j) {
-      const int x = j * kPsThreads + tid;
-      st[j] = base + x / kPerRec < rec1 ? __ldg(recs + (size_t)base * kPerRec + x) : make_uint4(0u, 0u, 0u, 0u);
-    }
-  };
-  fetch(rec0);
-  const float ln_full = logf((float)p.B);
-  const float half_s2 = (p.flags & 2u) ? 0.f : 0.5f * p.sm_scale * p.sm_scale;
-  for (int base = rec0; base < rec1; base += kPsRec) {
-    __syncthreads();                                           // the previous records have been read
+      for (int j = 0; j < D / 8; ++j) raw[j] = live ? __ldg(qr + j) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-    for (int j = 0; j < kPieces; ++j) {
-      const int x = j * kPsThreads + tid, rec = x / kPerRec, pc16 = x % kPerRec;
-      const bool var = pc16 >= kPerRec / 2;
-      __nv_bfloat16* dst = (var ? vs : ms) + (size_t)rec * LD;
-      const int piece = var ? pc16 - kPerRec / 2 : pc16;
-      if constexpr (R16) {
-        *reinterpret_cast<uint4*>(dst + piece * 8) = st[j];
-      } else {
-        const float f0 = __uint_as_float(st[j].x), f1 = __uint_as_float(st[j].y), f2 = __uint_as_float(st[j].z), f3 = __uint_as_float(st[j].w);
-        const uint32_t h0 = pack_bf16(f0, f1), h1 = pack_bf16(f2, f3);
-        const float a0 = f0 - bf16_lo(h0), a1 = f1 - bf16_hi(h0), a2 = f2 - bf16_lo(h1), a3 = f3 - bf16_hi(h1);
-        const uint32_t m0 = pack_bf16(a0, a1), m1 = pack_bf16(a2, a3);
-        const uint32_t l0 = pack_bf16(a0 - bf16_lo(m0), a1 - bf16_hi(m0)), l1 = pack_bf16(a2 - bf16_lo(m1), a3 - bf16_hi(m1));
-        *reinterpret_cast<uint2*>(dst + piece * 4) = make_uint2(h0, h1);
-        *reinterpret_cast<uint2*>(dst + (size_t)kPsRec * LD + piece * 4) = make_uint2(m0, m1);
-        *reinterpret_cast<uint2*>(dst + (size_t)2 * kPsRec * LD + piece * 4) = make_uint2(l0, l1);
+      for (int c = 0; c < D / 32; ++c) {                       // 32 channels = 16 columns
+        uint32_t w[16], h[16], l[16];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const uint4 x = raw[c * 4 + j];
+          w[4 * j] = x.x; w[4 * j + 1] = x.y; w[4 * j + 2] = x.z; w[4 * j + 3] = x.w;
+        }
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {                         // q^2 in two bf16 parts: exact
+          const float a = bf16_lo(w[j]), b = bf16_hi(w[j]), a2 = a * a, b2 = b * b;
+          h[j] = pack_bf16(a2, b2);
+          l[j] = pack_bf16(a2 - bf16_lo(h[j]), b2 - bf16_hi(h[j]));
+        }
+        tmem_st16(tQ + lane_off + c * 16, w);
+        tmem_st16(tQ + lane_off + D / 2 + c * 16, h);
+        tmem_st16(tQ + lane_off + D + c * 16, l);
       }
+      tmem_st_wait();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive1(q_ready);
     }
-    __syncthreads();
-    if (base + kPsRec < rec1) fetch(base + kPsRec);
-    float cm[4][4], cv[4][4];
+    const size_t slot = ((size_t)r.u * pc.ns + (sb - pc.s0)) * pc.SB + (live ? pos - sb_start : 0);
+    float* dst = pc.ell + (slot * G + row % G) * pc.stride + rec0;
+    const float ln_full = logf((float)p.B);
+    const float half_s2 = (p.flags & 2u) ? 0.f : 0.5f * p.sm_scale * p.sm_scale;
+#pragma unroll 1
+    for (int i = 0; i < n_tiles && !warp_aborted(abort_flag); ++i) {
+      const int b = i & 1;
+      if (!warp_waits(&c_full[b], (i >> 1) & 1, lim)) { ok = false; break; }
+      tc_fence_after();
+#pragma unroll 1
+      for (int c = 0; c < kPsRec && rec0 + i * kPsRec + c < rec1; c += 32) {   // (a row of ell has room for whole groups of 32)
+        uint32_t m[32], v[32];
+        tmem_ld32_async(tmem + b * 128 + lane_off + c, m);
+        tmem_ld32_async(tmem + b * 128 + 64 + lane_off + c, v);
+        tmem_ld_wait32(m);
+        tmem_ld_wait32(v);
+        if (live) {
 #pragma unroll
-    for (int n = 0; n < 4; ++n)
+          for (int x = 0; x < 32; x += 8) {
+            float e[8];
 #pragma unroll
-      for (int x = 0; x < 4; ++x) { cm[n][x] = 0.f; cv[n][x] = 0.f; }
-    // ldmatrix: lane addresses row (lane & 7) of matrix lane / 8: matrices (rec 0-7, k 0-7), (rec 0-7, k 8-15), (rec 8-15, ...)
-    const uint32_t lane_off = (uint32_t)(((((lane >> 4) & 1) * 8 + (lane & 7)) * LD + ((lane >> 3) & 1) * 8) * 2);
-    const uint32_t ms0 = smem_u32(ms) + lane_off, vs0 = smem_u32(vs) + lane_off;
-#pragma unroll
-    for (int kk = 0; kk < KS; ++kk) {
-      uint32_t qh[4], ql[4];                                   // q^2 in two bf16 parts: exact
-#pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        const float a = bf16_lo(qa[kk][x]), b = bf16_hi(qa[kk][x]);
-        const float a2 = a * a, b2 = b * b;
-        qh[x] = pack_bf16(a2, b2);
-        ql[x] = pack_bf16(a2 - bf16_lo(qh[x]), b2 - bf16_hi(qh[x]));
-      }
-#pragma unroll
-      for (int np = 0; np < 2; ++np) {
-        const uint32_t off = (uint32_t)((np * 16 * LD + kk * 16) * 2);
-#pragma unroll
-        for (int part = 0; part < NP; ++part) {
-          uint32_t m[4], v[4];
-          ldm_x4(m, ms0 + off + (uint32_t)(part * kPsRec * LD * 2));
-          ldm_x4(v, vs0 + off + (uint32_t)(part * kPsRec * LD * 2));
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            mma_bf16(cm[2 * np + e], qa[kk][0], qa[kk][1], qa[kk][2], qa[kk][3], m[2 * e], m[2 * e + 1]);
-            mma_bf16(cv[2 * np + e], qh[0], qh[1], qh[2], qh[3], v[2 * e], v[2 * e + 1]);
-            if (part < 2) mma_bf16(cv[2 * np + e], ql[0], ql[1], ql[2], ql[3], v[2 * e], v[2 * e + 1]);
+            for (int j = 0; j < 8; ++j)
+              e[j] = ln_full + __uint_as_float(m[x + j]) * p.sm_scale + __logf(1.f + half_s2 * __uint_as_float(v[x + j]));
+            store8(dst + i * kPsRec + c + x, e);
           }
         }
+        __syncwarp();
       }
+      tc_fence_before();
+      if (lane == 0) mbar_arrive1(&c_empty[b]);
     }
+  } else if (warp < 12) {
+    // ---------------------------------------------------------------- records: 16-byte pieces, cut into bf16 parts ----
+    constexpr int kPerRec = 2 * D * (R16 ? 2 : 4) / 16;        // pieces of a record
+    constexpr int kStep = kPsLoaders / kPerRec;                // records between a thread's pieces
+    constexpr int kPieces = kPsRec / kStep;                    // per thread and tile: 16 (d = 128, fp32) .. 4
+    const int t = tid - 128, rec_t = t / kPerRec, pc16 = t % kPerRec;
+    const bool var = pc16 >= kPerRec / 2;
+    const int ch = (var ? pc16 - kPerRec / 2 : pc16) * (R16 ? 8 : 4);   // first channel of the thread's pieces
+    const uint4* recs = reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned char*>(p.stats) +
+                                                       (size_t)r.u * p.max_blocks * 2 * D * (R16 ? 2 : 4));
+    uint4 st[kPieces];
+    auto fetch = [&](int base) {
 #pragma unroll
-    for (int hf = 0; hf < 2; ++hf) {
-      if (!ok_r[hf]) continue;
-      const int row = warp * 16 + g8 + 8 * hf;
-      const size_t slot = ((size_t)r.u * pc.ns + (sb - pc.s0)) * pc.SB + (pos_r[hf] - sb_start);
-      float* dst = pc.ell + (slot * G + row % G) * pc.stride + base + 2 * t4;
+      for (int j = 0; j < kPieces; ++j) {
+        const int rec = base + j * kStep + rec_t;
+        st[j] = rec < rec1 ? __ldg(recs + (size_t)rec * kPerRec + pc16) : make_uint4(0u, 0u, 0u, 0u);
+      }
+    };
+    fetch(rec0);
+    unsigned char* dst0 = smem + (var ? NP * SM::kPart : 0) + (ch >> 6) * SM::kHalf + (ch & 4) * 2;
+#pragma unroll 1
+    for (int i = 0; i < n_tiles && !warp_aborted(abort_flag); ++i) {
+      const int b = i & 1;
+      if (i >= 2 && !warp_waits(&r_empty[b], ((i >> 1) - 1) & 1, lim)) { ok = false; break; }
+      unsigned char* stage = dst0 + b * SM::kStage;
 #pragma unroll
-      for (int n = 0; n < 4; ++n)
-        *reinterpret_cast<float2*>(dst + n * 8) =
-            make_float2(ln_full + cm[n][2 * hf] * p.sm_scale + __logf(1.f + half_s2 * cv[n][2 * hf]),
-                        ln_full + cm[n][2 * hf + 1] * p.sm_scale + __logf(1.f + half_s2 * cv[n][2 * hf + 1]));
+      for (int j = 0; j < kPieces; ++j) {
+        const int rec = j * kStep + rec_t;
+        unsigned char* dst = stage + rec * 128 + ((((ch & 63) >> 3) ^ (rec & 7)) << 4);
+        if constexpr (R16) {
+          *reinterpret_cast<uint4*>(dst) = st[j];
+        } else {
+          const float f0 = __uint_as_float(st[j].x), f1 = __uint_as_float(st[j].y), f2 = __uint_as_float(st[j].z), f3 = __uint_as_float(st[j].w);
+          const uint32_t h0 = pack_bf16(f0, f1), h1 = pack_bf16(f2, f3);
+          const float a0 = f0 - bf16_lo(h0), a1 = f1 - bf16_hi(h0), a2 = f2 - bf16_lo(h1), a3 = f3 - bf16_hi(h1);
+          const uint32_t m0 = pack_bf16(a0, a1), m1 = pack_bf16(a2, a3);
+          const uint32_t l0 = pack_bf16(a0 - bf16_lo(m0), a1 - bf16_hi(m0)), l1 = pack_bf16(a2 - bf16_lo(m1), a3 - bf16_hi(m1));
+          *reinterpret_cast<uint2*>(dst) = make_uint2(h0, h1);
+          *reinterpret_cast<uint2*>(dst + SM::kPart) = make_uint2(m0, m1);
+          *reinterpret_cast<uint2*>(dst + 2 * SM::kPart) = make_uint2(l0, l1);
+        }
+      }
+      proxy_fence();                                           // -> visible to the tensor core
+      __syncwarp();
+      if (lane == 0) mbar_arrive1(&r_full[b]);
+      if (i + 1 < n_tiles) fetch(rec0 + (i + 1) * kPsRec);
     }
+  } else {
+    // ---------------------------------------------------------------- products (a converged warp, one lane issues) ----
+    constexpr uint32_t idesc = umma_idesc(true, false, false, kPfRows, kPsRec);
+    constexpr int kProducts = R16 ? 3 : 8;                     // q x NP parts, head of q^2 x NP, its remainder x the first one or two
+    const uint32_t one = elect_one();
+    const uint32_t lo0 = umma_desc_lo(smem_u32(smem), 16);
+    ok = warp_waits(q_ready, 0, lim);
+#pragma unroll 1
+    for (int i = 0; i < n_tiles && ok && !warp_aborted(abort_flag); ++i) {
+      const int b = i & 1;
+      if (!warp_waits(&r_full[b], (i >> 1) & 1, lim) || (i >= 2 && !warp_waits(&c_empty[b], ((i >> 1) - 1) & 1, lim))) { ok = false; break; }
+      tc_fence_after();
+#pragma unroll 1
+      for (int x = kProducts - 1; x >= 0; --x) {               // (small terms first)
+        const uint32_t a = tQ + (x < NP ? 0 : x < 2 * NP ? D / 2 : D);
+        const uint32_t part = x < 2 * NP ? x : x - NP;
+        const uint32_t lo = lo0 + (uint32_t)(b * SM::kStage) / 16 + part * (SM::kPart / 16);
+        const uint32_t acc = x != kProducts - 1 && x != NP - 1;
+#pragma unroll
+        for (int hh = 0; hh < H; ++hh)
+          umma_ts4_one<8, 2>(one, tmem + b * 128 + (x < NP ? 0 : 64), a + hh * 32, lo + hh * (SM::kHalf / 16), idesc, hh > 0 ? 1u : acc);
+      }
+      umma_commit_one(one, &r_empty[b]);
+      umma_commit_one(one, &c_full[b]);
+    }
+    umma_commit_one(one, done);
+    if (!warp_waits(done, 0, lim)) ok = false;                 // nothing in flight when tensor memory is released
   }
+  if (!ok) {
+    *abort_flag = 1;
+    if (lane == 0) atomicExch(p.status, kStatusTimeout);
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 12) tmem_free(tmem, kPsTmemCols);
 }
 
 // Selection of one position by W warps (W = 1: one warp per position, up to 32 NK blocks; W = 8: a CTA per position, up to
@@ -303,17 +392,21 @@ __global__ void __launch_bounds__(256, 2) prefill_select_kernel(const Params p, 
 
 template <int D, bool R16>
 cudaError_t score_d(const Params& p, const PrefillChunk& c, const void* q, int max_blocks_seen, int sm_count, cudaStream_t s) {
-  const size_t smem = (size_t)2 * (R16 ? 1 : 3) * kPsRec * (D + 8) * 2;
+  constexpr size_t smem = PsSmem<D, R16>::kBytes;
   auto kern = prefill_score_kernel<D, R16>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  // records per CTA: as many as leave about two waves of CTAs, at least 64 (the query rows are loaded once per CTA)
-  const int U = p.batch * p.Hkv;
-  const long long tiles = (long long)c.ns * c.nt * U;
-  int rec = 64;
-  while (rec < 1024 && tiles * ((max_blocks_seen + rec - 1) / rec) > 4LL * sm_count) rec *= 2;
-  const int ny = (max_blocks_seen + rec - 1) / rec;
-  kern<<<dim3(ny < 1 ? 1 : ny, c.ns * c.nt, U), kPsThreads, smem, s>>>(p, c, reinterpret_cast<const __nv_bfloat16*>(q), rec);
+  // Tiles of records per CTA: what leaves the fewest tile times, a CTA's start counted as one (one CTA per SM).
+  const int U = p.batch * p.Hkv, all = (max_blocks_seen + kPsRec - 1) / kPsRec;
+  const long long row_tiles = (long long)c.ns * c.nt * U;
+  int per = all;
+  long long best = -1;
+  for (int ny = 1; ny <= all; ++ny) {
+    const int n = (all + ny - 1) / ny;
+    const long long cost = (row_tiles * ((all + n - 1) / n) + sm_count - 1) / sm_count * (n + 1);
+    if (best < 0 || cost < best) { best = cost; per = n; }
+  }
+  kern<<<dim3((all + per - 1) / per, c.ns * c.nt, U), kPsThreads, smem, s>>>(p, c, reinterpret_cast<const __nv_bfloat16*>(q), per * kPsRec);
   ++g_launch_count;
   return cudaGetLastError();
 }
