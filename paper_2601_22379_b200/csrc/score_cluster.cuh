@@ -197,6 +197,9 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
 
   const int chunk = p.chunk;                      // blocks per CTA, at most (and the stride of its table of log masses)
   const int NW = WIN ? p.NW : 1;                  // selection windows per block; a "record" is one window
+  int share = chunk;                              // blocks of a CTA; where the length is known before the streaming: see below
+  int cta_blk0 = rank * share;                    // first block of this CTA's share
+  int rec_begin = cta_blk0 * NW;                  // (a CTA that has records starts at its share's first block)
   const ST* stats_u = reinterpret_cast<const ST*>(p.stats) + (size_t)u * p.max_blocks * NW * 2 * D;
   if (tid == 0) {                               // nothing here depends on the preceding kernel
     if constexpr (SM::kMma) { for (int s = 0; s < SM::kSlots; ++s) mbar_init(&full[s], 1); }
@@ -314,9 +317,11 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
   // over the cluster, so that its CTAs finish together (64 sequences of 4K to 64K tokens on clusters of two: with fixed
   // shares the first CTA had up to 512 blocks and the second what was left; score launch 97 -> 80 us).  EARLY: the CTAs may have
   // read different lengths, the shares are the fixed ones.
-  const int share = EARLY ? chunk : min(chunk, ((nblk + CS - 1) / CS + 7) / 8 * 8);
-  const int cta_blk0 = rank * share;              // first block of the share
-  const int rec_begin = cta_blk0 * NW;            // (a CTA that has records starts at its share's first block)
+  if constexpr (!EARLY) {
+    share = min(chunk, ((nblk + CS - 1) / CS + 7) / 8 * 8);
+    cta_blk0 = rank * share;
+    rec_begin = cta_blk0 * NW;
+  }
   const int nblk_stream = EARLY ? max(0, L0 - pending_new) / p.B : nblk;    // blocks whose records the ring may fetch
   const int n_stream = max(0, min(cta_blk0 + share, nblk_stream) - cta_blk0) * NW;
   int blk_begin = min(nblk, cta_blk0);
@@ -683,6 +688,7 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
     // lane w * GP + g takes the pair of warp w and head g; the warps of a head are folded with shuffles (32 / GP >= 8
     // warps fit a pass for groups of up to four heads, else two passes); lanes 0 .. G - 1 then send head `lane`
     float m = -INFINITY, s = 0.f;
+#pragma unroll 1
     for (int e = lane; e < kCsConsumers * GP; e += 32) lse_merge(m, s, wred[e * 2], wred[e * 2 + 1]);
 #pragma unroll
     for (int o = GP; o < 32; o <<= 1) {
@@ -741,6 +747,7 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
   float lse_r[GP];
   {
     float m = -INFINITY, sm = 0.f;
+#pragma unroll 1
     for (int pr = lane; pr < CS * GP; pr += 32) {
       const int g = pr % GP;
       if (g < G) lse_merge(m, sm, all_part[pr * 2], all_part[pr * 2 + 1]);
@@ -763,6 +770,7 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
     float* scores_u = p.scores + (size_t)u * p.max_blocks;
     const uint32_t keys0 = smem_u32(keys), bar = smem_u32(kbar);
     const int n_dest = sel_share ? CS : 1;
+#pragma unroll 1
     for (int li = tid * 2; li < nb_my; li += 128 * 2) {
       float sc0 = 0.f, sc1 = 0.f;
 #pragma unroll
