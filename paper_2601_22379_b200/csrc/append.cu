@@ -119,6 +119,8 @@ __global__ void __launch_bounds__(kStatThreads) append_block_kernel(const Params
   __shared__ float red_s[kStatThreads / D][D];
   __shared__ float mean_s[D];
   constexpr int VEC = D / 32;
+  pdl_wait();
+  pdl_launch_dependents();
   constexpr int CH = D * (int)sizeof(T) / 16;        // 16-byte chunks per token
   T* tile = reinterpret_cast<T*>(tile_raw);          // [B][D]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -189,6 +191,8 @@ __global__ void __launch_bounds__(D) append_state_kernel(const Params p, const T
                                                          const T* __restrict__ v_new, const int* __restrict__ n_new,
                                                          int max_new) {
   __shared__ float phi_s[kStateTokens][kStateRows];
+  pdl_wait();
+  pdl_launch_dependents();
   const int u = blockIdx.y, b = u / p.Hkv;
   const int L = p.seq_lens[b];
   const int n = tokens_to_add(p, n_new, max_new, b, L);
@@ -224,6 +228,8 @@ __global__ void __launch_bounds__(D) append_state_kernel(const Params p, const T
 }
 
 __global__ void append_lengths_kernel(const Params p, const int* __restrict__ n_new, int max_new) {
+  pdl_wait();
+  pdl_launch_dependents();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= p.batch) return;
   const int L = p.seq_lens[b];
@@ -403,16 +409,14 @@ static cudaError_t launch_typed(const Params& p, const void* k_new, const void* 
     const size_t tile_bytes = (size_t)p.B * D * sizeof(T);
     auto kern = append_block_kernel<T, D>;
     if (tile_bytes > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_bytes);
-    kern<<<dim3((max_new + p.B - 1) / p.B + 1, U), kStatThreads, tile_bytes, stream>>>(p, kn, vn, n_new, max_new);
-    ++g_launch_count;
+    const cudaError_t e = launch_ex(kern, dim3((max_new + p.B - 1) / p.B + 1, U), dim3(kStatThreads), tile_bytes, stream, 0, true, p, kn, vn, n_new, max_new);
+    if (e != cudaSuccess) return e;
   }
   if (!(p.flags & 4u)) {
-    append_state_kernel<T, D><<<dim3(D / kStateRows, U), D, 0, stream>>>(p, kn, vn, n_new, max_new);
-    ++g_launch_count;
+    const cudaError_t e = launch_ex(append_state_kernel<T, D>, dim3(D / kStateRows, U), dim3(D), 0, stream, 0, true, p, kn, vn, n_new, max_new);
+    if (e != cudaSuccess) return e;
   }
-  append_lengths_kernel<<<(p.batch + 127) / 128, 128, 0, stream>>>(p, n_new, max_new);
-  ++g_launch_count;
-  return cudaGetLastError();
+  return launch_ex(append_lengths_kernel, dim3((p.batch + 127) / 128), dim3(128), 0, stream, 0, true, p, n_new, max_new);
 }
 
 cudaError_t launch_append(const Params& p, const void* k_new, const void* v_new, const int* n_new, int max_new,

@@ -25,6 +25,8 @@ __global__ void __launch_bounds__(kAttendThreads) attend_merge_kernel(const Para
   constexpr int NWARP = kAttendThreads / 32;
   constexpr int TS = kAttendThreads / D;        // token slices in the value pass
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  pdl_wait();
+  pdl_launch_dependents();
 
   const int vu = blockIdx.y, item = blockIdx.x;     // vu: index into the workspace (a virtual unit in a prefill launch)
   const UnitRef ur = unit_ref(p, vu);
@@ -265,9 +267,7 @@ static cudaError_t launch_one(const Params& p, const void* q, int qb, const floa
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   dim3 grid(p.top_k, p.batch * p.Hkv * (p.vT > 0 ? p.vT : 1));
-  kern<<<grid, kAttendThreads, smem, stream>>>(p, q, qb, w, out, ds, dr);
-  ++g_launch_count;
-  return cudaGetLastError();
+  return launch_ex(kern, grid, dim3(kAttendThreads), smem, stream, 0, true, p, q, qb, w, out, ds, dr);
 }
 
 template <typename T, int D>

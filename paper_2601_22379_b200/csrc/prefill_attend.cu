@@ -205,6 +205,8 @@ __global__ void __launch_bounds__(kPaThreads, 1)
   float* lse_s = reinterpret_cast<float*>(smem + SM::kLse);
   float* l_s = reinterpret_cast<float*>(smem + SM::kQ);           // (the queries are dead by then)
 
+  pdl_wait();
+  pdl_launch_dependents();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wg = warp >> 2;
   const int G = p.G, B = p.B;
   const PrefillUnit r = prefill_unit_of(p, pc, blockIdx.y);
@@ -760,11 +762,11 @@ cudaError_t attend_d(const Params& p, const PrefillChunk& c, const AttendMaps& m
   auto kern = prefill_attend_kernel<D, RLA>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, PaSmem<D>::kBytes);
   if (e != cudaSuccess) return e;
-  kern<<<dim3(c.ns * c.nt, p.batch * p.Hkv), kPaThreads, PaSmem<D>::kBytes, s>>>(
-      p, c, *reinterpret_cast<const CUtensorMap*>(maps.k), *reinterpret_cast<const CUtensorMap*>(maps.v),
-      reinterpret_cast<const __nv_bfloat16*>(q), w, out);
-  ++g_launch_count;
-  return cudaGetLastError();
+  // Launched ahead of the selection's end up to two waves of CTAs (288: 294 -> 290 us per chunk; 2064: 1553 -> 1569 us).
+  const bool ahead = (long long)c.ns * c.nt * p.batch * p.Hkv <= 2 * 148;
+  return launch_ex(kern, dim3(c.ns * c.nt, p.batch * p.Hkv), dim3(kPaThreads), PaSmem<D>::kBytes, s, 0, ahead,
+                   p, c, *reinterpret_cast<const CUtensorMap*>(maps.k), *reinterpret_cast<const CUtensorMap*>(maps.v),
+                   reinterpret_cast<const __nv_bfloat16*>(q), w, out);
 }
 
 }  // namespace

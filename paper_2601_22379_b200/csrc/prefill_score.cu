@@ -60,6 +60,8 @@ __global__ void __launch_bounds__(kPsThreads, 1) prefill_score_kernel(const Para
   uint64_t *r_full = bars, *r_empty = bars + 2, *c_full = bars + 4, *c_empty = bars + 6, *q_ready = bars + 8, *done = bars + 9;
   uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(smem + SM::kMisc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + SM::kMisc + 4);
+  pdl_wait();
+  pdl_launch_dependents();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const PrefillUnit r = prefill_unit_of(p, pc, blockIdx.z);
   const int G = p.G;
@@ -254,6 +256,8 @@ __global__ void __launch_bounds__(256, 2) prefill_select_kernel(const Params p, 
   __shared__ float red_s[8][2];
   __shared__ int cnt_s[2][8];
   constexpr int L = W * 32;                                    // lanes of a position
+  pdl_wait();
+  pdl_launch_dependents();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const PrefillUnit r = prefill_unit_of(p, pc, blockIdx.y);
   const int G = p.G;
@@ -406,17 +410,14 @@ cudaError_t score_d(const Params& p, const PrefillChunk& c, const void* q, int m
     const long long cost = (row_tiles * ((all + n - 1) / n) + sm_count - 1) / sm_count * (n + 1);
     if (best < 0 || cost < best) { best = cost; per = n; }
   }
-  kern<<<dim3((all + per - 1) / per, c.ns * c.nt, U), kPsThreads, smem, s>>>(p, c, reinterpret_cast<const __nv_bfloat16*>(q), per * kPsRec);
-  ++g_launch_count;
-  return cudaGetLastError();
+  return launch_ex(kern, dim3((all + per - 1) / per, c.ns * c.nt, U), dim3(kPsThreads), smem, s, 0, true,
+                   p, c, reinterpret_cast<const __nv_bfloat16*>(q), per * kPsRec);
 }
 
 template <int W, int NK>
 cudaError_t select_w(const Params& p, const PrefillChunk& c, int* sel_user, cudaStream_t s) {
   const int slots = c.ns * c.SB;
-  prefill_select_kernel<W, NK><<<dim3((slots + 8 / W - 1) / (8 / W), p.batch * p.Hkv), 256, 0, s>>>(p, c, sel_user);
-  ++g_launch_count;
-  return cudaGetLastError();
+  return launch_ex(prefill_select_kernel<W, NK>, dim3((slots + 8 / W - 1) / (8 / W), p.batch * p.Hkv), dim3(256), 0, s, 0, true, p, c, sel_user);
 }
 
 }  // namespace

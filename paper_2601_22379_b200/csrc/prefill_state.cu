@@ -30,6 +30,7 @@ __global__ void __launch_bounds__(kOwnThreads) prefill_own_kernel(const Params p
   float* mean_s = reinterpret_cast<float*>(smem_raw);          // [kOwnGroup][D]
   float* var_s = mean_s + kOwnGroup * D;                       // [kOwnGroup][D]
   __shared__ float inv_s[128];
+  pdl_launch_dependents();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const PrefillUnit r = prefill_unit_of(p, pc, blockIdx.y);
   const int G = p.G;
@@ -133,6 +134,8 @@ __global__ void __launch_bounds__(256) prefill_local_state_kernel(const Params p
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __nv_bfloat16* phi = reinterpret_cast<__nv_bfloat16*>(smem_raw);    // [3][64][LD]
   __nv_bfloat16* vs = phi + 3 * 64 * LD;                              // [64][LD]
+  pdl_wait();
+  pdl_launch_dependents();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const PrefillUnit r = prefill_unit_of(p, pc, blockIdx.y);
   const int start = prefill_range_start(pc, r, blockIdx.x);
@@ -214,6 +217,8 @@ __global__ void __launch_bounds__(256) prefill_local_state_kernel(const Params p
 template <int D>
 __global__ void __launch_bounds__(128) prefill_scan_state_kernel(const Params p, const PrefillChunk pc) {
   constexpr int N2 = D * D / 2, AHEAD = 8;
+  pdl_wait();
+  pdl_launch_dependents();
   const int idx = blockIdx.x * 128 + threadIdx.x;
   const int u = blockIdx.y;
   float2* st = reinterpret_cast<float2*>(p.state + (size_t)u * D * D) + idx;
@@ -245,10 +250,10 @@ __global__ void __launch_bounds__(128) prefill_scan_state_kernel(const Params p,
 template <int D>
 cudaError_t own_d(const Params& p, const PrefillChunk& c, const void* q, float* out, int* sel_user, cudaStream_t s) {
   const size_t smem = (size_t)2 * kOwnGroup * D * 4;
-  prefill_own_kernel<D><<<dim3((c.T + p.B - 2) / p.B + 1, p.batch * p.Hkv), kOwnThreads, smem, s>>>(
-      p, c, reinterpret_cast<const __nv_bfloat16*>(q), out, sel_user);
-  ++g_launch_count;
-  return cudaGetLastError();
+  // (not launched ahead of the append's end like the others: its CTAs would crowd onto the SMs that are free first; 512 tokens
+  // on 32768 x 2: 293 us so, 306 us launched ahead)
+  return launch_ex(prefill_own_kernel<D>, dim3((c.T + p.B - 2) / p.B + 1, p.batch * p.Hkv), dim3(kOwnThreads), smem, s, 0, false,
+                   p, c, reinterpret_cast<const __nv_bfloat16*>(q), out, sel_user);
 }
 
 template <int D>
@@ -257,11 +262,9 @@ cudaError_t state_d(const Params& p, const PrefillChunk& c, cudaStream_t s) {
   auto kern = prefill_local_state_kernel<D>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<dim3(c.n_sb, p.batch * p.Hkv), 256, smem, s>>>(p, c);
-  ++g_launch_count;
-  prefill_scan_state_kernel<D><<<dim3(D * D / 2 / 128, p.batch * p.Hkv), 128, 0, s>>>(p, c);
-  ++g_launch_count;
-  return cudaGetLastError();
+  e = launch_ex(kern, dim3(c.n_sb, p.batch * p.Hkv), dim3(256), smem, s, 0, true, p, c);
+  if (e != cudaSuccess) return e;
+  return launch_ex(prefill_scan_state_kernel<D>, dim3(D * D / 2 / 128, p.batch * p.Hkv), dim3(128), 0, s, 0, true, p, c);
 }
 
 }  // namespace

@@ -108,3 +108,14 @@ def test_a_wait_that_runs_out_is_reported_and_leaves_the_device_usable():
     assert cache.sync_status() == binding.SPLA_ERR_TIMEOUT
     a, _, _ = _run(w, K0, V0, k, v, q, 0)
     assert torch.isfinite(a).all()
+
+
+EDGES = [(1, 2, 4, 64 if n % 2 else 128, 16, 8, 1, 2, 16 * n + 3, 20, flags)   # n complete records: edges of the score's tiles of 64
+         for n in (1, 63, 64, 65, 128, 129) for flags in (0, binding.SPLA_STATS_BF16)]
+EDGES += [(1, 2, 16, 64, 64, 8, 1, 2, 0, t, 0) for t in (17 * 64, 18 * 64)]    # 288 and 304 row tiles: either side of two waves
+
+
+@pytest.mark.parametrize("case", EDGES, ids=lambda c: "-".join(map(str, c)))
+def test_score_tiles_and_launch_sizes_at_their_edges(case):
+    """Same bounds as the first test: one record tile more or less, rows for one launch rule or the other."""
+    test_tensor_core_prefill_equals_the_general_kernels(case)
