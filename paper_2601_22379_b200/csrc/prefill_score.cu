@@ -250,11 +250,17 @@ __global__ void __launch_bounds__(kPsThreads, 1) prefill_score_kernel(const Para
 // Selection of one position by W warps (W = 1: one warp per position, up to 32 NK blocks; W = 8: a CTA per position, up to
 // 256 NK).  Each lane keeps the keys of its NK blocks in registers.  The k-th best key is found bit by bit from the top
 // (counting the keys at or above a candidate, with a stop as soon as exactly k are), which needs no scratch and no sort;
-// the list then comes out in ascending order by ballots.
+// the list then comes out in ascending order by ballots.  A warp with 16 or more keys per lane first bounds the k-th best key
+// from below by that of the 64 best ones of half a lane each, and ranks the few keys that reach the bound instead (513
+// blocks, 512 positions x 16 units: 55 -> 42 us, bound by instructions issued).
+constexpr int kFew = 64;
 template <int W, int NK>
 __global__ void __launch_bounds__(256, 2) prefill_select_kernel(const Params p, const PrefillChunk pc, int* __restrict__ sel_user) {
   __shared__ float red_s[8][2];
   __shared__ int cnt_s[2][8];
+  constexpr bool FEW = W == 1 && NK >= 16;
+  __shared__ __align__(16) unsigned long long flat_s[FEW ? 8 : 1][kFew];   // keys that reach the bound, with their blocks
+  __shared__ __align__(16) int pick_s[FEW ? 8 : 1][kFew];
   constexpr int L = W * 32;                                    // lanes of a position
   pdl_wait();
   pdl_launch_dependents();
@@ -327,6 +333,71 @@ __global__ void __launch_bounds__(256, 2) prefill_select_kernel(const Params p, 
     const int i = k * L + l;
     key[k] = i >= nblk ? 0u : (i < p.n_sink || i >= nblk - p.n_local) ? 0xffffffffu : __float_as_uint(sc[k]) + 1u;
   }
+  int* sel_w = pc.sel + ((size_t)r.u * pc.T + t) * p.top_k;
+  int* sel_o = sel_user ? sel_user + (((size_t)r.b * pc.T + t) * p.Hkv + r.h) * p.top_k : nullptr;
+  if constexpr (FEW) {
+    if (k_eff < nblk) {
+      uint32_t m0 = 0u, m1 = 0u;
+#pragma unroll
+      for (int k = 0; k < NK; k += 2) { m0 = max(m0, key[k]); m1 = max(m1, key[k + 1]); }
+      uint32_t low = 0u;                                       // k_eff of the 64 maxima, of different blocks, are at least this
+#pragma unroll 1
+      for (int bit = 31; bit >= 0; --bit) {
+        const uint32_t cand = low | (1u << bit);
+        const int c = __popc(__ballot_sync(0xffffffffu, m0 >= cand)) + __popc(__ballot_sync(0xffffffffu, m1 >= cand));
+        if (c >= k_eff) low = cand;
+        if (c == k_eff) break;
+      }
+      int c = 0;
+#pragma unroll
+      for (int k = 0; k < NK; ++k) c += key[k] >= low;
+      int dst = c;                                             // where the lane's keys start: the sum of the lanes before
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, dst, o);
+        if (lane >= o) dst += x;
+      }
+      const int total = __shfl_sync(0xffffffffu, dst, 31);
+      if (low > 0u && total <= kFew) {
+        unsigned long long* flat = flat_s[warp];
+        int* pick = pick_s[warp];
+        flat[lane] = flat[32 + lane] = 0ull;
+        __syncwarp();
+        dst -= c;
+#pragma unroll
+        for (int k = 0; k < NK; ++k)
+          if (key[k] >= low) flat[dst++] = ((unsigned long long)key[k] << 32) | (uint32_t)(0x7fffffff - (k * L + l));   // (ties: the smaller block first)
+        __syncwarp();
+        const unsigned long long a0 = flat[lane], a1 = flat[32 + lane];
+        int r0 = 0, r1 = 0;
+#pragma unroll 4
+        for (int j = 0; j < total; j += 2) {
+          const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(flat + j);
+          r0 += (x.x > a0) + (x.y > a0);
+          r1 += (x.x > a1) + (x.y > a1);
+        }
+        const bool take0 = lane < total && r0 < k_eff, take1 = 32 + lane < total && r1 < k_eff;
+        const int i0 = 0x7fffffff - (int)(uint32_t)a0, i1 = 0x7fffffff - (int)(uint32_t)a1;
+        pick[lane] = take0 ? i0 : 0x7fffffff;
+        pick[32 + lane] = take1 ? i1 : 0x7fffffff;
+        __syncwarp();
+        int p0 = 0, p1 = 0;
+#pragma unroll 4
+        for (int j = 0; j < total; j += 4) {
+          const int4 x = *reinterpret_cast<const int4*>(pick + j);
+          p0 += (x.x < i0) + (x.y < i0) + (x.z < i0) + (x.w < i0);
+          p1 += (x.x < i1) + (x.y < i1) + (x.z < i1) + (x.w < i1);
+        }
+        if (take0) { sel_w[p0] = i0; if (sel_o) sel_o[p0] = i0; }
+        if (take1) { sel_w[p1] = i1; if (sel_o) sel_o[p1] = i1; }
+        for (int s = k_eff + l; s < p.top_k; s += L) {
+          sel_w[s] = -1;
+          if (sel_o) sel_o[s] = -1;
+        }
+        return;
+      }
+    }
+  }
   uint32_t thr = 1u;
   int n_eq = k_eff;                                            // of the keys equal to thr, the first n_eq are taken
   if (k_eff < nblk) {
@@ -351,8 +422,6 @@ __global__ void __launch_bounds__(256, 2) prefill_select_kernel(const Params p, 
     }
   }
   // ascending list: position = number of taken blocks with a smaller index (blocks are dealt to lanes in index order)
-  int* sel_w = pc.sel + ((size_t)r.u * pc.T + t) * p.top_k;
-  int* sel_o = sel_user ? sel_user + (((size_t)r.b * pc.T + t) * p.Hkv + r.h) * p.top_k : nullptr;
   int base = 0, eq_base = 0;
   const uint32_t below = (1u << lane) - 1u;
 #pragma unroll
@@ -431,7 +500,7 @@ cudaError_t launch_prefill_score(const Params& p, const PrefillChunk& c, const v
 }
 
 // Selection for the same positions.  Up to 1024 blocks a warp holds a position's keys; above, a CTA does (513 blocks, 512 positions x 16
-// units: 121 us by CTAs, whose barriers cost more than the wider registers of one warp, 55 us by warps).
+// units: 121 us by CTAs, whose barriers cost more than the wider registers of one warp, 42 us by warps).
 cudaError_t launch_prefill_select(const Params& p, const PrefillChunk& c, int max_blocks_seen, int* sel_user, cudaStream_t s) {
   if (max_blocks_seen <= 32 * 2) return select_w<1, 2>(p, c, sel_user, s);
   if (max_blocks_seen <= 32 * 4) return select_w<1, 4>(p, c, sel_user, s);

@@ -119,3 +119,17 @@ EDGES += [(1, 2, 16, 64, 64, 8, 1, 2, 0, t, 0) for t in (17 * 64, 18 * 64)]    #
 def test_score_tiles_and_launch_sizes_at_their_edges(case):
     """Same bounds as the first test: one record tile more or less, rows for one launch rule or the other."""
     test_tensor_core_prefill_equals_the_general_kernels(case)
+
+
+@pytest.mark.parametrize("k", [8, 32, 64])                # few keys reach the bound, about as many as are ranked, too many
+@pytest.mark.parametrize("blocks", [257, 513, 1023])
+def test_selection_from_the_keys_that_reach_a_bound(blocks, k):
+    test_tensor_core_prefill_equals_the_general_kernels((1, 2, 4, 64, 16, k, 1, 2, 16 * blocks + 3, 20, 0))
+
+
+def test_selection_among_equal_scores_takes_the_first_blocks():
+    """All keys alike: every free block ties, the bound keeps them all, and the list is the forced blocks and the first free ones."""
+    w, K0, V0, k, v, q = _inputs((1, 2, 4, 64, 16, 16, 1, 2, 16 * 300, 5, 0))
+    _, sel, _ = _run(w, torch.ones_like(K0), V0, torch.ones_like(k), v, q, 0)
+    want = list(range(14)) + [299, 300]
+    assert (sel.cpu() == torch.tensor(want, dtype=torch.int32)).all()
