@@ -66,7 +66,7 @@ struct PaSmem {
   static constexpr int kBitmap = kPhi + 4 * kTileBytes;          // [512] words: the union of the selected blocks
   static constexpr int kLse = kBitmap + kPfMaxBlocks / 8;        // float [2][64]
   static constexpr int kBars = kLse + 2 * kPaTile * 4;
-  static constexpr int kMisc = kBars + 22 * 8;                   // tensor-memory base, abort flag, tile count
+  static constexpr int kMisc = kBars + 23 * 8;                   // tensor-memory base, abort flag, tile count
   static constexpr int kBytes = kMisc + 32;
   static_assert(kBytes <= 227 * 1024, "shared memory of the attend kernel");
   static_assert(2 * H * D * 128 <= 4 * kTileBytes, "S_base fits the phi(K) ring");
@@ -197,7 +197,8 @@ __global__ void __launch_bounds__(kPaThreads, 1)
   extern __shared__ __align__(1024) unsigned char smem[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SM::kBars);
   uint64_t *k_full = bars, *k_empty = bars + 2, *v_full = bars + 4, *v_empty = bars + 6, *phi_ready = bars + 8, *phi_empty = bars + 10,
-           *s_full = bars + 12, *a_full = bars + 14, *p_ready = bars + 16, *c_ready = bars + 18, *r_full = bars + 20, *r_empty = bars + 21;
+           *s_full = bars + 12, *a_full = bars + 14, *p_ready = bars + 16, *c_ready = bars + 18, *r_full = bars + 20, *r_empty = bars + 21,
+           *done = bars + 22;
   uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(smem + SM::kMisc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + SM::kMisc + 4);
   int* n_set_s = reinterpret_cast<int*>(smem + SM::kMisc + 8);
@@ -230,6 +231,7 @@ __global__ void __launch_bounds__(kPaThreads, 1)
     }
     mbar_init(r_full, 1);
     mbar_init(r_empty, 4);
+    mbar_init(done, 1);
     mbar_init_done();
     *abort_flag = 0;
     *n_set_s = 0;
@@ -374,8 +376,8 @@ __global__ void __launch_bounds__(kPaThreads, 1)
         }
         issued = i + 1;
       }
-      if (*abort_flag)                                            // let the copies in flight land before the CTA leaves
-        for (int j = max(0, issued - 2); j < issued; ++j) mbar_wait(&full[j & 1], (j >> 1) & 1, lim);
+      // every copy has landed before the CTA leaves, whatever the other roles do
+      for (int j = max(0, issued - 2); j < issued; ++j) mbar_wait(&full[j & 1], (j >> 1) & 1, lim);
     } else if (warp == 1) {
       // ------------------------------------------------------------ MMA issuer -------------------------------------
       constexpr uint32_t id_s = umma_idesc(true, false, false, kPfRows, kPaTile);
@@ -446,8 +448,12 @@ __global__ void __launch_bounds__(kPaThreads, 1)
           cv(tR, a + 64, v, !fresh);
         }
         umma_commit_one(one, &v_empty[b]);
-        if (i % kFlush == kFlush - 1 || i == n_tiles - 1) umma_commit_one(one, r_full);
+        if (RLA && (i % kFlush == kFlush - 1 || i == n_tiles - 1)) umma_commit_one(one, r_full);
       }
+      // This warp reaches the CTA-wide barrier before the merge only when all its products are complete: the merge reads O,
+      // stages rows over the K and V tiles, and tensor memory is released after it, on expiry of a wait too.
+      umma_commit_one(one, done);
+      if (!warp_waits(done, 0, lim)) ok = false;
       if (!ok) *abort_flag = 1;
     }
   } else if (wg == 1) {
@@ -640,11 +646,9 @@ __global__ void __launch_bounds__(kPaThreads, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive1(&c_ready[b]);
       }
-    } else {
-      if (!warp_waits(r_full, ((n_tiles - 1) / kFlush) & 1, lim)) ok = false;
     }
     if (!ok) *abort_flag = 1;
-    __syncthreads();                                              // l of every row is there
+    __syncthreads();                                              // l of every row is there; every product is complete (see the issuer)
     tc_fence_after();
     if (!warp_aborted(abort_flag)) {
       // merge: out = O / l + gamma R rsqrt(mean R^2 + eps); rows staged in shared memory (16-byte pieces swizzled by row)

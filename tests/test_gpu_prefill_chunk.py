@@ -133,3 +133,19 @@ def test_selection_among_equal_scores_takes_the_first_blocks():
     _, sel, _ = _run(w, torch.ones_like(K0), V0, torch.ones_like(k), v, q, 0)
     want = list(range(14)) + [299, 300]
     assert (sel.cpu() == torch.tensor(want, dtype=torch.int32)).all()
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("tiles", [1, 4, 5, 8, 9, 13, 17])
+def test_without_the_residual_the_merge_waits_for_the_last_products(tiles, d):
+    """A chunk of 5 positions that select all `tiles` blocks of 64: the accumulator is complete when the merge reads it, however
+    many groups of four tiles the walk has (the same bits every time, and those of the general kernels to the usual bound)."""
+    case = (2, 2, 4, d, 64, tiles, 0, 1, 64 * (tiles - 1) + 3, 5, binding.SPLA_NO_RLA)
+    w, K0, V0, k, v, q = _inputs(case)
+    a, sel_a, _ = _run(w, K0, V0, k, v, q, case[-1])
+    assert (sel_a >= 0).sum(dim=-1).eq(tiles).all()
+    for _ in range(10):
+        again, _, _ = _run(w, K0, V0, k, v, q, case[-1])
+        assert torch.equal(again, a)
+    b, _, _ = _run(w, K0, V0, k, v, q, case[-1] | binding.SPLA_GENERAL_KERNELS)
+    np.testing.assert_allclose(a.cpu().numpy(), b.cpu().numpy(), rtol=RTOL, atol=ATOL)
