@@ -29,8 +29,8 @@
 // fit the SM's instruction cache (fewer rows or tokens per loop body cost more in latency than they gain there).
 //
 // Every wait is an mbarrier poll with an iteration limit; a role whose wait runs out raises the CTA's abort flag and leaves its
-// loop, the others then run into their own limits; tensor memory is released and the time-out status is latched.  No
-// multicast anywhere.
+// loop, the others then run into their own limits; the copies and products in flight are waited for, tensor memory is
+// released, the share counts as zero in S_bar and the time-out status is latched.  No multicast anywhere.
 #include "spla_internal.h"
 #include "umma.cuh"
 
@@ -53,15 +53,12 @@ constexpr int kAbTmemCols = 256;                             // two 128-column a
 constexpr int kAbPhi = kAbStages * 2 * kAbTileBytes;
 constexpr int kAbRed = kAbPhi + 2 * kAbMaxParts * kAbTileBytes; // float [2 passes][2 parities][128]
 constexpr int kAbBars = kAbRed + 2 * 2 * kAbD * 4;
-constexpr int kAbNumBars = 2 * kAbStages + 8;
+constexpr int kAbNumBars = 2 * kAbStages + 9;
 constexpr int kAbMisc = kAbBars + kAbNumBars * 8;            // tensor-memory base, abort flag
 constexpr int kAbSmem = kAbMisc + 16;
 static_assert(kAbSmem <= 227 * 1024, "shared memory of the bulk append");
 
 constexpr uint32_t kAbIdesc = umma_idesc(true, true, true, kAbD, kAbD);   // A and B MN-major bf16, 128 x 128
-
-__device__ __forceinline__ bool warp_waits(uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait(bar, parity)); }
-__device__ __forceinline__ bool warp_aborted(volatile int* flag) { return __any_sync(0xffffffffu, *flag != 0); }
 
 // One TMA box from shared memory into the cache (its own bulk group is committed by the caller).
 __device__ __forceinline__ void tma_store_box(const CUtensorMap* map, int x, int y, uint32_t src) {
@@ -82,6 +79,7 @@ __global__ void __launch_bounds__(kAbThreads, 1)
   uint64_t* phi_empty = phi_ready + 2;                            // [2] MMA -> transform
   uint64_t* acc_full = phi_empty + 2;                             // [2] MMA -> drain: a group's accumulator is complete
   uint64_t* acc_empty = acc_full + 2;                             // [2] drain -> MMA: it may be overwritten
+  uint64_t* done = acc_empty + 2;                                 // every product issued has completed
   uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(smem + kAbMisc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kAbMisc + 4);
 
@@ -95,6 +93,7 @@ __global__ void __launch_bounds__(kAbThreads, 1)
     for (int s = 0; s < 2; ++s) {
       mbar_init(&phi_ready[s], 4); mbar_init(&phi_empty[s], 1); mbar_init(&acc_full[s], 1); mbar_init(&acc_empty[s], 8);
     }
+    mbar_init(done, 1);
     mbar_init_done();
     *abort_flag = 0;
   }
@@ -136,6 +135,7 @@ __global__ void __launch_bounds__(kAbThreads, 1)
   auto whole = [&](int i) { const int t0 = (tile0 + i) * kAbTile; return t0 >= L && t0 + kAbTile <= L + n; };   // every row is new
   const uint32_t sbase = smem_u32(smem);
   const uint32_t tmem = rla ? *tmem_base_s : 0u;
+  const int lim = p.wait_limit;
 
   if (n_tiles > 0) {
     if (wg == 0) {
@@ -145,10 +145,10 @@ __global__ void __launch_bounds__(kAbThreads, 1)
         int issued = 0;
         for (int i = 0; i < n_tiles && !*abort_flag; ++i) {
           const int s = i % kAbStages;
-          if (i >= kAbStages && !mbar_wait(&empty[s], ((i / kAbStages) - 1) & 1)) { *abort_flag = 1; break; }
+          if (i >= kAbStages && !mbar_wait(&empty[s], ((i / kAbStages) - 1) & 1, lim)) { *abort_flag = 1; break; }
           const uint32_t base = sbase + s * 2 * kAbTileBytes;
           const int row = (int)((long long)u * max_new + ((tile0 + i) * kAbTile - L));   // (rows that are not new: of a neighbour, or zeros)
-          mbar_expect_tx(&full[s], 2 * kAbTileBytes);
+          mbar_expect_tx(&full[s], 2 * kAbTileBytes + (uint32_t)p.dbg_tx_extra);
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             tma_load_box(base + h * kAbHalf, &map_kn, h * 64, row, &full[s]);
@@ -156,8 +156,8 @@ __global__ void __launch_bounds__(kAbThreads, 1)
           }
           issued = i + 1;
         }
-        if (*abort_flag)                                 // let the copies in flight land before the CTA leaves
-          for (int j = max(0, issued - kAbStages); j < issued; ++j) mbar_wait(&full[j % kAbStages], (j / kAbStages) & 1);
+        // every copy has landed before the CTA leaves, whatever the other roles do
+        for (int j = max(0, issued - kAbStages); j < issued; ++j) mbar_wait(&full[j % kAbStages], (j / kAbStages) & 1, lim);
       } else if (warp == 1 && rla) {
         // -------------------------------------------------------------- products (whole warp, one lane issues) ---------
         const uint32_t one = elect_one();
@@ -167,8 +167,8 @@ __global__ void __launch_bounds__(kAbThreads, 1)
           const int s = i % kAbStages, pb = i & 1;
           const int g = i / kAbGroup, ab = g & 1;
           const bool first = i % kAbGroup == 0, last = i % kAbGroup == kAbGroup - 1 || i == n_tiles - 1;
-          if (first && g >= 2 && !warp_waits(&acc_empty[ab], ((g >> 1) - 1) & 1)) { ok = false; break; }
-          if (!warp_waits(&phi_ready[pb], (i >> 1) & 1)) { ok = false; break; }   // (the tile itself arrived before that)
+          if (first && g >= 2 && !warp_waits(&acc_empty[ab], ((g >> 1) - 1) & 1, lim)) { ok = false; break; }
+          if (!warp_waits(&phi_ready[pb], (i >> 1) & 1, lim)) { ok = false; break; }   // (the tile itself arrived before that)
           tc_fence_after();
           const uint32_t a = umma_desc_lo(sbase + kAbPhi + pb * PARTS * kAbTileBytes, kAbHalf);
           const uint32_t v = umma_desc_lo(sbase + s * 2 * kAbTileBytes + kAbTileBytes, kAbHalf);
@@ -179,13 +179,15 @@ __global__ void __launch_bounds__(kAbThreads, 1)
           umma_commit_one(one, &empty[s]);
           if (last) umma_commit_one(one, &acc_full[ab]);
         }
+        umma_commit_one(one, done);                      // nothing in flight when tensor memory is released, on expiry of a wait too
+        if (!warp_waits(done, 0, lim)) ok = false;
         if (!ok) *abort_flag = 1;
       } else if (warp == 2 && lane == 0) {
         // -------------------------------------------------------------- whole tiles into the cache --------------------
         bool ok = true;
         for (int i = 0; i < n_tiles && !*abort_flag; ++i) {
           const int s = i % kAbStages;
-          if (!mbar_wait(&full[s], (i / kAbStages) & 1)) { ok = false; break; }
+          if (!mbar_wait(&full[s], (i / kAbStages) & 1, lim)) { ok = false; break; }
           int row = (int)(unit_tok0 + (size_t)(tile0 + i) * kAbTile);
           bool store = whole(i);
           if ((p.flags & kDebugBounds) && store && (tile0 + i + 1) * kAbTile > p.max_blocks * p.B) {   // checked build
@@ -235,8 +237,8 @@ __global__ void __launch_bounds__(kAbThreads, 1)
           const int s = i % kAbStages;
           const int t0 = (tile0 + i) * kAbTile;
           const bool edge = !whole(i);
-          if (!warp_waits(&full[s], (i / kAbStages) & 1)) { ok = false; break; }
-          if (rla && i >= 2 && !warp_waits(&phi_empty[wt], ((i >> 1) - 1) & 1)) { ok = false; break; }
+          if (!warp_waits(&full[s], (i / kAbStages) & 1, lim)) { ok = false; break; }
+          if (rla && i >= 2 && !warp_waits(&phi_empty[wt], ((i >> 1) - 1) & 1, lim)) { ok = false; break; }
           unsigned char* kt = smem + s * 2 * kAbTileBytes + tg * 16;
           unsigned char* ph = smem + kAbPhi + wt * PARTS * kAbTileBytes + tg * 16;
 #pragma unroll 1
@@ -373,7 +375,7 @@ __global__ void __launch_bounds__(kAbThreads, 1)
         const int upto = more ? i / kAbGroup : n_groups;
 #pragma unroll 1
         for (; drained < upto && ok; ++drained) {
-          if (!warp_waits(&acc_full[drained & 1], (drained >> 1) & 1)) { ok = false; break; }
+          if (!warp_waits(&acc_full[drained & 1], (drained >> 1) & 1, lim)) { ok = false; break; }
           tc_fence_after();
 #pragma unroll
           for (int cb = 0; cb < 2; ++cb) {
@@ -417,7 +419,7 @@ __global__ void __launch_bounds__(kAbThreads, 1)
       for (int i = 0; i < n_tiles; i += gran) {
         bool go = true;
         const int have = min(gran, n_tiles - i);
-        for (int j = 0; j < have && go; ++j) go = warp_waits(&full[(i + j) % kAbStages], ((i + j) / kAbStages) & 1);
+        for (int j = 0; j < have && go; ++j) go = warp_waits(&full[(i + j) % kAbStages], ((i + j) / kAbStages) & 1, lim);
         uint32_t stop;                                                 // one decision for the four warps: barrier counts must match
         asm volatile(
             "{\n\t.reg .pred p, q;\n\t"
@@ -536,7 +538,7 @@ __global__ void __launch_bounds__(kAbThreads, 1)
     tmem_free(tmem, kAbTmemCols);
   }
   if (tid == 0 && *abort_flag) atomicExch(p.status, kStatusTimeout);
-  if (n_tiles == 0 && rla && S > 1) {                    // (an empty share adds nothing)
+  if ((n_tiles == 0 || *abort_flag) && rla && S > 1) {   // an empty share adds nothing, nor does one that gave up (no old sums)
     float4* part = reinterpret_cast<float4*>(p.state_part + ((size_t)u * S + share) * D * D);
     for (int idx = tid; idx < D * D / 4; idx += kAbThreads) part[idx] = make_float4(0.f, 0.f, 0.f, 0.f);
   }

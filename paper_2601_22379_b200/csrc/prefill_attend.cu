@@ -78,11 +78,6 @@ __device__ __forceinline__ uint32_t pack_h2(float lo, float hi) {
 }
 __device__ __forceinline__ float h2_lo(uint32_t x) { return __low2float(*reinterpret_cast<const __half2*>(&x)); }
 __device__ __forceinline__ float h2_hi(uint32_t x) { return __high2float(*reinterpret_cast<const __half2*>(&x)); }
-// Warp-uniform forms: every lane of a warp goes on, or every lane gives up (the tensor-memory instructions want whole warps).
-__device__ __forceinline__ bool warp_waits(uint64_t* bar, uint32_t parity, int limit) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit));
-}
-__device__ __forceinline__ bool warp_aborted(volatile int* flag) { return __any_sync(0xffffffffu, *flag != 0); }
 __device__ __forceinline__ uint64_t low_bits(int n) { return n >= 64 ? ~0ull : (n <= 0 ? 0ull : (1ull << n) - 1ull); }
 
 // Walks the tiles of 64 tokens over the set bits of the bitmap.  Blocks of 64 tokens or more: one block, token offset

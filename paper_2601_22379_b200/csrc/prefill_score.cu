@@ -30,10 +30,6 @@ struct PsSmem {
   static constexpr int kBytes = kMisc + 16;
 };
 
-__device__ __forceinline__ bool warp_waits(uint64_t* bar, uint32_t parity, int limit) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit));
-}
-__device__ __forceinline__ bool warp_aborted(volatile int* flag) { return __any_sync(0xffffffffu, *flag != 0); }
 __device__ __forceinline__ void store8(float* dst, const float (&v)[8]) {
   asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
                "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])

@@ -166,6 +166,12 @@ __device__ __forceinline__ void tma_load_box(uint32_t dst, const CUtensorMap* ma
 __device__ __forceinline__ void mbar_arrive1(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// Warp-uniform bounded waits of kernels with roles: every lane of a warp goes on, or every lane gives up (the tensor-memory
+// instructions want whole warps).  `limit` as for mbar_wait.
+__device__ __forceinline__ bool warp_waits(uint64_t* bar, uint32_t parity, int limit) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit));
+}
+__device__ __forceinline__ bool warp_aborted(volatile int* flag) { return __any_sync(0xffffffffu, *flag != 0); }
 // Generic-proxy accesses to shared memory before this are ordered before asynchronous-proxy ones (TMA, tensor core) after it.
 __device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 

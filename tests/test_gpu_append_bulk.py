@@ -81,3 +81,34 @@ def test_one_pass_append_skips_and_reports_a_sequence_that_would_overflow():
     assert cache.sync_status() == binding.SPLA_ERR_CAPACITY
     assert cache.bufs.seq_lens.cpu().tolist() == [200, 300]
     assert torch.equal(cache.bufs.rla_state[0], before[0]) and not torch.equal(cache.bufs.rla_state[1], before[1])
+
+
+@pytest.mark.parametrize("batch", [1, 80], ids=["shares", "one_share"])      # 16 shares of a unit, added by a second kernel; one share
+def test_a_wait_that_runs_out_is_reported_and_adds_nothing_to_the_state(batch):
+    """The copies' barriers are told to expect more than arrives: every role gives up, the state is left as it was (no partial
+    sum of an earlier append reaches it), and the next append of the same cache is right."""
+    hkv, n = 2, 64 * 20
+    w = synth.Workload("case", 7, batch=batch, n_q_heads=hkv, n_kv_heads=hkv, head_dim=128, block_size=64, top_k=8, context=2 * n)
+    cache, want = (binding.SplaCache(runner.config_for(w), DEV) for _ in range(2))
+    for c in (cache, want):
+        c.bufs.k_cache.zero_()
+        c.bufs.v_cache.zero_()
+    g = torch.Generator(device=DEV).manual_seed(4)
+    parts = [torch.randn(batch, hkv, n, 128, generator=g, device=DEV).to(torch.bfloat16) for _ in range(4)]
+    cache.append_tokens(parts[0], parts[1])
+    lens, state = cache.bufs.seq_lens.clone(), cache.bufs.rla_state.clone()
+    cache.debug_wait_hook(500, 16)
+    cache.append_tokens(parts[2], parts[3])
+    torch.cuda.synchronize()
+    assert cache.sync_status() == binding.SPLA_ERR_TIMEOUT
+    assert torch.equal(cache.bufs.rla_state, state)
+    cache.debug_wait_hook(0, 0)
+    cache.bufs.seq_lens.copy_(lens)
+    cache.set_length_bound(n)
+    cache.append_tokens(parts[2], parts[3])
+    want.append_tokens(parts[0], parts[1])
+    want.append_tokens(parts[2], parts[3])
+    torch.cuda.synchronize()
+    assert cache.sync_status() == 0
+    for name in ("seq_lens", "k_cache", "v_cache", "stats", "tok_lse", "rla_state"):
+        assert torch.equal(getattr(cache.bufs, name), getattr(want.bufs, name)), name
