@@ -16,20 +16,27 @@ constexpr int kOwnRows = 4;                // (position, head) rows a warp works
 template <int VEC> struct QueryVec { using type = uint2; };      // a lane's VEC query elements
 template <> struct QueryVec<2> { using type = uint32_t; };
 
-// One CTA per (block the chunk touches, unit).  D threads walk the block's tokens, one channel each: running sum and
-// running sum of squared deviations (each token's deviation from the mean before and after it: Welford's update, no
-// cancellation), so that the statistics of ALL prefixes of the block cost one pass instead of one pass per prefix.
-// After every 32 tokens the eight warps form the dots of those prefixes with their positions' queries.
-// Bound by that serial chain and the load latencies around it.
+// One CTA per (block the chunk touches, unit).  The statistics of ALL prefixes of the block that end inside the chunk, each by
+// the two exact passes and in the summation order of the append kernels (256 / D running sums of every 256 / D-th token, added
+// in order), so that a position's own record has the bits a token-by-token append would have left there: with 16-bit records
+// a last-bit difference would round to the other neighbour, 2^-8 away.  The block's keys are staged in shared memory; thread
+// (channel pair, slot) takes every kSlots-th position of a group of kOwnGroup: running sums give the means, then one walk
+// over the older tokens serves all its positions.  After every group the eight warps form the dots of those prefixes with
+// their positions' queries.
+// Bound by instructions issued and the load latencies around them.
 template <int D>
 __global__ void __launch_bounds__(kOwnThreads) prefill_own_kernel(const Params p, const PrefillChunk pc,
                                                                   const __nv_bfloat16* __restrict__ q, float* __restrict__ out,
                                                                   int* __restrict__ sel_user) {
   constexpr int VEC = D / 32;
+  constexpr int TG = kOwnThreads / D;                          // running sums of a prefix
+  constexpr int kSlots = kOwnThreads / (D / 2);
+  constexpr int NP = kOwnGroup / kSlots;                       // positions of a thread
+  static_assert(kSlots % TG == 0 && kOwnGroup % TG == 0, "a position's newest token is of the same sum in every group");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* mean_s = reinterpret_cast<float*>(smem_raw);          // [kOwnGroup][D]
   float* var_s = mean_s + kOwnGroup * D;                       // [kOwnGroup][D]
-  __shared__ float inv_s[128];
+  uint32_t* key_s = reinterpret_cast<uint32_t*>(var_s + kOwnGroup * D);   // [B][D / 2] channel pairs
   pdl_launch_dependents();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const PrefillUnit r = prefill_unit_of(p, pc, blockIdx.y);
@@ -51,10 +58,8 @@ __global__ void __launch_bounds__(kOwnThreads) prefill_own_kernel(const Params p
     return;
   }
   const int cnt = min(p.B, r.L_end - t0);
-  if (tid < 128) inv_s[tid] = 1.f / (float)(tid + 1);
-  const __nv_bfloat16* kc = reinterpret_cast<const __nv_bfloat16*>(p.k_cache) + ((size_t)r.u * p.max_blocks * p.B + t0) * D;
+  const uint4* kc = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.k_cache) + ((size_t)r.u * p.max_blocks * p.B + t0) * D);
   const bool round16 = (p.flags & kStatsBf16) != 0;
-  float sum = 0.f, m2 = 0.f, mean = 0.f;
   // Queries of kOwnRows (position, head) rows of the group that starts at token g0, requested before they are needed:
   // fetched one row at a time where they are used, their latency was half of this kernel's time (33 -> 15 us for 144 CTAs).
   using QV = typename QueryVec<VEC>::type;
@@ -68,26 +73,90 @@ __global__ void __launch_bounds__(kOwnThreads) prefill_own_kernel(const Params p
       qn[i] = ok ? __ldg(reinterpret_cast<const QV*>(q + off)) : QV();
     }
   };
-  fetch(0, warp * kOwnRows, min(kOwnGroup, cnt));
+  const int g_begin = max(0, r.L0 - t0) / kOwnGroup * kOwnGroup;   // the first group with a position of the chunk
+  fetch(g_begin, warp * kOwnRows, min(kOwnGroup, cnt - g_begin));
+  {
+    uint4* dst = reinterpret_cast<uint4*>(key_s);              // rows past the end: zeros, in no prefix
+#pragma unroll 4
+    for (int x = tid; x < p.B * (D / 8); x += kOwnThreads) dst[x] = x < cnt * (D / 8) ? kc[x] : make_uint4(0u, 0u, 0u, 0u);
+  }
   __syncthreads();
+  const int cp = tid % (D / 2), slot = tid / (D / 2);
+  const uint32_t* col = key_s + cp;
+  auto key2 = [&](int t) { const uint32_t w = col[t * (D / 2)]; return make_float2(bf16_lo(w), bf16_hi(w)); };
+  float2 run[TG];                                              // running sums over the tokens before the group
+#pragma unroll
+  for (int g = 0; g < TG; ++g) run[g] = make_float2(0.f, 0.f);
   for (int g0 = 0; g0 < cnt; g0 += kOwnGroup) {
     const int ng = min(kOwnGroup, cnt - g0);
-    if (tid < D) {
-      __nv_bfloat16 x[kOwnGroup];
+    const bool wanted = g0 >= g_begin;
+    float2 nm[NP];                                             // minus the mean of each of the thread's positions
 #pragma unroll
-      for (int j = 0; j < kOwnGroup; ++j) x[j] = j < ng ? kc[(size_t)(g0 + j) * D + tid] : __nv_bfloat16();
+    for (int b = 0; b < kOwnGroup; b += kSlots) {              // (p.B is a multiple of kSlots: the reads stay inside the block)
+      if (g0 + b < p.B) {
 #pragma unroll
-      for (int j = 0; j < kOwnGroup; ++j) {
-        const float v = __bfloat162float(x[j]), inv = inv_s[min(g0 + j, 127)];
-        const float before = v - mean;
-        sum += v;
-        mean = sum * inv;
-        m2 = g0 + j == 0 ? 0.f : fmaf(before, v - mean, m2);
-        float mm = mean, vv = m2 * inv;
-        if (round16) { mm = __bfloat162float(__float2bfloat16_rn(mm)); vv = __bfloat162float(__float2bfloat16_rn(vv)); }
-        mean_s[j * D + tid] = mm;
-        var_s[j * D + tid] = vv;
+        for (int j = 0; j < kSlots; ++j) {
+          run[j % TG] = __fadd2_rn(run[j % TG], key2(g0 + b + j));
+          if (j == slot) {
+            float2 tot = run[0];
+#pragma unroll
+            for (int g = 1; g < TG; ++g) tot = __fadd2_rn(tot, run[g]);
+            nm[b / kSlots] = tot;
+          }
+        }
+      } else {
+        nm[b / kSlots] = make_float2(0.f, 0.f);
       }
+    }
+    if (!wanted) continue;
+    float2 ss[NP][TG];
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      const float n = (float)(g0 + i * kSlots + slot + 1);
+      nm[i] = make_float2(-(nm[i].x / n), -(nm[i].y / n));
+#pragma unroll
+      for (int g = 0; g < TG; ++g) ss[i][g] = make_float2(0.f, 0.f);
+    }
+    auto add = [&](int i, int g, float2 x) {
+      const float2 dv = __fadd2_rn(x, nm[i]);
+      ss[i][g] = __ffma2_rn(dv, dv, ss[i][g]);
+    };
+#pragma unroll 1
+    for (int t = 0; t < g0; t += TG) {                         // tokens of earlier groups: in every prefix of this one
+#pragma unroll
+      for (int g = 0; g < TG; ++g) {
+        const float2 x = key2(t + g);
+#pragma unroll
+        for (int i = 0; i < NP; ++i) add(i, g, x);
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < NP; ++b) {                             // the group's own tokens: those up to the position
+      if (g0 + b * kSlots < p.B) {
+#pragma unroll
+        for (int j = 0; j < kSlots; ++j) {
+          const float2 x = key2(g0 + b * kSlots + j);
+          if (j <= slot) add(b, j % TG, x);
+#pragma unroll
+          for (int i = b + 1; i < NP; ++i) add(i, j % TG, x);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      const int j = i * kSlots + slot;
+      const float n = (float)(g0 + j + 1);
+      float2 tot = ss[i][0];
+#pragma unroll
+      for (int g = 1; g < TG; ++g) tot = __fadd2_rn(tot, ss[i][g]);
+      float2 mm = make_float2(-nm[i].x, -nm[i].y), vv = make_float2(tot.x / n, tot.y / n);
+      if (round16) {
+        const uint32_t m16 = pack_bf16(mm.x, mm.y), v16 = pack_bf16(vv.x, vv.y);
+        mm = make_float2(bf16_lo(m16), bf16_hi(m16));
+        vv = make_float2(bf16_lo(v16), bf16_hi(v16));
+      }
+      *reinterpret_cast<float2*>(mean_s + j * D + 2 * cp) = mm;
+      *reinterpret_cast<float2*>(var_s + j * D + 2 * cp) = vv;
     }
     __syncthreads();
     for (int row0 = warp * kOwnRows; row0 < ng * G; row0 += kOwnRows * (kOwnThreads / 32)) {
@@ -249,10 +318,13 @@ __global__ void __launch_bounds__(128) prefill_scan_state_kernel(const Params p,
 
 template <int D>
 cudaError_t own_d(const Params& p, const PrefillChunk& c, const void* q, float* out, int* sel_user, cudaStream_t s) {
-  const size_t smem = (size_t)2 * kOwnGroup * D * 4;
+  const size_t smem = (size_t)2 * kOwnGroup * D * 4 + (size_t)p.B * D * 2;
+  auto kern = prefill_own_kernel<D>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
   // (not launched ahead of the append's end like the others: its CTAs would crowd onto the SMs that are free first; 512 tokens
   // on 32768 x 2: 293 us so, 306 us launched ahead)
-  return launch_ex(prefill_own_kernel<D>, dim3((c.T + p.B - 2) / p.B + 1, p.batch * p.Hkv), dim3(kOwnThreads), smem, s, 0, false,
+  return launch_ex(kern, dim3((c.T + p.B - 2) / p.B + 1, p.batch * p.Hkv), dim3(kOwnThreads), smem, s, 0, false,
                    p, c, reinterpret_cast<const __nv_bfloat16*>(q), out, sel_user);
 }
 
