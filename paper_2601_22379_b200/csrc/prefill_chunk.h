@@ -17,8 +17,8 @@ struct PrefillChunk {
   int n_sb;             // SB ranges of the chunk, at most
   int s0, ns;           // ... of this launch
   int stride;           // floats per (position, head) row of ell
-  float* ell;           // [U][ns * SB][G][stride]  log masses of the complete blocks, for the positions of this launch
-  float* ell_own;       // [U][T][G]                log mass of every position's own, growing block
+  float* ell;           // [U][ns * SB][G][stride]  log masses of the complete blocks less ln B, for the positions of this launch
+  float* ell_own;       // [U][T][G]                log mass of every position's own, growing block, less ln B
   float* snap;          // [U][n_sb][d][d]          the recurrent state at the start of every SB range (the first: of the chunk)
   int* sel;             // [U][T][top_k]            selected blocks, ascending, padded with -1
 };

@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kOwnThreads) prefill_own_kernel(const Params p
       if (p.flags & 2u) dv = 0.f;
       const int row = row0 + (lane >> 2), j = row / G, pos = t0 + g0 + j;
       if (lane < 16 && (lane & 3) == 0 && row < ng * G && pos >= r.L0)
-        pc.ell_own[((size_t)r.u * pc.T + (pos - r.first)) * G + row % G] = logf((float)(g0 + j + 1)) + vals[0] + __logf(1.f + dv);
+        pc.ell_own[((size_t)r.u * pc.T + (pos - r.first)) * G + row % G] = logf((float)(g0 + j + 1) / (float)p.B) + vals[0] + __logf(1.f + dv);
     }
     if (g0 + kOwnGroup < cnt) fetch(g0 + kOwnGroup, warp * kOwnRows, min(kOwnGroup, cnt - g0 - kOwnGroup));   // ... or the first of the next
     __syncthreads();

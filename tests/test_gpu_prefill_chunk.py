@@ -170,6 +170,6 @@ def test_a_positions_own_block_has_the_record_that_a_step_stores(d, B, flags):
         pos = K0.shape[2] + t
         mean, var = step.bufs.stats[0, :, pos // B].double().unbind(1)
         x = q[0, t].double().view(2, G, d) / d ** 0.5
-        want = np.log(pos % B + 1) + (x * mean[:, None]).sum(-1) + torch.log1p((0.5 * x * x * var[:, None]).sum(-1))
+        want = np.log((pos % B + 1) / B) + (x * mean[:, None]).sum(-1) + torch.log1p((0.5 * x * x * var[:, None]).sum(-1))
         worst = max(worst, (got[:, t] - want).abs().max().item())
     assert worst < 2e-6, worst
