@@ -209,14 +209,18 @@ int spla_decode_selected(spla_cache_t *cache, const void *q, const float *rms_we
  *                 reports for this T; with more (up to `good_bytes`) more positions are processed per kernel launch.
  * bf16 caches and queries with at most 16384 blocks per sequence run on the tensor cores (all positions of a chunk as
  * contractions); fp32, longer sequences and SPLA_GENERAL_KERNELS take the general kernels, one virtual unit per
- * position.  Strided selection windows are not supported (SPLA_ERR_UNSUPPORTED).  Returns SPLA_ERR_CAPACITY, with nothing enqueued, if the chunk does not fit.
+ * position.  (The latter also serve a call whose scratch is below `min_bytes` but enough for them.)  Strided selection
+ * windows are not supported (SPLA_ERR_UNSUPPORTED).  Returns SPLA_ERR_CAPACITY, with nothing enqueued, if the chunk does not
+ * fit.
  */
 int spla_prefill(spla_cache_t *cache, const void *k_new, const void *v_new, const void *q, int32_t T,
                  const float *rms_weight, float *out, int32_t *sel_idx, void *workspace, size_t workspace_bytes,
                  void *stream);
 
 /* Workspace of spla_prefill for chunks of T tokens: the least it runs with, and a size that lets it work efficiently.
- * HOST pointers; either may be NULL. */
+ * On the tensor cores: for every range of 64 (or 128) positions of every KV head a recurrent state, for every position its
+ * selection, and the block log masses of as many row tiles (at most 128 query rows of one KV head) as are worked on at once:
+ * one at the least, 256 MB's worth at best.  Results do not depend on the size.  HOST pointers; either may be NULL. */
 int spla_query_prefill_workspace(const spla_config_t *config, int32_t T, size_t *min_bytes, size_t *good_bytes);
 
 /* Block scores of the last spla_decode: DEVICE fp32 [batch][H_kv][max_blocks] copy-out (entries >= nblk are 0). */

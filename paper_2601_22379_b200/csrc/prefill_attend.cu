@@ -205,9 +205,9 @@ __global__ void __launch_bounds__(kPaThreads, 1)
   pdl_launch_dependents();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wg = warp >> 2;
   const int G = p.G, B = p.B;
-  const PrefillUnit r = prefill_unit_of(p, pc, blockIdx.y);
+  const PrefillUnit r = prefill_unit_of(p, pc, pc.u0 + blockIdx.y);
   // the last positions of a chunk see most: their tiles start first
-  const int sb = pc.s0 + (pc.ns - 1 - (int)blockIdx.x / pc.nt), tile = pc.nt - 1 - (int)blockIdx.x % pc.nt;
+  const int tq = pc.q0 + pc.nq - 1 - (int)blockIdx.x, sb = tq / pc.nt, tile = tq % pc.nt;
   const int sb_start = prefill_range_start(pc, r, sb);
   const int pos0 = sb_start + tile * pc.P;
   const int pos_lo = max(pos0, r.L0), pos_hi = min(min(pos0 + pc.P, sb_start + pc.SB), r.L_end);
@@ -762,8 +762,8 @@ cudaError_t attend_d(const Params& p, const PrefillChunk& c, const AttendMaps& m
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, PaSmem<D>::kBytes);
   if (e != cudaSuccess) return e;
   // Launched ahead of the selection's end up to two waves of CTAs (288: 294 -> 290 us per chunk; 2064: 1553 -> 1569 us).
-  const bool ahead = (long long)c.ns * c.nt * p.batch * p.Hkv <= 2 * 148;
-  return launch_ex(kern, dim3(c.ns * c.nt, p.batch * p.Hkv), dim3(kPaThreads), PaSmem<D>::kBytes, s, 0, ahead,
+  const bool ahead = (long long)c.nq * c.nu <= 2 * 148;
+  return launch_ex(kern, dim3(c.nq, c.nu), dim3(kPaThreads), PaSmem<D>::kBytes, s, 0, ahead,
                    p, c, *reinterpret_cast<const CUtensorMap*>(maps.k), *reinterpret_cast<const CUtensorMap*>(maps.v),
                    reinterpret_cast<const __nv_bfloat16*>(q), w, out);
 }

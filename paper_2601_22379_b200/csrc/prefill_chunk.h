@@ -14,10 +14,11 @@ constexpr int kPfMaxBlocks = 16384;      // blocks per sequence the path serves 
 struct PrefillChunk {
   int T;                // positions per sequence
   int SB, P, nt;
-  int n_sb;             // SB ranges of the chunk, at most
-  int s0, ns;           // ... of this launch
+  int n_sb;             // SB ranges of the chunk, at most; nt row tiles each
+  int q0, nq;           // row tiles of this launch ...
+  int u0, nu;           // ... and units
   int stride;           // floats per (position, head) row of ell
-  float* ell;           // [U][ns * SB][G][stride]  log masses of the complete blocks less ln B, for the positions of this launch
+  float* ell;           // [nu][nq * P][G][stride]  log masses of the complete blocks less ln B, for the positions of this launch
   float* ell_own;       // [U][T][G]                log mass of every position's own, growing block, less ln B
   float* snap;          // [U][n_sb][d][d]          the recurrent state at the start of every SB range (the first: of the chunk)
   int* sel;             // [U][T][top_k]            selected blocks, ascending, padded with -1

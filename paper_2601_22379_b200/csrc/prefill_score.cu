@@ -62,9 +62,9 @@ __global__ void __launch_bounds__(kPsThreads, 1) prefill_score_kernel(const Para
   pdl_wait();
   pdl_launch_dependents();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const PrefillUnit r = prefill_unit_of(p, pc, blockIdx.z);
+  const PrefillUnit r = prefill_unit_of(p, pc, pc.u0 + blockIdx.z);
   const int G = p.G;
-  const int sb = pc.s0 + blockIdx.y / pc.nt, tile = blockIdx.y % pc.nt;
+  const int sb = (pc.q0 + (int)blockIdx.y) / pc.nt, tile = (pc.q0 + (int)blockIdx.y) % pc.nt;
   const int sb_start = prefill_range_start(pc, r, sb);
   const int pos0 = sb_start + tile * pc.P;                     // position of row 0 (may lie before the chunk)
   const int pos_hi = min(min(pos0 + pc.P, sb_start + pc.SB), r.L_end);   // one past the last position
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(kPsThreads, 1) prefill_score_kernel(const Para
       __syncwarp();
       if (lane == 0) mbar_arrive1(q_ready);
     }
-    const size_t slot = ((size_t)r.u * pc.ns + (sb - pc.s0)) * pc.SB + (live ? pos - sb_start : 0);
+    const size_t slot = ((size_t)blockIdx.z * pc.nq + blockIdx.y) * pc.P + (live ? pos - pos0 : 0);
     float* dst = pc.ell + (slot * G + row % G) * pc.stride + rec0;
     const float half_s2 = (p.flags & 2u) ? 0.f : 0.5f * p.sm_scale * p.sm_scale;
 #pragma unroll 1
@@ -263,12 +263,12 @@ __global__ void __launch_bounds__(256, 2) prefill_select_kernel(const Params p, 
   pdl_wait();
   pdl_launch_dependents();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const PrefillUnit r = prefill_unit_of(p, pc, blockIdx.y);
+  const PrefillUnit r = prefill_unit_of(p, pc, pc.u0 + blockIdx.y);
   const int G = p.G;
-  const int slot = blockIdx.x * (8 / W) + (W == 1 ? warp : 0);   // position within the launch's SB ranges
-  const int sb_start = prefill_range_start(pc, r, pc.s0 + slot / pc.SB);
-  const int pos = sb_start + slot % pc.SB;
-  if (slot >= pc.ns * pc.SB || pos < r.L0 || pos >= r.L_end) return;   // uniform over the position's warps
+  const int slot = blockIdx.x * (8 / W) + (W == 1 ? warp : 0);   // position within the launch's row tiles
+  const int tq = pc.q0 + slot / pc.P, in_range = tq % pc.nt * pc.P + slot % pc.P;
+  const int pos = prefill_range_start(pc, r, tq / pc.nt) + in_range;
+  if (slot >= pc.nq * pc.P || in_range >= pc.SB || pos < r.L0 || pos >= r.L_end) return;   // uniform over the position's warps
   const int t = pos - r.first;
   const int own = pos / p.B, nblk = own + 1;
   const int k_eff = min(p.top_k, nblk);
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(256, 2) prefill_select_kernel(const Params p, 
   float sc[NK];
 #pragma unroll
   for (int k = 0; k < NK; ++k) sc[k] = 0.f;
-  const float* ell = pc.ell + (((size_t)r.u * pc.ns * pc.SB + slot) * G) * pc.stride;
+  const float* ell = pc.ell + (((size_t)blockIdx.y * pc.nq * pc.P + slot) * G) * pc.stride;
   for (int g = 0; g < G; ++g) {
     const float e_own = pc.ell_own[((size_t)r.u * pc.T + t) * G + g];
     float e[NK], mx = -INFINITY;
@@ -468,8 +468,8 @@ cudaError_t score_d(const Params& p, const PrefillChunk& c, const void* q, int m
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   // Tiles of records per CTA: what leaves the fewest tile times, a CTA's start counted as one (one CTA per SM).
-  const int U = p.batch * p.Hkv, all = (max_blocks_seen + kPsRec - 1) / kPsRec;
-  const long long row_tiles = (long long)c.ns * c.nt * U;
+  const int all = (max_blocks_seen + kPsRec - 1) / kPsRec;
+  const long long row_tiles = (long long)c.nq * c.nu;
   int per = all;
   long long best = -1;
   for (int ny = 1; ny <= all; ++ny) {
@@ -477,19 +477,19 @@ cudaError_t score_d(const Params& p, const PrefillChunk& c, const void* q, int m
     const long long cost = (row_tiles * ((all + n - 1) / n) + sm_count - 1) / sm_count * (n + 1);
     if (best < 0 || cost < best) { best = cost; per = n; }
   }
-  return launch_ex(kern, dim3((all + per - 1) / per, c.ns * c.nt, U), dim3(kPsThreads), smem, s, 0, true,
+  return launch_ex(kern, dim3((all + per - 1) / per, c.nq, c.nu), dim3(kPsThreads), smem, s, 0, true,
                    p, c, reinterpret_cast<const __nv_bfloat16*>(q), per * kPsRec);
 }
 
 template <int W, int NK>
 cudaError_t select_w(const Params& p, const PrefillChunk& c, int* sel_user, cudaStream_t s) {
-  const int slots = c.ns * c.SB;
-  return launch_ex(prefill_select_kernel<W, NK>, dim3((slots + 8 / W - 1) / (8 / W), p.batch * p.Hkv), dim3(256), 0, s, 0, true, p, c, sel_user);
+  const int slots = c.nq * c.P;
+  return launch_ex(prefill_select_kernel<W, NK>, dim3((slots + 8 / W - 1) / (8 / W), c.nu), dim3(256), 0, s, 0, true, p, c, sel_user);
 }
 
 }  // namespace
 
-// Log masses of the complete blocks, for the positions of SB ranges c.s0 .. c.s0 + c.ns - 1.  max_blocks_seen: blocks of the
+// Log masses of the complete blocks, for the row tiles and units of one launch.  max_blocks_seen: blocks of the
 // longest sequence after the chunk.
 cudaError_t launch_prefill_score(const Params& p, const PrefillChunk& c, const void* q, int max_blocks_seen, int sm_count, cudaStream_t s) {
   if (p.flags & kStatsBf16)

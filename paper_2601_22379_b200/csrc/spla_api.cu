@@ -502,12 +502,12 @@ static int prefill_batch_cap(const spla_config_t* c) {   // virtual units are th
   return (int)(65535 / U);
 }
 
-// Workspace of the tensor-core path: tables for the whole chunk, then the log masses of `ns` ranges of SB positions.
+// Workspace of the tensor-core path: tables for the whole chunk, then the log masses of `tiles` row tiles (of any units).
 struct PrefillChunkLayout {
   size_t ell_own, snap, sel, ell, total;
 };
 
-static PrefillChunkLayout prefill_chunk_layout(const spla_config_t* c, int T, int ns) {
+static PrefillChunkLayout prefill_chunk_layout(const spla_config_t* c, int T, size_t tiles) {
   PrefillChunkLayout w;
   const size_t U = (size_t)c->batch * c->n_kv_heads, G = c->n_q_heads / c->n_kv_heads, d = c->head_dim;
   const size_t max_blocks = ((size_t)c->max_context + c->block_size - 1) / c->block_size;
@@ -518,7 +518,7 @@ static PrefillChunkLayout prefill_chunk_layout(const spla_config_t* c, int T, in
   w.ell_own = take(U * T * G * 4);
   w.snap = take((c->flags & SPLA_NO_RLA) ? 0 : U * prefill_ranges(T, SB) * d * d * 4);
   w.sel = take(U * T * c->top_k * 4);
-  w.ell = take(U * ns * SB * G * align_up(max_blocks, 32) * 4);
+  w.ell = take(tiles * P * G * align_up(max_blocks, 32) * 4);
   w.total = off;
   return w;
 }
@@ -531,13 +531,14 @@ extern "C" int spla_query_prefill_workspace(const spla_config_t* config, int32_t
   const bool fast = prefill_on_tensor_cores(config);
   int SB, P, nt;
   prefill_tiling(config->n_q_heads / config->n_kv_heads, config->block_size, &SB, &P, &nt);
-  auto total = [&](int units) { return fast ? prefill_chunk_layout(config, T, units).total : prefill_layout(config, T, units).total; };
+  // tensor cores: whole ranges of all units at a time (at the least, one row tile of one unit); else positions
+  const size_t range_tiles = (size_t)config->batch * config->n_kv_heads * nt;
+  auto total = [&](int n) { return fast ? prefill_chunk_layout(config, T, n * range_tiles).total : prefill_layout(config, T, n).total; };
   const long long most = fast ? prefill_ranges(T, SB) : (T < prefill_batch_cap(config) ? T : prefill_batch_cap(config));
-  const size_t one = total(1);
-  if (min_bytes) *min_bytes = one;
+  if (min_bytes) *min_bytes = fast ? prefill_chunk_layout(config, T, 1).total : total(1);
   if (good_bytes) {
     // about 256 MB of per-batch scratch, at most the whole chunk at once
-    const size_t per = total(2) - one;
+    const size_t per = total(2) - total(1);
     long long n = (long long)((256ull << 20) / (per ? per : 1));
     if (n < 1) n = 1;
     if (n > most) n = most;
@@ -557,24 +558,28 @@ static int prefill_chunked(spla_cache* c, const void* q, int T, const float* rms
   const PrefillChunkLayout w = prefill_chunk_layout(&c->cfg, T, 1);
   const int blocks = (int)((c->len_bound + c->p.B - 1) / c->p.B);
   pc.stride = (int)align_up(blocks, 32);
-  // SB ranges per launch: as many as the workspace holds at this sequence length
-  const size_t per = (size_t)c->p.batch * c->p.Hkv * pc.SB * c->p.G * pc.stride * 4;
-  long long ns = (long long)((workspace_bytes - w.ell) / per);
-  if (ns > pc.n_sb) ns = pc.n_sb;
-  if (ns > 65535 / pc.nt) ns = 65535 / pc.nt;             // (a grid dimension)
-  if (ns < 1) ns = 1;                                     // (the minimum workspace holds one range at the largest length)
+  // row tiles per launch: as many as the workspace holds at this sequence length (the minimum one holds one at the largest),
+  // of all units if it holds that many
+  const int U = c->p.batch * c->p.Hkv, n_tiles = pc.n_sb * pc.nt;
+  const size_t fit = (workspace_bytes - w.ell) / ((size_t)pc.P * c->p.G * pc.stride * 4);
+  const int nu = fit < (size_t)U ? (int)fit : U;
+  size_t nq = fit / nu;
+  if (nq > (size_t)n_tiles) nq = n_tiles;
+  if (nq > 65535) nq = 65535;                             // (a grid dimension)
   pc.ell_own = (float*)(ws + w.ell_own);
   pc.snap = (float*)(ws + w.snap);
   pc.sel = (int*)(ws + w.sel);
   pc.ell = (float*)(ws + w.ell);
   cudaError_t e = launch_prefill_own(c->p, pc, q, out, sel_idx, s);
   if (e == cudaSuccess && !(c->cfg.flags & SPLA_NO_RLA)) e = launch_prefill_state(c->p, pc, s);
-  for (int s0 = 0; s0 < pc.n_sb && e == cudaSuccess; s0 += (int)ns) {
-    pc.s0 = s0;
-    pc.ns = (int)(ns < pc.n_sb - s0 ? ns : pc.n_sb - s0);
-    e = launch_prefill_score(c->p, pc, q, blocks, c->sm_count, s);
-    if (e == cudaSuccess) e = launch_prefill_select(c->p, pc, blocks, sel_idx, s);
-    if (e == cudaSuccess) e = launch_prefill_attend(c->p, pc, c->prefill_maps, q, rms_weight, out, s);
+  for (pc.q0 = 0; pc.q0 < n_tiles && e == cudaSuccess; pc.q0 += (int)nq) {
+    pc.nq = (int)nq < n_tiles - pc.q0 ? (int)nq : n_tiles - pc.q0;
+    for (pc.u0 = 0; pc.u0 < U && e == cudaSuccess; pc.u0 += nu) {
+      pc.nu = nu < U - pc.u0 ? nu : U - pc.u0;
+      e = launch_prefill_score(c->p, pc, q, blocks, c->sm_count, s);
+      if (e == cudaSuccess) e = launch_prefill_select(c->p, pc, blocks, sel_idx, s);
+      if (e == cudaSuccess) e = launch_prefill_attend(c->p, pc, c->prefill_maps, q, rms_weight, out, s);
+    }
   }
   return e == cudaSuccess ? SPLA_OK : cuda_fail(e, "spla_prefill");
 }
@@ -590,10 +595,11 @@ extern "C" int spla_prefill(spla_cache_t* c, const void* k_new, const void* v_ne
   if (c->len_bound + T > c->cfg.max_context) return SPLA_ERR_CAPACITY;
   const int cap = prefill_batch_cap(&c->cfg);
   if (cap < 1) return SPLA_ERR_UNSUPPORTED;
-  const bool fast = prefill_on_tensor_cores(&c->cfg);
-  if (fast && !c->prefill_maps.valid) return SPLA_ERR_UNSUPPORTED;   // (the driver refused the tensor maps)
-  const size_t one = fast ? prefill_chunk_layout(&c->cfg, T, 1).total : prefill_layout(&c->cfg, T, 1).total;
-  if (workspace_bytes < one) return SPLA_ERR_INVALID_ARG;
+  // On the general kernels also where the driver refused the tensor maps, or where the scratch is enough for those only (less
+  // than the reported minimum, with few tokens and a short selection)
+  const size_t one = prefill_layout(&c->cfg, T, 1).total;
+  const bool fast = prefill_on_tensor_cores(&c->cfg) && c->prefill_maps.valid && workspace_bytes >= prefill_chunk_layout(&c->cfg, T, 1).total;
+  if (!fast && workspace_bytes < one) return SPLA_ERR_INVALID_ARG;
   char* ws = reinterpret_cast<char*>(workspace);
   cudaStream_t s = (cudaStream_t)stream;
   const int qb = c->cfg.q_dtype == SPLA_BF16;

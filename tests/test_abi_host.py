@@ -110,3 +110,21 @@ def test_null_and_misaligned_buffers_are_rejected_before_any_launch(lib):
 def test_missing_library_fails_loudly(tmp_path):
     with pytest.raises(RuntimeError, match="no fallback"):
         binding.load(str(tmp_path / "libspla.so"))
+
+
+@pytest.mark.parametrize("kw,T", [
+    (dict(batch=64, n_q_heads=32, n_kv_heads=8, head_dim=128, block_size=64, top_k=32, max_context=65536), 16),
+    (dict(batch=8, n_q_heads=32, n_kv_heads=8, head_dim=128, block_size=64, top_k=32, max_context=1 << 20), 1),
+    (dict(batch=1, n_q_heads=32, n_kv_heads=8, head_dim=128, block_size=64, top_k=32, max_context=131072), 4096),
+    (dict(batch=4, n_q_heads=128, n_kv_heads=8, head_dim=128, block_size=32, top_k=64, max_context=32768), 200),
+])
+def test_prefill_needs_no_more_scratch_than_the_general_kernels(lib, kw, T):
+    """At the least: one row tile's log masses, whatever the number of units and the configured context."""
+    sizes = []
+    for flags in (0, binding.SPLA_GENERAL_KERNELS):
+        lo, good = C.c_size_t(), C.c_size_t()
+        cfg = binding.make_config(flags=flags, **kw)
+        assert lib.spla_query_prefill_workspace(C.byref(cfg), T, C.byref(lo), C.byref(good)) == 0
+        assert 0 < lo.value <= good.value
+        sizes.append(lo.value)
+    assert sizes[0] <= sizes[1]

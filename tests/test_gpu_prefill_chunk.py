@@ -5,6 +5,8 @@ Tolerance: probabilities and linear coefficients enter their products as two bf1
 22 bits, everything else in fp32, so single outputs agree to a few 1e-5; the residual's error is that of its operands,
 2^-17 |o_bar|, times the RMSNorm's amplification 1 / |o_rla|, which the sizes below keep under about 10 (near-complete
 selection, where it is larger, is the last case, with its own bound)."""
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
@@ -173,3 +175,28 @@ def test_a_positions_own_block_has_the_record_that_a_step_stores(d, B, flags):
         want = np.log((pos % B + 1) / B) + (x * mean[:, None]).sum(-1) + torch.log1p((0.5 * x * x * var[:, None]).sum(-1))
         worst = max(worst, (got[:, t] - want).abs().max().item())
     assert worst < 2e-6, worst
+
+
+def test_scratch_that_is_enough_for_the_general_kernels_only():
+    """Few tokens of small groups: the general kernels need less than the tensor-core path (a state per range); a call with their
+    minimum runs on them, one with less is refused."""
+    case = (2, 2, 1, 128, 64, 1, 0, 0, 300, 3, 0)
+    w, K0, V0, k, v, q = _inputs(case)
+    gamma = synth.gamma(w).to(DEV)
+    want, sel, _ = _run(w, K0, V0, k, v, q, binding.SPLA_GENERAL_KERNELS)
+    sizes = []
+    for flags in (0, binding.SPLA_GENERAL_KERNELS):
+        lo = C.c_size_t()
+        assert binding.load().spla_query_prefill_workspace(C.byref(runner.config_for(w, flags=flags)), 3, C.byref(lo), None) == 0
+        sizes.append(lo.value)
+    assert sizes[1] < sizes[0]
+    for size, status in ((sizes[1], 0), (sizes[1] - 1, binding.SPLA_ERR_INVALID_ARG)):
+        cache = binding.SplaCache(runner.config_for(w), DEV)
+        cache.append_tokens(K0, V0)
+        ws, out = torch.empty(size, dtype=torch.uint8, device=DEV), torch.empty_like(want)
+        assert cache.lib.spla_prefill(cache.handle, k.data_ptr(), v.data_ptr(), q.data_ptr(), 3, gamma.data_ptr(), out.data_ptr(),
+                                      None, ws.data_ptr(), size, torch.cuda.current_stream().cuda_stream) == status
+        torch.cuda.synchronize()
+        assert cache.sync_status() == 0
+        if status == 0:
+            np.testing.assert_allclose(out.cpu().numpy(), want.cpu().numpy(), rtol=RTOL, atol=ATOL)
