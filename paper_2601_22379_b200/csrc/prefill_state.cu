@@ -11,8 +11,14 @@ namespace spla {
 namespace {
 
 constexpr int kOwnThreads = 256;
-constexpr int kOwnGroup = 32;              // positions whose prefix statistics are in shared memory together
+constexpr int kOwnGroup = 16;              // positions whose prefix statistics are in shared memory together
 constexpr int kOwnRows = 4;                // (position, head) rows a warp works on side by side
+// a / n, correctly rounded, from y = 1 / n correctly rounded: one step of refinement with exact remainder (Markstein 1990; the
+// quotients here are far from the ends of the exponent range).  The plain division was a third of the kernel's instructions.
+__device__ __forceinline__ float2 div_by_count(float2 a, float n, float y) {
+  const float2 yy = make_float2(y, y), q = __fmul2_rn(a, yy);
+  return __ffma2_rn(__ffma2_rn(q, make_float2(-n, -n), a), yy, q);
+}
 template <int VEC> struct QueryVec { using type = uint2; };      // a lane's VEC query elements
 template <> struct QueryVec<2> { using type = uint32_t; };
 
@@ -23,9 +29,11 @@ template <> struct QueryVec<2> { using type = uint32_t; };
 // (channel pair, slot) takes every kSlots-th position of a group of kOwnGroup: running sums give the means, then one walk
 // over the older tokens serves all its positions.  After every group the eight warps form the dots of those prefixes with
 // their positions' queries.
-// Bound by instructions issued and the load latencies around them.
+// Bound by instructions issued (three quarters of the issue slots): 8192 tokens x 8 units, G = 4, 60 us (a running mean with
+// reciprocals, other bits, took 51); 512 tokens x 16 units 14 us, as that did.  Without the division by refinement, row / G by
+// multiplication and the packed dots it was 87 and 18 us; three CTAs an SM (80 registers, a few spilled) are no faster than two.
 template <int D>
-__global__ void __launch_bounds__(kOwnThreads) prefill_own_kernel(const Params p, const PrefillChunk pc,
+__global__ void __launch_bounds__(kOwnThreads, 2) prefill_own_kernel(const Params p, const PrefillChunk pc,
                                                                   const __nv_bfloat16* __restrict__ q, float* __restrict__ out,
                                                                   int* __restrict__ sel_user) {
   constexpr int VEC = D / 32;
@@ -34,6 +42,7 @@ __global__ void __launch_bounds__(kOwnThreads) prefill_own_kernel(const Params p
   constexpr int NP = kOwnGroup / kSlots;                       // positions of a thread
   static_assert(kSlots % TG == 0 && kOwnGroup % TG == 0, "a position's newest token is of the same sum in every group");
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ float inv_s[128], ln_s[128];                      // 1 / n, correctly rounded; ln(n / B)
   float* mean_s = reinterpret_cast<float*>(smem_raw);          // [kOwnGroup][D]
   float* var_s = mean_s + kOwnGroup * D;                       // [kOwnGroup][D]
   uint32_t* key_s = reinterpret_cast<uint32_t*>(var_s + kOwnGroup * D);   // [B][D / 2] channel pairs
@@ -64,13 +73,16 @@ __global__ void __launch_bounds__(kOwnThreads) prefill_own_kernel(const Params p
   // fetched one row at a time where they are used, their latency was half of this kernel's time (33 -> 15 us for 144 CTAs).
   using QV = typename QueryVec<VEC>::type;
   QV qn[kOwnRows];
+  const uint32_t g_inv = 65536u / G + 1u;
+  auto of_row = [&](int row) { return (int)(row * g_inv >> 16); };   // row / G: exact for G <= 16 and rows below 4096
+  const __nv_bfloat16* q_unit = q + ((size_t)r.b * pc.T * p.Hq + (size_t)r.h * G) * D + lane * VEC;
+  const size_t q_step = (size_t)p.Hq * D;
   auto fetch = [&](int g0, int row0, int ng) {
 #pragma unroll
     for (int i = 0; i < kOwnRows; ++i) {
-      const int row = row0 + i, pos = t0 + g0 + row / G;
+      const int row = row0 + i, j = of_row(row), pos = t0 + g0 + j;
       const bool ok = row < ng * G && pos >= r.L0;
-      const size_t off = (((size_t)r.b * pc.T + (ok ? pos - r.first : 0)) * p.Hq + (size_t)r.h * G + row % G) * D + lane * VEC;
-      qn[i] = ok ? __ldg(reinterpret_cast<const QV*>(q + off)) : QV();
+      qn[i] = ok ? __ldg(reinterpret_cast<const QV*>(q_unit + (size_t)(pos - r.first) * q_step + (row - j * G) * D)) : QV();
     }
   };
   const int g_begin = max(0, r.L0 - t0) / kOwnGroup * kOwnGroup;   // the first group with a position of the chunk
@@ -79,6 +91,10 @@ __global__ void __launch_bounds__(kOwnThreads) prefill_own_kernel(const Params p
     uint4* dst = reinterpret_cast<uint4*>(key_s);              // rows past the end: zeros, in no prefix
 #pragma unroll 4
     for (int x = tid; x < p.B * (D / 8); x += kOwnThreads) dst[x] = x < cnt * (D / 8) ? kc[x] : make_uint4(0u, 0u, 0u, 0u);
+  }
+  if (tid < 128) {
+    inv_s[tid] = __frcp_rn((float)(tid + 1));
+    ln_s[tid] = logf((float)(tid + 1) / (float)p.B);
   }
   __syncthreads();
   const int cp = tid % (D / 2), slot = tid / (D / 2);
@@ -92,28 +108,23 @@ __global__ void __launch_bounds__(kOwnThreads) prefill_own_kernel(const Params p
     const bool wanted = g0 >= g_begin;
     float2 nm[NP];                                             // minus the mean of each of the thread's positions
 #pragma unroll
-    for (int b = 0; b < kOwnGroup; b += kSlots) {              // (p.B is a multiple of kSlots: the reads stay inside the block)
-      if (g0 + b < p.B) {
+    for (int b = 0; b < NP; ++b)                               // (blocks are whole groups: the reads stay inside the block)
 #pragma unroll
-        for (int j = 0; j < kSlots; ++j) {
-          run[j % TG] = __fadd2_rn(run[j % TG], key2(g0 + b + j));
-          if (j == slot) {
-            float2 tot = run[0];
+      for (int j = 0; j < kSlots; ++j) {
+        run[j % TG] = __fadd2_rn(run[j % TG], key2(g0 + b * kSlots + j));
+        if (j == slot) {
+          nm[b] = run[0];
 #pragma unroll
-            for (int g = 1; g < TG; ++g) tot = __fadd2_rn(tot, run[g]);
-            nm[b / kSlots] = tot;
-          }
+          for (int g = 1; g < TG; ++g) nm[b] = __fadd2_rn(nm[b], run[g]);
         }
-      } else {
-        nm[b / kSlots] = make_float2(0.f, 0.f);
       }
-    }
     if (!wanted) continue;
     float2 ss[NP][TG];
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
-      const float n = (float)(g0 + i * kSlots + slot + 1);
-      nm[i] = make_float2(-(nm[i].x / n), -(nm[i].y / n));
+      const int j = g0 + i * kSlots + slot;
+      const float2 mean = div_by_count(nm[i], (float)(j + 1), inv_s[j]);
+      nm[i] = make_float2(-mean.x, -mean.y);
 #pragma unroll
       for (int g = 0; g < TG; ++g) ss[i][g] = make_float2(0.f, 0.f);
     }
@@ -121,7 +132,7 @@ __global__ void __launch_bounds__(kOwnThreads) prefill_own_kernel(const Params p
       const float2 dv = __fadd2_rn(x, nm[i]);
       ss[i][g] = __ffma2_rn(dv, dv, ss[i][g]);
     };
-#pragma unroll 1
+#pragma unroll 2
     for (int t = 0; t < g0; t += TG) {                         // tokens of earlier groups: in every prefix of this one
 #pragma unroll
       for (int g = 0; g < TG; ++g) {
@@ -131,25 +142,21 @@ __global__ void __launch_bounds__(kOwnThreads) prefill_own_kernel(const Params p
       }
     }
 #pragma unroll
-    for (int b = 0; b < NP; ++b) {                             // the group's own tokens: those up to the position
-      if (g0 + b * kSlots < p.B) {
+    for (int b = 0; b < NP; ++b)                               // the group's own tokens: those up to the position
 #pragma unroll
-        for (int j = 0; j < kSlots; ++j) {
-          const float2 x = key2(g0 + b * kSlots + j);
-          if (j <= slot) add(b, j % TG, x);
+      for (int j = 0; j < kSlots; ++j) {
+        const float2 x = key2(g0 + b * kSlots + j);
+        if (j <= slot) add(b, j % TG, x);
 #pragma unroll
-          for (int i = b + 1; i < NP; ++i) add(i, j % TG, x);
-        }
+        for (int i = b + 1; i < NP; ++i) add(i, j % TG, x);
       }
-    }
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
       const int j = i * kSlots + slot;
-      const float n = (float)(g0 + j + 1);
       float2 tot = ss[i][0];
 #pragma unroll
       for (int g = 1; g < TG; ++g) tot = __fadd2_rn(tot, ss[i][g]);
-      float2 mm = make_float2(-nm[i].x, -nm[i].y), vv = make_float2(tot.x / n, tot.y / n);
+      float2 mm = make_float2(-nm[i].x, -nm[i].y), vv = div_by_count(tot, (float)(g0 + j + 1), inv_s[g0 + j]);
       if (round16) {
         const uint32_t m16 = pack_bf16(mm.x, mm.y), v16 = pack_bf16(vv.x, vv.y);
         mm = make_float2(bf16_lo(m16), bf16_hi(m16));
@@ -163,27 +170,28 @@ __global__ void __launch_bounds__(kOwnThreads) prefill_own_kernel(const Params p
       float vals[2 * kOwnRows];
 #pragma unroll
       for (int i = 0; i < kOwnRows; ++i) {
-        const int j = min((row0 + i) / G, ng - 1);
-        float x[VEC], mv[VEC], vv[VEC], dm = 0.f, dv = 0.f;
+        const int j = min(of_row(row0 + i), ng - 1);
+        float x[VEC], mv[VEC], vv[VEC];
         load_vec<VEC>(reinterpret_cast<const __nv_bfloat16*>(&qn[i]), x);
         load_vec<VEC>(mean_s + j * D + lane * VEC, mv);
         load_vec<VEC>(var_s + j * D + lane * VEC, vv);
+        float2 dm = make_float2(0.f, 0.f), dv = dm;
 #pragma unroll
-        for (int v = 0; v < VEC; ++v) {
-          const float qh = x[v] * p.sm_scale;
-          dm = fmaf(qh, mv[v], dm);
-          dv = fmaf(0.5f * qh * qh, vv[v], dv);
+        for (int v = 0; v < VEC; v += 2) {
+          const float2 qh = __fmul2_rn(make_float2(x[v], x[v + 1]), make_float2(p.sm_scale, p.sm_scale));
+          dm = __ffma2_rn(qh, make_float2(mv[v], mv[v + 1]), dm);
+          dv = __ffma2_rn(__fmul2_rn(qh, qh), make_float2(vv[v], vv[v + 1]), dv);
         }
-        vals[i] = dm;
-        vals[kOwnRows + i] = dv;
+        vals[i] = dm.x + dm.y;
+        vals[kOwnRows + i] = dv.x + dv.y;
       }
       fetch(g0, row0 + kOwnRows * (kOwnThreads / 32), ng);       // the next rows of this group ...
       warp_reduce_multi<2 * kOwnRows>(vals, lane);               // value lane / 4: the mean dots, then the variance dots
       float dv = __shfl_xor_sync(0xffffffffu, vals[0], 16);
       if (p.flags & 2u) dv = 0.f;
-      const int row = row0 + (lane >> 2), j = row / G, pos = t0 + g0 + j;
+      const int row = row0 + (lane >> 2), j = of_row(row), pos = t0 + g0 + j;
       if (lane < 16 && (lane & 3) == 0 && row < ng * G && pos >= r.L0)
-        pc.ell_own[((size_t)r.u * pc.T + (pos - r.first)) * G + row % G] = logf((float)(g0 + j + 1) / (float)p.B) + vals[0] + __logf(1.f + dv);
+        pc.ell_own[((size_t)r.u * pc.T + (pos - r.first)) * G + (row - j * G)] = ln_s[g0 + j] + vals[0] + __logf(fmaf(0.5f, dv, 1.f));
     }
     if (g0 + kOwnGroup < cnt) fetch(g0 + kOwnGroup, warp * kOwnRows, min(kOwnGroup, cnt - g0 - kOwnGroup));   // ... or the first of the next
     __syncthreads();
