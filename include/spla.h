@@ -208,8 +208,9 @@ int spla_decode_selected(spla_cache_t *cache, const void *q, const float *rms_we
  *   workspace:    DEVICE scratch, 256-byte aligned, of at least the `min_bytes` that spla_query_prefill_workspace
  *                 reports for this T; with more (up to `good_bytes`) more positions are processed per kernel launch.
  * bf16 caches and queries with at most 16384 blocks per sequence run on the tensor cores (all positions of a chunk as
- * contractions); fp32, longer sequences and SPLA_GENERAL_KERNELS take the general kernels, one virtual unit per
- * position.  (The latter also serve a call whose scratch is below `min_bytes` but enough for them.)  Strided selection
+ * contractions); fp32, longer sequences, SPLA_GENERAL_KERNELS and chunks of so few positions that it is faster take the
+ * general kernels, one virtual unit per position.  (The latter also serve a call whose scratch is below `min_bytes` but
+ * enough for them.)  Strided selection
  * windows are not supported (SPLA_ERR_UNSUPPORTED).  Returns SPLA_ERR_CAPACITY, with nothing enqueued, if the chunk does not
  * fit.
  */
@@ -220,7 +221,8 @@ int spla_prefill(spla_cache_t *cache, const void *k_new, const void *v_new, cons
 /* Workspace of spla_prefill for chunks of T tokens: the least it runs with, and a size that lets it work efficiently.
  * On the tensor cores: for every range of 64 (or 128) positions of every KV head a recurrent state, for every position its
  * selection, and the block log masses of as many row tiles (at most 128 query rows of one KV head) as are worked on at once:
- * one at the least, 256 MB's worth at best.  Results do not depend on the size.  HOST pointers; either may be NULL. */
+ * one at the least, 256 MB's worth at best.  A chunk short enough for either path is given enough for both.  Results do not
+ * depend on the size.  HOST pointers; either may be NULL. */
 int spla_query_prefill_workspace(const spla_config_t *config, int32_t T, size_t *min_bytes, size_t *good_bytes);
 
 /* Block scores of the last spla_decode: DEVICE fp32 [batch][H_kv][max_blocks] copy-out (entries >= nblk are 0). */

@@ -523,6 +523,33 @@ static PrefillChunkLayout prefill_chunk_layout(const spla_config_t* c, int T, si
   return w;
 }
 
+// Chunks of few positions on a long selection.  The tensor-core path walks the blocks that a row tile's positions selected one
+// after the other on one CTA per tile, about 1.8 us per 64 tokens at d = 128 however few rows the tile has; the general kernels
+// take a CTA per (position, KV head, selected block), which few positions spread over the device.  Measured over 3588 sizes (1 to
+// 128 positions x 1 to 32 units, groups of 1 to 16, blocks of 16 to 128, selections of 8 to 64 blocks, contexts of 2000 and
+// 30000): 1 position x 8 units, 64 blocks of 128, G = 4: 124 us on the general kernels, 290 on the tensor cores; 8 positions 253
+// and 519; 32 positions 747 and 611.  Both times in us as fitted there, to 12 % on average; the path that is faster by them is the
+// faster one, or within 5 % of it, in 96 % of the sizes (37 % off at most; always the tensor cores: up to 4.5 times).  Above
+// kShortRows virtual units the general kernels hardly ever won.
+constexpr long long kShortRows = 256;
+static bool prefill_short(const spla_config_t* c, int T) { return (long long)c->batch * c->n_kv_heads * T <= kShortRows; }
+static bool prefill_faster_on_general(const spla_config_t* c, int T, int64_t blocks) {
+  if (!prefill_short(c, T)) return false;
+  const int G = c->n_q_heads / c->n_kv_heads, U = c->batch * c->n_kv_heads;
+  int SB, P, nt;
+  prefill_tiling(G, c->block_size, &SB, &P, &nt);
+  const double gp = padded_group(G), d = c->head_dim / 128.0, picked = (double)(c->top_k < blocks ? c->top_k : blocks);
+  const int rows = T < P ? T : P, tiles = (T + rows - 1) / rows;
+  // the walk: neighbouring positions share most blocks, the more so the larger the blocks and the share of them that each selects
+  const double few = log2(blocks / picked), spread = c->block_size < 64 ? 0.22 * (few < 5 ? few : 5) : 0.14 * (few < 3.8 ? few : 3.8);
+  const double walk = picked * (1 + spread * log2((double)rows)) * c->block_size / 64;
+  const double waves = (double)U * tiles > 148 ? U * tiles / 148.0 : 1.0;
+  const double tensor = 44 + 16 * d + walk * waves * (0.5 + 1.3 * d);
+  const double general = 57 + 11 * gp * d * ((T + 31) / 32) + 1.3 * T +
+                         U * T * d * (picked * c->block_size * (0.067 * gp + 0.106) + blocks * (0.13 * gp + 0.14)) / 1000;
+  return general < tensor;
+}
+
 extern "C" int spla_query_prefill_workspace(const spla_config_t* config, int32_t T, size_t* min_bytes, size_t* good_bytes) {
   int rc = validate_config(config);
   if (rc) return rc;
@@ -533,17 +560,23 @@ extern "C" int spla_query_prefill_workspace(const spla_config_t* config, int32_t
   prefill_tiling(config->n_q_heads / config->n_kv_heads, config->block_size, &SB, &P, &nt);
   // tensor cores: whole ranges of all units at a time (at the least, one row tile of one unit); else positions
   const size_t range_tiles = (size_t)config->batch * config->n_kv_heads * nt;
-  auto total = [&](int n) { return fast ? prefill_chunk_layout(config, T, n * range_tiles).total : prefill_layout(config, T, n).total; };
-  const long long most = fast ? prefill_ranges(T, SB) : (T < prefill_batch_cap(config) ? T : prefill_batch_cap(config));
-  if (min_bytes) *min_bytes = fast ? prefill_chunk_layout(config, T, 1).total : total(1);
-  if (good_bytes) {
+  size_t lo = 0, good = 0;
+  for (int path = 0; path < 2; ++path) {                   // a short chunk may take either (by its length when it is called)
+    const bool tensor = path == 0;
+    if (tensor ? !fast : fast && !prefill_short(config, T)) continue;
+    auto total = [&](int n) { return tensor ? prefill_chunk_layout(config, T, n * range_tiles).total : prefill_layout(config, T, n).total; };
+    const long long most = tensor ? prefill_ranges(T, SB) : (T < prefill_batch_cap(config) ? T : prefill_batch_cap(config));
+    const size_t least = tensor ? prefill_chunk_layout(config, T, 1).total : total(1);
     // about 256 MB of per-batch scratch, at most the whole chunk at once
     const size_t per = total(2) - total(1);
     long long n = (long long)((256ull << 20) / (per ? per : 1));
     if (n < 1) n = 1;
     if (n > most) n = most;
-    *good_bytes = total((int)n);
+    if (lo < least) lo = least;
+    if (good < total((int)n)) good = total((int)n);
   }
+  if (min_bytes) *min_bytes = lo;
+  if (good_bytes) *good_bytes = good;
   return SPLA_OK;
 }
 
@@ -598,8 +631,9 @@ extern "C" int spla_prefill(spla_cache_t* c, const void* k_new, const void* v_ne
   // On the general kernels also where the driver refused the tensor maps, or where the scratch is enough for those only (less
   // than the reported minimum, with few tokens and a short selection)
   const size_t one = prefill_layout(&c->cfg, T, 1).total;
-  const bool fast = prefill_on_tensor_cores(&c->cfg) && c->prefill_maps.valid && workspace_bytes >= prefill_chunk_layout(&c->cfg, T, 1).total;
+  bool fast = prefill_on_tensor_cores(&c->cfg) && c->prefill_maps.valid && workspace_bytes >= prefill_chunk_layout(&c->cfg, T, 1).total;
   if (!fast && workspace_bytes < one) return SPLA_ERR_INVALID_ARG;
+  if (fast && workspace_bytes >= one) fast = !prefill_faster_on_general(&c->cfg, T, (c->len_bound + T + c->cfg.block_size - 1) / c->cfg.block_size);
   char* ws = reinterpret_cast<char*>(workspace);
   cudaStream_t s = (cudaStream_t)stream;
   const int qb = c->cfg.q_dtype == SPLA_BF16;

@@ -63,21 +63,32 @@ def _run(w, K0, V0, k, v, q, flags, **kw):
         cache.append_tokens(K0, V0)
     T = k.shape[2]
     sel = torch.full((w.batch, T, w.n_kv_heads, w.top_k), -7, dtype=torch.int32, device=DEV)
+    n0 = binding.launch_count()
     out = cache.prefill(k, v, q, synth.gamma(w).to(DEV), sel_idx=sel, **kw)
+    cache.launches = binding.launch_count() - n0
     torch.cuda.synchronize()
     assert cache.sync_status() == 0
     return out, sel, cache
+
+
+def _launches(w, T, flags, tensor):
+    """Kernels of one prefill whose scratch holds the whole chunk: the append, then own-block masses, states, scan, scores,
+    selection and attention, or (general) statistics, scan, scores and attention."""
+    one_pass = tensor and w.head_dim == 128 and w.batch * w.n_kv_heads * T >= 64
+    rla = not flags & binding.SPLA_NO_RLA
+    return (1 if T <= 32 or one_pass else 2) + (4 + 2 * rla if tensor else 3 + rla)
 
 
 @pytest.mark.parametrize("case", CASES, ids=lambda c: "-".join(map(str, c)))
 def test_tensor_core_prefill_equals_the_general_kernels(case):
     w, K0, V0, k, v, q = _inputs(case)
     flags = case[-1]
-    n0 = binding.launch_count()
     a, sel_a, ca = _run(w, K0, V0, k, v, q, flags)
-    n1 = binding.launch_count()
     b, sel_b, cb = _run(w, K0, V0, k, v, q, flags | binding.SPLA_GENERAL_KERNELS)
-    assert n1 > n0 and torch.isfinite(a).all()
+    assert ca.launches == _launches(w, k.shape[2], flags, True)
+    batches, odd = divmod(cb.launches - _launches(w, k.shape[2], flags, False), 2)   # (batches of positions beyond the first)
+    assert batches in (0, 1) and not odd
+    assert torch.isfinite(a).all()
     same = (sel_a == sel_b).all(dim=-1)                 # [batch, T, hkv]; near-ties may fall the other way
     assert same.float().mean().item() >= 0.99
     rows = same.repeat_interleave(w.group, dim=2)
@@ -126,7 +137,8 @@ def test_score_tiles_and_launch_sizes_at_their_edges(case):
 @pytest.mark.parametrize("k", [8, 32, 64])                # few keys reach the bound, about as many as are ranked, too many
 @pytest.mark.parametrize("blocks", [257, 513, 1023])
 def test_selection_from_the_keys_that_reach_a_bound(blocks, k):
-    test_tensor_core_prefill_equals_the_general_kernels((1, 2, 4, 64, 16, k, 1, 2, 16 * blocks + 3, 20, 0))
+    T = 20 if k < 64 else 60                              # (20 positions of the longest selection take the general kernels)
+    test_tensor_core_prefill_equals_the_general_kernels((1, 2, 4, 64, 16, k, 1, 2, 16 * blocks + 3, T, 0))
 
 
 def test_selection_among_equal_scores_takes_the_first_blocks():
@@ -200,3 +212,23 @@ def test_scratch_that_is_enough_for_the_general_kernels_only():
         assert cache.sync_status() == 0
         if status == 0:
             np.testing.assert_allclose(out.cpu().numpy(), want.cpu().numpy(), rtol=RTOL, atol=ATOL)
+
+
+@pytest.mark.parametrize("case,tensor", [
+    ((1, 2, 4, 128, 128, 40, 1, 4, 128 * 60, 1, 0), False),       # 80 tiles of 64 tokens one after the other, or 80 CTAs
+    ((1, 2, 4, 128, 128, 40, 1, 4, 128 * 60, 64, 0), True),
+    ((2, 4, 1, 64, 64, 64, 1, 4, 64 * 150, 8, 0), False),
+    ((2, 4, 1, 64, 64, 64, 1, 4, 64 * 150, 33, 0), True),         # more than 256 virtual units
+    ((1, 4, 8, 128, 64, 8, 1, 4, 64 * 150, 4, 0), True),          # a short selection
+], ids=str)
+def test_a_short_chunk_takes_the_path_that_is_faster_for_it(case, tensor):
+    w, K0, V0, k, v, q = _inputs(case)
+    a, sel_a, ca = _run(w, K0, V0, k, v, q, 0)
+    b, sel_b, cb = _run(w, K0, V0, k, v, q, binding.SPLA_GENERAL_KERNELS)
+    T = k.shape[2]
+    assert ca.launches - (_launches(w, T, 0, True) - 6) == (6 if tensor else 4)     # (the appends differ; not what follows)
+    rows = (sel_a == sel_b).all(dim=-1).repeat_interleave(w.group, dim=2)
+    assert rows.float().mean().item() >= 0.99
+    np.testing.assert_allclose(a[rows].cpu().numpy(), b[rows].cpu().numpy(), rtol=RTOL, atol=ATOL)
+    least, _, _ = _run(w, K0, V0, k, v, q, 0, workspace_bytes=1)
+    assert torch.equal(least, a)
