@@ -402,8 +402,12 @@ static cudaError_t launch_typed(const Params& p, const void* k_new, const void* 
     return launch_ex(kern, dim3(n_copy + n_stats + n_state, U), dim3(kFusedThreads), 0, stream, 0, true,
                      p, kn, vn, n_new, max_new, n_copy, n_stats);
   }
-  // bf16 with d = 128: everything in one pass, the state on the tensor cores; the rest in three kernels
-  if (sizeof(T) == 2 && D == 128 && maps && maps->valid && fresh_maps && fresh_maps->valid)
+  // bf16 with d = 128: everything in one pass, the state on the tensor cores; the rest in three kernels.  Among those a few tokens
+  // of many sequences of different lengths: the pass takes a CTA per unit and SM whatever a unit adds, 0.2 us per unit, the
+  // kernels take less the less there is (1 to 33, 40, 48, 64 tokens, 512 units: 42, 50, 58, 60 us against 59 to 61; 1024 units 71,
+  // 83, 89, 99 against 104; 256 units 32 to 42 against 33 to 35; all at the longest: 65, 69, 75, 93 against 64).
+  const bool few_of_many = n_new && U > 2 * 148 && max_new < 48;
+  if (sizeof(T) == 2 && D == 128 && maps && maps->valid && fresh_maps && fresh_maps->valid && !few_of_many)
     return launch_append_bulk(p, *maps, *fresh_maps, n_new, max_new, stream);
   {
     const size_t tile_bytes = (size_t)p.B * D * sizeof(T);

@@ -112,3 +112,22 @@ def test_a_wait_that_runs_out_is_reported_and_adds_nothing_to_the_state(batch):
     assert cache.sync_status() == 0
     for name in ("seq_lens", "k_cache", "v_cache", "stats", "tok_lse", "rla_state"):
         assert torch.equal(getattr(cache.bufs, name), getattr(want.bufs, name)), name
+
+
+@pytest.mark.parametrize("n,ragged,launches", [(47, True, 3), (48, True, 1), (47, False, 1)])
+def test_few_tokens_of_many_sequences_of_different_lengths_take_the_three_kernels(n, ragged, launches):
+    """75 x 4 units, more than two waves of the one-pass kernel's CTAs; the same statistics, log-sum-exps and state either way."""
+    w = synth.Workload("case", 8, batch=75, n_q_heads=4, n_kv_heads=4, head_dim=128, block_size=64, top_k=8, context=200)
+    caches = [binding.SplaCache(runner.config_for(w, flags=f), DEV) for f in (0, binding.SPLA_GENERAL_KERNELS)]
+    g = torch.Generator(device=DEV).manual_seed(9)
+    k, v = (torch.randn(75, 4, n, 128, generator=g, device=DEV).to(torch.bfloat16) for _ in range(2))
+    n_new = torch.randint(0, n + 1, (75,), generator=torch.Generator().manual_seed(n), dtype=torch.int32).to(DEV) if ragged else None
+    for i, c in enumerate(caches):
+        before = binding.launch_count()
+        c.append_tokens(k, v, n_new)
+        assert binding.launch_count() - before == (launches, 3)[i]
+    torch.cuda.synchronize()
+    a, b = caches
+    assert a.sync_status() == 0 and torch.equal(a.bufs.seq_lens, b.bufs.seq_lens)
+    assert torch.equal(a.bufs.stats, b.bufs.stats) and torch.equal(a.bufs.tok_lse, b.bufs.tok_lse)
+    assert parity.rel_l2(a.bufs.rla_state.cpu().numpy(), b.bufs.rla_state.cpu().numpy()) < 2 * parity.STATE_TOL_FMA
