@@ -15,7 +15,7 @@
 //   warp 2      TMA stores of whole tiles from the ring into the cache;
 //   warps 4-11  two groups taking the tiles in turn: log-sum-exp and phi(k) = exp(phi_scale k - lse) of a row by the eight
 //               lanes that hold it; on tiles that are not wholly new also the row-wise cache writes and the zeroing of what
-//               is not new.  They also drain the accumulator into fp32 registers every two tiles: the tensor core does not
+//               is not new.  They also drain the accumulator into fp32 registers every tile or two: the tensor core does not
 //               round to nearest when it adds (1e-4 relative after a chain of 4000 instructions);
 //   warps 12-15 block statistics: two exact passes in the summation order of the other append kernels (same bits), one
 //               channel pair and every second token per thread.
@@ -47,7 +47,10 @@ constexpr int kAbHalf = kAbTile * 128;                       // one TMA box: 64 
 constexpr int kAbTileBytes = 2 * kAbHalf;                    // 16 KB: all 128 channels
 constexpr int kAbMaxParts = 3;                               // bf16 parts of phi, at most
 constexpr int kAbTwoParts = 256;                             // new tokens per sequence from which two parts are used
-constexpr int kAbGroup = 2;                                  // tiles accumulated in tensor memory before a drain
+// Tiles accumulated in tensor memory before a drain: two; one where phi has all its bits, whose sums would otherwise show the
+// cuts of the tensor core's adder (S_bar after 40 to 255 tokens, against 64 bits: 1.0e-7 to 1.4e-7 so, 3.4e-7 to 4.5e-7 after two
+// tiles and the largest terms first, 2.6e-7 to 5.9e-7 from the fp32 kernels; 255 tokens x 512 units 90 -> 92 us).
+template <int PARTS> constexpr int kAbGroupOf = PARTS == 3 ? 1 : 2;
 constexpr int kAbTmemCols = 256;                             // two 128-column accumulators, used in turn
 // shared memory: ring [stage][K, V], phi [2][part], reduction buffers of the statistics, barriers
 constexpr int kAbPhi = kAbStages * 2 * kAbTileBytes;
@@ -71,7 +74,7 @@ __global__ void __launch_bounds__(kAbThreads, 1)
     append_bulk_kernel(const Params p, const __grid_constant__ CUtensorMap map_kn, const __grid_constant__ CUtensorMap map_vn,
                        const __grid_constant__ CUtensorMap map_kc, const __grid_constant__ CUtensorMap map_vc,
                        const int* __restrict__ n_new, int max_new) {
-  constexpr int D = kAbD;
+  constexpr int D = kAbD, kAbGroup = kAbGroupOf<PARTS>;
   extern __shared__ __align__(1024) unsigned char smem[];
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + kAbBars);   // TMA -> everybody
   uint64_t* empty = full + kAbStages;                             // everybody -> TMA
@@ -173,8 +176,10 @@ __global__ void __launch_bounds__(kAbThreads, 1)
           const uint32_t a = umma_desc_lo(sbase + kAbPhi + pb * PARTS * kAbTileBytes, kAbHalf);
           const uint32_t v = umma_desc_lo(sbase + s * 2 * kAbTileBytes + kAbTileBytes, kAbHalf);
 #pragma unroll
-          for (int part = 0; part < PARTS; ++part)    // 16 tokens (two swizzle atoms of 8 rows) per instruction
-            umma_ss4_one<2048 / 16, 2048 / 16>(one, tmem + ab * D, a + part * (kAbTileBytes / 16), v, kAbIdesc, !first || part > 0);
+          for (int x = 0; x < PARTS; ++x) {           // 16 tokens (two swizzle atoms of 8 rows) per instruction
+            const int part = PARTS == 3 ? PARTS - 1 - x : x;   // (small terms first)
+            umma_ss4_one<2048 / 16, 2048 / 16>(one, tmem + ab * D, a + part * (kAbTileBytes / 16), v, kAbIdesc, !first || x > 0);
+          }
           umma_commit_one(one, &phi_empty[pb]);
           umma_commit_one(one, &empty[s]);
           if (last) umma_commit_one(one, &acc_full[ab]);

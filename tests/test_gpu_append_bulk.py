@@ -131,3 +131,23 @@ def test_few_tokens_of_many_sequences_of_different_lengths_take_the_three_kernel
     assert a.sync_status() == 0 and torch.equal(a.bufs.seq_lens, b.bufs.seq_lens)
     assert torch.equal(a.bufs.stats, b.bufs.stats) and torch.equal(a.bufs.tok_lse, b.bufs.tok_lse)
     assert parity.rel_l2(a.bufs.rla_state.cpu().numpy(), b.bufs.rla_state.cpu().numpy()) < 2 * parity.STATE_TOL_FMA
+
+
+@pytest.mark.parametrize("outlier", [1.0, 10.0])
+@pytest.mark.parametrize("n,times", [(40, 1), (100, 1), (255, 1), (200, 10)])
+def test_state_below_256_tokens_is_no_less_exact_than_the_fp32_kernels(n, times, outlier):
+    """Against 64 bits; phi enters the products with all its bits, and no sum is longer than a tile."""
+    errs = []
+    for flags in (0, binding.SPLA_GENERAL_KERNELS):
+        w = synth.Workload("case", 9, batch=2, n_q_heads=4, n_kv_heads=4, head_dim=128, block_size=64, top_k=8, context=n * times)
+        cache = binding.SplaCache(runner.config_for(w, flags=flags), DEV)
+        g = torch.Generator(device=DEV).manual_seed(6)
+        state = torch.zeros(2, 4, 128, 128, dtype=torch.float64, device=DEV)
+        for _ in range(times):
+            k, v = (torch.randn(2, 4, n, 128, generator=g, device=DEV) for _ in range(2))
+            k[..., :4] *= outlier
+            k, v = k.to(torch.bfloat16), v.to(torch.bfloat16)
+            cache.append_tokens(k, v)
+            state += torch.softmax(k.double(), dim=-1).transpose(-1, -2) @ v.double()
+        errs.append(((cache.bufs.rla_state.double() - state).norm() / state.norm()).item())
+    assert errs[0] <= errs[1], errs
