@@ -232,3 +232,29 @@ def test_a_short_chunk_takes_the_path_that_is_faster_for_it(case, tensor):
     np.testing.assert_allclose(a[rows].cpu().numpy(), b[rows].cpu().numpy(), rtol=RTOL, atol=ATOL)
     least, _, _ = _run(w, K0, V0, k, v, q, 0, workspace_bytes=1)
     assert torch.equal(least, a)
+
+
+@pytest.mark.parametrize("d,B,G", [(128, 64, 4), (64, 16, 4), (128, 128, 2), (128, 32, 1)])
+def test_a_value_that_is_not_finite_reaches_only_the_positions_that_attend_to_it(d, B, G):
+    """Without the residual: a NaN in a late token of the chunk, an infinity in one old block.  Positions before the token, and
+    those that did not select the block, are as if the values were finite; the others are not finite in those channels."""
+    T = 300                                                   # (more than the short chunks that take the general kernels)
+    case = (1, 2, G, d, B, 4, 0, 1, B * 12 + 5, T, binding.SPLA_NO_RLA)
+    w, K0, V0, k, v, q = _inputs(case)
+    clean, sel, cache = _run(w, K0, V0, k, v, q, case[-1])
+    assert cache.launches == _launches(w, T, case[-1], True)
+    V1, v1 = V0.clone(), v.clone()
+    blk = next(x for x in range(12) if 0 < (sel[:, :, 0] == x).sum() < T)     # an old block that some positions select
+    late = 41
+    V1[:, 0, B * blk + 1, 7] = float("inf")
+    v1[:, 1, late, d - 1] = float("nan")
+    a, sel_a, _ = _run(w, K0, V1, k, v1, q, case[-1])
+    b, _, _ = _run(w, K0, V1, k, v1, q, case[-1] | binding.SPLA_GENERAL_KERNELS)
+    assert torch.equal(sel_a, sel)
+    hit = torch.zeros_like(a, dtype=torch.bool)
+    hit[:, :, :G, 7] = (sel[:, :, 0] == blk).any(-1)[..., None]
+    seen = (sel[:, :, 1] == (K0.shape[2] + late) // B).any(-1) & (torch.arange(T, device=DEV) >= late)
+    hit[:, :, G:, d - 1] = seen[..., None]
+    assert seen.any()
+    assert torch.equal(~torch.isfinite(a), hit) and torch.equal(~torch.isfinite(b), hit)
+    assert torch.equal(a[~hit], clean[~hit])
