@@ -36,8 +36,8 @@ CASES = [
     (1, 2, 4, 128, 64, 64, 1, 4, 64 * 90, 100, 0),     # longest selection
     (1, 1, 4, 128, 64, 8, 1, 2, 700, 90, binding.SPLA_FIRST_ORDER),
     (1, 1, 4, 128, 64, 8, 0, 0, 700, 90, binding.SPLA_NO_RLA),
-    (1, 1, 4, 128, 16, 8, 1, 4, 16 * 600, 40, 0),      # more than 512 blocks: a CTA selects
-    (1, 1, 4, 64, 16, 8, 1, 4, 16 * 1100, 33, binding.SPLA_DEBUG_BOUNDS),
+    (1, 1, 4, 128, 16, 8, 1, 4, 16 * 600, 40, 0),      # more than 512 blocks: 32 keys per lane of a warp
+    (1, 1, 4, 64, 16, 8, 1, 4, 16 * 1100, 33, binding.SPLA_DEBUG_BOUNDS),   # more than 1024: a CTA selects
 ]
 
 
@@ -258,3 +258,24 @@ def test_a_value_that_is_not_finite_reaches_only_the_positions_that_attend_to_it
     assert seen.any()
     assert torch.equal(~torch.isfinite(a), hit) and torch.equal(~torch.isfinite(b), hit)
     assert torch.equal(a[~hit], clean[~hit])
+
+
+@pytest.mark.parametrize("blocks", [1024, 1025, 4096, 4097, 16384])
+def test_selection_by_a_warp_and_by_a_cta_up_to_the_longest_sequence(blocks):
+    """Either side of each instance of the selection kernel, and of the tiles' bitmap of selected blocks at its last word."""
+    for more in (0, 1):                                       # a chunk that ends with a block, and inside one
+        test_tensor_core_prefill_equals_the_general_kernels((1, 1, 4, 64, 16, 8, 1, 2, 16 * blocks - 20 - 7 * more, 20, 0))
+
+
+def test_above_the_longest_sequence_of_the_tensor_core_path():
+    """16385 blocks: the general kernels, and their scratch."""
+    w, K0, V0, k, v, q = _inputs((1, 1, 4, 64, 16, 8, 1, 2, 16 * 16384 - 19, 20, 0))
+    sizes = []
+    for flags in (0, binding.SPLA_GENERAL_KERNELS):
+        lo = C.c_size_t()
+        assert binding.load().spla_query_prefill_workspace(C.byref(runner.config_for(w, flags=flags)), 20, C.byref(lo), None) == 0
+        sizes.append(lo.value)
+    assert sizes[0] == sizes[1]
+    a, sel_a, ca = _run(w, K0, V0, k, v, q, 0)
+    b, sel_b, cb = _run(w, K0, V0, k, v, q, binding.SPLA_GENERAL_KERNELS)
+    assert ca.launches == cb.launches and torch.equal(a, b) and torch.equal(sel_a, sel_b)
