@@ -3,8 +3,8 @@
     python bench_prefill.py [--workload long_128k] [--batch N] [--reps R] [--general]
 
 One JSON line: milliseconds per append of the whole context (CUDA events on the launching stream, after a
-warm-up call, each repetition into a fresh cache so that every token is new), tokens/s, and the K/V bytes the
-state kernel has to read over the time of the whole append.  `--general` forces the FMA state kernel.
+warm-up call, each repetition into a fresh cache so that every token is new), tokens/s, and the new tokens' K/V bytes (read
+once; the cache takes as many again) over the time of the whole append.  `--general` takes the three general kernels (state on the FMA pipe).
 """
 from __future__ import annotations
 

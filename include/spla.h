@@ -267,10 +267,10 @@ int spla_select_blocks_noalloc(const spla_config_t *config, const float *stats, 
                                const void *q, int32_t *sel_idx, float *scores_out, int32_t *status_out, void *stream);
 
 /*
- * Test hook for the failure path of the kernels' bounded waits (no counterpart in the paper).  Every wait of a decode
- * kernel on one of its asynchronous copies polls a barrier a bounded number of times (2^22 by default) and, when the
- * limit is reached, latches SPLA_ERR_TIMEOUT, skips the arithmetic and returns normally.  This call sets that limit
- * for the decode kernels of `cache` (max_wait_polls > 0; 0 restores the default) and makes their copy barriers expect
+ * Test hook for the failure path of the kernels' bounded waits (no counterpart in the paper).  Every wait of a kernel
+ * on one of its asynchronous copies polls a barrier a bounded number of times (2^22 by default) and, when the limit is
+ * reached, latches SPLA_ERR_TIMEOUT, skips the arithmetic and returns normally.  This call sets that limit for the
+ * decode, prefill and bulk append kernels of `cache` (max_wait_polls > 0; 0 restores the default) and makes their copy barriers expect
  * extra_expected_bytes more than will ever arrive (>= 0, a multiple of 16; 0 in normal use), so that a test can watch a
  * wait run out without any fault, trap or endless loop on the device.  HOST values; affects later calls only.
  */

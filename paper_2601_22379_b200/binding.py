@@ -309,7 +309,7 @@ class SplaCache:
             return self.lib.spla_sync_status(self.handle, _stream())
 
     def debug_wait_hook(self, max_wait_polls: int, extra_expected_bytes: int):
-        """Test hook: wait limit of the decode kernels' copy barriers and bytes they expect in excess (see spla.h)."""
+        """Test hook: wait limit of the kernels' copy barriers (decode, prefill, bulk append) and bytes they expect in excess (see spla.h)."""
         _check(self.lib.spla_debug_wait_hook(self.handle, max_wait_polls, extra_expected_bytes), "spla_debug_wait_hook")
 
     def set_length_bound(self, n: int):

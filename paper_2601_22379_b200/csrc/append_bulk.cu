@@ -24,8 +24,8 @@
 //
 // Bound by HBM: every token is read once and written once.  Before, one kernel copied (K staged once more for the
 // statistics) and a second read everything again for the state.
-// 131072 tokens x 32 units (4.3 GB in and out): copy and state kernels 1.44 ms, this one 0.92 ms = 4.7 TB/s; 50 to 700 tokens x
-// 128 units on a history: 45 -> 32 us.  What keeps it from the copy rate: 16 warps in five roles issue from code that does not
+// 131072 tokens x 32 units (4.3 GB in and out): copy and state kernels 1.44 ms, this one 0.84 ms a call = 5.1 TB/s, 0.79 of the
+// measured copy rate; 50 to 700 tokens x 128 units on a history: 45 -> 32 us.  What keeps it from the copy rate: 16 warps in five roles issue from code that does not
 // fit the SM's instruction cache (fewer rows or tokens per loop body cost more in latency than they gain there).
 //
 // Every wait is an mbarrier poll with an iteration limit; a role whose wait runs out raises the CTA's abort flag and leaves its
@@ -574,7 +574,7 @@ __global__ void __launch_bounds__(kAbMergeThreads) append_merge_state_kernel(con
 
 // Shares of a unit's tokens.  One CTA fits an SM, and per CTA the work is bounded by the roles' latencies, so what counts is
 // that all 148 SMs have the same: either one wave, or, where that leaves many SMs idle (32 units: 4 x 32 = 128 CTAs) and
-// the shares stay long (16 tiles), two (9 x 32 = 288 of 296 places; 131072 tokens x 32 units: 0.95 -> 0.92 ms).  A fixed SM
+// the shares stay long (16 tiles), two (9 x 32 = 288 of 296 places; 131072 tokens x 32 units as first built: 0.95 -> 0.92 ms).  A fixed SM
 // count, because the partial buffer is sized from the configuration alone, before any device is known.
 constexpr int kAbMaxShares = 72;
 static int shares_in_waves(int units, int waves) {

@@ -31,8 +31,8 @@
 // each scheduler, so code size counts (with every loop unrolled 43 % of all stalls were instruction fetches, 9000 cycles per
 // tile; with 16-token loop bodies 3600), and the MMA warp runs converged with one elected lane (a one-lane branch cost 75 to
 // 110 cycles per MMA instead of 50 to 65).  A prompt of 8192 tokens (8 KV heads, G = 4, d = 128, 32 of up to 128 blocks of
-// 64): 60.6 ms as one virtual unit per position on the general kernels, 2.87 ms with this kernel unrolled, 1.65 ms now, of
-// which it takes 1.3 ms.
+// 64): 60.6 ms as one virtual unit per position on the general kernels, 2.87 ms with this kernel unrolled, 1.62 ms now, of
+// which it takes 1.27 ms.
 //
 // Every wait is an mbarrier poll with an iteration limit; on expiry the CTA raises its abort flag, all roles leave their
 // loops, tensor memory is released and the time-out status is latched.  No multicast anywhere.
@@ -661,12 +661,12 @@ __global__ void __launch_bounds__(kPaThreads, 1)
           tmem_st16(src + 16 * c, pk);
         };
 #pragma unroll 1
-      for (int c = 0; c < 4; ++c) {                               // (rolled, like the other roles' loops: see the top)
-        uint32_t cur16[16];
-        tmem_ld16_async(src + 16 * c, cur16);
-        tmem_ld_wait16(cur16);
-        coefs(cur16, c);
-      }
+        for (int c = 0; c < 4; ++c) {                             // (rolled, like the other roles' loops: see the top)
+          uint32_t cur16[16];
+          tmem_ld16_async(src + 16 * c, cur16);
+          tmem_ld_wait16(cur16);
+          coefs(cur16, c);
+        }
         tmem_st_wait();
         tc_fence_before();
         __syncwarp();

@@ -69,7 +69,7 @@ struct Params {
   const float* vstats;                  // [U][vTtot][2][d] statistics of each position's own (last, partial) block as of that position
   const float* vobar;                   // [U][vTtot][G][d] o_bar = phi(q_t) S_bar_t of every position
   int wait_limit;                       // iterations a bounded barrier wait polls before it gives up (0: kWaitLimitDefault)
-  int dbg_tx_extra;                     // test hook: bytes added to what the decode kernels' copy barriers expect (0 in use)
+  int dbg_tx_extra;                     // test hook: bytes added to what the copy barriers of decode, prefill and bulk append expect (0 in use)
 };
 
 __device__ __forceinline__ float to_float(float x) { return x; }
