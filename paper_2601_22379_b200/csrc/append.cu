@@ -9,14 +9,15 @@
 //            shared memory once; from there the new tokens go to the cache (k_new, v_new -> cache), their
 //            logsumexp of phi_scale * k to tok_lse, and the block's mean / variance records are recomputed (two
 //            exact passes, so the result does not depend on how the tokens were split across append calls)
-//   state  : rank-n update of S_bar (rows tiled over CTAs on the FMA pipe)
+//   state  : rank-n update of S_bar on the FMA pipe, shares of the tokens side by side and then added
 //   lengths: seq_lens += n_new
 #include "spla_internal.h"
 
 namespace spla {
 
-constexpr int kStateRows = 16;     // rows of S_bar per CTA
+constexpr int kStateRows = 16;     // rows of S_bar per CTA where there are few units
 constexpr int kStateTokens = 32;   // tokens staged per inner step
+constexpr int kStateShare = 256;   // tokens per share of a unit, at least (below, a share's fixed cost outweighs what it takes off)
 
 __device__ __forceinline__ int tokens_to_add(const Params& p, const int* n_new, int max_new, int b, int L) {
   int n = n_new ? n_new[b] : max_new;
@@ -120,7 +121,6 @@ __global__ void __launch_bounds__(kStatThreads) append_block_kernel(const Params
   __shared__ float mean_s[D];
   constexpr int VEC = D / 32;
   pdl_wait();
-  pdl_launch_dependents();
   constexpr int CH = D * (int)sizeof(T) / 16;        // 16-byte chunks per token
   T* tile = reinterpret_cast<T*>(tile_raw);          // [B][D]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -184,47 +184,133 @@ __global__ void __launch_bounds__(kStatThreads) append_block_kernel(const Params
                               [&](int t) { return to_float(tile[(size_t)t * D + c]); });
     __syncthreads();                                 // the next window reuses the reduction buffers
   }
+  // Only now: the small CTAs of the state kernel, started earlier, crowd onto the SMs that have room first (bf16, d = 64, 255 tokens
+  // x 32 units: 57 us a call against 33).
+  pdl_launch_dependents();
 }
 
-template <typename T, int D>
-__global__ void __launch_bounds__(D) append_state_kernel(const Params p, const T* __restrict__ k_new,
-                                                         const T* __restrict__ v_new, const int* __restrict__ n_new,
-                                                         int max_new) {
-  __shared__ float phi_s[kStateTokens][kStateRows];
+// S_bar += phi(K)^T V on the FMA pipe: ROWS rows of S_bar per CTA over one share of a unit's new tokens, staged kStateTokens at a
+// time (the next ones are on their way to registers meanwhile); a thread owns RT x 8 outputs, so that a staged value feeds eight
+// or RT products.  Every output adds its tokens in order; shares are added in share order by append_merge_state_kernel.
+// Bound by issuing FMAs (two per instruction).  One CTA per 16 rows used to walk all tokens, one load per token in the chain:
+// fp32, d = 64, 16384 tokens x 4 units 1860 -> 52 us a call, 255 tokens 37 -> 19; fp32, d = 128 3399 -> 109.
+template <typename T, int D, int ROWS, int RT>
+__global__ void __launch_bounds__(ROWS / RT * (D / 8)) append_state_kernel(const Params p, const T* __restrict__ k_new,
+                                                                           const T* __restrict__ v_new,
+                                                                           const int* __restrict__ n_new, int max_new) {
+  constexpr int NT = ROWS / RT * (D / 8);
+  constexpr int E = 16 / (int)sizeof(T);                    // elements per 16-byte piece
+  constexpr int CHK = ROWS / E, CHV = D / E;                // pieces per token: of the CTA's channels of K, of V
+  constexpr int NK = (kStateTokens * CHK + NT - 1) / NT, NV = (kStateTokens * CHV + NT - 1) / NT;
+  __shared__ __align__(16) float phi_s[kStateTokens][ROWS];
+  __shared__ __align__(16) float v_s[kStateTokens][D];
   pdl_wait();
   pdl_launch_dependents();
-  const int u = blockIdx.y, b = u / p.Hkv;
+  const int u = blockIdx.y, b = u / p.Hkv, tid = threadIdx.x;
   const int L = p.seq_lens[b];
-  const int n = tokens_to_add(p, n_new, max_new, b, L);
-  if (n <= 0) return;
-  const int row0 = blockIdx.x * kStateRows;
-  const int j = threadIdx.x;
+  const int n = max(0, tokens_to_add(p, n_new, max_new, b, L));
+  const int S = gridDim.z, share = blockIdx.z;
+  const int per = ((n + S - 1) / S + kStateTokens - 1) / kStateTokens * kStateTokens;
+  const int t_lo = min(n, share * per), t_hi = min(n, t_lo + per);
+  const int row0 = blockIdx.x * ROWS;
+  if (S == 1 && n == 0) return;
   const float a2 = p.phi_scale * kLog2e;
   const float* lse = p.tok_lse + (size_t)u * p.max_blocks * p.B + L;
-  const T* kn = k_new + (size_t)u * max_new * D;
+  const T* kn = k_new + (size_t)u * max_new * D + row0;
   const T* vn = v_new + (size_t)u * max_new * D;
-  float acc[kStateRows];
+  uint4 kr[NK], vr[NV];
+  float lr[NK];
+  auto fetch = [&](int t0) {
 #pragma unroll
-  for (int r = 0; r < kStateRows; ++r) acc[r] = 0.f;
-  for (int t0 = 0; t0 < n; t0 += kStateTokens) {
-    const int nt = min(kStateTokens, n - t0);
+    for (int j = 0; j < NK; ++j) {
+      const int x = j * NT + tid, t = x / CHK, c = x % CHK;
+      const bool in = t < kStateTokens && t0 + t < t_hi;
+      kr[j] = in ? __ldg(reinterpret_cast<const uint4*>(kn + (size_t)(t0 + t) * D) + c) : make_uint4(0u, 0u, 0u, 0u);
+      lr[j] = in ? -__ldcg(lse + t0 + t) * kLog2e : -INFINITY;    // (phi of a token that is not there: 0)
+    }
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      const int x = j * NT + tid, t = x / CHV, c = x % CHV;
+      const bool in = t < kStateTokens && t0 + t < t_hi;
+      vr[j] = in ? __ldg(reinterpret_cast<const uint4*>(vn + (size_t)(t0 + t) * D) + c) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  auto floats = [](const uint4& r, float (&x)[E]) {
+    if constexpr (E == 4) {
+      x[0] = __uint_as_float(r.x); x[1] = __uint_as_float(r.y); x[2] = __uint_as_float(r.z); x[3] = __uint_as_float(r.w);
+    } else {
+      x[0] = bf16_lo(r.x); x[1] = bf16_hi(r.x); x[2] = bf16_lo(r.y); x[3] = bf16_hi(r.y);
+      x[4] = bf16_lo(r.z); x[5] = bf16_hi(r.z); x[6] = bf16_lo(r.w); x[7] = bf16_hi(r.w);
+    }
+  };
+  const int rg = tid / (D / 8) * RT, c4 = tid % (D / 8) * 4;  // the thread's rows; its columns c4 .. + 3 and D / 2 + c4 .. + 3
+  float2 acc[RT][4];
+#pragma unroll
+  for (int r = 0; r < RT; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[r][c] = make_float2(0.f, 0.f);
+  if (t_lo < t_hi) fetch(t_lo);
+  for (int t0 = t_lo; t0 < t_hi; t0 += kStateTokens) {
     __syncthreads();
-    for (int idx = j; idx < kStateTokens * kStateRows; idx += D) {
-      const int t = idx / kStateRows, r = idx % kStateRows;
-      float f = 0.f;
-      if (t < nt) f = exp2f(fmaf(to_float(kn[(size_t)(t0 + t) * D + row0 + r]), a2, -lse[t0 + t] * kLog2e));
-      phi_s[t][r] = f;
+#pragma unroll
+    for (int j = 0; j < NK; ++j) {
+      const int x = j * NT + tid, t = x / CHK, c = x % CHK;
+      if (t < kStateTokens) {
+        float k[E];
+        floats(kr[j], k);
+#pragma unroll
+        for (int e = 0; e < E; ++e) k[e] = exp2f(fmaf(k[e], a2, lr[j]));
+#pragma unroll
+        for (int e = 0; e < E; e += 4) *reinterpret_cast<float4*>(&phi_s[t][c * E + e]) = make_float4(k[e], k[e + 1], k[e + 2], k[e + 3]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      const int x = j * NT + tid, t = x / CHV, c = x % CHV;
+      if (t < kStateTokens) {
+        float v[E];
+        floats(vr[j], v);
+#pragma unroll
+        for (int e = 0; e < E; e += 4) *reinterpret_cast<float4*>(&v_s[t][c * E + e]) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+      }
     }
     __syncthreads();
+    if (t0 + kStateTokens < t_hi) fetch(t0 + kStateTokens);
+    const int nt = min(kStateTokens, t_hi - t0);
+#pragma unroll 2
     for (int t = 0; t < nt; ++t) {
-      const float v = to_float(vn[(size_t)(t0 + t) * D + j]);
+      float f[RT];
 #pragma unroll
-      for (int r = 0; r < kStateRows; ++r) acc[r] = fmaf(phi_s[t][r], v, acc[r]);
+      for (int r = 0; r < RT; r += 2) {
+        if constexpr (RT % 4 == 0) {
+          if (r % 4 == 0) {
+            const float4 x = *reinterpret_cast<const float4*>(&phi_s[t][rg + r]);
+            f[r] = x.x; f[r + 1] = x.y; f[r + 2] = x.z; f[r + 3] = x.w;
+          }
+        } else {
+          const float2 x = *reinterpret_cast<const float2*>(&phi_s[t][rg + r]);
+          f[r] = x.x; f[r + 1] = x.y;
+        }
+      }
+      const float4 v0 = *reinterpret_cast<const float4*>(&v_s[t][c4]), v1 = *reinterpret_cast<const float4*>(&v_s[t][D / 2 + c4]);
+      const float2 v[4] = {make_float2(v0.x, v0.y), make_float2(v0.z, v0.w), make_float2(v1.x, v1.y), make_float2(v1.z, v1.w)};
+#pragma unroll
+      for (int r = 0; r < RT; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[r][c] = __ffma2_rn(make_float2(f[r], f[r]), v[c], acc[r][c]);
     }
   }
-  float* S = p.state + (size_t)u * D * D + (size_t)row0 * D + j;
+  float* dst = (S > 1 ? p.state_part + ((size_t)u * S + share) * D * D : p.state + (size_t)u * D * D) + (size_t)(row0 + rg) * D + c4;
 #pragma unroll
-  for (int r = 0; r < kStateRows; ++r) S[(size_t)r * D] += acc[r];
+  for (int r = 0; r < RT; ++r) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float4* d4 = reinterpret_cast<float4*>(dst + (size_t)r * D + h * (D / 2));
+      float4 o = S > 1 ? make_float4(0.f, 0.f, 0.f, 0.f) : *d4;
+      o.x += acc[r][2 * h].x; o.y += acc[r][2 * h].y; o.z += acc[r][2 * h + 1].x; o.w += acc[r][2 * h + 1].y;
+      *d4 = o;
+    }
+  }
 }
 
 __global__ void append_lengths_kernel(const Params p, const int* __restrict__ n_new, int max_new) {
@@ -417,7 +503,14 @@ static cudaError_t launch_typed(const Params& p, const void* k_new, const void* 
     if (e != cudaSuccess) return e;
   }
   if (!(p.flags & 4u)) {
-    const cudaError_t e = launch_ex(append_state_kernel<T, D>, dim3(D / kStateRows, U), dim3(D), 0, stream, 0, true, p, kn, vn, n_new, max_new);
+    const int most = append_max_shares(U), want = (max_new + kStateShare - 1) / kStateShare, S = want < most ? want : most;
+    // All rows per CTA where units and shares fill the device (less is staged more than once), 16 rows where they do not.
+    cudaError_t e;
+    if ((long long)U * S >= 148)
+      e = launch_ex(append_state_kernel<T, D, D, D / 16>, dim3(1, U, S), dim3(2 * D), 0, stream, 0, true, p, kn, vn, n_new, max_new);
+    else
+      e = launch_ex(append_state_kernel<T, D, kStateRows, 2>, dim3(D / kStateRows, U, S), dim3(D), 0, stream, 0, true, p, kn, vn, n_new, max_new);
+    if (e == cudaSuccess && S > 1) e = launch_append_merge_state(p, S, stream);
     if (e != cudaSuccess) return e;
   }
   return launch_ex(append_lengths_kernel, dim3((p.batch + 127) / 128), dim3(128), 0, stream, 0, true, p, n_new, max_new);

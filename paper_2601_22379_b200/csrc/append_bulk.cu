@@ -552,11 +552,11 @@ __global__ void __launch_bounds__(kAbThreads, 1)
 // Shares of every unit onto S_bar, in share order.
 constexpr int kAbMergeThreads = 256;
 __global__ void __launch_bounds__(kAbMergeThreads) append_merge_state_kernel(const Params p, int S) {
-  constexpr int N4 = kAbD * kAbD / 4;
+  const int N4 = p.d * p.d / 4;
   pdl_wait();
   const int idx = blockIdx.x * kAbMergeThreads + threadIdx.x, u = blockIdx.y;
-  const float4* part = reinterpret_cast<const float4*>(p.state_part + (size_t)u * S * kAbD * kAbD) + idx;
-  float4* st = reinterpret_cast<float4*>(p.state + (size_t)u * kAbD * kAbD) + idx;
+  const float4* part = reinterpret_cast<const float4*>(p.state_part) + (size_t)u * S * N4 + idx;
+  float4* st = reinterpret_cast<float4*>(p.state) + (size_t)u * N4 + idx;
   float4 a = make_float4(0.f, 0.f, 0.f, 0.f), o = *st;
   for (int s0 = 0; s0 < S; s0 += 16) {
     float4 x[16];
@@ -588,9 +588,15 @@ static int append_bulk_shares(int units, int tiles) {
   return s < tiles ? s : tiles;
 }
 
+int append_max_shares(int units) { return shares_in_waves(units, 2); }
+
 size_t append_bulk_part_bytes(int units, int d) {
-  const int s = shares_in_waves(units, 2);
+  const int s = append_max_shares(units);
   return s > 1 ? (size_t)units * s * d * d * 4 : 0;
+}
+
+cudaError_t launch_append_merge_state(const Params& p, int S, cudaStream_t stream) {
+  return launch_ex(append_merge_state_kernel, dim3(p.d * p.d / 4 / kAbMergeThreads, p.batch * p.Hkv), dim3(kAbMergeThreads), 0, stream, 0, true, p, S);
 }
 
 // cache: maps of the K / V cache, fresh: of k_new / v_new as [units * max_new][128]; boxes of 64 rows x 64 columns.
@@ -607,8 +613,7 @@ cudaError_t launch_append_bulk(const Params& p, const AttendMaps& cache, const A
   e = launch_ex(kern, dim3(S, U), dim3(kAbThreads), kAbSmem, stream, 0, true, p,
                 *reinterpret_cast<const CUtensorMap*>(fresh.k), *reinterpret_cast<const CUtensorMap*>(fresh.v),
                 *reinterpret_cast<const CUtensorMap*>(cache.k), *reinterpret_cast<const CUtensorMap*>(cache.v), n_new, max_new);
-  if (e == cudaSuccess && S > 1 && !(p.flags & 4u))
-    e = launch_ex(append_merge_state_kernel, dim3(kAbD * kAbD / 4 / kAbMergeThreads, U), dim3(kAbMergeThreads), 0, stream, 0, true, p, S);
+  if (e == cudaSuccess && S > 1 && !(p.flags & 4u)) e = launch_append_merge_state(p, S, stream);
   return e;
 }
 

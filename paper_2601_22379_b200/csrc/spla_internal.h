@@ -88,7 +88,9 @@ struct AttendMaps {                      // TMA tensor maps (CUtensorMap) of the
   bool valid;
 };
 // append_bulk.cu (one-pass bulk append with S_bar on the tensor cores: bf16 cache, d = 128; maps with boxes of 64 tokens)
+int append_max_shares(int units);            // partial sums of S_bar per unit that the workspace holds
 size_t append_bulk_part_bytes(int units, int d);
+cudaError_t launch_append_merge_state(const Params& p, int S, cudaStream_t stream);   // S partial sums per unit onto S_bar, in order
 cudaError_t launch_append_bulk(const Params& p, const AttendMaps& cache, const AttendMaps& fresh, const int* n_new, int max_new,
                                cudaStream_t stream);
 // attend_merge.cu

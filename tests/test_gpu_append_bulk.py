@@ -151,3 +151,31 @@ def test_state_below_256_tokens_is_no_less_exact_than_the_fp32_kernels(n, times,
             state += torch.softmax(k.double(), dim=-1).transpose(-1, -2) @ v.double()
         errs.append(((cache.bufs.rla_state.double() - state).norm() / state.norm()).item())
     assert errs[0] <= errs[1], errs
+
+
+@pytest.mark.parametrize("dtype,d,batch,hkv,sizes,ragged", [
+    ("f32", 64, 1, 1, [33, 255, 257], False),       # one share, the last token of it, two; 16 rows per CTA
+    ("f32", 64, 2, 2, [256 * 74 + 31], False),      # as many shares as the workspace holds, ragged at their end
+    ("bf16", 64, 2, 2, [40, 700], True),            # shares sized by the longest: some of a short sequence are empty
+    ("f32", 128, 3, 20, [300, 770], True),          # all rows per CTA, two and four shares
+    ("bf16", 64, 40, 4, [513], False),              # ... and one share, more units than SMs
+])
+def test_state_of_the_three_kernel_append(dtype, d, batch, hkv, sizes, ragged):
+    """S_bar against 64 bits at the edges of staged tokens and of shares; the tolerance of fp32 sums."""
+    w = synth.Workload("case", 10, batch=batch, n_q_heads=hkv, n_kv_heads=hkv, head_dim=d, block_size=64, top_k=8,
+                       context=sum(sizes), kv_dtype=dtype)
+    cache = binding.SplaCache(runner.config_for(w), DEV)
+    g = torch.Generator(device=DEV).manual_seed(8)
+    state = torch.zeros(batch, hkv, d, d, dtype=torch.float64, device=DEV)
+    for n in sizes:
+        k, v = (torch.randn(batch, hkv, n, d, generator=g, device=DEV).to(w.torch_dtype) for _ in range(2))
+        n_new = torch.randint(0, n + 1, (batch,), generator=torch.Generator().manual_seed(n), dtype=torch.int32).to(DEV) if ragged else None
+        cache.append_tokens(k, v, n_new)
+        phi = torch.softmax(k.double(), dim=-1)
+        if ragged:
+            phi = phi * (torch.arange(n, device=DEV)[None, :] < n_new[:, None])[:, None, :, None]
+        state += phi.transpose(-1, -2) @ v.double()
+    torch.cuda.synchronize()
+    assert cache.sync_status() == 0
+    err = (cache.bufs.rla_state.double() - state).flatten(2).norm(dim=-1) / state.flatten(2).norm(dim=-1).clamp_min(1e-30)
+    assert err.max().item() < parity.STATE_TOL_FMA
