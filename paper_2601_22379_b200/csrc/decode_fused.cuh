@@ -68,6 +68,7 @@ static cudaError_t fused_launch_win(const Params& p, const AttendMaps& maps, con
   size_t smem = (size_t)SM::kEll + (size_t)p.G * p.chunk * sizeof(float);
   const size_t smem_attend = attend_mma_ring_bytes(p.tile_rows, D, 1);     // (the merge's receive area lies in phase 1's layout)
   if (smem_attend > smem) smem = smem_attend;
+  if ((size_t)SM::kMergeRecv + SM::kMergeRecvBytes > smem) smem = (size_t)SM::kMergeRecv + SM::kMergeRecvBytes;
   auto kern = decode_fused_kernel<D, GP, WIN, EARLY, ST>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess && p.cs > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);

@@ -103,9 +103,14 @@ struct Smem {
   // K/V tile ring (at most 66 KB) over this area, and the tile copies must stay clear of the fixed region below, which
   // holds this phase's mbarrier objects (never invalidated: overwriting them with tile data corrupted value rows, found
   // with NaN-filled memory), and of the o_bar scratch, which may still be in use when the first tiles arrive.
-  static constexpr int kMergeRecv = kAreaEnd;                       // the attend phase's receive area (fused kernel)
+  // Behind it, or where the ring is no longer than that area anyway (16-bit records) over the table of log masses, the attend
+  // phase's receive area (fused kernel): a sibling stores there once it has attended, so after this CTA's keys, formed from that
+  // table, have reached it.  (G = 8, 48 units of 1580 blocks:
+  // one CTA per SM in clusters of three became two in clusters of six, 98 -> 49 us a step.)
+  static constexpr bool kRecvOverEll = kStreamBytes <= kAreaEnd;
   static constexpr int kMergeRecvBytes = (16 * (2 * D + 2) * 4 + 1023) / 1024 * 1024;
-  static constexpr int kRingBytes = kStreamBytes > kMergeRecv + kMergeRecvBytes ? kStreamBytes : kMergeRecv + kMergeRecvBytes;
+  static constexpr int kRecvInRing = kRecvOverEll ? kAreaEnd : kAreaEnd + kMergeRecvBytes;
+  static constexpr int kRingBytes = kStreamBytes > kRecvInRing ? kStreamBytes : kRecvInRing;
   static_assert(kStateScratch >= 68 * 1024, "the attend phase's tile ring must end below the o_bar scratch");
   // fixed region after the ring:
   static constexpr int kAllPart = kRingBytes;                       // float [16][GP][2]  every CTA's (max, sum exp) per head
@@ -117,7 +122,8 @@ struct Smem {
   // word), kept here instead of in 32 more registers per thread)
   static constexpr int kBfrag = (kBars + kNumBars * 8 + 15) / 16 * 16;
   static constexpr int kBfragBytes = (sizeof(ST) == 2 && GP > 4) ? 2 * (D * 2 / 64) * 4 * 32 * 4 : 0;
-  static constexpr int kEll = kBfrag + kBfragBytes;                                // float [G][chunk]
+  static constexpr int kEll = (kBfrag + kBfragBytes + 15) / 16 * 16;                // float [G][chunk]
+  static constexpr int kMergeRecv = kRecvOverEll ? kEll : kAreaEnd;
 };
 
 }  // namespace
