@@ -291,7 +291,7 @@ cudaError_t launch_attend_merge(const Params& p, const AttendMaps* maps, const v
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  if (p.kv_bf16 && q_is_bf16 && p.G <= 8 && maps && maps->valid && p.acs > 0)
+  if (p.kv_bf16 && q_is_bf16 && maps && maps->valid && p.acs > 0)
     return launch_attend_mma(p, *maps, q, rms_weight, out, dbg_o_sparse, dbg_o_rla, stream);
   const int GP = padded_group(p.G);
   if (p.kv_bf16) {

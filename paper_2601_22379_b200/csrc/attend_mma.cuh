@@ -1,4 +1,4 @@
-// Sparse attention + fused residual-linear term for bf16 K/V on tensor cores (GQA groups of up to 8 heads).
+// Sparse attention + fused residual-linear term for bf16 K/V on tensor cores.
 //
 // The CTAs that serve one (sequence, KV head) unit form a thread-block cluster; CTA r of the cluster walks the
 // selected blocks r, r + CS, r + 2 CS, ... through a shared-memory ring that TMA fills (tiled tensor copies with
@@ -74,12 +74,15 @@ __device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
 __device__ __forceinline__ float f16_lo(uint32_t x) { return __low2float(*reinterpret_cast<const __half2*>(&x)); }
 __device__ __forceinline__ float f16_hi(uint32_t x) { return __high2float(*reinterpret_cast<const __half2*>(&x)); }
 
+constexpr float kPhiScaleWide = 16384.f;   // groups of more than eight heads: phi times 2^14 (at most 2^14 then) keeps both fp16 parts clear of the subnormals
 constexpr int kPad = 8;   // floats of padding per row of the cross-warp reduction buffer
 
 // Bytes of the tile ring (reused for the cross-warp fold); as a kernel of its own the receive area of the merge follows.
-__host__ __device__ constexpr size_t attend_mma_ring_bytes(int B, int D, int groups) {
+// `wide`: groups of more than eight heads, whose two branches take 32 rows.
+__host__ __device__ constexpr size_t attend_mma_ring_bytes(int B, int D, int groups, bool wide = false) {
   const size_t ring = (size_t)(2 * groups) * ((2 * (size_t)B * D * 2 + (size_t)B * 4 + 1023) / 1024 * 1024);
-  const size_t fold = (size_t)(groups * (kAttendThreads / 32) * (16 * (D + kPad) + 16)) * sizeof(float);
+  const int rows = wide ? 32 : 16;
+  const size_t fold = (size_t)(groups * (kAttendThreads / 32) * (rows * (D + kPad) + rows)) * sizeof(float);
   return (ring > fold ? ring : fold);
 }
 constexpr size_t attend_mma_recv_bytes(int D) { return (size_t)16 * (2 * D + 2) * 4; }
@@ -88,7 +91,10 @@ constexpr size_t attend_mma_recv_bytes(int D) { return (size_t)16 * (2 * D + 2) 
 
 // PACK: the group has at most 4 heads, so accumulator rows 4..7 and 12..15 are padding; rows 12..15 then carry
 // the bf16 remainder of the linear coefficients and no extra products are needed for it.
-template <int D, bool PACK, int NG, bool FUSED>
+// WIDE: the group has more than 8 heads: S and A take all 16 rows of a product of their own, and the probabilities keep 24 bits
+// like the linear coefficients (three bf16 parts; every slice's sums start at zero and are added in fp32), as on the general
+// kernel, which served such groups before.
+template <int D, bool PACK, int NG, bool FUSED, bool WIDE = false>
 __device__ __forceinline__ void attend_mma_body(const Params& p, const CUtensorMap& map_k, const CUtensorMap& map_v,
                                                 const __nv_bfloat16* __restrict__ q, const float* __restrict__ rms_weight,
                                                 float* __restrict__ out, float* __restrict__ dbg_sparse,
@@ -99,6 +105,8 @@ __device__ __forceinline__ void attend_mma_body(const Params& p, const CUtensorM
   constexpr int NT = D / 8;         // n-tiles of the PV-type product
   constexpr int NTHR = NG * kAttendThreads;
   constexpr int NWARP = NTHR / 32;
+  constexpr int RW = WIDE ? 16 : 8;             // accumulator rows of one branch
+  static_assert(!WIDE || (!PACK && NG == 1 && !FUSED), "groups of more than eight heads have one shape");
   __shared__ __align__(8) uint64_t full_own[kMaxSlots + 1];
   uint64_t* full = full_ext ? full_ext : full_own;      // (the fused kernel initialises its barriers at its start)
   uint64_t* mbar_merge = full + kMaxSlots;              // completes when every sibling's partial results have arrived here
@@ -133,9 +141,48 @@ __device__ __forceinline__ void attend_mma_body(const Params& p, const CUtensorM
   // fl_s (groups of more than 4 heads only): the fp16 remainder of phi(q), a second left operand, kept in shared
   // memory (the same for every warp) to stay clear of the register limit; in the packed layout rows 12..15 of fa
   // carry that remainder for heads 0..3 instead.
-  __shared__ uint32_t fl_s[PACK ? 1 : KS][2][32];
-  uint32_t qa[KS][2], fa[KS][2];
+  // WIDE: rows g and g + 8 are heads g and g + 8; phi(q), head and remainder, in shared memory.
+  __shared__ __align__(16) uint32_t fl_s[PACK ? 1 : KS][WIDE ? 32 : 2][WIDE ? 8 : 32];
+  uint32_t qa[KS][WIDE ? 4 : 2], fa[KS][WIDE ? 1 : 2];
   auto make_fragments = [&]() {
+    if constexpr (WIDE) {
+      const float a2 = p.phi_scale * kLog2e;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int head = g + 8 * j;
+        const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + ((size_t)b * p.Hq + (size_t)h * G + (head < G ? head : 0)) * D);
+        float mx = -INFINITY, sum = 0.f;
+#pragma unroll
+        for (int kk = 0; kk < KS; ++kk)
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            const uint32_t w = head < G ? __ldg(qrow + 8 * kk + 4 * x + t) : 0u;
+            qa[kk][2 * x + j] = w;
+            mx = fmaxf(mx, fmaxf(bf16_lo(w), bf16_hi(w)));
+          }
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+#pragma unroll
+        for (int kk = 0; kk < KS; ++kk)
+#pragma unroll
+          for (int x = 0; x < 2; ++x) sum += exp2f((bf16_lo(qa[kk][2 * x + j]) - mx) * a2) + exp2f((bf16_hi(qa[kk][2 * x + j]) - mx) * a2);
+        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+        sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+        const float inv = (head < G && rla_on) ? kPhiScaleWide / sum : 0.f;
+        if (warp == 0) {                                    // (visible after a barrier below)
+#pragma unroll
+          for (int kk = 0; kk < KS; ++kk)
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+              const float f0 = exp2f((bf16_lo(qa[kk][2 * x + j]) - mx) * a2) * inv, f1 = exp2f((bf16_hi(qa[kk][2 * x + j]) - mx) * a2) * inv;
+              const uint32_t hd = pack_f16(f0, f1);
+              fl_s[kk][lane][2 * x + j] = hd;
+              fl_s[kk][lane][4 + 2 * x + j] = pack_f16(f0 - f16_lo(hd), f1 - f16_hi(hd));
+            }
+        }
+      }
+      return;
+    } else {
     const bool hv = g < G;
     const bool rem_row = PACK && g >= 4;                  // this lane's row 8 + g holds the remainder of head g - 4
     const int hq = rem_row ? g - 4 : g;                   // head whose phi(q) this lane forms
@@ -178,6 +225,7 @@ __device__ __forceinline__ void attend_mma_body(const Params& p, const CUtensorM
         fa[kk][0] = h0; fa[kk][1] = h1;
         if (warp == 0) { fl_s[kk][0][lane] = l0; fl_s[kk][1][lane] = l1; }   // (visible after a barrier below)
       }
+    }
     }
   };
   // As a kernel of its own the fragments are formed first (under programmatic dependent launch this overlaps the
@@ -250,6 +298,10 @@ __device__ __forceinline__ void attend_mma_body(const Params& p, const CUtensorM
   float o[NT][4];
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt) { o[nt][0] = o[nt][1] = o[nt][2] = o[nt][3] = 0.f; }
+  float m_run2 = -INFINITY, l_run2 = 0.f;    // WIDE: row g + 8; the linear branch has accumulators of its own
+  float ol[WIDE ? NT : 1][4];
+#pragma unroll
+  for (int nt = 0; nt < (WIDE ? NT : 1); ++nt) { ol[nt][0] = ol[nt][1] = ol[nt][2] = ol[nt][3] = 0.f; }
   const float sc2 = p.sm_scale * kLog2e;
   const float a2 = p.phi_scale * kLog2e;
   const int spb = TB / 16;                   // slices per tile
@@ -288,6 +340,108 @@ __device__ __forceinline__ void attend_mma_body(const Params& p, const CUtensorM
       const int tok0 = sl * 16;
       if (tok0 >= ntok || dead) break;
       const float lse2_0 = lse_s[tok0 + g] * kLog2e, lse2_1 = lse_s[tok0 + 8 + g] * kLog2e;
+      if constexpr (WIDE) {
+        float sacc[2][4], aacc[2][4];
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) sacc[nt][c] = aacc[nt][c] = 0.f;
+        const uint32_t krow = ks + (tok0 + (mi >> 1) * 8 + r8) * 128;
+#pragma unroll
+        for (int kk = 0; kk < KS; ++kk) {
+          uint32_t kb[4], pb[4], pl[4];
+          const int ch = 2 * kk + (mi & 1);
+          ldmatrix_x4(kb, krow + (ch >> 3) * half_bytes + (((ch & 7) ^ r8) << 4));
+          // (the tensor core cuts off when it adds: every k-step starts at zero and is added in fp32)
+          float ts[2][4], ta[2][4];
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) ts[nt][c] = ta[nt][c] = 0.f;
+          mma_bf16(ts[0], qa[kk][0], qa[kk][1], qa[kk][2], qa[kk][3], kb[0], kb[1]);
+          mma_bf16(ts[1], qa[kk][0], qa[kk][1], qa[kk][2], qa[kk][3], kb[2], kb[3]);
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            const float ls = x < 2 ? lse2_0 : lse2_1;
+            const float e0 = ex2(fmaf(bf16_lo(kb[x]), a2, -ls)) * kPhiScaleWide, e1 = ex2(fmaf(bf16_hi(kb[x]), a2, -ls)) * kPhiScaleWide;
+            pb[x] = pack_f16(e0, e1);
+            pl[x] = pack_f16(e0 - f16_lo(pb[x]), e1 - f16_hi(pb[x]));
+          }
+          const uint4 fh = *reinterpret_cast<const uint4*>(&fl_s[kk][lane][0]), fr = *reinterpret_cast<const uint4*>(&fl_s[kk][lane][4]);
+          mma_f16(ta[0], fr.x, fr.y, fr.z, fr.w, pb[0], pb[1]);
+          mma_f16(ta[1], fr.x, fr.y, fr.z, fr.w, pb[2], pb[3]);
+          mma_f16(ta[0], fh.x, fh.y, fh.z, fh.w, pl[0], pl[1]);
+          mma_f16(ta[1], fh.x, fh.y, fh.z, fh.w, pl[2], pl[3]);
+          mma_f16(ta[0], fh.x, fh.y, fh.z, fh.w, pb[0], pb[1]);
+          mma_f16(ta[1], fh.x, fh.y, fh.z, fh.w, pb[2], pb[3]);
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) { sacc[nt][c] += ts[nt][c]; aacc[nt][c] += ta[nt][c]; }
+        }
+        float corr[2], mxr[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          float mx = -INFINITY;
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+              const bool valid = tok0 + nt * 8 + 2 * t + c < ntok;
+              sacc[nt][2 * j + c] = valid ? sacc[nt][2 * j + c] : -INFINITY;
+              aacc[nt][2 * j + c] = valid ? aacc[nt][2 * j + c] * (1.f / (kPhiScaleWide * kPhiScaleWide)) : 0.f;
+              mx = fmaxf(mx, sacc[nt][2 * j + c]);
+            }
+          mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+          mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+          float& mr = j ? m_run2 : m_run;
+          float& lr = j ? l_run2 : l_run;
+          mxr[j] = fmaxf(mr, mx * sc2);                    // finite: the slice has at least one valid token (sc2 > 0)
+          corr[j] = ex2(mr - mxr[j]);
+          mr = mxr[j];
+          float psum = 0.f;
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) { sacc[nt][2 * j + c] = ex2(fmaf(sacc[nt][2 * j + c], sc2, -mxr[j])); psum += sacc[nt][2 * j + c]; }
+          lr = fmaf(lr, corr[j], psum);
+        }
+        // P and the coefficients as three bf16 parts each: words (row g, first 8 tokens), (row g + 8, ..), then the last 8 tokens
+        uint32_t pp[3][4], cc[3][4];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          float a = sacc[x >> 1][2 * (x & 1)], bb = sacc[x >> 1][2 * (x & 1) + 1], c = aacc[x >> 1][2 * (x & 1)], d = aacc[x >> 1][2 * (x & 1) + 1];
+#pragma unroll
+          for (int pt = 0; pt < 3; ++pt) {
+            pp[pt][x] = pack_bf16(a, bb);
+            a -= bf16_lo(pp[pt][x]); bb -= bf16_hi(pp[pt][x]);
+            cc[pt][x] = pack_bf16(c, d);
+            c -= bf16_lo(cc[pt][x]); d -= bf16_hi(cc[pt][x]);
+          }
+        }
+        const uint32_t vrow = vs + (tok0 + (mi & 1) * 8 + r8) * 128;
+#pragma unroll
+        for (int np = 0; np < NT / 2; ++np) {
+          uint32_t vb[4];
+          const int ch = 2 * np + (mi >> 1);
+          ldmatrix_x4_trans(vb, vrow + (ch >> 3) * half_bytes + (((ch & 7) ^ r8) << 4));
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            float ts[4] = {0.f, 0.f, 0.f, 0.f}, tl[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int pt = 2; pt >= 0; --pt) {              // (small terms first)
+              mma_bf16(ts, pp[pt][0], pp[pt][1], pp[pt][2], pp[pt][3], vb[2 * e], vb[2 * e + 1]);
+              mma_bf16(tl, cc[pt][0], cc[pt][1], cc[pt][2], cc[pt][3], vb[2 * e], vb[2 * e + 1]);
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              o[2 * np + e][c] = fmaf(o[2 * np + e][c], corr[c >> 1], ts[c]);
+              ol[2 * np + e][c] += tl[c];
+            }
+          }
+        }
+        continue;
+      } else {
       // two accumulator tiles per n-tile (one per product) so that the dependent chain of each is half as long;
       // rows 0..7 of the first and rows 8..15 of the second are the meaningful halves
       float sacc[2][4], aacc[2][4];
@@ -391,6 +545,7 @@ __device__ __forceinline__ void attend_mma_body(const Params& p, const CUtensorM
           }
         }
       }
+      }
     }
     group_sync();                                      // every warp of the group is done with this slot
     if (gtid == 0 && i + ns < nb && !dead) {
@@ -406,28 +561,37 @@ __device__ __forceinline__ void attend_mma_body(const Params& p, const CUtensorM
   // ---- fold the four warps together ------------------------------------------------------------------------
   l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
   l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
+  if constexpr (WIDE) {
+    l_run2 += __shfl_xor_sync(0xffffffffu, l_run2, 1);
+    l_run2 += __shfl_xor_sync(0xffffffffu, l_run2, 2);
+  }
   cta_sync();                                   // the ring is dead: its space becomes the reduction buffer
-  float* red_o = reinterpret_cast<float*>(smem_raw);                    // [NWARP][16][D + kPad]
-  float* red_m = red_o + NWARP * 16 * (D + kPad);                       // [NWARP][8]
-  float* red_l = red_m + NWARP * 8;                                     // [NWARP][8]
+  float* red_o = reinterpret_cast<float*>(smem_raw);                    // [NWARP][2 RW][D + kPad]
+  float* red_m = red_o + NWARP * 2 * RW * (D + kPad);                   // [NWARP][RW]
+  float* red_l = red_m + NWARP * RW;                                    // [NWARP][RW]
   // Where the partial results of head hd go: into the CTA that merges it, hd % CS, entry (hd / CS) * CS + sender of
   // its receive area (at most 16 entries: [2][D] floats each, then the (max, sum) pairs), as asynchronous stores that
   // count their bytes on that CTA's merge barrier.
   constexpr int kRecvEntries = 16;
   float* recv = recv_raw ? reinterpret_cast<float*>(recv_raw)
-                         : reinterpret_cast<float*>(smem_raw + attend_mma_ring_bytes(TB, D, NG));  // [16][2][D], [16][2]
+                         : reinterpret_cast<float*>(smem_raw + attend_mma_ring_bytes(TB, D, NG, WIDE));  // [16][2][D], [16][2]
   float* recv_ml = recv + kRecvEntries * 2 * D;
   const int my_heads = G > rank ? (G - rank + CS - 1) / CS : 0;         // heads this CTA merges
   if (tid == 0 && my_heads > 0) mbar_expect_tx(mbar_merge, (uint32_t)(my_heads * CS * (2 * D * 4 + 8)));
   // every warp leaves its rows as they are, with its running maximum and sum; the combiner rescales (one barrier less
   // than agreeing on the maximum first)
-  if (t == 0) { red_m[warp * 8 + g] = m_run; red_l[warp * 8 + g] = l_run; }
+  if (t == 0) { red_m[warp * RW + g] = m_run; red_l[warp * RW + g] = l_run; }
+  if (WIDE && t == 0) { red_m[warp * RW + 8 + g] = m_run2; red_l[warp * RW + 8 + g] = l_run2; }
   {
-    float* ro = red_o + (size_t)warp * 16 * (D + kPad);
+    float* ro = red_o + (size_t)warp * 2 * RW * (D + kPad);
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) {
       *reinterpret_cast<float2*>(ro + (size_t)g * (D + kPad) + nt * 8 + 2 * t) = make_float2(o[nt][0], o[nt][1]);
       *reinterpret_cast<float2*>(ro + (size_t)(g + 8) * (D + kPad) + nt * 8 + 2 * t) = make_float2(o[nt][2], o[nt][3]);
+      if constexpr (WIDE) {
+        *reinterpret_cast<float2*>(ro + (size_t)(g + 16) * (D + kPad) + nt * 8 + 2 * t) = make_float2(ol[nt][0], ol[nt][1]);
+        *reinterpret_cast<float2*>(ro + (size_t)(g + 24) * (D + kPad) + nt * 8 + 2 * t) = make_float2(ol[nt][2], ol[nt][3]);
+      }
     }
   }
   cta_sync();
@@ -435,19 +599,19 @@ __device__ __forceinline__ void attend_mma_body(const Params& p, const CUtensorM
   const uint32_t recv0 = smem_u32(recv), recv_ml0 = smem_u32(recv_ml), bar0 = smem_u32(mbar_merge);
   for (int idx = tid; idx < 2 * G * (D / 4); idx += NTHR) {             // four columns per thread and step
     const int br = idx / (G * (D / 4)), hd = (idx / (D / 4)) % G, c4 = (idx % (D / 4)) * 4;   // branch, head, first column
-    const int rr = br * 8 + hd;
+    const int rr = br * RW + hd;
     float fw[NWARP];                                                    // 0 for a warp that saw no token
     {
       float M = red_m[hd];
 #pragma unroll
-      for (int w = 1; w < NWARP; ++w) M = fmaxf(M, red_m[w * 8 + hd]);
+      for (int w = 1; w < NWARP; ++w) M = fmaxf(M, red_m[w * RW + hd]);
 #pragma unroll
-      for (int w = 0; w < NWARP; ++w) fw[w] = (br == 0 && M > -INFINITY) ? ex2(red_m[w * 8 + hd] - M) : (br == 0 ? 0.f : 1.f);
+      for (int w = 0; w < NWARP; ++w) fw[w] = (br == 0 && M > -INFINITY) ? ex2(red_m[w * RW + hd] - M) : (br == 0 ? 0.f : 1.f);
     }
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int w = 0; w < NWARP; ++w) {
-      const float4 a = *reinterpret_cast<const float4*>(red_o + ((size_t)w * 16 + rr) * (D + kPad) + c4);
+      const float4 a = *reinterpret_cast<const float4*>(red_o + ((size_t)w * 2 * RW + rr) * (D + kPad) + c4);
       s.x += a.x * fw[w]; s.y += a.y * fw[w]; s.z += a.z * fw[w]; s.w += a.w * fw[w];
       if (PACK && br == 1) {                                              // the second and third parts of the coefficients
         const float4 b2 = *reinterpret_cast<const float4*>(red_o + ((size_t)w * 16 + rr + 4) * (D + kPad) + c4);
@@ -463,9 +627,9 @@ __device__ __forceinline__ void attend_mma_body(const Params& p, const CUtensorM
   if (tid < G) {
     float Mg = red_m[tid], Lg = 0.f;
 #pragma unroll
-    for (int w = 1; w < NWARP; ++w) Mg = fmaxf(Mg, red_m[w * 8 + tid]);
+    for (int w = 1; w < NWARP; ++w) Mg = fmaxf(Mg, red_m[w * RW + tid]);
 #pragma unroll
-    for (int w = 0; w < NWARP; ++w) Lg += Mg > -INFINITY ? red_l[w * 8 + tid] * ex2(red_m[w * 8 + tid] - Mg) : 0.f;
+    for (int w = 0; w < NWARP; ++w) Lg += Mg > -INFINITY ? red_l[w * RW + tid] * ex2(red_m[w * RW + tid] - Mg) : 0.f;
     const uint32_t dest = (uint32_t)(tid % CS);
     const int entry = (tid / CS) * CS + rank;
     st_async_v2(map_to_rank(recv_ml0 + (uint32_t)(entry * 8), dest), __float_as_uint(Mg), __float_as_uint(Lg),

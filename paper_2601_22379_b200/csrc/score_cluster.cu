@@ -4,10 +4,10 @@
 namespace spla {
 
 // Blocks per CTA when `cs` CTAs share a sequence of at most max_seq_blocks blocks, or 0 if the cluster kernel cannot
-// serve that (groups above 8, more than 1024 blocks per CTA, shared memory).  The share is the exact quotient rounded
+// serve that (more than 1024 blocks per CTA, shared memory).  The share is the exact quotient rounded
 // up to a multiple of 8, so that the CTAs of a cluster stream equal amounts.
 int score_cluster_chunk(long long max_seq_blocks, int cs, int NW, int G, int d) {
-  if (G > 8 || cs < 1 || cs > kMaxCluster) return 0;
+  if (G > kMaxGroup || cs < 1 || cs > kMaxCluster) return 0;
   if (max_seq_blocks < 1) max_seq_blocks = 1;
   const long long chunk = ((max_seq_blocks + cs - 1) / cs + 7) / 8 * 8;
   if (chunk > 1024) return 0;

@@ -81,7 +81,7 @@ struct Smem {
   static constexpr int kStageBytes = kStageRec * kRecBytes;
   // tensor-core streaming (16-bit records; fp32 records for groups of more than four heads, where the FMA pipe cannot
   // keep up): the ring is cut into slots of 16 records, one MMA row tile each
-  static constexpr bool kMma = sizeof(ST) == 2 || GP > 4;
+  static constexpr bool kMma = GP <= 8 && (sizeof(ST) == 2 || GP > 4);   // (groups of more than eight heads: fp32 FMAs, as ever)
   static constexpr int kSlotBytes = kSlotRec * kRecBytes;
   static constexpr int kSlots = sizeof(ST) == 2 ? NWP : 6;         // one ring position per streaming warp (6 x 16 KB with fp32 records)
   static constexpr int kStreamBytes = kMma ? kSlots * kSlotBytes : kStages * kStageBytes;
@@ -107,7 +107,7 @@ struct Smem {
   // phase's receive area (fused kernel): a sibling stores there once it has attended, so after this CTA's keys, formed from that
   // table, have reached it.  (G = 8, 48 units of 1580 blocks:
   // one CTA per SM in clusters of three became two in clusters of six, 98 -> 49 us a step.)
-  static constexpr bool kRecvOverEll = kStreamBytes <= kAreaEnd;
+  static constexpr bool kRecvOverEll = kStreamBytes <= kAreaEnd || GP > 8;   // (groups of more than eight heads never run fused)
   static constexpr int kMergeRecvBytes = (16 * (2 * D + 2) * 4 + 1023) / 1024 * 1024;
   static constexpr int kRecvInRing = kRecvOverEll ? kAreaEnd : kAreaEnd + kMergeRecvBytes;
   static constexpr int kRingBytes = kStreamBytes > kRecvInRing ? kStreamBytes : kRecvInRing;
@@ -121,7 +121,7 @@ struct Smem {
   // (tensor-core path with two column tiles: the B fragments of the variance dots, one word per lane and (tile, chunk,
   // word), kept here instead of in 32 more registers per thread)
   static constexpr int kBfrag = (kBars + kNumBars * 8 + 15) / 16 * 16;
-  static constexpr int kBfragBytes = (sizeof(ST) == 2 && GP > 4) ? 2 * (D * 2 / 64) * 4 * 32 * 4 : 0;
+  static constexpr int kBfragBytes = (kMma && sizeof(ST) == 2 && GP > 4) ? 2 * (D * 2 / 64) * 4 * 32 * 4 : 0;
   static constexpr int kEll = (kBfrag + kBfragBytes + 15) / 16 * 16;                // float [G][chunk]
   static constexpr int kMergeRecv = kRecvOverEll ? kEll : kAreaEnd;
 };
@@ -172,15 +172,19 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
                                                    int* __restrict__ sel_user, int pending_new, unsigned char* smem_raw,
                                                    int* sel_share = nullptr, float* obar_local = nullptr) {
   using SM = Smem<D, GP, ST, NWP>;
+  // Groups of more than eight heads are dealt out to two teams of warps, eight heads each (that many queries fit a warp's
+  // registers); a team takes every record of a stage.
+  constexpr int GT = GP > 8 ? 8 : GP;           // heads of a team, padded
+  constexpr int TEAMS = GP / GT;
   constexpr int kCsConsumers = NWP;             // warps; all consume, lane 0 of warp 0 also feeds the ring
   constexpr int kCsThreads = NWP * 32;
   constexpr int kStageRec = SM::kStageRec;
-  constexpr int UNR = kRecPerWarp;              // records per warp per stage
+  constexpr int UNR = kRecPerWarp * TEAMS;      // records per warp per stage
   constexpr int W = GP <= 4 ? 16 : 32;          // lanes that share one record
   constexpr int NGRP = 32 / W;                  // records a warp works on side by side
-  constexpr int PASSES = UNR / NGRP;
+  constexpr int PASSES = kRecPerWarp / NGRP;    // ... held in registers together
   constexpr int VECW = D / W;                   // floats of the mean (and of the variance) per lane
-  constexpr int NV = 2 * GP;
+  constexpr int NV = 2 * GT;
   constexpr int LPV = W / NV;                   // lanes holding a copy of each reduced value
   constexpr int FB = LPV < PASSES ? LPV : PASSES;
   static_assert(LPV >= 1, "group too large for the lane layout");
@@ -189,6 +193,8 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
   const int CS = gridDim.x;
   const int rank = blockIdx.x;
   const int G = p.G;
+  const int team_warp = warp % (NWP / TEAMS);   // warp of its team
+  const int g0 = TEAMS > 1 ? warp / (NWP / TEAMS) * GT : 0;   // the team's first head
   const int u = blockIdx.y;
   const int b = u / p.Hkv, h = u % p.Hkv;
 
@@ -248,7 +254,7 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
   constexpr bool BVS = MMA && NT2 == 2 && !MMAF;
   uint32_t bq[MMA ? NT2 : 1][MMA ? NJ : 1][BW], bv[(MMA && !BVS) ? NT2 : 1][(MMA && !BVS) ? NJ : 1][BW];
   uint32_t* bv_s = reinterpret_cast<uint32_t*>(smem_raw + SM::kBfrag);   // [NT2][NJ][BW][32 lanes]
-  float qm[GP][VECW], qv[GP][VECW];
+  float qm[GT][VECW], qv[GT][VECW];
   if constexpr (MMA) {
 #pragma unroll
     for (int nt = 0; nt < NT2; ++nt) {
@@ -289,9 +295,9 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
     }
   }
 #pragma unroll
-  for (int g = 0; g < GP && !MMA; ++g) {
-    if (g < G) {
-      const size_t qrow = ((size_t)b * p.Hq + (size_t)h * G + g) * D;
+  for (int g = 0; g < GT && !MMA; ++g) {
+    if (g0 + g < G) {
+      const size_t qrow = ((size_t)b * p.Hq + (size_t)h * G + g0 + g) * D;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         float x[CW];
@@ -366,7 +372,7 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
     else { for (int r = 0; r < min(kStages, n_rounds); ++r) issue(r); }
   }
 #pragma unroll
-  for (int g = 0; g < GP && !MMA; ++g) {
+  for (int g = 0; g < GT && !MMA; ++g) {
 #pragma unroll
     for (int v = 0; v < VECW; ++v) {
       qm[g][v] *= p.sm_scale;
@@ -381,7 +387,7 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
     // After the group reduction the first W/2 lanes of a group hold the mean dots and the others the variance
     // dots, value index (hl % (W/2)) / LPV, each on LPV lanes.  Copy lane `sub` keeps the result of pass `sub`,
     // so the log / exp work of FB passes runs side by side.
-    const int my_g = (hl % (W / 2)) / LPV;
+    const int my_g = g0 + (hl % (W / 2)) / LPV;
     const int sub = hl % LPV;
     const bool fin_lane = hl < W / 2 && sub < FB && my_g < G;
     const float ln_full = logf((float)p.B);
@@ -502,10 +508,10 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
           for (int pp = 0; pp < FB; ++pp) {
             float vals[NV];
 #pragma unroll
-            for (int g = 0; g < GP; ++g) {
+            for (int g = 0; g < GT; ++g) {
               // packed fp32 FMAs (two products per instruction): even and odd channels accumulate side by side
               float2 am = make_float2(0.f, 0.f), av = make_float2(0.f, 0.f);
-              if (GP <= 4 || g < G) {              // (groups of 5 to 7 heads: the padded heads' products are skipped)
+              if (GP <= 4 || g0 + g < G) {         // (the padded heads' products are skipped)
 #pragma unroll
                 for (int v = 0; v < VECW; v += 2) {
                   am = __ffma2_rn(make_float2(qm[g][v], qm[g][v + 1]), make_float2(mean[p0 + pp][v], mean[p0 + pp][v + 1]), am);
@@ -513,7 +519,7 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
                 }
               }
               vals[g] = am.x + am.y;
-              vals[GP + g] = av.x + av.y;
+              vals[GT + g] = av.x + av.y;
             }
             group_reduce_multi<NV, W>(vals, lane);
             const float other = __shfl_xor_sync(0xffffffffu, vals[0], W / 2);   // variance dot of the same head
@@ -545,13 +551,16 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
     for (int r = 0; r < (MMA ? 0 : n_rounds); ++r) {
       const int s = r % kStages;
       if (!mbar_wait(&full[s], (r / kStages) & 1, p.wait_limit)) { if (lane == 0) atomicExch(&err_s, 1); break; }
-      const int l0 = r * kStageRec + warp * UNR;                       // first record of this warp, CTA-local
-      const ST* st = reinterpret_cast<const ST*>(smem_raw + (size_t)s * SM::kStageBytes) + (size_t)(warp * UNR) * 2 * D;
+      const int l0 = r * kStageRec + team_warp * UNR;                  // first record of this warp, CTA-local
+      const ST* st = reinterpret_cast<const ST*>(smem_raw + (size_t)s * SM::kStageBytes) + (size_t)(team_warp * UNR) * 2 * D;
+#pragma unroll 1
+      for (int part = 0; part < TEAMS; ++part, st += (size_t)kRecPerWarp * 2 * D) {
+      const int l1 = l0 + part * kRecPerWarp;
       float mean[PASSES][VECW], var[PASSES][VECW];
 #pragma unroll
       for (int ps = 0; ps < PASSES; ++ps) {
         const int rec = ps * NGRP + grp;
-        if (l0 + rec < n_stream) {
+        if (l1 + rec < n_stream) {
 #pragma unroll
           for (int c = 0; c < NC; ++c) {
             float a[CW], bb[CW];
@@ -565,14 +574,17 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
           for (int v = 0; v < VECW; ++v) { mean[ps][v] = 0.f; var[ps][v] = 0.f; }
         }
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&empty[s]);                            // the stage is in registers: hand it back
-      if (tid == 0 && r + kStages < n_rounds) {                         // refill it once every warp has done the same
-        if (mbar_wait(&empty[s], (r / kStages) & 1, p.wait_limit)) issue(r + kStages);
-        else atomicExch(&err_s, 1);
+      if (part == TEAMS - 1) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[s]);                          // the stage is in registers: hand it back
+        if (tid == 0 && r + kStages < n_rounds) {                       // refill it once every warp has done the same
+          if (mbar_wait(&empty[s], (r / kStages) & 1, p.wait_limit)) issue(r + kStages);
+          else atomicExch(&err_s, 1);
+        }
+        __syncwarp();
       }
-      __syncwarp();
-      if (l0 < n_stream) finish_passes(l0, n_stream, mean, var);
+      if (l1 < n_stream) finish_passes(l1, n_stream, mean, var);
+      }
     }
     if constexpr (EARLY) {
       // now the append must be complete: final length, and the blocks it wrote to (the last ones of the sequence, a
@@ -597,9 +609,9 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
         if constexpr (MMA)
           for (int base = warp * kSlotRec; base < n_late; base += kCsConsumers * kSlotRec)
             consume_slot(smem_raw + (size_t)base * SM::kRecBytes, n_stream + base, n_my);
-        for (int base = 0; base < (MMA ? 0 : n_late); base += kStageRec) {
-          const int l0 = n_stream + base + warp * UNR;
-          const ST* st = reinterpret_cast<const ST*>(smem_raw) + (size_t)(base + warp * UNR) * 2 * D;
+        for (int base = 0; base < (MMA ? 0 : n_late); base += kStageRec / TEAMS) {
+          const int l0 = n_stream + base + team_warp * kRecPerWarp;
+          const ST* st = reinterpret_cast<const ST*>(smem_raw) + (size_t)(base + team_warp * kRecPerWarp) * 2 * D;
           float mean[PASSES][VECW], var[PASSES][VECW];
 #pragma unroll
           for (int ps = 0; ps < PASSES; ++ps) {
@@ -679,6 +691,10 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
       wred[(warp * GP + my_g) * 2 + 0] = run_max;
       wred[(warp * GP + my_g) * 2 + 1] = run_sum;
     }
+    if (TEAMS > 1 && !WIN && lane < GT) {          // the other team's heads
+      wred[(warp * GP + (g0 ^ GT) + lane) * 2 + 0] = -INFINITY;
+      wred[(warp * GP + (g0 ^ GT) + lane) * 2 + 1] = 0.f;
+    }
   }
   // (fused decode kernel: TMA tiles will overwrite the ring area; what all eight warps did there is ordered before
   // those copies here, the barrier passes the order on)
@@ -694,12 +710,20 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
     // lane w * GP + g takes the pair of warp w and head g; the warps of a head are folded with shuffles (32 / GP >= 8
     // warps fit a pass for groups of up to four heads, else two passes); lanes 0 .. G - 1 then send head `lane`
     float m = -INFINITY, s = 0.f;
+    if constexpr (GP > 8) {                       // (see the fold over the CTAs below)
+      for (int e = lane; e < kCsConsumers * GP; e += 32) m = fmaxf(m, wred[e * 2]);
+      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+      for (int e = lane; e < kCsConsumers * GP; e += 32)
+        if (wred[e * 2] > -INFINITY) s = fmaf(wred[e * 2 + 1], __expf(wred[e * 2] - m), s);
+      s += __shfl_xor_sync(0xffffffffu, s, 16);
+    } else {
 #pragma unroll 1
     for (int e = lane; e < kCsConsumers * GP; e += 32) lse_merge(m, s, wred[e * 2], wred[e * 2 + 1]);
 #pragma unroll
     for (int o = GP; o < 32; o <<= 1) {
       const float m2 = __shfl_xor_sync(0xffffffffu, m, o), s2 = __shfl_xor_sync(0xffffffffu, s, o);
       lse_merge(m, s, m2, s2);
+    }
     }
     if (lane < G) {
       const uint32_t mine = smem_u32(all_part + ((size_t)rank * GP + lane) * 2), bar = smem_u32(pbar);
@@ -753,6 +777,16 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
   float lse_r[GP];
   {
     float m = -INFINITY, sm = 0.f;
+    if constexpr (GP > 8) {
+      // one factor per partial sum (a pair at a time each merge rounds twice more: aggregated scores 1.0 to 1.2 times as far from 64
+      // bits as on the general kernel, which served such groups before)
+      const int end = lane % GP < G ? CS * GP : 0;  // (the padded heads' lanes have nothing to read)
+      for (int pr = lane; pr < end; pr += 32) m = fmaxf(m, all_part[pr * 2]);
+      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+      for (int pr = lane; pr < end; pr += 32)
+        if (all_part[pr * 2] > -INFINITY) sm = fmaf(all_part[pr * 2 + 1], __expf(all_part[pr * 2] - m), sm);
+      sm += __shfl_xor_sync(0xffffffffu, sm, 16);
+    } else {
 #pragma unroll 1
     for (int pr = lane; pr < CS * GP; pr += 32) {
       const int g = pr % GP;
@@ -762,6 +796,7 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
     for (int o = GP; o < 32; o <<= 1) {
       const float m2 = __shfl_xor_sync(0xffffffffu, m, o), s2 = __shfl_xor_sync(0xffffffffu, sm, o);
       lse_merge(m, sm, m2, s2);
+    }
     }
     const float lse = m + __logf(sm);
 #pragma unroll
@@ -986,7 +1021,8 @@ static cudaError_t launch_d(const Params& p, int GP, const void* q, int qb, int*
     case 1: return launch_one<D, 1, NWP>(p, q, qb, sel_user, pending_new, s, occ);
     case 2: return launch_one<D, 2, NWP>(p, q, qb, sel_user, pending_new, s, occ);
     case 4: return launch_one<D, 4, NWP>(p, q, qb, sel_user, pending_new, s, occ);
-    default: return launch_one<D, 8, NWP>(p, q, qb, sel_user, pending_new, s, occ);
+    case 8: return launch_one<D, 8, NWP>(p, q, qb, sel_user, pending_new, s, occ);
+    default: return launch_one<D, 16, NWP>(p, q, qb, sel_user, pending_new, s, occ);
   }
 }
 

@@ -348,7 +348,7 @@ static void plan_score_grid(spla_cache* c, Params* p, bool fused = false) {
 // phase is built for) whenever the cluster score plan exists.
 static bool fused_eligible(const spla_cache* c) {
   return !(c->cfg.flags & SPLA_GENERAL_KERNELS) && c->p.kv_bf16 && c->cfg.q_dtype == SPLA_BF16 &&
-         c->p.G <= 8 && c->maps.valid && attend_mma_smem_bytes(c->p.tile_rows, c->p.d, 1) + 4096 <= (size_t)113 * 1024;
+         c->p.G <= 8 && c->maps.valid && attend_mma_smem_bytes(c->p.tile_rows, c->p.d, 1, c->p.G) + 4096 <= (size_t)113 * 1024;
 }
 
 
@@ -363,7 +363,7 @@ static void plan_attend(spla_cache* c, Params* p) {
   p->acs = 0;
   if (c->cfg.flags & SPLA_GENERAL_KERNELS) return;
   const long long U = (long long)c->p.batch * c->p.Hkv;
-  const size_t smem = attend_mma_smem_bytes(c->p.tile_rows, c->p.d, 1) + 2048;
+  const size_t smem = attend_mma_smem_bytes(c->p.tile_rows, c->p.d, 1, c->p.G) + 2048;
   long long per_sm = (227 * 1024) / (long long)smem;
   if (per_sm > 2) per_sm = 2;                     // the kernel is compiled for two CTAs per SM (no register spills)
   if (per_sm < 1) return;                         // the tiles do not fit: use the general kernel

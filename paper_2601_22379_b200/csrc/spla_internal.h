@@ -76,7 +76,7 @@ int device_sm_count();   // multiprocessors of the current device (148 if the qu
 // score_select.cu
 int score_chunk_for(long long units, long long max_seq_blocks, int sm_count);
 cudaError_t launch_score_select(const Params& p, const void* q, int q_is_bf16, int* sel_user, cudaStream_t stream);
-// score_cluster.cu (G <= 8, at most 16 x 1024 blocks per sequence)
+// score_cluster.cu (at most 16 x 1024 blocks per sequence)
 int score_cluster_chunk(long long max_seq_blocks, int cs, int NW, int G, int d);   // blocks per CTA, 0: not servable
 // Clusters of the score kernel (p.cs CTAs each, p.chunk blocks per CTA) the device holds at once; -1 if unknown.
 int score_cluster_max_clusters(const Params& p);
@@ -97,8 +97,8 @@ cudaError_t launch_append_bulk(const Params& p, const AttendMaps& cache, const A
 cudaError_t launch_attend_merge(const Params& p, const AttendMaps* maps, const void* q, int q_is_bf16,
                                 const float* rms_weight, const int* sel_in, float* out, float* dbg_o_sparse,
                                 float* dbg_o_rla, cudaStream_t stream);
-// attend_mma.cu (bf16 K/V and q, G <= 8)
-size_t attend_mma_smem_bytes(int B, int D, int groups);
+// attend_mma.cu (bf16 K/V and q)
+size_t attend_mma_smem_bytes(int B, int D, int groups, int G);
 int attend_mma_max_clusters(const Params& p);   // clusters of p.acs CTAs resident at once; -1 if unknown
 cudaError_t launch_attend_mma(const Params& p, const AttendMaps& maps, const void* q, const float* rms_weight, float* out,
                               float* dbg_o_sparse, float* dbg_o_rla, cudaStream_t stream);

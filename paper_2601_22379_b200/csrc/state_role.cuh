@@ -61,12 +61,25 @@ __device__ __forceinline__ void state_role(const Params& p, int u, int s, const 
 #pragma unroll
         for (int r = 0; r < RB; ++r) sv[r] = __ldcs(S + (size_t)(r0 + r) * RG * D);
       }
+      // (groups of more than eight heads: a sum per batch of rows, no longer than those of twice the threads on the general kernel)
+      float part[GP > 8 ? GP : 1];
+      if constexpr (GP > 8) {
+#pragma unroll
+        for (int g = 0; g < GP; ++g) part[g] = 0.f;
+      }
 #pragma unroll
       for (int r = 0; r < RB; ++r) {
         const int row = s * (D / kStateSplits) + rg + (r0 + r) * RG;
 #pragma unroll
         for (int g = 0; g < GP; ++g)
-          if (g < G) acc[g] = fmaf(phiq[g * D + row], sv[r], acc[g]);
+          if (g < G) {
+            if constexpr (GP > 8) part[g] = fmaf(phiq[g * D + row], sv[r], part[g]);
+            else acc[g] = fmaf(phiq[g * D + row], sv[r], acc[g]);
+          }
+      }
+      if constexpr (GP > 8) {
+#pragma unroll
+        for (int g = 0; g < GP; ++g) acc[g] += part[g];
       }
     }
 #pragma unroll

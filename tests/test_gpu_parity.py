@@ -562,3 +562,42 @@ def test_equal_scores_select_the_lowest_block_indices(ctx, top_k, flags):
                              stats_bf16=bool(flags & binding.SPLA_STATS_BF16))
     assert res["sel"].tolist() == want
     parity.check_outputs("out", out[0, :w.group], res["out"], w.kv_dtype)
+
+
+@pytest.mark.parametrize("G,d,B,k,ctx,flags,window", [
+    (9, 128, 64, 8, 64 * 3 + 1, 0, None),             # nine heads; fewer blocks than picks
+    (16, 128, 64, 17, 64 * 20 + 5, 0, None),          # a CTA of the attention with two picks, others with one
+    (16, 64, 32, 8, 32 * 700 + 31, 0, None),          # several CTAs of the scores
+    (12, 128, 128, 16, 128 * 40, 0, None),            # blocks of two tiles
+    (16, 128, 16, 64, 16 * 300 + 9, binding.SPLA_STATS_BF16, None),
+    (16, 128, 64, 8, 64 * 90 + 40, 0, (32, 16)),
+    (16, 128, 64, 8, 64 * 90 + 40, binding.SPLA_NO_RLA, None),
+    (16, 128, 64, 8, 64 * 90 + 40, binding.SPLA_DEBUG_BOUNDS, None),
+])
+def test_groups_of_more_than_eight_heads_equal_the_general_kernels(G, d, B, k, ctx, flags, window):
+    """Scores and attention of 9 to 16 heads on the cluster and tensor-core kernels against the general ones (fp32 throughout), a step
+    at a time; every operand there has 22 bits or more, so the two agree to fp32 sums times the residual's amplification."""
+    w = synth.Workload("case", 12, batch=2, n_q_heads=2 * G, n_kv_heads=2, head_dim=d, block_size=B, top_k=k, context=ctx,
+                       n_outlier_channels=4, outlier_scale=3.0, n_steps=3)
+    K, V, _ = runner.generate_prefill(w, "cuda:0")
+    gamma = synth.gamma(w).to("cuda:0")
+    caches = [binding.SplaCache(runner.config_for(w, flags=f, window=window), "cuda:0") for f in (flags, flags | binding.SPLA_GENERAL_KERNELS)]
+    for c in caches:
+        for t in (c.bufs.k_cache, c.bufs.v_cache):
+            t.fill_(float("nan"))
+        c.append_tokens(K, V)
+    caches[1].bufs.rla_state.copy_(caches[0].bufs.rla_state)
+    for step in range(3):
+        q = synth.step_queries(w, step, "cuda:0")
+        res = []
+        for c in caches:
+            k1, v1 = synth.step_kv(w, step, "cuda:0")
+            sel = c.new_sel_buffer()
+            res.append((c.append_decode(k1, v1, q, gamma, sel_idx=sel), sel, c.scores()))
+        torch.cuda.synchronize()
+        nblk = (ctx + step + B) // B
+        torch.testing.assert_close(res[0][2][:, :, :nblk], res[1][2][:, :, :nblk], rtol=5e-6, atol=1e-9)   # (logarithms of 10 rounded to 1e-6)
+        rows = (res[0][1] == res[1][1]).all(-1).repeat_interleave(G, dim=1)
+        assert rows.float().mean() >= 0.75
+        torch.testing.assert_close(res[0][0][rows], res[1][0][rows], rtol=1e-4, atol=3e-5)
+    assert [c.sync_status() for c in caches] == [0, 0]
