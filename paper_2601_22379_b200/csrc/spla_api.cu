@@ -370,6 +370,20 @@ static void plan_attend(spla_cache* c, Params* p) {
   const long long slots = per_sm * c->sm_count;
   int cs = 1;
   while (cs * 2 <= 16 && cs * 2 <= c->p.top_k && U * cs * 2 <= slots) cs *= 2;
+  // More units than places: several waves, of which the last may be nearly empty.  Waves times (a CTA's start and end, about 8 tiles'
+  // time, and its tiles): 320 units of 64 picks of 128 tokens, 128 tiles, in clusters of one (two waves, 24 CTAs in the second) 429 us
+  // a step, of four (five waves) 359; 320 units of 64 picks of 64: 290, 239.  512 units of 16 tiles stay at one (184 us; clusters of
+  // two and four 9 and 32 us longer).
+  if (U > slots) {
+    const long long tiles = (long long)c->p.top_k * (c->p.B / c->p.tile_rows);
+    long long best = 0;
+    for (int x = 1; x <= 16 && x <= c->p.top_k; x *= 2) {
+      const long long cost = (U * x + slots - 1) / slots * (8 + (tiles + x - 1) / x);
+      if (x == 1 || cost < best) { best = cost; cs = x; }
+    }
+    p->acs = cs;
+    return;
+  }
   // all clusters of the launch must be resident together (see plan_score_clusters): ask the device
   for (; cs > 1; cs /= 2) {
     int lg = 0;
