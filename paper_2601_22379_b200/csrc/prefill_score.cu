@@ -301,60 +301,59 @@ __global__ void __launch_bounds__(256, 2) prefill_select_kernel(const Params p, 
     return c;
   };
 
-  // aggregated score of the lane's blocks: per head softmax over the position's blocks, summed over the group.  With few keys per lane
-  // only as many as the position has blocks, and the next head's log masses are on their way meanwhile (511 tokens x 4 units, G = 8:
-  // 82.2 -> 79.9 us a call; 77 tokens x 4 units 48.8 -> 47.8; with 16 keys and more the same gave nothing).
-  constexpr int KB = NK <= 8 ? 1 : NK;
-  constexpr bool AHEAD = NK <= 8;
+  // aggregated score of the lane's blocks: per head softmax over the position's blocks, summed over the group.  Up to 64 blocks, where
+  // latency counts, the next head's log masses are on their way meanwhile, and only as many keys as the position has blocks (511
+  // tokens x 4 units, G = 8: 82.3 -> 79.9 us a call; 77 tokens x 4 units 48.3 -> 47.5; with more keys it is instructions that count: the
+  // 8192-token prompt, four keys, 1680 -> 1690).
+  constexpr bool AHEAD = NK <= 2;
   float sc[NK];
 #pragma unroll
   for (int k = 0; k < NK; ++k) sc[k] = 0.f;
   const float* ell = pc.ell + (((size_t)blockIdx.y * pc.nq * pc.P + slot) * G) * pc.stride;
+  const float* own_row = pc.ell_own + ((size_t)r.u * pc.T + t) * G;
   float nxt[AHEAD ? NK : 1];
-  auto fetch = [&](int g, float (&e)[NK]) {
-    const float* row = ell + (size_t)g * pc.stride;
-    const float* e_own = pc.ell_own + ((size_t)r.u * pc.T + t) * G + g;
+  auto ahead = [&](int g) {
 #pragma unroll
-    for (int k0 = 0; k0 < NK; k0 += KB) {
-      if (k0 > 0 && k0 * L >= nblk) break;                     // (uniform)
-#pragma unroll
-      for (int k = k0; k < k0 + KB; ++k) {
-        const int i = k * L + l;
-        e[k] = i < nblk ? *(i < own ? row + i : e_own) : -INFINITY;
-      }
+    for (int k = 0; k < (AHEAD ? NK : 0); ++k) {
+      if (k > 0 && k * L >= nblk) break;                       // (uniform)
+      const int i = k * L + l;
+      nxt[k] = i < nblk ? *(i < own ? ell + (size_t)g * pc.stride + i : own_row + g) : -INFINITY;
     }
   };
-  if constexpr (AHEAD) fetch(0, nxt);
-#pragma unroll 1
+  if constexpr (AHEAD) ahead(0);
   for (int g = 0; g < G; ++g) {
     float e[NK], mx = -INFINITY;
     if constexpr (AHEAD) {
 #pragma unroll
       for (int k = 0; k < NK; ++k) e[k] = nxt[k];
-      if (g + 1 < G) fetch(g + 1, nxt);
+      if (g + 1 < G) ahead(g + 1);
+#pragma unroll
+      for (int k = 0; k < NK; ++k) {
+        if (k > 0 && k * L >= nblk) break;
+        mx = fmaxf(mx, e[k]);
+      }
     } else {
-      fetch(g, e);
-    }
+      const float e_own = own_row[g];
 #pragma unroll
-    for (int k0 = 0; k0 < NK; k0 += KB) {
-      if (k0 > 0 && k0 * L >= nblk) break;
-#pragma unroll
-      for (int k = k0; k < k0 + KB; ++k) mx = fmaxf(mx, e[k]);
+      for (int k = 0; k < NK; ++k) {
+        const int i = k * L + l;
+        e[k] = i < own ? ell[(size_t)g * pc.stride + i] : (i == own ? e_own : -INFINITY);
+        mx = fmaxf(mx, e[k]);
+      }
     }
     mx = reduce(mx, true);
     float sum = 0.f;
 #pragma unroll
-    for (int k0 = 0; k0 < NK; k0 += KB) {
-      if (k0 > 0 && k0 * L >= nblk) break;
-#pragma unroll
-      for (int k = k0; k < k0 + KB; ++k) { e[k] = __expf(e[k] - mx); sum += e[k]; }
+    for (int k = 0; k < NK; ++k) {
+      if (AHEAD && k > 0 && k * L >= nblk) break;
+      e[k] = __expf(e[k] - mx);
+      sum += e[k];
     }
     const float inv = 1.f / reduce(sum, false);
 #pragma unroll
-    for (int k0 = 0; k0 < NK; k0 += KB) {
-      if (k0 > 0 && k0 * L >= nblk) break;
-#pragma unroll
-      for (int k = k0; k < k0 + KB; ++k) sc[k] = fmaf(e[k], inv, sc[k]);
+    for (int k = 0; k < NK; ++k) {
+      if (AHEAD && k > 0 && k * L >= nblk) break;
+      sc[k] = fmaf(e[k], inv, sc[k]);
     }
   }
   // keys: 0 for blocks that do not exist, all ones for the forced ones, else the score's bits + 1 (positive floats order
