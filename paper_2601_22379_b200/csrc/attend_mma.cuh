@@ -559,8 +559,8 @@ __device__ __forceinline__ void attend_mma_body(const Params& p, const CUtensorM
   }
   if (tid == 0 && err_s) atomicExch(p.status, kStatusTimeout);
 
-  // (a kernel input the merge needs at its very end: requested now, it arrives under the fold)
-  const float gamma0 = (rank < G && tid < D) ? __ldg(rms_weight + ((size_t)h * G + rank) * D + tid) : 0.f;
+  // (a kernel input the merge needs at its very end: requested now, it arrives under the fold; null is allowed without the residual)
+  const float gamma0 = (rla_on && rank < G && tid < D) ? __ldg(rms_weight + ((size_t)h * G + rank) * D + tid) : 0.f;
 
   // ---- fold the four warps together ------------------------------------------------------------------------
   l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
@@ -693,8 +693,10 @@ __device__ __forceinline__ void attend_mma_body(const Params& p, const CUtensorM
       if (col < D) {
         const size_t oidx = ((size_t)b * p.Hq + (size_t)h * G + hd) * D + col;
         float res = o_sp;
-        const float gamma = hd == rank ? gamma0 : rms_weight[((size_t)h * G + hd) * D + col];
-        if (rla) res += gamma * r_ * rsqrtf(tot / D + p.rms_eps);
+        if (rla) {
+          const float gamma = hd == rank ? gamma0 : rms_weight[((size_t)h * G + hd) * D + col];
+          res += gamma * r_ * rsqrtf(tot / D + p.rms_eps);
+        }
         out[oidx] = res;
         if (dbg_sparse) dbg_sparse[oidx] = o_sp;
         if (dbg_rla) dbg_rla[oidx] = r_;

@@ -181,3 +181,28 @@ def test_many_ragged_units_deal_their_blocks_out_evenly(batch, lo, hi):
         assert parity.rel_l2(oa[rows].cpu().numpy(), ob[rows].cpu().numpy()) < 5e-3
         assert torch.equal(a.bufs.stats, b.bufs.stats)
         assert parity.rel_l2(a.bufs.rla_state.cpu().numpy(), b.bufs.rla_state.cpu().numpy()) < 2 * parity.STATE_TOL_TENSOR   # (the contexts went in on different kernels)
+
+
+@pytest.mark.parametrize("G", [4, 8, 12, 16])
+@pytest.mark.parametrize("batch", [2, 160])         # the fused kernel up to eight heads; scores and attention as two launches
+def test_without_the_residual_no_norm_weight_is_needed(G, batch):
+    """SPLA_NO_RLA with a null rms_weight: the same outputs, bit for bit, as with a weight, from every entry point."""
+    w = synth.Workload("case", 21, batch=batch, n_q_heads=2 * G, n_kv_heads=2, head_dim=128, block_size=32, top_k=8, context=32 * 11 + 5,
+                       n_steps=2 + 7)
+    K, V, _ = runner.generate_prefill(w, DEV)
+    q = [synth.step_queries(w, i, DEV) for i in range(2)]
+    kv = [synth.step_kv(w, i, DEV) for i in range(2)]
+    qp = torch.stack([synth.step_queries(w, i, DEV) for i in range(7)], dim=1).contiguous()
+    kp, vp = (K[:, :, :7].contiguous(), V[:, :, :7].contiguous())
+    res = []
+    for gamma in (synth.gamma(w).to(DEV), None):
+        c = binding.SplaCache(runner.config_for(w, flags=binding.SPLA_NO_RLA), DEV)
+        c.append_tokens(K, V)
+        sel = c.new_sel_buffer()
+        outs = [c.append_decode(*kv[0], q[0], gamma, sel_idx=sel), c.decode(q[1], gamma), c.decode_selected(q[1], gamma, sel)]
+        outs.append(c.prefill(kp, vp, qp, gamma))
+        torch.cuda.synchronize()
+        assert c.sync_status() == 0
+        res.append([o.clone() for o in outs])
+    assert all(torch.equal(a, b) for a, b in zip(*res))
+    assert all(torch.isfinite(a).all() for a in res[0])
