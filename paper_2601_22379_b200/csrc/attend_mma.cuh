@@ -71,6 +71,12 @@ __device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
   __half2 v = __floats2half2_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
 }
+// Two bf16 values, each the nearest finite one (any, for a NaN).
+__device__ __forceinline__ uint32_t finite_bf16(uint32_t x) {
+  const __nv_bfloat162 top = __halves2bfloat162(__ushort_as_bfloat16(0x7f7f), __ushort_as_bfloat16(0x7f7f));
+  const __nv_bfloat162 v = __hmin2(__hmax2(*reinterpret_cast<const __nv_bfloat162*>(&x), __hneg2(top)), top);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
 __device__ __forceinline__ float f16_lo(uint32_t x) { return __low2float(*reinterpret_cast<const __half2*>(&x)); }
 __device__ __forceinline__ float f16_hi(uint32_t x) { return __high2float(*reinterpret_cast<const __half2*>(&x)); }
 
@@ -397,9 +403,11 @@ __device__ __forceinline__ void attend_mma_body(const Params& p, const CUtensorM
           mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
           float& mr = j ? m_run2 : m_run;
           float& lr = j ? l_run2 : l_run;
-          mxr[j] = fmaxf(mr, mx * sc2);                    // finite: the slice has at least one valid token (sc2 > 0)
+          const float mr0 = fmaxf(mr, mx * sc2);
+          // (-inf: every score so far is; such tokens weigh nothing, whatever comes after them)
+          mxr[j] = mr0 > -INFINITY ? mr0 : 0.f;
           corr[j] = ex2(mr - mxr[j]);
-          mr = mxr[j];
+          mr = mr0;
           float psum = 0.f;
 #pragma unroll
           for (int nt = 0; nt < 2; ++nt)
@@ -431,7 +439,9 @@ __device__ __forceinline__ void attend_mma_body(const Params& p, const CUtensorM
             float ts[4] = {0.f, 0.f, 0.f, 0.f}, tl[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
             for (int pt = 2; pt >= 0; --pt) {              // (small terms first)
-              mma_bf16(ts, pp[pt][0], pp[pt][1], pp[pt][2], pp[pt][3], vb[2 * e], vb[2 * e + 1]);
+              // the second and third part of a probability may be zero or negative: a value that is not finite meets the first only
+              mma_bf16(ts, pp[pt][0], pp[pt][1], pp[pt][2], pp[pt][3], pt ? finite_bf16(vb[2 * e]) : vb[2 * e],
+                       pt ? finite_bf16(vb[2 * e + 1]) : vb[2 * e + 1]);
               mma_bf16(tl, cc[pt][0], cc[pt][1], cc[pt][2], cc[pt][3], vb[2 * e], vb[2 * e + 1]);
             }
 #pragma unroll

@@ -601,3 +601,34 @@ def test_groups_of_more_than_eight_heads_equal_the_general_kernels(G, d, B, k, c
         assert rows.float().mean() >= 0.75
         torch.testing.assert_close(res[0][0][rows], res[1][0][rows], rtol=1e-4, atol=3e-5)
     assert [c.sync_status() for c in caches] == [0, 0]
+
+
+@pytest.mark.parametrize("flags,k", [(binding.SPLA_NO_RLA, 8), (0, 16)])     # without the residual; with everything selected
+@pytest.mark.parametrize("G,d,B", [(9, 128, 64), (16, 128, 128), (16, 64, 32), (12, 128, 16)])
+def test_values_and_scores_that_are_not_finite_in_groups_of_more_than_eight_heads(G, d, B, flags, k):
+    """An infinite value gives the outputs that attend to it that infinity, in its column only; tokens of score -inf weigh nothing, a
+    run of them at the start of a block included.  As on the general kernels, over the same selection."""
+    nblk = 12
+    w = synth.Workload("case", 31, batch=2, n_q_heads=2 * G, n_kv_heads=2, head_dim=d, block_size=B, top_k=k, context=nblk * B - 3, n_steps=1)
+    K, V, _ = runner.generate_prefill(w, DEV)
+    V[0, 0, 3 * B + 5, 7], V[0, 0, 4 * B, 9], V[0, 1, 2 * B + 15, d - 1] = float("inf"), -float("inf"), float("nan")
+    V[0, 1, 5 * B + 1, 0] = V[0, 1, 5 * B + 2, 0] = float("inf")
+    K[1, :, 3 * B:3 * B + 15, 3] = -float("inf")                 # up to a slice of 16 tokens less one, more than one, the whole tail
+    K[1, :, 6 * B:6 * B + min(B - 1, 37), 3] = -float("inf")
+    K[1, :, 11 * B + 1:, 3] = -float("inf")
+    q = synth.step_queries(w, 0, DEV)
+    q[..., 3] = q[..., 3].abs() + 0.5
+    q[1, 1, 3] = -1.0                                            # this head's scores there are +inf: no output of it is a number
+    gamma = synth.gamma(w).to(DEV)
+    sel = torch.tensor([0, 2, 3, 4, 5, 6, 10, 11] if k == 8 else list(range(nblk)) + [-1] * (k - nblk), dtype=torch.int32, device=DEV)
+    sel = sel.expand(2, 2, k).contiguous()
+    res = []
+    for f in (0, binding.SPLA_GENERAL_KERNELS):
+        c = binding.SplaCache(runner.config_for(w, flags=flags | f), DEV)
+        c.append_tokens(K, V)
+        res.append(c.decode_selected(q, gamma, sel).clone())
+        torch.cuda.synchronize()
+        assert c.sync_status() == 0
+    assert res[1][0, :G, 7].eq(float("inf")).all() and res[1][0, :G, 9].eq(-float("inf")).all() and res[1][0, :G, 8].isfinite().all()
+    assert res[1][1, 0].isfinite().all() and res[1][1, 1].isnan().all()
+    torch.testing.assert_close(res[0], res[1], rtol=1e-5, atol=1e-6, equal_nan=True)      # (fp32 sums in another order)
