@@ -715,7 +715,7 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
       for (int e = lane; e < kCsConsumers * GP; e += 32) m = fmaxf(m, wred[e * 2]);
       m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
       for (int e = lane; e < kCsConsumers * GP; e += 32)
-        if (wred[e * 2] > -INFINITY) s = fmaf(wred[e * 2 + 1], __expf(wred[e * 2] - m), s);
+        if (wred[e * 2 + 1] != 0.f) s = fmaf(wred[e * 2 + 1], __expf(wred[e * 2] - m), s);   // (a NaN is kept: see below)
       s += __shfl_xor_sync(0xffffffffu, s, 16);
     } else {
 #pragma unroll 1
@@ -780,12 +780,13 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
     float m = -INFINITY, sm = 0.f;
     if constexpr (GP > 8) {
       // one factor per partial sum (a pair at a time each merge rounds twice more: aggregated scores 1.0 to 1.2 times as far from 64
-      // bits as on the general kernel, which served such groups before)
+      // bits as on the general kernel, which served such groups before).  A sum of zero has no blocks; one that is NaN, of blocks
+      // whose masses all are, may have the maximum -inf and counts: every score of the head is NaN then.
       const int end = lane % GP < G ? CS * GP : 0;  // (the padded heads' lanes have nothing to read)
       for (int pr = lane; pr < end; pr += 32) m = fmaxf(m, all_part[pr * 2]);
       m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
       for (int pr = lane; pr < end; pr += 32)
-        if (all_part[pr * 2] > -INFINITY) sm = fmaf(all_part[pr * 2 + 1], __expf(all_part[pr * 2] - m), sm);
+        if (all_part[pr * 2 + 1] != 0.f) sm = fmaf(all_part[pr * 2 + 1], __expf(all_part[pr * 2] - m), sm);
       sm += __shfl_xor_sync(0xffffffffu, sm, 16);
     } else {
 #pragma unroll 1

@@ -632,3 +632,29 @@ def test_values_and_scores_that_are_not_finite_in_groups_of_more_than_eight_head
     assert res[1][0, :G, 7].eq(float("inf")).all() and res[1][0, :G, 9].eq(-float("inf")).all() and res[1][0, :G, 8].isfinite().all()
     assert res[1][1, 0].isfinite().all() and res[1][1, 1].isnan().all()
     torch.testing.assert_close(res[0], res[1], rtol=1e-5, atol=1e-6, equal_nan=True)      # (fp32 sums in another order)
+
+
+@pytest.mark.parametrize("G,B,ctx,bad", [
+    (16, 64, 64 * 3 + 20, range(1, 2)),
+    (9, 64, 64 * 20, range(8, 16)),                     # all records of a warp, and of a CTA
+    (12, 32, 32 * 700 + 3, range(40, 100)),             # ... of a CTA of several warps
+])
+def test_scores_that_are_not_numbers_in_groups_of_more_than_eight_heads(G, B, ctx, bad):
+    """Blocks whose log masses are NaN leave no score of the sequence a number and the other sequences as they are: like the general
+    kernels, whichever warp or CTA the blocks fall to."""
+    w = synth.Workload("case", 33, batch=2, n_q_heads=2 * G, n_kv_heads=2, head_dim=128, block_size=B, top_k=8, context=ctx, n_steps=1)
+    K, V, _ = runner.generate_prefill(w, DEV)
+    for i in bad:
+        K[1, 0, i * B + 3] = float("inf")
+    q = synth.step_queries(w, 0, DEV)
+    res = []
+    for f in (0, binding.SPLA_GENERAL_KERNELS):
+        c = binding.SplaCache(runner.config_for(w, flags=f), DEV)
+        c.append_tokens(K, V)
+        sel = c.select(q).clone()
+        res.append((c.scores()[..., :(ctx + B - 1) // B], sel))
+        torch.cuda.synchronize()
+        assert c.sync_status() == 0
+    assert res[1][0][1, 0].isnan().all() and res[1][0][1, 1].isfinite().all() and res[1][0][0].isfinite().all()
+    torch.testing.assert_close(res[0][0], res[1][0], rtol=5e-6, atol=1e-9, equal_nan=True)
+    assert torch.equal(res[0][1][0], res[1][1][0]) and torch.equal(res[0][1][1, 1], res[1][1][1, 1])
