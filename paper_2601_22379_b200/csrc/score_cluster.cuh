@@ -543,7 +543,9 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
                 const int cnt = min(p.win_C, n_last - w * p.win_s);
                 ln_n = cnt > 0 ? logf((float)cnt) : -INFINITY;
               }
-              atomicMax(reinterpret_cast<uint32_t*>(ell_s) + my_g * chunk + lb, float_order_key(ln_n + dm_keep + __logf(1.f + dv_keep)));
+              // (groups of more than eight heads: a window whose mass is NaN counts as empty, as on the general kernels)
+              const float ell = ln_n + dm_keep + __logf(1.f + dv_keep);
+              atomicMax(reinterpret_cast<uint32_t*>(ell_s) + my_g * chunk + lb, float_order_key(GP > 8 ? fmaxf(ell, -INFINITY) : ell));
             }
           }
         }

@@ -658,3 +658,25 @@ def test_scores_that_are_not_numbers_in_groups_of_more_than_eight_heads(G, B, ct
     assert res[1][0][1, 0].isnan().all() and res[1][0][1, 1].isfinite().all() and res[1][0][0].isfinite().all()
     torch.testing.assert_close(res[0][0], res[1][0], rtol=5e-6, atol=1e-9, equal_nan=True)
     assert torch.equal(res[0][1][0], res[1][1][0]) and torch.equal(res[0][1][1, 1], res[1][1][1, 1])
+
+
+@pytest.mark.parametrize("flags", [0, binding.SPLA_STATS_BF16])
+def test_windows_whose_score_is_not_a_number_in_groups_of_more_than_eight_heads(flags):
+    """A window of NaN mass leaves its block the masses of the others and every other block its score; a block of such windows only
+    has the score zero.  Like the general kernels."""
+    w = synth.Workload("case", 35, batch=1, n_q_heads=32, n_kv_heads=2, head_dim=128, block_size=64, top_k=8, context=64 * 30 + 9, n_steps=1)
+    K, V, _ = runner.generate_prefill(w, DEV)
+    K[0, 0, 64 * 4 + 3] = K[0, 0, 64 * 9 + 20] = K[0, 0, 64 * 11 + 63] = float("inf")     # one window, two, one
+    K[0, 1, 64 * 6 + 30] = K[0, 1, 64 * 6 + 33] = float("inf")                            # all three
+    q = synth.step_queries(w, 0, DEV)
+    res = []
+    for f in (0, binding.SPLA_GENERAL_KERNELS):
+        c = binding.SplaCache(runner.config_for(w, flags=flags | f, window=(32, 16)), DEV)
+        c.append_tokens(K, V)
+        sel = c.select(q).clone()
+        res.append((c.scores()[..., :31], sel))
+        torch.cuda.synchronize()
+        assert c.sync_status() == 0
+    assert res[1][0].isfinite().all() and res[1][0][0, 1, 6] == 0 and (res[1][0][0, 0] > 0).all()
+    torch.testing.assert_close(res[0][0], res[1][0], rtol=5e-6, atol=1e-9)
+    assert torch.equal(res[0][1], res[1][1])
