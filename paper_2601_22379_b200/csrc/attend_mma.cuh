@@ -153,39 +153,43 @@ __device__ __forceinline__ void attend_mma_body(const Params& p, const CUtensorM
   uint32_t qa[KS][WIDE ? 4 : 2], fa[KS][WIDE ? 1 : 2];
   auto make_fragments = [&]() {
     if constexpr (WIDE) {
-      const float a2 = p.phi_scale * kLog2e;
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         const int head = g + 8 * j;
         const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + ((size_t)b * p.Hq + (size_t)h * G + (head < G ? head : 0)) * D);
-        float mx = -INFINITY, sum = 0.f;
 #pragma unroll
         for (int kk = 0; kk < KS; ++kk)
 #pragma unroll
-          for (int x = 0; x < 2; ++x) {
-            const uint32_t w = head < G ? __ldg(qrow + 8 * kk + 4 * x + t) : 0u;
-            qa[kk][2 * x + j] = w;
-            mx = fmaxf(mx, fmaxf(bf16_lo(w), bf16_hi(w)));
-          }
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+          for (int x = 0; x < 2; ++x) qa[kk][2 * x + j] = head < G ? __ldg(qrow + 8 * kk + 4 * x + t) : 0u;
+      }
+      // phi(q) by the very sums that o_bar's is formed with (state_role): what rounding it carries then cancels in o_bar - o_tilde
+      // (formed in another order, the residual of queries of four times the usual size was up to 25 % further off)
+      constexpr int VEC = D / 32;
+      const float a2 = p.phi_scale * kLog2e;
+      for (int hd = warp; hd < 16; hd += NWARP) {           // (visible after a barrier below)
+        float x[VEC] = {};
+        if (hd < G && rla_on) {
+          load_vec<VEC>(q + ((size_t)b * p.Hq + (size_t)h * G + hd) * D + lane * VEC, x);
+          float mx = -INFINITY;
 #pragma unroll
-        for (int kk = 0; kk < KS; ++kk)
+          for (int v = 0; v < VEC; ++v) { x[v] *= a2; mx = fmaxf(mx, x[v]); }
+          mx = warp_max(mx);
+          float sum = 0.f;
 #pragma unroll
-          for (int x = 0; x < 2; ++x) sum += exp2f((bf16_lo(qa[kk][2 * x + j]) - mx) * a2) + exp2f((bf16_hi(qa[kk][2 * x + j]) - mx) * a2);
-        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-        sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-        const float inv = (head < G && rla_on) ? kPhiScaleWide / sum : 0.f;
-        if (warp == 0) {                                    // (visible after a barrier below)
+          for (int v = 0; v < VEC; ++v) { x[v] = exp2f(x[v] - mx); sum += x[v]; }
+          sum = warp_sum(sum);
+          const float inv = 1.f / sum;
 #pragma unroll
-          for (int kk = 0; kk < KS; ++kk)
+          for (int v = 0; v < VEC; ++v) x[v] *= inv;
+        }
 #pragma unroll
-            for (int x = 0; x < 2; ++x) {
-              const float f0 = exp2f((bf16_lo(qa[kk][2 * x + j]) - mx) * a2) * inv, f1 = exp2f((bf16_hi(qa[kk][2 * x + j]) - mx) * a2) * inv;
-              const uint32_t hd = pack_f16(f0, f1);
-              fl_s[kk][lane][2 * x + j] = hd;
-              fl_s[kk][lane][4 + 2 * x + j] = pack_f16(f0 - f16_lo(hd), f1 - f16_hi(hd));
-            }
+        for (int v = 0; v < VEC; v += 2) {
+          const int c = lane * VEC + v;                     // channels c, c + 1 of the k-step c / 16
+          const float f0 = x[v] * kPhiScaleWide, f1 = x[v + 1] * kPhiScaleWide;
+          const uint32_t hi = pack_f16(f0, f1);
+          uint32_t* w = &fl_s[c / 16][(hd & 7) * 4 + c % 8 / 2][c % 16 / 8 * 2 + (hd >> 3)];
+          w[0] = hi;
+          w[4] = pack_f16(f0 - f16_lo(hi), f1 - f16_hi(hi));
         }
       }
       return;
