@@ -71,11 +71,11 @@ __device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
   __half2 v = __floats2half2_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
 }
-// Two bf16 values, each the nearest finite one (any, for a NaN).
+// Two bf16 values, each the nearest finite one (any, for a NaN): the smaller magnitude of it and the largest finite value, its sign.
 __device__ __forceinline__ uint32_t finite_bf16(uint32_t x) {
-  const __nv_bfloat162 top = __halves2bfloat162(__ushort_as_bfloat16(0x7f7f), __ushort_as_bfloat16(0x7f7f));
-  const __nv_bfloat162 v = __hmin2(__hmax2(*reinterpret_cast<const __nv_bfloat162*>(&x), __hneg2(top)), top);
-  return *reinterpret_cast<const uint32_t*>(&v);
+  uint32_t y;
+  asm("min.xorsign.abs.bf16x2 %0, %1, %2;" : "=r"(y) : "r"(x), "r"(0x7f7f7f7fu));
+  return y;
 }
 __device__ __forceinline__ float f16_lo(uint32_t x) { return __low2float(*reinterpret_cast<const __half2*>(&x)); }
 __device__ __forceinline__ float f16_hi(uint32_t x) { return __high2float(*reinterpret_cast<const __half2*>(&x)); }
