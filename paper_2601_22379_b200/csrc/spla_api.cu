@@ -344,8 +344,8 @@ static void plan_score_grid(spla_cache* c, Params* p, bool fused = false) {
   p->n_chunks_cap = (int)((blocks * p->NW + p->chunk - 1) / p->chunk);
 }
 
-// The fused decode kernel serves bf16 caches and queries with groups of up to 8 heads (what the tensor-core attend
-// phase is built for) whenever the cluster score plan exists.
+// The fused decode kernel serves bf16 caches and queries with groups of up to 8 heads (larger ones need all registers of the attend
+// phase for accumulators and run it as a kernel of its own) whenever the cluster score plan exists.
 static bool fused_eligible(const spla_cache* c) {
   return !(c->cfg.flags & SPLA_GENERAL_KERNELS) && c->p.kv_bf16 && c->cfg.q_dtype == SPLA_BF16 &&
          c->p.G <= 8 && c->maps.valid && attend_mma_smem_bytes(c->p.tile_rows, c->p.d, 1, c->p.G) + 4096 <= (size_t)113 * 1024;
@@ -356,36 +356,26 @@ static cudaError_t launch_score(const Params& p, const void* q, int qb, int* sel
   return p.cs > 0 ? launch_score_cluster(p, q, qb, sel_user, pending_new, s) : launch_score_select(p, q, qb, sel_user, s);
 }
 
-// Cluster size of the tensor-core attend kernel as a launch of its own, written to p->acs: the largest power of two (at
-// most 16 and at most top_k) for which all CTAs are resident at once; each CTA of a cluster then walks top_k / size
-// selected blocks.
+// Cluster size of the tensor-core attend kernel as a launch of its own, written to p->acs.  A CTA of a cluster walks every size-th
+// tile of the unit's selected blocks.
+//   One wave: the largest power of two (at most 16 and at most top_k) for which all CTAs are resident at once.
+//   More units than places: waves, of which the last may be nearly empty, times a CTA's start, end and share of the tiles, in tokens;
+//   the size with the least, from how many clusters of each size the device holds (fewer the larger they are: 296, 148, 71, 33 and 14
+//   at d = 128).  Over 400 sizes (300 to 900 units, 4 to 16 heads, d = 64 and 128, selections of 6 to 64 blocks of 16 to 128 tokens,
+//   contexts of 900 and 9000) times of a step are 5 to 6 % below clusters of one on average (320 units, G = 4, d = 128, 64 blocks of 128:
+//   485 us in two waves of single CTAs, 341 in clusters of four) and nowhere more than 1 % above; 9 % above the best size at most.
+//   With a CTA's start and end as eight tiles, as measured at three sizes, two places per SM and top_k blocks however short the
+//   sequences, d = 64 was up to 12 % slower than clusters of one.
 static void plan_attend(spla_cache* c, Params* p) {
   p->acs = 0;
   if (c->cfg.flags & SPLA_GENERAL_KERNELS) return;
   const long long U = (long long)c->p.batch * c->p.Hkv;
   const size_t smem = attend_mma_smem_bytes(c->p.tile_rows, c->p.d, 1, c->p.G) + 2048;
   long long per_sm = (227 * 1024) / (long long)smem;
-  if (per_sm > 2) per_sm = 2;                     // the kernel is compiled for two CTAs per SM (no register spills)
+  if (per_sm > 2) per_sm = 2;                     // (a third fits at d = 64: one wave of fewer, longer CTAs is no slower)
   if (per_sm < 1) return;                         // the tiles do not fit: use the general kernel
   const long long slots = per_sm * c->sm_count;
-  int cs = 1;
-  while (cs * 2 <= 16 && cs * 2 <= c->p.top_k && U * cs * 2 <= slots) cs *= 2;
-  // More units than places: several waves, of which the last may be nearly empty.  Waves times (a CTA's start and end, about 8 tiles'
-  // time, and its tiles): 320 units of 64 picks of 128 tokens, 128 tiles, in clusters of one (two waves, 24 CTAs in the second) 429 us
-  // a step, of four (five waves) 359; 320 units of 64 picks of 64: 290, 239.  512 units of 16 tiles stay at one (184 us; clusters of
-  // two and four 9 and 32 us longer).
-  if (U > slots) {
-    const long long tiles = (long long)c->p.top_k * (c->p.B / c->p.tile_rows);
-    long long best = 0;
-    for (int x = 1; x <= 16 && x <= c->p.top_k; x *= 2) {
-      const long long cost = (U * x + slots - 1) / slots * (8 + (tiles + x - 1) / x);
-      if (x == 1 || cost < best) { best = cost; cs = x; }
-    }
-    p->acs = cs;
-    return;
-  }
-  // all clusters of the launch must be resident together (see plan_score_clusters): ask the device
-  for (; cs > 1; cs /= 2) {
+  auto resident = [&](int cs) {                   // clusters of that size resident at once; -1 if unknown
     int lg = 0;
     while ((1 << lg) < cs) ++lg;
     if (c->attend_occ[lg] == -2) {
@@ -393,7 +383,27 @@ static void plan_attend(spla_cache* c, Params* p) {
       probe.acs = cs;
       c->attend_occ[lg] = attend_mma_max_clusters(probe);
     }
-    if (c->attend_occ[lg] < 0 || U <= c->attend_occ[lg]) break;
+    return c->attend_occ[lg];
+  };
+  int cs = 1;
+  if (U > slots) {
+    const long long blocks = (c->len_bound + c->p.B - 1) / c->p.B;
+    const long long tiles = (c->p.top_k < blocks ? c->p.top_k : blocks) * (c->p.B / c->p.tile_rows);
+    constexpr long long kEnds = 5 * 64;           // start and end of a CTA, in tokens
+    long long best = 0;
+    for (int x = 1; x <= 16 && x <= c->p.top_k && (x == 1 || x <= tiles); x *= 2) {
+      const int n = resident(x);
+      if (n <= 0 && x > 1) continue;
+      const long long places = n > 0 ? n : slots;
+      const long long cost = (U + places - 1) / places * (kEnds + (tiles + x - 1) / x * c->p.tile_rows);
+      if (x == 1 || cost < best) { best = cost; cs = x; }
+    }
+  } else {
+    while (cs * 2 <= 16 && cs * 2 <= c->p.top_k && U * cs * 2 <= slots) cs *= 2;
+    for (; cs > 1; cs /= 2) {                     // all clusters of the launch must be resident together (see plan_score_clusters)
+      const int n = resident(cs);
+      if (n < 0 || U <= n) break;
+    }
   }
   p->acs = cs;
 }

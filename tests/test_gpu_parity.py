@@ -727,3 +727,27 @@ def test_groups_of_more_than_eight_heads_are_no_less_exact_than_the_general_kern
         errs.append([_errors_against_64_bits(w, f, scale) for f in (0, binding.SPLA_GENERAL_KERNELS)])
     for name, new, old in zip(("scores", "o_sparse", "o_rla"), *np.mean(errs, axis=0)):
         assert new <= 1.1 * old, (name, new, old)
+
+
+@pytest.mark.parametrize("G,d,B,k,ctx", [
+    (4, 128, 16, 64, 16 * 80 + 3),       # clusters of two
+    (4, 128, 64, 64, 64 * 70),           # of four, every CTA 16 tiles
+    (8, 64, 128, 32, 128 * 40 + 5),      # of four, 32 blocks of one tile
+    (16, 128, 32, 16, 32 * 30 + 31),
+    (4, 128, 64, 64, 64 * 6 + 1),        # short sequences: fewer blocks than picks, clusters of one
+])
+def test_attention_in_several_waves_of_clusters(G, d, B, k, ctx):
+    """320 units of 16 to 64 picks take the attend kernel in several waves of clusters; like the general kernels, over one selection."""
+    w = synth.Workload("case", 41, batch=80, n_q_heads=4 * G, n_kv_heads=4, head_dim=d, block_size=B, top_k=k, context=ctx, n_steps=1)
+    K, V, _ = runner.generate_prefill(w, DEV)
+    q, gamma = synth.step_queries(w, 0, DEV), synth.gamma(w).to(DEV)
+    caches = [binding.SplaCache(runner.config_for(w, flags=f), DEV) for f in (0, binding.SPLA_GENERAL_KERNELS)]
+    for c in caches:
+        c.append_tokens(K, V)
+    caches[1].bufs.rla_state.copy_(caches[0].bufs.rla_state)
+    sel = caches[0].new_sel_buffer()
+    out = caches[0].decode(q, gamma, sel_idx=sel)
+    want = caches[1].decode_selected(q, gamma, sel)
+    torch.cuda.synchronize()
+    assert [c.sync_status() for c in caches] == [0, 0]
+    parity.check_outputs("out", out.cpu().numpy(), want.cpu().numpy(), w.kv_dtype)
