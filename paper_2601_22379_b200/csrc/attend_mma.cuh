@@ -166,26 +166,37 @@ __device__ __forceinline__ void attend_mma_body(const Params& p, const CUtensorM
       // (formed in another order, the residual of queries of four times the usual size was up to 25 % further off)
       constexpr int VEC = D / 32;
       const float a2 = p.phi_scale * kLog2e;
-      for (int hd = warp; hd < 16; hd += NWARP) {           // (visible after a barrier below)
-        float x[VEC] = {};
-        if (hd < G && rla_on) {
-          load_vec<VEC>(q + ((size_t)b * p.Hq + (size_t)h * G + hd) * D + lane * VEC, x);
-          float mx = -INFINITY;
+      constexpr int HW = 16 / NWARP;                        // heads per warp, side by side
+      float x[HW][VEC], mx[HW], sum[HW];
 #pragma unroll
-          for (int v = 0; v < VEC; ++v) { x[v] *= a2; mx = fmaxf(mx, x[v]); }
-          mx = warp_max(mx);
-          float sum = 0.f;
+      for (int i = 0; i < HW; ++i) {
+        const int hd = warp + i * NWARP;
 #pragma unroll
-          for (int v = 0; v < VEC; ++v) { x[v] = exp2f(x[v] - mx); sum += x[v]; }
-          sum = warp_sum(sum);
-          const float inv = 1.f / sum;
+        for (int v = 0; v < VEC; ++v) x[i][v] = 0.f;
+        if (hd < G) load_vec<VEC>(q + ((size_t)b * p.Hq + (size_t)h * G + hd) * D + lane * VEC, x[i]);
+      }
 #pragma unroll
-          for (int v = 0; v < VEC; ++v) x[v] *= inv;
-        }
+      for (int i = 0; i < HW; ++i) {
+        mx[i] = -INFINITY;
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) { x[i][v] *= a2; mx[i] = fmaxf(mx[i], x[i][v]); }
+        mx[i] = warp_max(mx[i]);
+      }
+#pragma unroll
+      for (int i = 0; i < HW; ++i) {
+        sum[i] = 0.f;
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) { x[i][v] = exp2f(x[i][v] - mx[i]); sum[i] += x[i][v]; }
+        sum[i] = warp_sum(sum[i]);
+      }
+#pragma unroll
+      for (int i = 0; i < HW; ++i) {                        // (visible after a barrier below)
+        const int hd = warp + i * NWARP;
+        const float inv = hd < G && rla_on ? 1.f / sum[i] : 0.f;
 #pragma unroll
         for (int v = 0; v < VEC; v += 2) {
           const int c = lane * VEC + v;                     // channels c, c + 1 of the k-step c / 16
-          const float f0 = x[v] * kPhiScaleWide, f1 = x[v + 1] * kPhiScaleWide;
+          const float f0 = x[i][v] * inv * kPhiScaleWide, f1 = x[i][v + 1] * inv * kPhiScaleWide;
           const uint32_t hi = pack_f16(f0, f1);
           uint32_t* w = &fl_s[c / 16][(hd & 7) * 4 + c % 8 / 2][c % 16 / 8 * 2 + (hd >> 3)];
           w[0] = hi;
