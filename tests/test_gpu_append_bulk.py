@@ -157,8 +157,10 @@ def test_state_below_256_tokens_is_no_less_exact_than_the_fp32_kernels(n, times,
     ("f32", 64, 1, 1, [33, 255, 257], False),       # one share, the last token of it, two; 16 rows per CTA
     ("f32", 64, 2, 2, [256 * 74 + 31], False),      # as many shares as the workspace holds, ragged at their end
     ("bf16", 64, 2, 2, [40, 700], True),            # shares sized by the longest: some of a short sequence are empty
-    ("f32", 128, 3, 20, [300, 770], True),          # all rows per CTA, two and four shares
-    ("bf16", 64, 40, 4, [513], False),              # ... and one share, more units than SMs
+    ("f32", 128, 3, 20, [300, 770], True),          # two shares, 16 rows per CTA; four, all rows
+    ("bf16", 64, 40, 4, [513], False),              # all rows and one share, more units than SMs
+    ("f32", 128, 38, 4, [255, 40], False),          # ... d = 128, twice onto the state in place
+    ("bf16", 128, 75, 4, [33, 47], True),           # a few tokens of many sequences of different lengths
 ])
 def test_state_of_the_three_kernel_append(dtype, d, batch, hkv, sizes, ragged):
     """S_bar against 64 bits at the edges of staged tokens and of shares; the tolerance of fp32 sums."""
