@@ -165,8 +165,8 @@ def test_noalloc_entry_rejects_bf16_statistics():
 
 @pytest.mark.parametrize("hq,hkv", [(1, 1), (2, 1), (3, 1), (5, 1), (8, 1), (16, 1), (6, 2)])
 def test_bf16_statistics_group_sizes(hq, hkv):
-    """Groups of 1-4 heads take the tensor-core score path (unused B columns are zero), 5-8 the FMA path of the
-    cluster kernel, 16 the general kernel."""
+    """Groups of 1-4 heads take one column tile of the tensor-core scores (unused B columns are zero), 5-8 two, 16 the FMA path of the
+    cluster kernel in two teams of warps."""
     w = synth.BY_NAME["gqa_32k"].scaled(batch=1, n_q_heads=hq, n_kv_heads=hkv, context=64 * 40 + 3, n_needles=3)
     cache, K, V, lens = runner.build_cache(w, DEV, flags=F16)
     gamma = synth.gamma(w).to(DEV)
@@ -218,3 +218,25 @@ def test_bf16_statistics_steps_across_block_boundaries_every_unit():
             parity.compare_unit(w, run(), out[b].cpu().numpy(), osp[b].cpu().numpy(), orla[b].cpu().numpy(),
                                 sel[b, h].cpu().numpy(), h, n_sink=w.n_sink, n_local=w.n_local, rerun=run,
                                 tie_band=parity.TIE_BAND_STATS_BF16)
+
+
+@pytest.mark.parametrize("hq,batch,blocks", [(64, 6, 200), (40, 6, 203), (64, 1, 1500), (32, 2, 3)])
+def test_partial_results_that_arrive_over_the_table_of_log_masses(hq, batch, blocks):
+    """With 16-bit records the fused kernel receives the siblings' partial results of the attention where the scores' log masses were.
+    The scores formed from that table and the outputs are those of the two kernels on their own, over steps (the outputs to the 8 bits
+    of the probabilities, which meet another running maximum there: 2^-9 each, and their mean over many)."""
+    w = synth.Workload("case", 51, batch=batch, n_q_heads=hq, n_kv_heads=8, head_dim=128, block_size=64, top_k=16, context=64 * blocks - 2,
+                       n_steps=4)
+    cache, _, _, _ = runner.build_cache(w, DEV, flags=F16)
+    gamma = synth.gamma(w).to(DEV)
+    for step in range(w.n_steps):
+        k1, v1 = synth.step_kv(w, step, DEV)
+        q = synth.step_queries(w, step, DEV)
+        sel = cache.new_sel_buffer()
+        out = cache.append_decode(k1, v1, q, gamma, sel_idx=sel)
+        nblk = (64 * blocks - 2 + step + 64) // 64
+        scores = cache.scores()[..., :nblk]
+        sel2 = cache.select(q)                              # the score kernel as a launch of its own, then the attention
+        torch.testing.assert_close(scores, cache.scores()[..., :nblk], rtol=2e-6, atol=1e-10)
+        assert parity.rel_l2(out.cpu().numpy(), cache.decode_selected(q, gamma, sel).cpu().numpy()) < 2 ** -9
+        assert (sel == sel2).all(-1).float().mean() > 0.95 and cache.sync_status() == 0
