@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(kStatThreads) append_block_kernel(const Params
     __syncthreads();                                 // the next window reuses the reduction buffers
   }
   // Only now: the small CTAs of the state kernel, started earlier, crowd onto the SMs that have room first (bf16, d = 64, 255 tokens
-  // x 32 units: 57 us a call against 33).
+  // x 32 units: 57 us a call against 21; 600 tokens x 400 units 138 against 100).
   pdl_launch_dependents();
 }
 
@@ -489,9 +489,11 @@ static cudaError_t launch_typed(const Params& p, const void* k_new, const void* 
                      p, kn, vn, n_new, max_new, n_copy, n_stats);
   }
   // bf16 with d = 128: everything in one pass, the state on the tensor cores; the rest in three kernels.  Among those a few tokens
-  // of many sequences of different lengths: the pass takes a CTA per unit and SM whatever a unit adds, 0.2 us per unit, the
-  // kernels take less the less there is (1 to 33, 40, 48, 64 tokens, 512 units: 42, 50, 58, 60 us against 59 to 61; 1024 units 71,
-  // 83, 89, 99 against 104; 256 units 32 to 42 against 33 to 35; all at the longest: 65, 69, 75, 93 against 64).
+  // of many sequences of different lengths: the pass takes a CTA per unit and SM whatever a unit adds, 0.1 us per unit, the
+  // kernels take less the less there is (1 to 33, 40 tokens, 512 units: 26, 28 us against 53; 1024 units 44, 47 against 96; 304 units
+  // 21, 21 against 39; all at the longest, 512 units: 33, 35 against 55).  The line was drawn where an earlier state kernel fell
+  // behind; with this one the kernels stay ahead further on, up to about 80 tokens and below 296 units too (1 to 48, 64, 80, 128
+  // tokens, 512 units: 31, 33, 41, 57 us against 53, 53, 54, 58; 296 units 22, 23, 30, 41 against 30, 30, 30, 35).
   const bool few_of_many = n_new && U > 2 * 148 && max_new < 48;
   if (sizeof(T) == 2 && D == 128 && maps && maps->valid && fresh_maps && fresh_maps->valid && !few_of_many)
     return launch_append_bulk(p, *maps, *fresh_maps, n_new, max_new, stream);

@@ -17,7 +17,8 @@
 // difference (Section 3.2, "Numerical Stability": the states stay in high precision): phi(q) and phi(k) enter
 // their product as an fp16 head plus an fp16 remainder each, and the coefficients phi(q).phi(k_t) enter the
 // product with V as three bf16 parts.  For groups of up to 4 heads the
-// extra parts ride in the accumulator rows that would otherwise be padding.
+// extra parts ride in the accumulator rows that would otherwise be padding; groups of 5 to 8 heads take more products; groups
+// of 9 to 16 fill all 16 rows of a product with heads, so that S and A, P V and o_tilde are products and accumulators of their own.
 //
 // Merge (Eq. rla-impl-3, Section 3.3): every CTA sends its partial results of head g into CTA g % CS of the cluster as
 // asynchronous stores (st.async) that count their bytes on a barrier there; that CTA goes on when all of them have
@@ -80,7 +81,10 @@ __device__ __forceinline__ uint32_t finite_bf16(uint32_t x) {
 __device__ __forceinline__ float f16_lo(uint32_t x) { return __low2float(*reinterpret_cast<const __half2*>(&x)); }
 __device__ __forceinline__ float f16_hi(uint32_t x) { return __high2float(*reinterpret_cast<const __half2*>(&x)); }
 
-constexpr float kPhiScaleWide = 16384.f;   // groups of more than eight heads: phi times 2^14 (at most 2^14 then) keeps both fp16 parts clear of the subnormals
+// Groups of more than eight heads: phi times 2^14 (at most 2^14 then) has 22 bits in its two fp16 parts from 2^-17 up; below, the
+// remainder is subnormal and the error 2^-39.  (The remainder times another 2^11, 22 bits down to 2^-28: no error against 64 bits
+// changed by a hundredth, outlier channels and queries of eight times the usual size included, and steps took 3 % longer.)
+constexpr float kPhiScaleWide = 16384.f;
 constexpr int kPad = 8;   // floats of padding per row of the cross-warp reduction buffer
 
 // Bytes of the tile ring (reused for the cross-warp fold); as a kernel of its own the receive area of the merge follows.
@@ -99,8 +103,9 @@ constexpr size_t attend_mma_recv_bytes(int D) { return (size_t)16 * (2 * D + 2) 
 // the bf16 remainder of the linear coefficients and no extra products are needed for it.
 // WIDE: the group has more than 8 heads: S and A take all 16 rows of a product of their own, and the probabilities keep 24 bits
 // like the linear coefficients (three bf16 parts; every slice's sums start at zero and are added in fp32), as on the general
-// kernel, which served such groups before: 8 units of 64 blocks, G = 16, 95 us there, a step of 7450 blocks with it and the cluster
-// score kernel 367 -> 165.  Two CTAs per SM with all 255 registers: two accumulators of 16 rows take 128 of them.
+// kernel, which served such groups before: with it and the cluster scores a step of 8 units of 7450 blocks, 64 picks, G = 16 takes
+// 162 us instead of 365.  Two CTAs per SM with all 255 registers: two accumulators of 16 rows take 128 of them.  (Without the residual
+// the linear products are formed and dropped.)
 template <int D, bool PACK, int NG, bool FUSED, bool WIDE = false>
 __device__ __forceinline__ void attend_mma_body(const Params& p, const CUtensorMap& map_k, const CUtensorMap& map_v,
                                                 const __nv_bfloat16* __restrict__ q, const float* __restrict__ rms_weight,

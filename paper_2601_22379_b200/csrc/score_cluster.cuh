@@ -106,7 +106,7 @@ struct Smem {
   // Behind it, or where the ring is no longer than that area anyway (16-bit records) over the table of log masses, the attend
   // phase's receive area (fused kernel): a sibling stores there once it has attended, so after this CTA's keys, formed from that
   // table, have reached it.  (G = 8, 48 units of 1580 blocks: one CTA per SM in clusters of three became two in clusters of six,
-  // 98 -> 49 us a step.)
+  // 98 -> 47 us a step.)
   static constexpr bool kRecvOverEll = kStreamBytes <= kAreaEnd || GP > 8;   // (groups of more than eight heads never run fused)
   static constexpr int kMergeRecvBytes = (16 * (2 * D + 2) * 4 + 1023) / 1024 * 1024;
   static constexpr int kRecvInRing = kRecvOverEll ? kAreaEnd : kAreaEnd + kMergeRecvBytes;
@@ -173,8 +173,10 @@ __device__ __forceinline__ void score_cluster_body(const Params& p, const void* 
                                                    int* sel_share = nullptr, float* obar_local = nullptr) {
   using SM = Smem<D, GP, ST, NWP>;
   // Groups of more than eight heads are dealt out to two teams of warps, eight heads each (that many queries fit a warp's
-  // registers); a team takes every record of a stage.  (8 units of 13000 blocks, G = 16: scores and selection 458 us on the general
-  // kernel, the whole step 225 now; bound by FMAs and the halving sums, 220 instructions per record and team pair.)
+  // registers); a team takes every record of a stage, also at G = 9, where the second has one head.  (8 units of 13000 blocks, G = 16: a
+  // step 500 us with the general kernels, 227 now; 64 units of 938 blocks, G = 9, 12, 16: 285, 302, 331 -> 95, 96, 101; no size of
+  // 9 to 16 heads tried, 1 to 320 units of 1000 to 800000 tokens, was faster on the general kernels.  Bound by FMAs and the halving
+  // sums, 220 instructions per record and team pair.)
   constexpr int GT = GP > 8 ? 8 : GP;           // heads of a team, padded
   constexpr int TEAMS = GP / GT;
   constexpr int kCsConsumers = NWP;             // warps; all consume, lane 0 of warp 0 also feeds the ring
