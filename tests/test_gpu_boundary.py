@@ -17,12 +17,13 @@ def _small(name="gqa_32k", **over):
     return synth.BY_NAME[name].scaled(**kw)
 
 
-@pytest.mark.parametrize("flags", [0, binding.SPLA_GENERAL_KERNELS])
-def test_a_wait_that_runs_out_is_reported_as_timeout_and_the_context_stays_usable(flags):
+@pytest.mark.parametrize("flags,group", [(0, 4), (0, 16), (binding.SPLA_GENERAL_KERNELS, 4)])
+def test_a_wait_that_runs_out_is_reported_as_timeout_and_the_context_stays_usable(flags, group):
     """The copy barriers of the decode kernels are told to expect 16 bytes more than will ever arrive and to give up
     after a few thousand polls: every wait runs out, the kernels skip their arithmetic, return, and latch
     SPLA_ERR_TIMEOUT.  With the hook cleared the same cache decodes correctly again."""
     w = _small()
+    w = w.scaled(n_q_heads=w.n_kv_heads * group)
     cache, K, V, lens = runner.build_cache(w, DEV, flags=flags)
     gamma = synth.gamma(w).to(DEV)
     q = synth.step_queries(w, 0, DEV)
@@ -73,11 +74,12 @@ def test_invalid_entries_of_a_given_selection_are_dropped_and_reported(flags):
     assert cache.sync_status() == 0 and torch.isfinite(out_none).all()
 
 
-@pytest.mark.parametrize("flags", [0, binding.SPLA_GENERAL_KERNELS])
-def test_a_corrupt_length_is_clamped_and_reported(flags):
+@pytest.mark.parametrize("flags,group", [(0, 4), (0, 16), (binding.SPLA_GENERAL_KERNELS, 4)])
+def test_a_corrupt_length_is_clamped_and_reported(flags, group):
     """seq_lens belongs to the caller.  A value above max_context (or below zero) is clamped by every decode kernel
     and reported; nothing is read outside the buffers, and the other sequence decodes as before."""
     w = _small()
+    w = w.scaled(n_q_heads=w.n_kv_heads * group)
     cache, K, V, lens = runner.build_cache(w, DEV, flags=flags)
     gamma = synth.gamma(w).to(DEV)
     q = synth.step_queries(w, 0, DEV)
